@@ -513,21 +513,16 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
     const int ntx = (L.nx + e.bx - 1) / e.bx;
     const int nty = (L.ny + e.by - 1) / e.by;
     const int64_t cols = (int64_t)ntx * nty * nshots;
-    const int64_t slots = (int64_t)nsm * per_sm;
-    // Split z only when the columns alone cannot fill the machine; keep every
-    // chunk long enough that the 2R-plane warm-up stays a small fraction.
-    // The narrow stencils (R <= 2) run at the HBM limit once three quarters
-    // of the slots are busy, so there a split only adds warm-up planes
-    // (512^3, so 4: 413 GPts/s unsplit, 396 in two chunks); the wider ones
-    // are limited per SM and gain from the finer units (so 8: 381 in two
-    // chunks, 357 unsplit).
+    // 2R warm-up planes, slightly cheaper than output planes; the load of a
+    // CTA as fitted per radius: 0.63 for 64 x 16 tiles at so 4, 0.25 and 0.30
+    // for 64 x 8 at so 8 and 12, 0.20 for 64 x 4 at so 16.
     int nzc = 1;
-    if (cols < slots && !(radius <= 2 && 4 * cols >= 3 * slots)) {
-        nzc = (int)((slots + cols - 1) / cols);
-        const int min_chunk = 8 * radius > 32 ? 8 * radius : 32;
-        const int max_nzc = L.nz / min_chunk > 1 ? L.nz / min_chunk : 1;
-        if (nzc > max_nzc) nzc = max_nzc;
-    }
+    if (L.nz > 1)
+        nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, 0.9 * 2 * radius,
+                            e.bx * e.by / (radius >= 8 ? 1280.0 : 1800.0));
+    const int min_nzc = (L.nz + 8191) / 8192;  // damp_z of a chunk: at most 32 KB
+    if (nzc < min_nzc) nzc = min_nzc;
+    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
     const int zchunk = (L.nz + nzc - 1) / nzc;
     nzc = (L.nz + zchunk - 1) / zchunk;
     if ((int64_t)nshots * nzc > 65535 || nty > 65535)

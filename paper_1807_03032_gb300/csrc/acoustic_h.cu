@@ -491,15 +491,13 @@ fd_status acoustic_h_plan(int radius, int config, const WaveLayout &L, int nshot
     const int ntx = (L.nx + e.bx - 1) / e.bx;
     const int nty = (L.ny + e.by - 1) / e.by;
     const int64_t cols = (int64_t)ntx * nty * nshots;
-    const int64_t slots = (int64_t)nsm * per_sm;
-    // split z only when the columns alone cannot fill the machine (as K1)
-    int nzc = 1;
-    if (cols < slots) {
-        nzc = (int)((slots + cols - 1) / cols);
-        const int min_chunk = 8 * radius > 32 ? 8 * radius : 32;
-        const int max_nzc = L.nz / min_chunk > 1 ? L.nz / min_chunk : 1;
-        if (nzc > max_nzc) nzc = max_nzc;
-    }
+    // the conversions make a plane of the wide stencils twice as dear per
+    // point (fitted: load 0.38 / 0.48 / 0.40 / 0.51 of the default tiles)
+    int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, (radius <= 4 ? 0.5 : 0.7) * 2 * radius,
+                            e.bx * e.by / (radius <= 4 ? 2400.0 : 1150.0));
+    const int min_nzc = (L.nz + 8191) / 8192;  // damp_z of a chunk: at most 32 KB
+    if (nzc < min_nzc) nzc = min_nzc;
+    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
     const int zchunk = (L.nz + nzc - 1) / nzc;
     nzc = (L.nz + zchunk - 1) / zchunk;
     if ((int64_t)nshots * nzc > 65535 || nty > 65535)

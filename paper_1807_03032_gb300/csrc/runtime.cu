@@ -3,6 +3,7 @@
 // driver entry point (no link-time dependency on libcuda), pointer
 // classification and the stream-ordered workspace.
 #include <cudaTypedefs.h>
+#include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -203,6 +204,37 @@ fd_status raise_smem_limit(const void *fn, size_t bytes) {
         cur = bytes;
     }
     return FD_OK;
+}
+
+int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load) {
+    const int64_t slots = (int64_t)nsm * per_sm;
+    // beyond a few waves more chunks only add warm-up planes
+    const int64_t most = 8 * slots / (cols > 0 ? cols : 1) + 8;
+    auto h = [&](double k) { return sqrt(1.0 + load * load * k * k); };
+    int best = 1;
+    double best_cost = 0.0;
+    int last_chunk = 0;
+    for (int n = 1; n <= nz && n <= most; ++n) {
+        const int chunk = (nz + n - 1) / n;
+        if (chunk == last_chunk) continue;
+        last_chunk = chunk;
+        const int64_t units = cols * ((nz + chunk - 1) / chunk);
+        const int64_t full = units / slots, rem = units - full * slots;
+        double waves = (double)full * h(per_sm);
+        if (rem) {
+            // the last wave: between the mean and the fullest SM's load
+            double k = (double)rem / nsm;
+            if (k < 1.0) k = 1.0;
+            waves += h(0.5 * (k + ceil(k)));
+        }
+        double cost = (chunk + warmup) * waves;
+        if (n == 1) cost *= 1.06;  // measured 3 - 6 % above the estimate
+        if (n == 1 || cost < best_cost) {
+            best_cost = cost;
+            best = n;
+        }
+    }
+    return best;
 }
 
 bool is_device_pointer(const void *p) {

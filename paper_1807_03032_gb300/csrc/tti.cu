@@ -535,26 +535,6 @@ bool tti_info(int radius, int stag, int config, TtiInfo *out) {
 
 }  // namespace
 
-// Number of z chunks per column for the TTI kernels.  Split z when the
-// columns alone cannot fill the machine (chunks of at least min_chunk
-// planes), and also cut the columns into chunks of at least 128 planes until
-// there are about six units per slot: both TTI schemes hold two CTAs per SM
-// and are limited per SM, so finer units balance the SMs' work (512^3, 512
-// columns on 304 slots: four chunks run so 4 / 8 / 12 / 16 at 76.0 / 61.8 /
-// 58.5 / 48.6 GPts/s against 67.8 / 59.1 / 53.3 / 44.7 unsplit).
-int tti_z_chunks(int64_t cols, int64_t slots, int nz, int min_chunk) {
-    int nzc = 1;
-    if (cols < slots) {
-        nzc = (int)((slots + cols - 1) / cols);
-        const int max_nzc = nz / min_chunk > 1 ? nz / min_chunk : 1;
-        if (nzc > max_nzc) nzc = max_nzc;
-    }
-    int64_t bal = (6 * slots + cols - 1) / cols;
-    const int max_bal = nz / 128 > 1 ? nz / 128 : 1;
-    if (bal > max_bal) bal = max_bal;
-    return nzc > bal ? nzc : (int)bal;
-}
-
 int tti_num_configs(int radius) {
     TtiInfo in;
     return tti_info(radius, 0, 0, &in) ? kTtiConfigs : 0;
@@ -586,8 +566,12 @@ fd_status tti_plan(int radius, const WaveLayout &L, int nshots, float *wave, flo
     FD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, in.p2, in.threads, in.smem2));
     if (per_sm < 1) return set_error(FD_ERR_CUDA, "TTI pass-2 kernel does not fit on an SM");
     const int ntx = (L.nx + in.bx - 1) / in.bx, nty = (L.ny + in.by - 1) / in.by;
-    const int64_t cols = (int64_t)ntx * nty * nshots, slots = (int64_t)nsm * per_sm;
-    int nzc = tti_z_chunks(cols, slots, L.nz, 8 * radius > 32 ? 8 * radius : 32);
+    const int64_t cols = (int64_t)ntx * nty * nshots;
+    // both passes together; their 2R warm-up planes only feed the z pipeline
+    // (fitted: 0.2 .. 0.44 of a plane each; load 0.64 .. 0.69 of 64 x 8
+    // tiles, 0.31 of 64 x 4)
+    int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, 0.35 * 2 * radius, in.bx * in.by / 800.0);
+    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
     const int zchunk = (L.nz + nzc - 1) / nzc;
     nzc = (L.nz + zchunk - 1) / zchunk;
     if ((int64_t)nshots * nzc > 65535 || nty > 65535)

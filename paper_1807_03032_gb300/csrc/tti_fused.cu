@@ -392,8 +392,10 @@ fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, 
     if (per_sm < 1) return set_error(FD_ERR_CUDA, "fused TTI kernel does not fit on an SM");
     const int bx = 64, by = in.by;
     const int ntx = (L.nx + bx - 1) / bx, nty = (L.ny + by - 1) / by;
-    const int64_t cols = (int64_t)ntx * nty * nshots, slots = (int64_t)nsm * per_sm;
-    int nzc = tti_z_chunks(cols, slots, L.nz, 16 * radius > 32 ? 16 * radius : 32);
+    const int64_t cols = (int64_t)ntx * nty * nshots;
+    // 4R warm-up planes, the first half of which only feed the z pipeline
+    int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, 0.55 * 4 * radius, bx * by / 950.0);
+    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
     const int zchunk = (L.nz + nzc - 1) / nzc;
     nzc = (L.nz + zchunk - 1) / zchunk;
     if ((int64_t)nshots * nzc > 65535 || nty > 65535)

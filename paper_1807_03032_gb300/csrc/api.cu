@@ -515,7 +515,6 @@ static fd_status acoustic_forward_impl(const fd_grid *grid, int so, double dt, i
     FD_STAGE(s, "acoustic: inputs staged");
 
     // ---- K0: coefficients, tables, validation
-    FD_CUDA_TRY(cudaMemsetAsync(bcoef, 0, (damp_field ? 2 : 1) * (size_t)L.vol * 4, s));
     FD_TRY(init_medium_stats(dstats, s));
     FD_TRY(setup_acoustic_coeffs(sm.dev, sdamp.dev, dt, L, bcoef, dps, dstats, s, damp_field));
     FD_STAGE(s, "acoustic: coefficients");
@@ -829,7 +828,6 @@ static fd_status acoustic_forward_h_impl(const fd_grid *grid, int so, double dt,
     FD_STAGE(s, "acoustic f16: inputs staged");
 
     // ---- K0: coefficients (FP64 -> FP32 as in the FP32 path, then binary16)
-    FD_CUDA_TRY(cudaMemsetAsync(b32, 0, (size_t)L.vol * 4, s));
     FD_CUDA_TRY(cudaMemsetAsync(bh, 0, (size_t)LH.vol * 2, s));
     FD_TRY(init_medium_stats(dstats, s));
     FD_TRY(setup_acoustic_coeffs(sm.dev, sdamp.dev, dt, L, b32, dps, dstats, s));
@@ -1036,7 +1034,6 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
     for (Staged *st : {&sm, &sdamp, &seps, &sdel, &sth, &sph, &ssxyz, &swav, &srxyz})
         FD_TRY(st->place(s));
 
-    FD_CUDA_TRY(cudaMemsetAsync(bcoef, 0, (size_t)6 * L.vol * 4, s));
     FD_TRY(init_medium_stats(dstats, s));
     FD_TRY(setup_acoustic_coeffs(sm.dev, sdamp.dev, dt, L, bcoef, dps, dstats, s));
     FD_TRY(setup_tti_coeffs(seps.dev, sdel.dev, sth.dev, sph.dev, L, acoef, scoef, nvec, dstats,
@@ -1214,7 +1211,6 @@ static fd_status acoustic_common_setup(const fd_grid *grid, int so, double dt, c
                                        SparsePoint *rec_tab, MediumStats *dstats,
                                        const char *what, cudaStream_t s) {
     const WaveLayout &L = gd.L;
-    FD_CUDA_TRY(cudaMemsetAsync(bcoef, 0, (size_t)L.vol * 4, s));
     FD_TRY(init_medium_stats(dstats, s));
     FD_TRY(setup_acoustic_coeffs(m, damp, dt, L, bcoef, dps, dstats, s));
     for (int sh = 0; sh < nshots; ++sh) {

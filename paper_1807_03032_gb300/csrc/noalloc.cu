@@ -139,9 +139,8 @@ fd_status noalloc_impl(const fd_grid *g, int so, double dt, int nt, int nshots, 
     MediumStats *dstats = c.take<MediumStats>(1);
     const size_t dense = (size_t)L.nx * L.ny * L.nz;
 
-    // setup: the scratch keeps the previous call's data, so zero what the
-    // kernels expect to start at zero (b padding, wavefields)
-    FD_CUDA_TRY(cudaMemsetAsync(bcoef, 0, (size_t)L.vol * 4, s));
+    // setup: the scratch keeps the previous call's data; the coefficient
+    // kernel writes all of b, and the wavefields are cleared below
     FD_TRY(init_medium_stats(dstats, s));
     FD_TRY(setup_acoustic_coeffs(m, damp, dt, L, bcoef, dps, dstats, s));
     for (int sh = 0; sh < nshots; ++sh) {

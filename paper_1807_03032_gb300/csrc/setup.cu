@@ -8,7 +8,8 @@
 //    update); damping profiles scaled by 1/dt.
 //  * TTI: a = 1 + 2 eps, s = sqrt(1 + 2 delta) and the symmetry axis
 //    n = (sin theta cos phi, sin theta sin phi, cos theta), precomputed once
-//    because they do not change with time.
+//    because they do not change with time; rounded once to FP32, formed in
+//    two-float arithmetic too.
 //  * Sparse tables: the trilinear corner and fractional offsets of every
 //    source and receiver, x1 = floor((x - o)/h) in FP64, clamped to n - 2.
 //  * Reductions for validation: min/max of m (stability bound), max eps,
@@ -84,54 +85,152 @@ __device__ __forceinline__ TwoFloat two_sum(float a, float b) {
     return TwoFloat{s, e};
 }
 
+__device__ __forceinline__ TwoFloat quick_two_sum(float a, float b) {  // |a| >= |b| or a = 0
+    const float s = __fadd_rn(a, b);
+    return TwoFloat{s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+__device__ __forceinline__ TwoFloat tf_mul(TwoFloat a, TwoFloat b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = fmaf(a.hi, b.hi, -p);
+    e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
+    return quick_two_sum(p, e);
+}
+
+__device__ __forceinline__ TwoFloat tf_add(TwoFloat a, TwoFloat b) {
+    const TwoFloat s = two_sum(a.hi, b.hi);
+    return quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+
+// sin x and cos x as two-floats for |x| <= kSincosRange, to about 2^-36 of
+// their size: x - k pi/2 with pi/2 as three floats and exact products (Cody
+// and Waite's reduction), then the Taylor series on [-pi/4, pi/4], the last
+// terms in plain FP32 and the leading ones in two-float arithmetic.  Against
+// 80-bit references over 2e7 angle pairs the rounded products sin cos, sin
+// sin and cos were within 0.5007 units in the last place, with the same root
+// mean square error (0.28866 units) as rounding the FP64 functions.
+constexpr float kSincosRange = 1000.f;
+__device__ __forceinline__ void sincos_two_float(float x, TwoFloat *sine, TwoFloat *cosine) {
+    const float k = rintf(__fmul_rn(x, 0x1.45f306p-1f));  // x / (pi/2)
+    constexpr float P1 = 0x1.921fb6p+0f, P2 = -0x1.777a5cp-25f, P3 = -0x1.ee59dap-50f;
+    const float p1 = __fmul_rn(k, P1), p1l = fmaf(k, P1, -p1);
+    const TwoFloat t1 = two_sum(__fsub_rn(x, p1), -p1l);  // x - p1 is exact
+    const float p2 = __fmul_rn(k, P2), p2l = fmaf(k, P2, -p2);
+    const TwoFloat t2 = two_sum(t1.hi, -p2);
+    const TwoFloat r =
+        quick_two_sum(t2.hi, __fsub_rn(__fadd_rn(t1.lo, t2.lo), fmaf(k, P3, p2l)));
+    const TwoFloat z = tf_mul(r, r);
+    const float y = z.hi;
+    // sin r = r + r z (-1/3! + z (1/5! + z (-1/7! + ... + z^3 / 13!)))
+    const float u =
+        __fmul_rn(y, fmaf(y, fmaf(y, fmaf(y, 1.f / 6227020800.f, -1.f / 39916800.f),
+                                  1.f / 362880.f), -1.f / 5040.f));
+    TwoFloat q = tf_add(TwoFloat{0x1.111112p-7f, -0x1.dddddep-32f}, TwoFloat{u, 0.f});
+    q = tf_add(TwoFloat{-0x1.555556p-3f, 0x1.555556p-28f}, tf_mul(z, q));
+    const TwoFloat s = tf_add(r, tf_mul(r, tf_mul(z, q)));
+    // cos r = 1 + z (-1/2! + z (1/4! + z (-1/6! + ... + z^3 / 12!)))
+    const float v =
+        __fmul_rn(y, fmaf(y, fmaf(y, fmaf(y, 1.f / 479001600.f, -1.f / 3628800.f),
+                                  1.f / 40320.f), -1.f / 720.f));
+    TwoFloat g = tf_add(TwoFloat{0x1.555556p-5f, -0x1.555556p-30f}, TwoFloat{v, 0.f});
+    g = tf_add(TwoFloat{-0.5f, 0.f}, tf_mul(z, g));
+    const TwoFloat c = tf_add(TwoFloat{1.f, 0.f}, tf_mul(z, g));
+    const int quadrant = (int)k & 3;
+    TwoFloat a = (quadrant & 1) ? c : s, b = (quadrant & 1) ? s : c;
+    if (quadrant & 2) a = TwoFloat{-a.hi, -a.lo};
+    if ((quadrant + 1) & 2) b = TwoFloat{-b.hi, -b.lo};
+    *sine = a;
+    *cosine = b;
+}
+
 // The nearest float to (A + a) / (X + x) for two-float numerator and
-// denominator (X > 0): q = A / X is within a few units of the answer; the
-// residual (A + a) - q (X + x), whose leading part A - q X is exact by FMA,
-// divided by X is the remaining correction, and q plus it is rounded once
-// (Markstein's final step).  The correction carries about 24 bits, so the
+// denominator (X > 0): q = A (1/X) is within two units of the answer; the
+// residual (A + a) - q (X + x), whose leading part A - q X FMA forms to 2^-47
+// of A, times 1/X is the remaining correction, and q plus it is rounded once
+// (Markstein's final step).  The correction carries about 23 bits, so the
 // result can differ from exact rounding only when the quotient lies within
 // about 2^-44 of its size of a rounding midpoint.
 __device__ __forceinline__ float div_two_float_rn(float A, float a, float X, float x) {
-    const float q = __fdiv_rn(A, X);
+    const float y = __frcp_rn(X);
+    const float q = __fmul_rn(A, y);
     float r = fmaf(-q, X, A);
     r = __fadd_rn(r, a);
     r = fmaf(-q, x, r);
-    return fmaf(r, __frcp_rn(X), q);
+    return fmaf(r, y, q);
 }
 
-// One grid row (j, k) per block iteration: the row index is split once per
-// row, not per point.  b = dt^2 / (m + (dx + dy + dz) dt / 2) is formed in
-// two-float FP32 arithmetic (dt^2 = A + a, dt / 2 = H + h): the damping sum
-// and its product with dt / 2 carried to about 2^-44, the quotient rounded
-// once (div_two_float_rn).  FP64 -- slow on this part -- remains for the
-// points that fail validation or lie outside the range where the two-float
-// steps are exact (m or a damping term negative, non-finite, or extreme).
+// Four consecutive x points of a dense [nz][ny][nx] row (zero beyond nx):
+// one 16-byte load where rows and base allow it.
+__device__ __forceinline__ void load_quad(const float *row, int i, int nx, bool vec, float v[4]) {
+    if (vec) {
+        const float4 f = __ldcs(reinterpret_cast<const float4 *>(row + i));
+        v[0] = f.x, v[1] = f.y, v[2] = f.z, v[3] = f.w;
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = i + e < nx ? __ldcs(row + i + e) : 0.f;
+}
+
+// The setup kernels walk the padded layout four x points at a time (rows are
+// whole 16-byte quads, fewer than 2^30 in all) and write its padding columns
+// as zero, so that the coefficient fields need no clearing.
+struct Quad {
+    int i, j, k;
+    unsigned int row;  // dense row k ny + j
+};
+__device__ __forceinline__ Quad quad_at(unsigned int q, const WaveLayout &L) {
+    const unsigned int nxq = (unsigned int)L.nxp / 4;
+    Quad p;
+    p.row = q / nxq;
+    p.i = 4 * (int)(q - p.row * nxq);
+    p.k = (int)(p.row / (unsigned int)L.ny);
+    p.j = (int)(p.row - (unsigned int)p.k * L.ny);
+    return p;
+}
+
+// b = dt^2 / (m + (dx + dy + dz) dt / 2) formed in two-float FP32 arithmetic
+// (dt^2 = A + a, dt / 2 = H + h): the damping sum and its product with dt / 2
+// carried to about 2^-44, the quotient rounded once (div_two_float_rn).  FP64
+// -- slow on this part -- remains for the points that fail validation or lie
+// outside the range where the two-float steps are exact (m or a damping term
+// negative, non-finite, or extreme).
 // With `zeta` non-null the damping is a 3-D field damp[nz][ny][nx] (d = damp
 // at the point) and zeta = fl(fl(d / dt) b) is stored beside b, the factor
 // the stencil kernel's damp-field variant reads instead of forming it from
 // per-axis profiles (the same two roundings as the profile path's
 // fl(fl(d_x/dt + (d_y/dt + d_z/dt)) b) when a single axis is damped).
-__global__ void acoustic_coeff_kernel(const float *__restrict__ m, const float *__restrict__ damp,
-                                      double dt, float dt2_hi, float dt2_lo, float hdt_hi,
-                                      float hdt_lo, WaveLayout L, float *__restrict__ bcoef,
-                                      float *__restrict__ zeta, StatsKeys *stats) {
-    const int64_t rows = (int64_t)L.ny * L.nz;
+// Bound by instruction issue (about 60 operations per point) next to HBM (8
+// bytes per point): at 384^3 172 us (67 us at the copy bandwidth), 396 us
+// with one row per block and one point per thread and load.
+__global__ void __launch_bounds__(256)
+    acoustic_coeff_kernel(const float *__restrict__ m, const float *__restrict__ damp,
+                          double dt, float dt2_hi, float dt2_lo, float hdt_hi, float hdt_lo,
+                          WaveLayout L, unsigned int nquads, int vec,
+                          float *__restrict__ bcoef, float *__restrict__ zeta,
+                          StatsKeys *stats) {
     const double dt2 = dt * dt;
+    const bool dense = zeta != nullptr;
     float lmin = __int_as_float(0x7f800000), lmax = 0.f;
     unsigned int bad = 0u;
-    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int j = (int)(r % L.ny);
-        const int k = (int)(r / L.ny);
-        const bool dense = zeta != nullptr;
-        const float dyf = damp && !dense ? damp[L.nx + j] : 0.f;
-        const float dzf = damp && !dense ? damp[L.nx + L.ny + k] : 0.f;
+    for (unsigned int n = blockIdx.x * blockDim.x + threadIdx.x; n < nquads;
+         n += gridDim.x * blockDim.x) {
+        const Quad p = quad_at(n, L);
+        const float dyf = damp && !dense ? __ldg(damp + L.nx + p.j) : 0.f;
+        const float dzf = damp && !dense ? __ldg(damp + L.nx + L.ny + p.k) : 0.f;
         const bool row_ok = dyf >= 0.f && dyf <= 1.0e30f && dzf >= 0.f && dzf <= 1.0e30f;
-        const float *mrow = m + r * L.nx;
-        const float *drow = dense && damp ? damp + r * L.nx : nullptr;
-        float *brow = bcoef + (int64_t)k * L.plane + (int64_t)j * L.nxp;
-        for (int i = threadIdx.x; i < L.nx; i += blockDim.x) {
-            const float mv = mrow[i];
-            const float dxf = drow ? drow[i] : (damp && !dense ? damp[i] : 0.f);
+        float mq[4], dq[4] = {0.f, 0.f, 0.f, 0.f}, bq[4], zq[4];
+        load_quad(m + (int64_t)p.row * L.nx, p.i, L.nx, vec, mq);
+        if (damp && dense) {
+            load_quad(damp + (int64_t)p.row * L.nx, p.i, L.nx, vec, dq);
+        } else if (damp) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dq[e] = p.i + e < L.nx ? __ldg(damp + p.i + e) : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            bq[e] = zq[e] = 0.f;
+            if (p.i + e >= L.nx) continue;
+            const float mv = mq[e], dxf = dq[e];
             lmin = fminf(lmin, mv);
             lmax = fmaxf(lmax, mv);
             if (row_ok && dxf >= 0.f && dxf <= 1.0e30f && mv >= 1.17549435e-38f &&
@@ -144,18 +243,20 @@ __global__ void acoustic_coeff_kernel(const float *__restrict__ m, const float *
                 float pl = fmaf(s2.hi, hdt_hi, -ph);
                 pl = __fadd_rn(pl, __fadd_rn(__fmul_rn(s2.hi, hdt_lo), __fmul_rn(dlo, hdt_hi)));
                 const TwoFloat xs = two_sum(mv, ph);
-                brow[i] = div_two_float_rn(dt2_hi, dt2_lo, xs.hi, __fadd_rn(xs.lo, pl));
+                bq[e] = div_two_float_rn(dt2_hi, dt2_lo, xs.hi, __fadd_rn(xs.lo, pl));
             } else {
                 double d = 0.0;
                 if (damp) d = (double)dxf + (double)dyf + (double)dzf;
                 if (!(mv > 0.f) || !isfinite(mv) || !(d >= 0.0) || !isfinite(d))
                     bad = DEV_ERR_MEDIUM;
-                brow[i] = (float)(dt2 * recip_newton((double)mv + 0.5 * d * dt));
+                bq[e] = (float)(dt2 * recip_newton((double)mv + 0.5 * d * dt));
             }
-            if (dense)
-                zeta[(int64_t)k * L.plane + (int64_t)j * L.nxp + i] =
-                    __fmul_rn((float)((double)dxf / dt), brow[i]);
+            if (dense) zq[e] = __fmul_rn((float)((double)dxf / dt), bq[e]);
         }
+        const int64_t o = (int64_t)4 * n;
+        *reinterpret_cast<float4 *>(bcoef + o) = make_float4(bq[0], bq[1], bq[2], bq[3]);
+        if (dense)
+            *reinterpret_cast<float4 *>(zeta + o) = make_float4(zq[0], zq[1], zq[2], zq[3]);
     }
     lmin = warp_min(lmin);
     lmax = warp_max(lmax);
@@ -172,33 +273,70 @@ __global__ void damp_scale_kernel(const float *__restrict__ damp, int n, double 
     if (i < n) dps[i] = damp ? (float)((double)damp[i] / dt) : 0.f;
 }
 
-__global__ void tti_coeff_kernel(const float *__restrict__ eps, const float *__restrict__ delta,
-                                 const float *__restrict__ theta, const float *__restrict__ phi,
-                                 WaveLayout L, float *__restrict__ acoef, float *__restrict__ scoef,
-                                 float *__restrict__ nvec, StatsKeys *stats) {
-    const int64_t n = (int64_t)L.nx * L.ny * L.nz;
+// n = (sin theta cos phi, sin theta sin phi, cos theta) of one point.
+__device__ __forceinline__ void axis_of(float th, float ph, float *nx, float *ny, float *nz) {
+    if (fabsf(th) <= kSincosRange && fabsf(ph) <= kSincosRange) {
+        TwoFloat st, ct, sp, cp;
+        sincos_two_float(th, &st, &ct);
+        sincos_two_float(ph, &sp, &cp);
+        *nx = tf_mul(st, cp).hi;
+        *ny = tf_mul(st, sp).hi;
+        *nz = ct.hi;
+        return;
+    }
+    double st, ct, sp, cp;
+    sincos((double)th, &st, &ct);
+    sincos((double)ph, &sp, &cp);
+    *nx = (float)(st * cp);
+    *ny = (float)(st * sp);
+    *nz = (float)ct;
+}
+
+// a = 1 + 2 eps and s = sqrt(1 + 2 delta) rounded once (1 + 2 delta as an
+// exact two-float, the FP32 root corrected by its exact residual), and the
+// symmetry axis.  Two-float FP32 throughout: with FP64 trigonometry the
+// kernel was bound by the FP64 pipe, 7390 us at 384^3 (14 % of a 59-step so 4
+// run) against 647 us (36 bytes per point: 302 us at the copy bandwidth).
+__global__ void __launch_bounds__(256)
+    tti_coeff_kernel(const float *__restrict__ eps, const float *__restrict__ delta,
+                     const float *__restrict__ theta, const float *__restrict__ phi,
+                     WaveLayout L, unsigned int nquads, int vec, float *__restrict__ acoef,
+                     float *__restrict__ scoef, float *__restrict__ nvec, StatsKeys *stats) {
     float lmax = -__int_as_float(0x7f800000);
     unsigned int bad = 0u;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(p % L.nx);
-        const int64_t r = p / L.nx;
-        const int j = (int)(r % L.ny);
-        const int k = (int)(r / L.ny);
-        const float e = eps[p], d = delta[p], th = theta[p], ph = phi[p];
-        if (!isfinite(e) || !isfinite(d) || !isfinite(th) || !isfinite(ph) || !(e >= d) ||
-            !(1.0f + 2.0f * d >= 0.f))
-            bad = DEV_ERR_MEDIUM;
-        lmax = fmaxf(lmax, e);
-        const int64_t q = (int64_t)k * L.plane + (int64_t)j * L.nxp + i;
-        acoef[q] = (float)(1.0 + 2.0 * (double)e);
-        scoef[q] = (float)sqrt(fmax(0.0, 1.0 + 2.0 * (double)d));
-        double st, ct, sp, cp;
-        sincos((double)th, &st, &ct);
-        sincos((double)ph, &sp, &cp);
-        nvec[q] = (float)(st * cp);
-        nvec[L.vol + q] = (float)(st * sp);
-        nvec[2 * L.vol + q] = (float)ct;
+    for (unsigned int n = blockIdx.x * blockDim.x + threadIdx.x; n < nquads;
+         n += gridDim.x * blockDim.x) {
+        const Quad p = quad_at(n, L);
+        const int64_t row = (int64_t)p.row * L.nx;
+        float eq[4], dq[4], tq[4], pq[4], av[4], sv[4], xv[4], yv[4], zv[4];
+        load_quad(eps + row, p.i, L.nx, vec, eq);
+        load_quad(delta + row, p.i, L.nx, vec, dq);
+        load_quad(theta + row, p.i, L.nx, vec, tq);
+        load_quad(phi + row, p.i, L.nx, vec, pq);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            av[e] = sv[e] = xv[e] = yv[e] = zv[e] = 0.f;
+            if (p.i + e >= L.nx) continue;
+            const float ev = eq[e], dv = dq[e], th = tq[e], ph = pq[e];
+            if (!isfinite(ev) || !isfinite(dv) || !isfinite(th) || !isfinite(ph) ||
+                !(ev >= dv) || !(1.0f + 2.0f * dv >= 0.f))
+                bad = DEV_ERR_MEDIUM;
+            lmax = fmaxf(lmax, ev);
+            av[e] = __fadd_rn(1.f, 2.f * ev);
+            const TwoFloat x = two_sum(1.f, 2.f * dv);
+            if (x.hi > 0.f) {
+                const float r = __fsqrt_rn(x.hi);
+                sv[e] = __fadd_rn(r, __fdividef(__fadd_rn(fmaf(-r, r, x.hi), x.lo), 2.f * r));
+            }
+            axis_of(th, ph, &xv[e], &yv[e], &zv[e]);
+        }
+        const int64_t o = (int64_t)4 * n;
+        *reinterpret_cast<float4 *>(acoef + o) = make_float4(av[0], av[1], av[2], av[3]);
+        *reinterpret_cast<float4 *>(scoef + o) = make_float4(sv[0], sv[1], sv[2], sv[3]);
+        *reinterpret_cast<float4 *>(nvec + o) = make_float4(xv[0], xv[1], xv[2], xv[3]);
+        *reinterpret_cast<float4 *>(nvec + L.vol + o) = make_float4(yv[0], yv[1], yv[2], yv[3]);
+        *reinterpret_cast<float4 *>(nvec + 2 * L.vol + o) =
+            make_float4(zv[0], zv[1], zv[2], zv[3]);
     }
     lmax = warp_max(lmax);
     if ((threadIdx.x & 31) == 0) atomicMax(&stats->eps_max, float_key(lmax));
@@ -266,6 +404,8 @@ __global__ void watchdog_kernel(const float *__restrict__ f, WaveLayout L, int n
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flags, DEV_ERR_NONFINITE);
 }
 
+bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 int grid_for(int64_t n, int threads) {
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
@@ -293,9 +433,11 @@ fd_status setup_acoustic_coeffs(const float *m, const float *damp, double dt,
     const double dt2 = dt * dt, hdt = 0.5 * dt;
     const float dt2_hi = (float)dt2, hdt_hi = (float)hdt;
     const float dt2_lo = (float)(dt2 - (double)dt2_hi), hdt_lo = (float)(hdt - (double)hdt_hi);
-    acoustic_coeff_kernel<<<grid_for((int64_t)L.ny * L.nz * 256, 256), 256, 0, stream>>>(
-        m, damp, dt, dt2_hi, dt2_lo, hdt_hi, hdt_lo, L, bcoef, damp_field ? bcoef + L.vol : nullptr,
-        keys);
+    const int64_t nquads = L.vol / 4;  // < 2^30 (validate_grid)
+    const int vec = L.nx % 4 == 0 && aligned16(m) && (!damp_field || aligned16(damp));
+    acoustic_coeff_kernel<<<grid_for(nquads, 256), 256, 0, stream>>>(
+        m, damp, dt, dt2_hi, dt2_lo, hdt_hi, hdt_lo, L, (unsigned int)nquads, vec, bcoef,
+        damp_field ? bcoef + L.vol : nullptr, keys);
     FD_CUDA_TRY(cudaGetLastError());
     note_launch(stream);
     const int nd = L.nx + L.ny + L.nz;
@@ -310,9 +452,11 @@ fd_status setup_tti_coeffs(const float *eps, const float *delta, const float *th
                            const float *phi, const WaveLayout &L, float *acoef, float *scoef,
                            float *nvec, MediumStats *dev_stats, cudaStream_t stream) {
     StatsKeys *keys = reinterpret_cast<StatsKeys *>(dev_stats);
-    const int64_t n = (int64_t)L.nx * L.ny * L.nz;
-    tti_coeff_kernel<<<grid_for(n, 256), 256, 0, stream>>>(eps, delta, theta, phi, L, acoef,
-                                                           scoef, nvec, keys);
+    const int64_t nquads = L.vol / 4;
+    const int vec = L.nx % 4 == 0 && aligned16(eps) && aligned16(delta) && aligned16(theta) &&
+                    aligned16(phi);
+    tti_coeff_kernel<<<grid_for(nquads, 256), 256, 0, stream>>>(
+        eps, delta, theta, phi, L, (unsigned int)nquads, vec, acoef, scoef, nvec, keys);
     FD_CUDA_TRY(cudaGetLastError());
     note_launch(stream);
     return FD_OK;

@@ -413,8 +413,8 @@ int64_t fd_launch_count(void);
  * merely in flight, the call returns FD_ERR_TIMEOUT and the device stays
  * usable (the copies already issued are still waited for, with their own
  * limit, before a stopped kernel exits).  Process-wide; it applies to the
- * stencil kernel's default launch configuration with per-axis damping (a
- * variant of it that reads the limit is launched while the setting is
+ * stencil kernel's launch configurations with per-axis damping (variants of
+ * them that read the limit are launched while the setting is
  * non-zero, so the production kernel keeps a constant limit), and to launches
  * enqueued after the call (a CUDA graph keeps the variant it was captured
  * with).
@@ -470,7 +470,8 @@ int fd_num_tti_configs(int so);
 /*
  * Tile configuration override for the acoustic stencil kernel (for tuning
  * sweeps): index into the compiled configuration table for the given space
- * order, or -1 for the built-in choice.  Returns FD_ERR_ARG if out of range.
+ * order, or -1 for the built-in choice (the configuration with the smallest
+ * estimated time for the grid).  Returns FD_ERR_ARG if out of range.
  */
 fd_status fd_set_acoustic_config(int so, int config);
 int fd_num_acoustic_configs(int so);

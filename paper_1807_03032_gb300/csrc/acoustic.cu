@@ -15,8 +15,16 @@
 // memory stages by cp.async.bulk.tensor, D planes ahead of use; the same stage
 // also receives the interior tiles of u^n, u^{n-1} and b for the output plane
 // p - R.  Each stage has a "full" mbarrier (TMA transaction count) and an
-// "empty" mbarrier (one arrival per warp), so warps run decoupled and thread 0
-// refills a stage as soon as every warp has released it.
+// "empty" mbarrier (one arrival per warp), so warps run decoupled; a producer
+// warp refills a stage as soon as every consumer warp has released it.  (With
+// a consumer thread as the producer, the wait for the stage and the four copy
+// issues, about 460 cycles, preceded that warp's share of every plane and set
+// the pace of all: 1024 cycles (0.5 us) per plane for a lone CTA of any
+// radius. With its own warp a plane takes 0.28 - 0.39 us.)
+//
+// One launch is one time step: extra blocks record the receivers of u^n, the
+// sources are injected by the CTAs that own their nodes, and the launch is
+// chained to the previous one (its prologue overlaps the other's last planes).
 //
 // The z-direction uses an accumulator pipeline: when plane p arrives, each
 // thread adds w_|p-z| u(p) to the 2R pending outputs z in [p-R, p+R) it holds
@@ -32,6 +40,7 @@
 
 #include "f32x2.cuh"
 #include "kernels.cuh"
+#include "receive.cuh"
 #include "runtime.cuh"
 
 namespace fdsweep {
@@ -56,13 +65,34 @@ struct AcCfg {
     static constexpr int STAGE = HALO + NINT * INT;  // [halo u^n][u^n][u^{n-1}][b][zeta]
     static constexpr uint32_t HALO_BYTES = PW * PH * 4;
     static constexpr uint32_t INT_BYTES = INT * 4;
-    static constexpr int THREADS = TX * TY;
-    static constexpr int WARPS = THREADS / 32;
+    static constexpr int CONSUMERS = TX * TY;        // threads that own points
+    static constexpr int WARPS = CONSUMERS / 32;
+    static constexpr int THREADS = CONSUMERS + 32;   // + the producer warp
     // stages, full/empty mbarriers, abort flag; + damp_z of the z chunk
     // (added at launch) and 128 bytes to align the base
     static constexpr size_t SMEM = (size_t)NSL * STAGE * 4 + NSL * 16 + 16 + 128;
     static_assert(PW <= 256 && PH <= 256 && BX <= 256 && BY <= 256, "TMA box dimension limit");
-    static_assert(INT % 32 == 0 && THREADS % 32 == 0, "tile shape");
+    static_assert(INT % 32 == 0 && CONSUMERS % 32 == 0, "tile shape");
+};
+
+// Position in a ring of N stages: from the plane index where N is a power of
+// two (constant stage addresses in an unrolled loop), counted otherwise.
+template <int N>
+struct RingPos {
+    int s = 0;
+    uint32_t ph = 0;
+    static constexpr bool POW2 = (N & (N - 1)) == 0;
+    __device__ __forceinline__ int slot(int j) const { return POW2 ? j % N : s; }
+    __device__ __forceinline__ uint32_t phase(int j) const {
+        return POW2 ? (uint32_t)(j / N) & 1u : ph;
+    }
+    __device__ __forceinline__ void next() {
+        if (POW2) return;
+        if (++s == N) {
+            s = 0;
+            ph ^= 1u;
+        }
+    }
 };
 
 // Source injection by the CTA that wrote a source's corners, after its
@@ -113,15 +143,21 @@ __device__ __noinline__ void inject_column(const AcousticStepArgs *a, const Acou
 // constant 2 s, which keeps the limit out of the plane loop's registers (a
 // limit read at run time cost 13 % at so 8).
 template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB = 0, bool WL = false>
-__global__ void __launch_bounds__(TX *TY, MINB)
+__global__ void __launch_bounds__(TX *TY + 32, MINB)
     acoustic_step_kernel(const __grid_constant__ CUtensorMap map_halo,
                          const __grid_constant__ CUtensorMap map_int,
                          const __grid_constant__ CUtensorMap map_b,
                          const __grid_constant__ AcousticStepArgs a,
-                         const __grid_constant__ AcousticInject inj, int zchunk, int nzc) {
+                         const __grid_constant__ AcousticInject inj,
+                         const __grid_constant__ ReceiveArgs rec, int zchunk, int nzc) {
     using C = AcCfg<R, TX, TY, VY, D, DF>;
-    // the divergence watchdog stopped the run: nothing more to compute
-    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;
+    if (blockIdx.z >= gridDim.z - rec.slices) {
+        chain_trigger();
+        chain_wait();
+        if (!(__ldcg(a.err) & DEV_ERR_NONFINITE))
+            record_receivers(&rec, a.wave, a.lps, a.lev_cur, a.lev_cur, &a.L);
+        return;
+    }
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *smem = reinterpret_cast<float *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
@@ -158,33 +194,44 @@ __global__ void __launch_bounds__(TX *TY, MINB)
     }
     for (int z = za + tid; z < zb; z += C::THREADS) sdz[z - za] = a.dpz[z];
     __syncthreads();
+    chain_wait();
+    // the divergence watchdog stopped the run: nothing more to compute
+    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;
 
-    // Producer (thread 0): stage for iteration jj = halo plane za-R+jj, plus
-    // the interior tiles of output plane za-2R+jj once jj >= 2R.
     int issued = 0;
-    auto issue = [&](int jj) -> bool {
-        const int slot = jj % C::NSL;
-        if (jj >= C::NSL &&
-            !mbar_wait_bounded(&empty[slot], (uint32_t)(((jj - C::NSL) / C::NSL) & 1), wait_ns))
-            return false;
-        const bool with_out = jj >= 2 * R;
-        mbar_arrive_expect_tx(&full[slot],
-                              C::HALO_BYTES + (with_out ? C::NINT * C::INT_BYTES : 0));
-        float *st = smem + slot * C::STAGE;
-        tma_load_4d(st, &map_halo, &full[slot], x0 - C::RA, y0 - R, za - R + jj, wcur);
-        if (with_out) {
-            const int zo = za - 2 * R + jj;
-            tma_load_4d(st + C::HALO, &map_int, &full[slot], x0, y0, zo, wcur);
-            tma_load_4d(st + C::HALO + C::INT, &map_int, &full[slot], x0, y0, zo, wprev);
-            tma_load_4d(st + C::HALO + 2 * C::INT, &map_b, &full[slot], x0, y0, zo, 0);
-            if (DF) tma_load_4d(st + C::HALO + 3 * C::INT, &map_b, &full[slot], x0, y0, zo, 1);
+    if (tid >= C::CONSUMERS) {
+        // Producer warp (one lane): stage jj = halo plane za-R+jj, plus the
+        // interior tiles of output plane za-2R+jj once jj >= 2R.
+        if (lane == 0) {
+            RingPos<C::NSL> pos;
+            for (int jj = 0; jj < nplanes && !*abort_flag; ++jj, pos.next()) {
+                const int slot = pos.slot(jj);
+                if (jj >= C::NSL &&
+                    !mbar_wait_bounded(&empty[slot], pos.phase(jj) ^ 1u, wait_ns)) {
+                    if (!*abort_flag) atomicOr(a.err, DEV_ERR_TIMEOUT);
+                    *abort_flag = 1;
+                    break;
+                }
+                const bool with_out = jj >= 2 * R;
+                mbar_arrive_expect_tx(&full[slot],
+                                      C::HALO_BYTES + (with_out ? C::NINT * C::INT_BYTES : 0));
+                float *st = smem + slot * C::STAGE;
+                tma_load_4d(st, &map_halo, &full[slot], x0 - C::RA, y0 - R, za - R + jj, wcur);
+                if (with_out) {
+                    const int zo = za - 2 * R + jj;
+                    tma_load_4d(st + C::HALO, &map_int, &full[slot], x0, y0, zo, wcur);
+                    tma_load_4d(st + C::HALO + C::INT, &map_int, &full[slot], x0, y0, zo, wprev);
+                    tma_load_4d(st + C::HALO + 2 * C::INT, &map_b, &full[slot], x0, y0, zo, 0);
+                    if (DF)
+                        tma_load_4d(st + C::HALO + 3 * C::INT, &map_b, &full[slot], x0, y0, zo, 1);
+                }
+                issued = jj + 1;
+            }
+            // the next launch may move in while the last planes are computed;
+            // earlier, its waiting blocks would take the place of this one's
+            chain_trigger();
         }
-        issued = jj + 1;
-        return true;
-    };
-    if (tid == 0)
-        for (int jj = 0; jj < D && jj < nplanes; ++jj) issue(jj);
-
+    } else {
     const bool xok = gx < a.L.nxp;
     float dpx4[4];
 #pragma unroll
@@ -209,18 +256,11 @@ __global__ void __launch_bounds__(TX *TY, MINB)
 #pragma unroll
         for (int v = 0; v < VY; ++v) acc[i][v] = Q4{0ull, 0ull};
 
-    bool failed = false;
+    RingPos<C::NSL> pos;
 #pragma unroll U
-    for (int j = 0; j < nplanes; ++j) {
-        if (tid == 0 && j + D < nplanes && !failed) {
-            if (!issue(j + D)) {
-                failed = true;
-                *abort_flag = 1;
-                atomicOr(a.err, DEV_ERR_TIMEOUT);
-            }
-        }
-        const int slot = j % C::NSL;
-        if (*abort_flag || !mbar_wait_bounded(&full[slot], (uint32_t)((j / C::NSL) & 1), wait_ns)) {
+    for (int j = 0; j < nplanes; ++j, pos.next()) {
+        const int slot = pos.slot(j);
+        if (*abort_flag || !mbar_wait_bounded(&full[slot], pos.phase(j), wait_ns)) {
             *abort_flag = 1;
             atomicOr(a.err, DEV_ERR_TIMEOUT);
             break;
@@ -356,8 +396,9 @@ __global__ void __launch_bounds__(TX *TY, MINB)
             acc[2 * R - 1][v] = Q4{f2_mul(wR2, cen[v].lo), f2_mul(wR2, cen[v].hi)};
         }
     }
+    }
     __syncthreads();
-    if (*abort_flag && tid == 0) {
+    if (*abort_flag && tid == C::CONSUMERS) {
         // The last NSL issued stages may still be in flight: give them a
         // bounded chance to land before the CTA's shared memory is released.
         for (int jj = issued - C::NSL; jj < issued; ++jj)
@@ -368,110 +409,102 @@ __global__ void __launch_bounds__(TX *TY, MINB)
         inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
 }
 
+// A launch configuration and what a launch of it costs (microseconds, fitted
+// to measured steps of 21 problems from 48^3 to 512^3, ragged and with up to
+// 8 shots, over all chunk counts): `launch` + (planes + warm 2R) x waves, a
+// plane costing sqrt(lat^2 + (k thr)^2) with k CTAs on the SM.
 struct ConfigEntry {
-    int radius, tx, ty, vy, d;
-    const void *fn;
+    int radius;
+    const void *fn, *fn_wl;  // fn_wl: the variant with the wait limit from the arguments
     size_t smem;
     int bx, by, pw, ph, threads;
+    float launch, lat, thr, warm;
     const char *name;
 };
 
-template <int R, int TX, int TY, int VY, int D, int U, bool DF = false, int MINB = 0,
-          bool WL = false>
-ConfigEntry make_entry(const char *name) {
+template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB>
+ConfigEntry make_entry(const char *name, float launch, float lat, float thr, float warm) {
     using C = AcCfg<R, TX, TY, VY, D, DF>;
-    return ConfigEntry{R,       TX,    TY,    VY,    D,
-                       (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, WL>,
-                       C::SMEM, C::BX, C::BY, C::PW, C::PH, C::THREADS, name};
+    const void *wl = nullptr;
+    if constexpr (!DF) wl = (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, true>;
+    return ConfigEntry{R,      (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB>,
+                       wl,     C::SMEM, C::BX, C::BY, C::PW, C::PH, C::THREADS,
+                       launch, lat, thr, warm, name};
 }
 
-#define FD_AC_ENTRY(R, TX, TY, VY, D, U)                                           \
-    make_entry<R, TX, TY, VY, D, U>("acoustic_step<" #R "," #TX "," #TY "," #VY "," #D \
-                                    "," #U ">")
-#define FD_AC_ENTRY_DF(R, TX, TY, VY, D, U, MB)                                              \
-    make_entry<R, TX, TY, VY, D, U, true, MB>("acoustic_step<" #R "," #TX "," #TY "," #VY "," #D \
-                                              "," #U ",damp field>")
+#define FD_AC_ENTRY(R, TX, TY, VY, D, U, MB, ...)                                               \
+    make_entry<R, TX, TY, VY, D, U, false, MB>("acoustic_step<" #R "," #TX "," #TY "," #VY "," \
+                                               #D "," #U ">",                                  \
+                                               __VA_ARGS__)
+#define FD_AC_ENTRY_DF(R, TX, TY, VY, D, U, MB, ...)                                           \
+    make_entry<R, TX, TY, VY, D, U, true, MB>("acoustic_step<" #R "," #TX "," #TY "," #VY "," \
+                                              #D "," #U ",damp field>",                       \
+                                              __VA_ARGS__)
 
-#define FD_AC_ENTRY_WL(R, TX, TY, VY, D, U)                                                 \
-    make_entry<R, TX, TY, VY, D, U, false, 0, true>("acoustic_step<" #R "," #TX "," #TY "," #VY \
-                                                    "," #D "," #U ",wait limit>")
-
-// The default configuration of each radius with the wait limit taken from the
-// arguments: launched instead of it while fd_set_wait_limit_ns is set.
-const ConfigEntry *config_table_wl(int radius) {
-    static const ConfigEntry r1 = FD_AC_ENTRY_WL(1, 16, 16, 1, 4, 1);
-    static const ConfigEntry r2 = FD_AC_ENTRY_WL(2, 16, 16, 1, 4, 4);
-    static const ConfigEntry r4 = FD_AC_ENTRY_WL(4, 16, 8, 1, 4, 4);
-    static const ConfigEntry r6 = FD_AC_ENTRY_WL(6, 16, 8, 1, 3, 4);
-    static const ConfigEntry r8 = FD_AC_ENTRY_WL(8, 16, 4, 1, 1, 4);
-    switch (radius) {
-        case 1: return &r1;
-        case 2: return &r2;
-        case 4: return &r4;
-        case 6: return &r6;
-        case 8: return &r8;
-        default: return nullptr;
-    }
-}
-
-// 3-D damping field: one configuration per radius, the default one's tiles,
-// with the prefetch depth and register bound chosen so that a 512^3 launch
-// still fits in one wave despite the fourth interior tile per stage (four
-// 128-thread or eight 64-thread CTAs per SM; with three 128-thread CTAs the
-// 512 columns need two waves: so 8 and 12 at 0.6 of the copy bandwidth).
-const ConfigEntry *config_table_df(int radius) {
-    static const ConfigEntry r1 = FD_AC_ENTRY_DF(1, 16, 16, 1, 4, 1, 0);
-    static const ConfigEntry r2 = FD_AC_ENTRY_DF(2, 16, 16, 1, 4, 4, 0);
-    static const ConfigEntry r4 = FD_AC_ENTRY_DF(4, 16, 8, 1, 3, 4, 0);
-    static const ConfigEntry r6 = FD_AC_ENTRY_DF(6, 16, 8, 1, 2, 4, 4);
-    static const ConfigEntry r8 = FD_AC_ENTRY_DF(8, 16, 4, 1, 1, 4, 8);
-    switch (radius) {
-        case 1: return &r1;
-        case 2: return &r2;
-        case 4: return &r4;
-        case 6: return &r6;
-        case 8: return &r8;
-        default: return nullptr;
-    }
-}
-
+// The configurations of each radius (template arguments R, TX, TY, VY, D, U,
+// minimum CTAs per SM); acoustic_plan takes the one with the smallest
+// estimated time for the grid.  Ring sizes are powers of two (D = 3), so that
+// the unrolled plane loop has constant stage addresses.
+//  * Small tiles fill the machine on small grids (64 x 4 at so 16: 128^3 17.8
+//    us per step, 64 x 8 19.4).
+//  * Two rows per thread (VY = 2) halve the shared-memory reads of the y
+//    neighbours, which bound the wide stencils: R y-rows above and below cost
+//    R + 1 reads per point instead of 2R.  At so 12 and 16 a few large CTAs
+//    pay best at large sizes: 64 x 28 tiles, one CTA of 224 + 32 threads with
+//    255 registers per SM, run 512^3 so 16 in 369 us (442 with 64 x 8, 472
+//    before the producer warp); 64 x 44 at so 12 in 340 us (387 and 402).
+//  * so 4 and 8 are at the HBM limit at 512^3 (306 and 318 us for 2.15 GB).
 const ConfigEntry *config_table(int radius, int *count) {
-    // Index 0 is the default; the others are kept for tuning sweeps
-    // (fd_set_acoustic_config).  Defaults measured on GB300 at 512^3 (template
-    // arguments R, TX, TY, VY, D, U): the plane-loop unroll U = 4 helps at every
-    // radius; a deeper prefetch suits R = 4 (D = 4, +10 %), a shallower one
-    // R = 8 (D = 1: more CTAs per SM), where 64 x 4 tiles of 64 threads (1024
-    // columns in two z chunks) beat 64 x 8 tiles by 4 % (281 against 269
-    // GPts/s; 32 x 8 tiles of 64 threads measured the same as 64 x 4).
-    static const ConfigEntry r1[] = {FD_AC_ENTRY(1, 16, 16, 1, 4, 1)};
+    static const ConfigEntry r1[] = {
+        FD_AC_ENTRY(1, 16, 16, 1, 3, 4, 0, 2.4f, 0.30f, 0.27f, 0.9f)};
     static const ConfigEntry r2[] = {
-        FD_AC_ENTRY(2, 16, 16, 1, 4, 4), FD_AC_ENTRY(2, 16, 16, 1, 4, 1),
-        FD_AC_ENTRY(2, 16, 8, 1, 6, 1),  FD_AC_ENTRY(2, 16, 8, 2, 4, 1),
-        FD_AC_ENTRY(2, 16, 16, 1, 4, 2), FD_AC_ENTRY(2, 16, 16, 1, 3, 4),
-        FD_AC_ENTRY(2, 16, 16, 1, 5, 4), FD_AC_ENTRY(2, 16, 8, 1, 6, 4)};
+        FD_AC_ENTRY(2, 16, 8, 1, 3, 4, 0, 3.57f, 0.278f, 0.162f, 0.40f),
+        FD_AC_ENTRY(2, 16, 16, 1, 4, 2, 0, 2.44f, 0.299f, 0.269f, 0.91f)};
     static const ConfigEntry r4[] = {
-        FD_AC_ENTRY(4, 16, 8, 1, 4, 4),  FD_AC_ENTRY(4, 16, 8, 1, 3, 1),
-        FD_AC_ENTRY(4, 16, 16, 1, 4, 1), FD_AC_ENTRY(4, 16, 8, 2, 3, 1),
-        FD_AC_ENTRY(4, 16, 8, 1, 3, 4),  FD_AC_ENTRY(4, 16, 16, 1, 3, 4),
-        FD_AC_ENTRY(4, 16, 8, 1, 5, 4),  FD_AC_ENTRY(4, 16, 8, 1, 6, 4),
-        FD_AC_ENTRY(4, 16, 8, 1, 4, 2),  FD_AC_ENTRY(4, 16, 8, 1, 4, 8)};
+        FD_AC_ENTRY(4, 16, 8, 1, 3, 8, 0, 3.23f, 0.346f, 0.152f, 0.68f),
+        FD_AC_ENTRY(4, 16, 4, 2, 3, 8, 0, 2.94f, 0.458f, 0.119f, 0.73f)};
     static const ConfigEntry r6[] = {
-        FD_AC_ENTRY(6, 16, 8, 1, 3, 4),  FD_AC_ENTRY(6, 16, 8, 1, 2, 4),
-        FD_AC_ENTRY(6, 16, 16, 1, 3, 1), FD_AC_ENTRY(6, 8, 16, 1, 3, 1),
-        FD_AC_ENTRY(6, 16, 8, 1, 2, 1),  FD_AC_ENTRY(6, 16, 8, 1, 3, 2),
-        FD_AC_ENTRY(6, 16, 8, 1, 4, 4),  FD_AC_ENTRY(6, 16, 8, 1, 1, 4)};
+        FD_AC_ENTRY(6, 16, 8, 1, 3, 4, 0, 3.05f, 0.394f, 0.147f, 0.91f),
+        FD_AC_ENTRY(6, 16, 8, 2, 3, 4, 2, 2.90f, 0.513f, 0.250f, 0.85f),
+        FD_AC_ENTRY(6, 16, 22, 2, 3, 4, 1, 1.67f, 0.501f, 0.697f, 0.96f)};
     static const ConfigEntry r8[] = {
-        FD_AC_ENTRY(8, 16, 4, 1, 1, 4),  FD_AC_ENTRY(8, 16, 8, 1, 1, 4),
-        FD_AC_ENTRY(8, 16, 8, 1, 2, 1),
-        FD_AC_ENTRY(8, 16, 16, 1, 3, 1), FD_AC_ENTRY(8, 8, 16, 1, 3, 1),
-        FD_AC_ENTRY(8, 16, 8, 1, 2, 4),  FD_AC_ENTRY(8, 16, 8, 1, 1, 2),
-        FD_AC_ENTRY(8, 8, 16, 1, 1, 4),  FD_AC_ENTRY(8, 16, 8, 1, 1, 8)};
+        FD_AC_ENTRY(8, 16, 8, 1, 3, 8, 3, 3.95f, 0.372f, 0.185f, 0.89f),
+        FD_AC_ENTRY(8, 16, 4, 1, 3, 4, 0, 2.86f, 0.386f, 0.078f, 0.98f),
+        FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 2.10f, 0.689f, 0.097f, 0.97f)};
     switch (radius) {
         case 1: *count = 1; return r1;
-        case 2: *count = 8; return r2;
-        case 4: *count = 10; return r4;
-        case 6: *count = 8; return r6;
-        case 8: *count = 9; return r8;
+        case 2: *count = 2; return r2;
+        case 4: *count = 2; return r4;
+        case 6: *count = 3; return r6;
+        case 8: *count = 3; return r8;
+        default: *count = 0; return nullptr;
+    }
+}
+
+// 3-D damping field: a fourth interior tile per stage (64 x 44 tiles at so 12
+// would need a shorter ring and measured slower than 64 x 16 up to 384^3);
+// the costs fitted to 10 problems.
+const ConfigEntry *config_table_df(int radius, int *count) {
+    static const ConfigEntry r1[] = {
+        FD_AC_ENTRY_DF(1, 16, 16, 1, 3, 4, 0, 2.7f, 0.28f, 0.38f, 0.5f)};
+    static const ConfigEntry r2[] = {
+        FD_AC_ENTRY_DF(2, 16, 8, 1, 3, 4, 0, 3.17f, 0.286f, 0.185f, 0.42f)};
+    static const ConfigEntry r4[] = {
+        FD_AC_ENTRY_DF(4, 16, 8, 1, 3, 8, 0, 3.33f, 0.291f, 0.193f, 0.57f),
+        FD_AC_ENTRY_DF(4, 16, 4, 2, 3, 8, 0, 3.91f, 0.342f, 0.181f, 0.42f)};
+    static const ConfigEntry r6[] = {
+        FD_AC_ENTRY_DF(6, 16, 8, 1, 3, 4, 0, 3.24f, 0.311f, 0.195f, 0.77f),
+        FD_AC_ENTRY_DF(6, 16, 8, 2, 3, 4, 2, 3.96f, 0.372f, 0.382f, 0.61f)};
+    static const ConfigEntry r8[] = {
+        FD_AC_ENTRY_DF(8, 16, 8, 1, 3, 8, 3, 3.20f, 0.297f, 0.218f, 0.89f),
+        FD_AC_ENTRY_DF(8, 16, 4, 1, 3, 4, 0, 4.22f, 0.314f, 0.107f, 0.87f),
+        FD_AC_ENTRY_DF(8, 16, 14, 2, 3, 8, 1, 1.41f, 0.712f, 0.058f, 0.91f)};
+    switch (radius) {
+        case 1: *count = 1; return r1;
+        case 2: *count = 1; return r2;
+        case 4: *count = 2; return r4;
+        case 6: *count = 2; return r6;
+        case 8: *count = 3; return r8;
         default: *count = 0; return nullptr;
     }
 }
@@ -484,47 +517,58 @@ int acoustic_num_configs(int radius) {
     return n;
 }
 
-int acoustic_default_config(int radius) {
-    (void)radius;
-    return 0;
-}
-
 fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots, int lps,
                         float *wave, const float *bcoef, AcousticPlan *plan, int map_shots,
                         bool damp_field) {
     if (map_shots < nshots) map_shots = nshots;
     int n = 0;
-    const ConfigEntry *tab = config_table(radius, &n);
+    const ConfigEntry *tab =
+        damp_field ? config_table_df(radius, &n) : config_table(radius, &n);
     if (!tab) return set_error(FD_ERR_SO, "no acoustic kernel for radius %d", radius);
-    if (config < 0 || config >= n || damp_field) config = acoustic_default_config(radius);
-    const ConfigEntry &e = damp_field ? *config_table_df(radius) : tab[config];
-    plan->radius = radius;
-    plan->config = config;
-    plan->damp_field = damp_field;
-    plan->name = e.name;
-    plan->smem = e.smem;
-    plan->block = dim3(e.threads, 1, 1);
-    FD_TRY(raise_smem_limit(e.fn, e.smem));
-    int dev = 0, nsm = 0, per_sm = 0;
+    if (config >= n || damp_field) config = -1;
+    int dev = 0, nsm = 0, max_smem = 0;
     FD_CUDA_TRY(cudaGetDevice(&dev));
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    FD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e.fn, e.threads, e.smem));
-    if (per_sm < 1) return set_error(FD_ERR_CUDA, "kernel %s does not fit on an SM", e.name);
+    FD_CUDA_TRY(
+        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // The configuration and chunk count with the smallest estimated time.
+    int best = -1, zchunk = 0;
+    double best_us = 0.0;
+    for (int i = 0; i < n; ++i) {
+        if (config >= 0 && i != config) continue;
+        const ConfigEntry &e = tab[i];
+        int per_sm = 0;
+        FD_TRY(raise_smem_limit(e.fn, e.smem));
+        FD_CUDA_TRY(
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e.fn, e.threads, e.smem));
+        if (per_sm < 1) return set_error(FD_ERR_CUDA, "kernel %s does not fit on an SM", e.name);
+        const int64_t cols = (int64_t)((L.nx + e.bx - 1) / e.bx) *
+                             ((L.ny + e.by - 1) / e.by) * nshots;
+        int nzc = 1;
+        double planes = 0.0;
+        nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat, &planes);
+        // damp_z of a chunk follows the stages in shared memory
+        const int max_chunk = (max_smem - (int)e.smem) / 4;
+        const int min_nzc = (L.nz + max_chunk - 1) / max_chunk;
+        if (nzc < min_nzc) nzc = min_nzc;
+        if (nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
+        if (nzc < min_nzc && config < 0 && i + 1 < n) continue;
+        const double us = e.launch + e.lat * planes;
+        if (best < 0 || us < best_us) {
+            best = i;
+            best_us = us;
+            zchunk = (L.nz + nzc - 1) / nzc;
+        }
+    }
+    const ConfigEntry &e = tab[best];
+    plan->radius = radius;
+    plan->config = best;
+    plan->damp_field = damp_field;
+    plan->name = e.name;
+    plan->block = dim3(e.threads, 1, 1);
     const int ntx = (L.nx + e.bx - 1) / e.bx;
     const int nty = (L.ny + e.by - 1) / e.by;
-    const int64_t cols = (int64_t)ntx * nty * nshots;
-    // 2R warm-up planes, slightly cheaper than output planes; the load of a
-    // CTA as fitted per radius: 0.63 for 64 x 16 tiles at so 4, 0.25 and 0.30
-    // for 64 x 8 at so 8 and 12, 0.20 for 64 x 4 at so 16.
-    int nzc = 1;
-    if (L.nz > 1)
-        nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, 0.9 * 2 * radius,
-                            e.bx * e.by / (radius >= 8 ? 1280.0 : 1800.0));
-    const int min_nzc = (L.nz + 8191) / 8192;  // damp_z of a chunk: at most 32 KB
-    if (nzc < min_nzc) nzc = min_nzc;
-    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
-    const int zchunk = (L.nz + nzc - 1) / nzc;
-    nzc = (L.nz + zchunk - 1) / zchunk;
+    const int nzc = (L.nz + zchunk - 1) / zchunk;
     if ((int64_t)nshots * nzc > 65535 || nty > 65535)
         return set_error(FD_ERR_ARG, "grid too large for the launch configuration");
     plan->grid = dim3(ntx, nty, nshots * nzc);
@@ -532,8 +576,7 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
     plan->nzc = nzc;
     plan->smem = e.smem + (size_t)zchunk * 4;
     FD_TRY(raise_smem_limit(e.fn, plan->smem));
-    if (!damp_field && config == acoustic_default_config(radius))
-        FD_TRY(raise_smem_limit(config_table_wl(radius)->fn, plan->smem));
+    if (e.fn_wl) FD_TRY(raise_smem_limit(e.fn_wl, plan->smem));
     FD_TRY(make_tensor_map_4d(&plan->map_halo, wave, L.nx, L.ny, L.nz, (uint64_t)map_shots * lps,
                               (uint64_t)L.nxp * 4, (uint64_t)L.plane * 4, (uint64_t)L.vol * 4,
                               e.pw, e.ph, 1, 1));
@@ -546,9 +589,11 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
 }
 
 fd_status acoustic_launch(const AcousticPlan &plan, const AcousticStepArgs &args,
-                          cudaStream_t stream, const AcousticInject *inject) {
+                          cudaStream_t stream, const AcousticInject *inject,
+                          const ReceiveArgs *receive) {
     int n = 0;
-    const ConfigEntry *tab = config_table(plan.radius, &n);
+    const ConfigEntry *tab =
+        plan.damp_field ? config_table_df(plan.radius, &n) : config_table(plan.radius, &n);
     if (!tab || plan.config >= n) return set_error(FD_ERR_SO, "bad acoustic plan");
     AcousticInject inj;
     memset(&inj, 0, sizeof(inj));
@@ -558,17 +603,25 @@ fd_status acoustic_launch(const AcousticPlan &plan, const AcousticStepArgs &args
                              kInjectMaxSources);
         inj = *inject;
     }
+    ReceiveArgs rec;
+    memset(&rec, 0, sizeof(rec));
+    dim3 grid = plan.grid;
+    if (receive && receive->nrec > 0) {
+        rec = *receive;
+        rec.slices = receive_slices(rec, grid.x, grid.y, plan.block.x);
+        if (grid.z >= 65535) return set_error(FD_ERR_ARG, "no grid slice left for receivers");
+        if ((int64_t)grid.z + rec.slices > 65535) rec.slices = 65535 - grid.z;
+        grid.z += rec.slices;
+    }
     int zchunk = plan.zchunk, nzc = plan.nzc;
     AcousticStepArgs a = args;
     if (!a.wait_ns) a.wait_ns = wait_limit_ns();
     void *params[] = {(void *)&plan.map_halo, (void *)&plan.map_int, (void *)&plan.map_b,
-                      (void *)&a, (void *)&inj, (void *)&zchunk, (void *)&nzc};
+                      (void *)&a, (void *)&inj, (void *)&rec, (void *)&zchunk, (void *)&nzc};
     const void *fn = tab[plan.config].fn;
-    if (plan.damp_field)
-        fn = config_table_df(plan.radius)->fn;
-    else if (a.wait_ns != 0 && plan.config == acoustic_default_config(plan.radius))
-        fn = config_table_wl(plan.radius)->fn;  // same tiles, ring and shared memory
-    FD_CUDA_TRY(cudaLaunchKernel(fn, plan.grid, plan.block, params, plan.smem, stream));
+    if (a.wait_ns != 0 && tab[plan.config].fn_wl)
+        fn = tab[plan.config].fn_wl;  // same tiles, ring and shared memory
+    FD_CUDA_TRY(launch_chained(fn, grid, plan.block, params, plan.smem, stream));
     note_launch(stream);
     return FD_OK;
 }

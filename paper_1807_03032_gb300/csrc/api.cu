@@ -132,6 +132,10 @@ WaveLayout wave_layout(const fd_grid &g) {
 namespace {
 
 constexpr int kGraphChunk = 16;  // steps per captured graph (even: parity repeats)
+// Steps from which a loop of one launch per step is captured: building the
+// graph costs about 70 us and a replayed step saves about 0.5 us (64^3, 99
+// steps: 841 us direct, 908 us captured; 256^3, 237 steps: 12.95 and 12.83 ms).
+constexpr int kSingleLaunchGraph = 144;
 
 // max over theta of the squared first-derivative symbol (2 sum c_k sin k theta)^2
 double first_symbol_sq_max(int r, const double *c) {
@@ -379,9 +383,10 @@ struct NoProgress {
 // units, and at the end.
 template <class StepFn, class ProgressFn = NoProgress>
 fd_status run_time_loop(int nsteps, cudaStream_t s, int *counter, bool allow_graph,
-                        StepFn step, ProgressFn progress = ProgressFn()) {
+                        StepFn step, ProgressFn progress = ProgressFn(),
+                        int graph_from = 2 * kGraphChunk) {
     int n = 0;
-    if (allow_graph && nsteps >= 2 * kGraphChunk) {
+    if (allow_graph && nsteps >= graph_from) {
         FD_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), s));
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
@@ -595,17 +600,20 @@ static fd_status acoustic_forward_impl(const fd_grid *grid, int so, double dt, i
     bool odd_tail = false;
     if (!tiled) {
         // The receivers of step n read only u^n, which the stencil kernel of
-        // step n reads too and the kernel of step n+1 overwrites: they run on
-        // a side stream concurrently with the stencil, and only the source
-        // injection into u^{n+1} stays between two stencil launches.
-        SideLane side;
-        const bool overlap = nrec > 0;
-        if (overlap) FD_TRY(side.begin());
-        // Up to kInjectMaxSources sources per shot are injected by the
-        // stencil kernel itself (the CTA that wrote the corners), which
-        // removes a dependent launch from every step; more go through the
-        // sparse kernel.
+        // step n reads too and the kernel of step n+1 overwrites: extra blocks
+        // of the stencil launch record them.  Up to kInjectMaxSources sources
+        // per shot are injected by the stencil kernel as well (the CTA that
+        // wrote the corners); more go through the sparse kernel.  A step is
+        // then a single launch, chained to the one before it.
         const bool inject_in_k1 = nsrc > 0 && nsrc <= kInjectMaxSources;
+        const bool record_in_k1 = nrec > 0 && plan.grid.z < 65535;
+        ReceiveArgs rec;
+        memset(&rec, 0, sizeof(rec));
+        rec.tab = rec_tab;
+        rec.out = srec.dev;
+        rec.nshots = nshots;
+        rec.nrec = record_in_k1 ? nrec : 0;
+        rec.nt = nt;
         auto step = [&](int i, int par, bool via_counter) -> fd_status {
             AcousticStepArgs ai = a;
             set_two_levels(ai, par);
@@ -623,23 +631,21 @@ static fd_status acoustic_forward_impl(const fd_grid *grid, int so, double dt, i
                 inj.step_base = si.step_base;
                 inj.step = i;
             }
-            if (overlap) {
-                FD_TRY(side.fork(s));
-                FD_TRY(sparse_launch(si, i, false, true, side.get()));
-            }
+            ReceiveArgs ri = rec;
+            ri.step_base = si.step_base;
+            ri.step = i;
             if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 0), s));
-            FD_TRY(acoustic_launch(plan, ai, s, &inj));
+            FD_TRY(acoustic_launch(plan, ai, s, &inj, &ri));
             if (!via_counter && trace_level() >= 2) FD_STAGE(s, "acoustic_step kernel");
             if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 1), s));
-            FD_TRY(sparse_launch(si, i, nsrc > 0 && !inject_in_k1, !overlap && nrec > 0, s));
+            FD_TRY(sparse_launch(si, i, nsrc > 0 && !inject_in_k1, nrec > 0 && !record_in_k1, s));
             if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 2), s));
-            if (overlap) FD_TRY(side.join(s));
             if (i % kWatchEvery == kWatchEvery - 1)
                 FD_TRY(watchdog_launch(wave, L, lps * nshots, &dstats->flags, s));
             return FD_OK;
         };
         FD_TRY(run_time_loop(nsteps, s, counter, graphs, step,
-                             [&](int n) { return traces.upto(n, s); }));
+                             [&](int n) { return traces.upto(n, s); }, kSingleLaunchGraph));
     } else {
         // Two steps per launch over four levels per shot: pair i (parity par)
         // reads u^n, u^{n-1} from levels (0, 1) or (3, 2) and writes u^{n+1},

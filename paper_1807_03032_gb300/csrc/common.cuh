@@ -50,6 +50,14 @@ fd_status make_tensor_map_4d(CUtensorMap *map, const float *base, uint64_t nx, u
                              uint64_t stride_z_bytes, uint64_t stride_w_bytes, uint32_t box_x,
                              uint32_t box_y, uint32_t box_z, uint32_t box_w);
 
+// Kernel launch that may start before the previous kernel of the stream has
+// drained (programmatic stream serialisation): its prologue overlaps the
+// previous kernel's tail.  Only for kernels that call chain_wait.  Not used
+// while per-launch events are recorded (fd_stats_enable), where every launch
+// is timed by itself.
+cudaError_t launch_chained(const void *fn, dim3 grid, dim3 block, void **params, size_t smem,
+                           cudaStream_t stream);
+
 // Launch accounting (fd_launch_count): call note_launch(stream) after every
 // kernel launch.  Launches recorded while the stream is being captured are
 // counted when the graph is replayed (take_captured / add_launches).
@@ -146,6 +154,19 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, u
         " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
         : "memory");
+}
+
+// Programmatic dependent launch (see launch_chained): the next launch of the
+// stream may start its blocks once every block of this one has called
+// chain_trigger or exited; chain_wait blocks until the previous launch is
+// complete and its writes are visible, and returns at once for a launch that
+// does not overlap.  Every thread of a chained kernel calls chain_wait before
+// it touches anything an earlier launch writes or reads.
+__device__ __forceinline__ void chain_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map) {

@@ -54,6 +54,8 @@ __device__ __forceinline__ float corner_w(const SparsePoint &p, int c) {
 
 // Threads [0, nactive*max_nrec) record traces; then nactive*max_nsrc*8 inject.
 __global__ void engine_sparse_kernel(const EngineSparseArgs e, int offset, int cur) {
+    chain_wait();
+    chain_trigger();
     const int G = *e.gstep + offset;
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nrec_all = (int64_t)e.nactive * e.max_nrec;
@@ -68,7 +70,7 @@ __global__ void engine_sparse_kernel(const EngineSparseArgs e, int offset, int c
         const float *u = e.wave + (int64_t)(2 * slot + cur) * e.L.vol;
         float acc = 0.f;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc = fmaf(corner_w(p, c), __ldg(u + corner_off(p, c, e.L)), acc);
+        for (int c = 0; c < 8; ++c) acc = fmaf(corner_w(p, c), __ldcg(u + corner_off(p, c, e.L)), acc);
         d.out[(int64_t)n * d.nrec + r] = acc;
         return;
     }
@@ -321,8 +323,10 @@ static fd_status engine_one_step(Engine *e, int offset, int cur) {
     sp.gstep = e->gstep;
     const int64_t total = (int64_t)e->nactive * (e->max_nrec + 8 * e->max_nsrc);
     if (total > 0) {
-        engine_sparse_kernel<<<(unsigned)((total + 255) / 256), 256, 0, e->stream>>>(sp, offset, cur);
-        FD_CUDA_TRY(cudaGetLastError());
+        void *params[] = {(void *)&sp, (void *)&offset, (void *)&cur};
+        FD_CUDA_TRY(launch_chained((const void *)&engine_sparse_kernel,
+                                   dim3((unsigned)((total + 255) / 256)), dim3(256), params, 0,
+                                   e->stream));
         note_launch(e->stream);
     }
     return FD_OK;

@@ -126,8 +126,20 @@ struct AcousticInject {
     int step;
 };
 
+// Receivers recorded by a stencil launch itself: extra blocks behind the
+// columns' (z slices of the grid) interpolate trace sample n = step +
+// *step_base from level u^n, which the launch only reads.
+struct ReceiveArgs {
+    const SparsePoint *tab;  // [nshots][nrec]
+    float *out;              // [nshots][nt][nrec]
+    int nshots, nrec, nt;    // nrec = 0: none
+    const int *step_base;
+    int step;
+    int mean;                // TTI: record the mean of p and r
+    int slices;              // z slices of receiver blocks (set by the launch)
+};
+
 int acoustic_num_configs(int radius);
-int acoustic_default_config(int radius);
 // `lps` levels per shot are addressable (buffers nshots * lps).  The launch
 // covers `nshots` shots; the tensor maps cover `map_shots` shots (default:
 // nshots) for callers that map launch shots to slots (slot_map).
@@ -137,7 +149,8 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
                         float *wave, const float *bcoef, AcousticPlan *plan, int map_shots = 0,
                         bool damp_field = false);
 fd_status acoustic_launch(const AcousticPlan &plan, const AcousticStepArgs &args,
-                          cudaStream_t stream, const AcousticInject *inject = nullptr);
+                          cudaStream_t stream, const AcousticInject *inject = nullptr,
+                          const ReceiveArgs *receive = nullptr);
 
 // ---------------------------------------------------------------- time-tiled K1
 

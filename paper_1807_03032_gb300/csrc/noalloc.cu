@@ -212,13 +212,21 @@ fd_status noalloc_impl(const fd_grid *g, int so, double dt, int nt, int nshots, 
         inj.nsrc = nsrc;
         inj.nt = nt;
     }
+    const bool record_in_k1 = nrec > 0 && plan.grid.z < 65535;
+    ReceiveArgs rec;
+    memset(&rec, 0, sizeof(rec));
+    rec.tab = rec_tab;
+    rec.out = rec_out;
+    rec.nshots = nshots;
+    rec.nrec = record_in_k1 ? nrec : 0;
+    rec.nt = nt;
     for (int n = 0; n + 1 < nt; ++n) {
         set_two_levels(a, n & 1);
-        inj.step = n;
-        FD_TRY(acoustic_launch(plan, a, s, &inj));
+        inj.step = rec.step = n;
+        FD_TRY(acoustic_launch(plan, a, s, &inj, &rec));
         sp.inj_level0 = 1 - (n & 1);
         sp.rec_level = n & 1;
-        FD_TRY(sparse_launch(sp, n, nsrc > 0 && !inject_in_k1, nrec > 0, s));
+        FD_TRY(sparse_launch(sp, n, nsrc > 0 && !inject_in_k1, nrec > 0 && !record_in_k1, s));
     }
     const int last = (nt - 1) & 1;
     sp.rec_level = last;

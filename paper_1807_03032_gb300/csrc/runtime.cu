@@ -46,6 +46,21 @@ void note_launch(cudaStream_t s) {
         g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
+cudaError_t launch_chained(const void *fn, dim3 grid, dim3 block, void **params, size_t smem,
+                           cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = stats_enabled() ? 0 : 1;
+    return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
 int64_t take_captured() {
     const int64_t n = t_captured;
     t_captured = 0;
@@ -206,7 +221,8 @@ fd_status raise_smem_limit(const void *fn, size_t bytes) {
     return FD_OK;
 }
 
-int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load) {
+int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load,
+                  double *planes) {
     const int64_t slots = (int64_t)nsm * per_sm;
     // beyond a few waves more chunks only add warm-up planes
     const int64_t most = 8 * slots / (cols > 0 ? cols : 1) + 8;
@@ -227,13 +243,13 @@ int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, doub
             if (k < 1.0) k = 1.0;
             waves += h(0.5 * (k + ceil(k)));
         }
-        double cost = (chunk + warmup) * waves;
-        if (n == 1) cost *= 1.06;  // measured 3 - 6 % above the estimate
+        const double cost = (chunk + warmup) * waves;
         if (n == 1 || cost < best_cost) {
             best_cost = cost;
             best = n;
         }
     }
+    if (planes) *planes = best_cost;
     return best;
 }
 

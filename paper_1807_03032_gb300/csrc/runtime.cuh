@@ -52,7 +52,9 @@ fd_status raise_smem_limit(const void *fn, size_t bytes);
 // acoustic 64^3 so 4 20.1 against 7.2 us per step, 256^3 so 8 77 against 53,
 // 384^3 so 8 170 against 142; TTI 48^3 so 4 85 against 15, 256^3 so 8 382
 // against 301.
-int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load);
+// `planes` (optional) receives the estimate.
+int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load,
+                  double *planes = nullptr);
 
 // Host-side fault injection for tests: with the environment variable
 // FDSWEEP_FAIL_ALLOC=1 every device allocation of the library (per-call

@@ -27,6 +27,8 @@ __device__ __forceinline__ int64_t corner_offset(const SparsePoint &p, int c, co
 // Threads [0, nrec_total) interpolate receivers (nrec_total = 0 when only
 // injecting); the following nshots*nsrc*8 threads inject.
 __global__ void sparse_kernel(const SparseArgs a, int step, int do_inject, int64_t nrec_total) {
+    chain_wait();
+    chain_trigger();
     const int n = step + (a.step_base ? *a.step_base : 0);
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid < nrec_total) {
@@ -42,12 +44,12 @@ __global__ void sparse_kernel(const SparseArgs a, int step, int do_inject, int64
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const int64_t o = corner_offset(p, c, a.L);
-                acc = fmaf(corner_weight(p, c), 0.5f * (__ldg(u + o) + __ldg(u2 + o)), acc);
+                acc = fmaf(corner_weight(p, c), 0.5f * (__ldcg(u + o) + __ldcg(u2 + o)), acc);
             }
         } else {
 #pragma unroll
             for (int c = 0; c < 8; ++c)
-                acc = fmaf(corner_weight(p, c), __ldg(u + corner_offset(p, c, a.L)), acc);
+                acc = fmaf(corner_weight(p, c), __ldcg(u + corner_offset(p, c, a.L)), acc);
         }
         a.rec_out[((int64_t)s * a.nt + ro) * a.nrec + i] = acc;
         return;
@@ -118,9 +120,11 @@ fd_status sparse_launch(const SparseArgs &a, int step, bool do_inject, bool do_i
     if (total == 0) return FD_OK;
     const int threads = 256;
     const int64_t blocks = (total + threads - 1) / threads;
-    sparse_kernel<<<(unsigned)blocks, threads, 0, stream>>>(a, step, do_inject ? 1 : 0,
-                                                            nrec_total);
-    FD_CUDA_TRY(cudaGetLastError());
+    int inject = do_inject ? 1 : 0;
+    int64_t nrec = nrec_total;
+    void *params[] = {(void *)&a, (void *)&step, (void *)&inject, (void *)&nrec};
+    FD_CUDA_TRY(launch_chained((const void *)&sparse_kernel, dim3((unsigned)blocks), dim3(threads),
+                               params, 0, stream));
     note_launch(stream);
     return FD_OK;
 }

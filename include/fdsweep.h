@@ -184,8 +184,9 @@ fd_status acoustic_forward_opts(const fd_grid *grid, int so, double dt, int nt, 
  *   rec_out   [nshots][nt][nrec] samples of p.
  *   Other arguments as for acoustic_forward.
  * The kernels: one fused kernel per step with the first-derivative
- * temporaries in shared memory for so <= 4, two passes with the temporaries
- * in device memory above (see tti_forward_opts).
+ * temporaries in shared memory for so <= 4 (from about 128^3 points), two
+ * passes with the temporaries in device memory otherwise (see
+ * tti_forward_opts).
  */
 fd_status tti_forward(const fd_grid *grid, int so, double dt, int nt, int nshots, const float *m,
                       const float *damp, const float *epsilon, const float *delta,
@@ -211,8 +212,9 @@ fd_status tti_forward(const fd_grid *grid, int so, double dt, int nt, int nshots
  *                   stability bound uses the staggered symbol.
  *   opts->receiver  FD_TTI_REC_P: receivers record p; FD_TTI_REC_MEAN: they
  *                   record (p + r)/2.
- *   opts->scheme    FD_TTI_AUTO (what tti_forward uses): FD_TTI_FUSED for
- *                   so <= 4, FD_TTI_TWO_PASS otherwise (the faster on GB300);
+ *   opts->scheme    FD_TTI_AUTO (what tti_forward uses): the faster on GB300:
+ *                   FD_TTI_TWO_PASS for so > 4 and for small grids (about
+ *                   128^3 and below), FD_TTI_FUSED otherwise;
  *                   FD_TTI_TWO_PASS: six first-derivative temporaries per
  *                   point are written to device memory once and
  *                   differentiated again by a second kernel (the default,
@@ -461,7 +463,7 @@ int fd_num_time_tiling_configs(int so);
  * given space order (0 .. fd_num_tti_configs(so) - 1), or -1 for the
  * built-in choice.  Applies to centred derivatives of the two-pass scheme
  * (the staggered reading always uses the built-in choice); for the fused
- * scheme configuration 1 selects 64 x 16 tiles instead of 64 x 8 (other
+ * scheme configuration 1 selects 64 x 8 tiles instead of 64 x 16 (other
  * values: the built-in choice).  Process-wide; FD_ERR_ARG if out of range.
  */
 fd_status fd_set_tti_config(int so, int config);

@@ -41,6 +41,7 @@
 #include "f32x2.cuh"
 #include "kernels.cuh"
 #include "receive.cuh"
+#include "ring.cuh"
 #include "runtime.cuh"
 
 namespace fdsweep {
@@ -73,26 +74,6 @@ struct AcCfg {
     static constexpr size_t SMEM = (size_t)NSL * STAGE * 4 + NSL * 16 + 16 + 128;
     static_assert(PW <= 256 && PH <= 256 && BX <= 256 && BY <= 256, "TMA box dimension limit");
     static_assert(INT % 32 == 0 && CONSUMERS % 32 == 0, "tile shape");
-};
-
-// Position in a ring of N stages: from the plane index where N is a power of
-// two (constant stage addresses in an unrolled loop), counted otherwise.
-template <int N>
-struct RingPos {
-    int s = 0;
-    uint32_t ph = 0;
-    static constexpr bool POW2 = (N & (N - 1)) == 0;
-    __device__ __forceinline__ int slot(int j) const { return POW2 ? j % N : s; }
-    __device__ __forceinline__ uint32_t phase(int j) const {
-        return POW2 ? (uint32_t)(j / N) & 1u : ph;
-    }
-    __device__ __forceinline__ void next() {
-        if (POW2) return;
-        if (++s == N) {
-            s = 0;
-            ph ^= 1u;
-        }
-    }
 };
 
 // Source injection by the CTA that wrote a source's corners, after its

@@ -132,10 +132,11 @@ WaveLayout wave_layout(const fd_grid &g) {
 namespace {
 
 constexpr int kGraphChunk = 16;  // steps per captured graph (even: parity repeats)
-// Steps from which a loop of one launch per step is captured: building the
-// graph costs about 70 us and a replayed step saves about 0.5 us (64^3, 99
-// steps: 841 us direct, 908 us captured; 256^3, 237 steps: 12.95 and 12.83 ms).
-constexpr int kSingleLaunchGraph = 144;
+// Steps from which a loop of one or two launches per step is captured:
+// building the graph costs about 70 us and a replayed step saves about 0.5 us
+// (64^3, 99 steps: 841 us direct, 908 us captured; 256^3, 237 steps: 12.95 and
+// 12.83 ms).
+constexpr int kFewLaunchesGraph = 144;
 
 // max over theta of the squared first-derivative symbol (2 sum c_k sin k theta)^2
 double first_symbol_sq_max(int r, const double *c) {
@@ -645,7 +646,7 @@ static fd_status acoustic_forward_impl(const fd_grid *grid, int so, double dt, i
             return FD_OK;
         };
         FD_TRY(run_time_loop(nsteps, s, counter, graphs, step,
-                             [&](int n) { return traces.upto(n, s); }, kSingleLaunchGraph));
+                             [&](int n) { return traces.upto(n, s); }, kFewLaunchesGraph));
     } else {
         // Two steps per launch over four levels per shot: pair i (parity par)
         // reads u^n, u^{n-1} from levels (0, 1) or (3, 2) and writes u^{n+1},
@@ -988,10 +989,12 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
          op.scheme != FD_TTI_RECOMPUTE && op.scheme != FD_TTI_FUSED))
         return set_error(FD_ERR_ARG, "tti_forward: options (%d, %d, %d) out of range", op.deriv,
                          op.receiver, op.scheme);
-    // automatic: the fused kernel where it was measured faster (so <= 4:
-    // 1.76 against 2.12 ms per 512^3 step at so 4), two passes otherwise
-    if (op.scheme == FD_TTI_AUTO)
-        op.scheme = (so <= 4 && tti_fused_supported(so / 2)) ? FD_TTI_FUSED : FD_TTI_TWO_PASS;
+    if (op.scheme == FD_TTI_AUTO) {
+        int scheme = kTtiTwoPass;
+        FD_TRY(tti_choose_scheme(so / 2, op.deriv == FD_TTI_STAGGERED, wave_layout(*grid), nshots,
+                                 &scheme));
+        op.scheme = scheme == kTtiFused ? FD_TTI_FUSED : FD_TTI_TWO_PASS;
+    }
     if (op.scheme == FD_TTI_FUSED && !tti_fused_supported(so / 2))
         return set_error(FD_ERR_ARG, "tti_forward: the fused scheme covers so <= 8 (so = %d)",
                          so);
@@ -1142,26 +1145,48 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
     const bool timing = stats_enabled();
     StepEvents evs;
     if (timing) FD_TRY(evs.create(nsteps, 4));
+    // the kernels inject and record themselves, like the acoustic step
+    const bool inject_in_step = (two_pass || fused) && nsrc > 0 && nsrc <= kInjectMaxSources;
+    const bool record_in_step = nrec > 0 && tti_records_receivers(tplan);
+    AcousticInject inj;
+    memset(&inj, 0, sizeof(inj));
+    if (inject_in_step) {
+        inj.src_tab = src_tab;
+        inj.src_wav = swav.dev;
+        inj.nsrc = nsrc;
+        inj.nt = nt;
+    }
+    ReceiveArgs rec;
+    memset(&rec, 0, sizeof(rec));
+    rec.tab = rec_tab;
+    rec.out = srec.dev;
+    rec.nshots = nshots;
+    rec.nrec = record_in_step ? nrec : 0;
+    rec.nt = nt;
+    rec.mean = sp.rec_mean;
     auto step = [&](int i, int par, bool via_counter) -> fd_status {
         TtiArgs ai = a;
         ai.cur = par;
         cudaEvent_t ev3[3];
         if (timing)
             for (int k = 0; k < 3; ++k) ev3[k] = evs.at(i, k);
-        FD_TRY(tti_launch(tplan, ai, s, timing ? ev3 : nullptr));
+        inj.step = rec.step = i;
+        inj.step_base = rec.step_base = via_counter ? counter : nullptr;
+        FD_TRY(tti_launch(tplan, ai, s, timing ? ev3 : nullptr, &inj, &rec));
         SparseArgs si = sp;
         si.inj_level0 = 1 - par;
         si.inj_level1 = 3 - par;
         si.rec_level = par;
         si.rec_level2 = 2 + par;
         si.step_base = via_counter ? counter : nullptr;
-        FD_TRY(sparse_launch(si, i, nsrc > 0, nrec > 0, s));
+        FD_TRY(sparse_launch(si, i, nsrc > 0 && !inject_in_step, nrec > 0 && !record_in_step, s));
         if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 3), s));
         if (i % kWatchEvery == kWatchEvery - 1)
             FD_TRY(watchdog_launch(wave, L, 4 * nshots, &dstats->flags, s));
         return FD_OK;
     };
-    FD_TRY(run_time_loop(nsteps, s, counter, !timing && trace_level() < 2, step));
+    FD_TRY(run_time_loop(nsteps, s, counter, !timing && trace_level() < 2, step, NoProgress(),
+                         kFewLaunchesGraph));
     FD_STAGE(s, "tti: time loop");
     const int last = nsteps & 1;
     {
@@ -1350,7 +1375,8 @@ static fd_status acoustic_adjoint_impl(const fd_grid *grid, int so, double dt, i
         FD_TRY(sparse_launch(si, i, nrec > 0, nsrc > 0, s));
         return FD_OK;
     };
-    FD_TRY(run_time_loop(nsteps, s, counter, trace_level() < 2, step));
+    FD_TRY(run_time_loop(nsteps, s, counter, trace_level() < 2, step, NoProgress(),
+                         kFewLaunchesGraph));
     FD_STAGE(s, "adjoint: time loop");
     FD_TRY(check_finite(wave, L, 2 * nshots, &dstats->flags, s));
     FD_TRY(sgrad.copy_back(s));

@@ -292,18 +292,27 @@ struct TtiArgs {
 
 enum TtiScheme { kTtiTwoPass = 0, kTtiRecompute = 1, kTtiFused = 2 };
 
+// Launch of one kernel of a TTI step.
+struct TtiPassPlan {
+    const void *fn = nullptr;
+    dim3 grid, block;
+    size_t smem = 0;
+    int zchunk = 0, nzc = 1;
+    int bx = 0, by = 0, pw = 0, ph = 0;  // tile, x-halo width, y-halo height
+    double est_us = 0.0;                 // estimated time
+};
+
 struct TtiPlan {
     int radius = 0;
     int stag = 0;    // 0: centred first derivatives, 1: staggered (D+ inner, D- outer)
     int scheme = kTtiTwoPass;
-    int config = 0;  // launch configuration of the two passes (tti_num_configs)
-    CUtensorMap map_wint, map_whalo;          // p/r buffers: interior, x+y halo boxes
-    CUtensorMap map_tint, map_tx, map_ty;     // temporaries: interior, x-halo, y-halo
-    CUtensorMap map_cint;                     // b, a, s, n_x, n_y, n_z: interior box
-    CUtensorMap map_fbox, map_fnbox;          // fused scheme: p/r plane box, n box
-    dim3 grid, block;
-    size_t smem1 = 0, smem2 = 0;
-    int zchunk = 0, nzc = 1;
+    int config = 0;  // tile choice of the fused scheme
+    TtiPassPlan p1, p2;                        // p1 alone: fused and recompute schemes
+    CUtensorMap map_wint, map_whalo;           // p, r of a level: interior, x+y halo boxes
+    CUtensorMap map_wlev;                      // p, r at both levels: interior box
+    CUtensorMap map_tint, map_tx, map_ty;      // temporaries: interior, x-halo, y-halo
+    CUtensorMap map_c1, map_c2;                // three coefficient fields: interior boxes
+    CUtensorMap map_fbox, map_fnbox;           // fused scheme: p/r plane box, n box
 };
 
 // coef: 6 consecutive fields b, a, s, n_x, n_y, n_z ([6][vol]).  scheme
@@ -319,9 +328,20 @@ int tti_num_configs(int radius);
 bool tti_fused_supported(int radius);
 fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, float *wave,
                          const float *coef, TtiPlan *plan, int config = 0);
-fd_status tti_fused_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream);
+fd_status tti_fused_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
+                           const AcousticInject &inj, const ReceiveArgs &receive);
+// inject, receive: done by the step's own kernels (not with the recompute
+// scheme; see tti_records_receivers); at most kInjectMaxSources sources.
+// Estimated time (us) of a fused step.
+fd_status tti_fused_time(int radius, int stag, const WaveLayout &L, int nshots, double *us);
+// The automatic scheme (kTtiTwoPass or kTtiFused) for a problem.
+fd_status tti_choose_scheme(int radius, int stag, const WaveLayout &L, int nshots, int *scheme);
 fd_status tti_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
-                     cudaEvent_t *ev /* 3 events or null */);
+                     cudaEvent_t *ev /* 3 events or null */,
+                     const AcousticInject *inject = nullptr,
+                     const ReceiveArgs *receive = nullptr);
+// Whether tti_launch can record receivers for this plan.
+bool tti_records_receivers(const TtiPlan &plan);
 
 // ---------------------------------------------------------------- binary16 storage
 

@@ -16,7 +16,7 @@ inline int receive_slices(const ReceiveArgs &r, int ntx, int nty, int threads) {
 
 // rec[n][i] = sum_c w_c u^n(node_c), or of (u + u2) / 2.  Reads through L2:
 // the launch may overlap the one that wrote u^n.
-__device__ __noinline__ void record_receivers(const ReceiveArgs *r, const float *wave, int lps,
+static __device__ __noinline__ void record_receivers(const ReceiveArgs *r, const float *wave, int lps,
                                               int lev, int lev2, const WaveLayout *L) {
     const int n = r->step + (r->step_base ? *r->step_base : 0);
     if (n < 0 || n >= r->nt) return;

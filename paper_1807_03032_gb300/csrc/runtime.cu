@@ -134,11 +134,11 @@ fd_status make_tensor_map_4d(CUtensorMap *map, const float *base, uint64_t nx, u
                                    stride_w_bytes, box_x, box_y, box_z, box_w);
 }
 
-fd_status make_tensor_map_4d_elem(CUtensorMap *map, const void *base, int elem_bytes,
-                                  uint64_t nx, uint64_t ny, uint64_t nz, uint64_t nw,
-                                  uint64_t stride_y_bytes, uint64_t stride_z_bytes,
-                                  uint64_t stride_w_bytes, uint32_t box_x, uint32_t box_y,
-                                  uint32_t box_z, uint32_t box_w) {
+namespace {
+
+fd_status encode_tensor_map(CUtensorMap *map, const void *base, int elem_bytes, int rank,
+                            const uint64_t *dims_in, const uint64_t *strides_in,
+                            const uint32_t *box_in) {
     if (elem_bytes != 4 && elem_bytes != 2)
         return set_error(FD_ERR_ARG, "tensor map: element size %d not supported", elem_bytes);
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -155,22 +155,43 @@ fd_status make_tensor_map_4d_elem(CUtensorMap *map, const void *base, int elem_b
     if (!encode)
         return set_error(FD_ERR_CUDA, "cuTensorMapEncodeTiled not available (%s)",
                          cudaGetErrorString(lookup_err));
-    cuuint64_t dims[4] = {nx, ny, nz, nw};
-    cuuint64_t strides[3] = {stride_y_bytes, stride_z_bytes, stride_w_bytes};
-    cuuint32_t box[4] = {box_x, box_y, box_z, box_w};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
+    cuuint64_t dims[5], strides[4];
+    cuuint32_t box[5], estr[5];
+    for (int d = 0; d < rank; ++d) {
+        dims[d] = dims_in[d];
+        box[d] = box_in[d];
+        estr[d] = 1;
+        if (d > 0) strides[d - 1] = strides_in[d - 1];
+    }
     const CUtensorMapDataType dtype =
         elem_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    CUresult r = encode(map, dtype, 4, const_cast<void *>(base), dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    CUresult r = encode(map, dtype, rank, const_cast<void *>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return set_error(FD_ERR_CUDA,
                          "cuTensorMapEncodeTiled failed (%d): dims %llu %llu %llu %llu box %u %u",
-                         (int)r, (unsigned long long)nx, (unsigned long long)ny,
-                         (unsigned long long)nz, (unsigned long long)nw, box_x, box_y);
+                         (int)r, (unsigned long long)dims[0], (unsigned long long)dims[1],
+                         (unsigned long long)dims[2], (unsigned long long)dims[3], box[0], box[1]);
     return FD_OK;
+}
+
+}  // namespace
+
+fd_status make_tensor_map_4d_elem(CUtensorMap *map, const void *base, int elem_bytes,
+                                  uint64_t nx, uint64_t ny, uint64_t nz, uint64_t nw,
+                                  uint64_t stride_y_bytes, uint64_t stride_z_bytes,
+                                  uint64_t stride_w_bytes, uint32_t box_x, uint32_t box_y,
+                                  uint32_t box_z, uint32_t box_w) {
+    const uint64_t dims[4] = {nx, ny, nz, nw};
+    const uint64_t strides[3] = {stride_y_bytes, stride_z_bytes, stride_w_bytes};
+    const uint32_t box[4] = {box_x, box_y, box_z, box_w};
+    return encode_tensor_map(map, base, elem_bytes, 4, dims, strides, box);
+}
+
+fd_status make_tensor_map_5d(CUtensorMap *map, const float *base, const uint64_t dims[5],
+                             const uint64_t strides[4], const uint32_t box[5]) {
+    return encode_tensor_map(map, base, 4, 5, dims, strides, box);
 }
 
 int trace_level() {

@@ -26,6 +26,11 @@ fd_status make_tensor_map_4d_elem(CUtensorMap *map, const void *base, int elem_b
                                   uint64_t stride_w_bytes, uint32_t box_x, uint32_t box_y,
                                   uint32_t box_z, uint32_t box_w);
 
+// TMA descriptor of a 5-D FP32 tensor (x, y, z, v, w) with x contiguous, for
+// copies of several fields at once; strides in bytes for dims 1..4.
+fd_status make_tensor_map_5d(CUtensorMap *map, const float *base, const uint64_t dims[5],
+                             const uint64_t strides[4], const uint32_t box[5]);
+
 // Raises a kernel's dynamic shared-memory limit on the current device to at
 // least `bytes`, never lowering it: the limit belongs to the function and is
 // shared by every thread and call, so one call must not lower the limit

@@ -19,20 +19,35 @@
 //
 // GB300 design (both passes, like the acoustic step): one CTA owns a BX x BY
 // column and marches it through z.  The z-derivatives use an accumulator
-// pipeline (2R pending outputs per point in registers, fed by the interior
-// tile of each arriving plane); the x/y derivatives of the output plane
-// s = p - R come from tiles staged with their halo.  Every operand arrives by
-// cp.async.bulk.tensor into a (D+1)-slot ring with full/empty mbarriers.  The
-// CTA has two thread groups: in K2a one differentiates p and the other r; in
-// K2b one builds A = Hxy p and the other B = Hz r, they exchange A and B
-// through shared memory, and update p and r respectively.
+// pipeline (2R pending outputs per point and field in registers, fed by the
+// interior tile of each arriving plane); the x/y derivatives of the output
+// plane s = p - R come from tiles staged with their halo.  Every operand
+// arrives by cp.async.bulk.tensor, several fields per copy (three copies per
+// plane in K2a, five in K2b), issued by a producer warp into a ring of stages
+// with full/empty mbarriers.  A thread owns four x points of BOTH fields: it
+// reads n (K2a) and b, a, s (K2b) once for the two, and K2b needs no exchange
+// of Hxy p and Hz r between threads, so warps never meet at a barrier.  (With
+// one thread group per field, one copy per field and tile and a consumer
+// thread as the producer, a plane of both passes took 1.4 us for a lone CTA;
+// see the launch tables for what this layout measures.)
+//
+// A time step is two launches, chained to each other: K2a's extra blocks
+// record the receivers of p^n (or (p + r)/2), K2b's CTAs inject the sources
+// into the nodes they own.
+#include <string.h>
+
 #include "kernels.cuh"
+#include "receive.cuh"
+#include "ring.cuh"
 #include "runtime.cuh"
+#include "tti_inject.cuh"
 #include "tti_stencil.cuh"
 
 namespace fdsweep {
 namespace {
 using namespace tti;
+
+constexpr int round32(int n) { return (n + 31) / 32 * 32; }
 
 template <int R, int TX, int TY, int D>
 struct TtiCfg {
@@ -42,22 +57,28 @@ struct TtiCfg {
     static constexpr int PW = BX + 2 * RA;       // x-halo width
     static constexpr int PH = BY + 2 * R;        // y-halo height
     static constexpr int NSL = D + 1;
-    static constexpr int GROUP = TX * TY;        // threads per group
-    static constexpr int THREADS = 2 * GROUP;
-    static constexpr int WARPS = THREADS / 32;
+    static constexpr int CONSUMERS = TX * TY;
+    static constexpr int WARPS = CONSUMERS / 32;
+    static constexpr int THREADS = CONSUMERS + 32;
     static constexpr int INT = BX * BY;
-    static constexpr int HXY = (PW * PH + 31) / 32 * 32;  // x+y halo tile
-    static constexpr int HX = (PW * BY + 31) / 32 * 32;   // x-halo tile
-    static constexpr int HY = (BX * PH + 31) / 32 * 32;   // y-halo tile
-    // pass 1 stage: [p(j)][r(j)] interiors, [p(s)][r(s)] xy-halo, [nx][ny][nz](s)
-    static constexpr int STAGE1 = 2 * INT + 2 * HXY + 3 * INT;
-    // pass 2 stage: [fz(j)][ez(j)], [fx(s)][ex(s)] x-halo, [fy(s)][ey(s)] y-halo,
-    //               [p][p-][r][r-][b][a][s](s)
-    static constexpr int STAGE2 = 2 * INT + 2 * HX + 2 * HY + 7 * INT;
+    static constexpr int HXY = PW * PH;  // x+y halo tile
+    static constexpr int HX = PW * BY;   // x-halo tile
+    static constexpr int HY = BX * PH;   // y-halo tile
+    // pass 1 stage: [p | r](j) interiors, [p | r](s) xy-halo, [nx | ny | nz](s)
+    static constexpr int OFF1_H = round32(2 * INT);
+    static constexpr int OFF1_N = OFF1_H + round32(2 * HXY);
+    static constexpr int STAGE1 = OFF1_N + round32(3 * INT);
+    // pass 2 stage: [fz | ez](j), [fx | ex](s) x-halo, [fy | ey](s) y-halo,
+    //               [p0 | p1 | r0 | r1](s) both levels, [b | a | s](s)
+    static constexpr int OFF2_X = round32(2 * INT);
+    static constexpr int OFF2_Y = OFF2_X + round32(2 * HX);
+    static constexpr int OFF2_W = OFF2_Y + round32(2 * HY);
+    static constexpr int OFF2_C = OFF2_W + round32(4 * INT);
+    static constexpr int STAGE2 = OFF2_C + round32(3 * INT);
     static constexpr size_t SMEM1 = (size_t)NSL * STAGE1 * 4 + NSL * 16 + 16 + 128;
-    static constexpr size_t SMEM2 = (size_t)NSL * STAGE2 * 4 + 4 * INT * 4 + NSL * 16 + 16 + 128;
+    static constexpr size_t SMEM2 = (size_t)NSL * STAGE2 * 4 + NSL * 16 + 16 + 128;
     static_assert(PW <= 256 && PH <= 256, "TMA box dimension limit");
-    static_assert(GROUP % 32 == 0, "thread groups must be whole warps");
+    static_assert(CONSUMERS % 32 == 0, "whole consumer warps");
 };
 
 struct Ring {
@@ -67,11 +88,11 @@ struct Ring {
 };
 
 template <int NSL, int WARPS>
-__device__ __forceinline__ Ring ring_init(unsigned char *raw, size_t stage_floats, int extra_floats) {
+__device__ __forceinline__ Ring ring_init(unsigned char *raw, size_t stage_floats) {
     Ring r;
     r.smem = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(raw) + 127) &
                                        ~static_cast<uintptr_t>(127));
-    r.full = reinterpret_cast<uint64_t *>(r.smem + NSL * stage_floats + extra_floats);
+    r.full = reinterpret_cast<uint64_t *>(r.smem + NSL * stage_floats);
     r.empty = r.full + NSL;
     r.abort_flag = reinterpret_cast<volatile int *>(r.empty + NSL);
     if (threadIdx.x == 0) {
@@ -85,272 +106,287 @@ __device__ __forceinline__ Ring ring_init(unsigned char *raw, size_t stage_float
     return r;
 }
 
+// The producer lane's loop: waits for each stage to be released by every
+// consumer warp and fills it with fill(jj, stage, barrier) (which announces
+// its bytes first).  Returns the number of stages issued.
+template <int NSL, class Fill>
+__device__ __forceinline__ int produce(const Ring &ring, size_t stage_floats, int nplanes,
+                                       unsigned int *err, Fill fill) {
+    int issued = 0;
+    RingPos<NSL> pos;
+    for (int jj = 0; jj < nplanes && !*ring.abort_flag; ++jj, pos.next()) {
+        const int slot = pos.slot(jj);
+        if (jj >= NSL && !mbar_wait_bounded(&ring.empty[slot], pos.phase(jj) ^ 1u)) {
+            if (!*ring.abort_flag) atomicOr(err, DEV_ERR_TIMEOUT);
+            *ring.abort_flag = 1;
+            break;
+        }
+        fill(jj, ring.smem + slot * stage_floats, &ring.full[slot]);
+        issued = jj + 1;
+    }
+    chain_trigger();  // the next launch may move in (see acoustic.cu)
+    return issued;
+}
+
+// After an aborted column: the copies in flight get a bounded chance to land
+// before the CTA's shared memory is released.
+template <int NSL>
+__device__ __forceinline__ void drain(const Ring &ring, int issued) {
+    for (int jj = issued - NSL; jj < issued; ++jj)
+        if (jj >= 0)
+            mbar_wait_bounded(&ring.full[jj % NSL], (uint32_t)((jj / NSL) & 1), 200000000ull);
+}
+
 // ---------------------------------------------------------------- pass 1
 
-template <int R, int TX, int TY, int D, int KIND, int U>
-__global__ void __launch_bounds__(2 * TX * TY)
+template <int R, int TX, int TY, int D, int KIND, int U, int MINB>
+__global__ void __launch_bounds__(TX *TY + 32, MINB)
     tti_pass1_kernel(const __grid_constant__ CUtensorMap map_wint,
                      const __grid_constant__ CUtensorMap map_whalo,
-                     const __grid_constant__ CUtensorMap map_cint, const TtiArgs a, int zchunk,
-                     int nzc) {
+                     const __grid_constant__ CUtensorMap map_cint,
+                     const __grid_constant__ TtiArgs a, const __grid_constant__ ReceiveArgs rec,
+                     int zchunk, int nzc) {
     using C = TtiCfg<R, TX, TY, D>;
-    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;  // stopped by the divergence watchdog
+    if (blockIdx.z >= gridDim.z - rec.slices) {
+        chain_trigger();
+        chain_wait();
+        if (!(__ldcg(a.err) & DEV_ERR_NONFINITE))
+            record_receivers(&rec, a.wave, 4, a.cur, 2 + a.cur, &a.L);
+        return;
+    }
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    Ring ring = ring_init<C::NSL, C::WARPS>(smem_raw, C::STAGE1, 0);
+    Ring ring = ring_init<C::NSL, C::WARPS>(smem_raw, C::STAGE1);
     const int tid = threadIdx.x, lane = tid & 31;
-    const int field = tid / C::GROUP;  // 0: p, 1: r
-    const int t = tid - field * C::GROUP;
-    const int tx = t % TX, ty = t / TX;
+    const int tx = tid % TX, ty = tid / TX;
     const int shot = blockIdx.z / nzc, chunk = blockIdx.z - shot * nzc;
     const int x0 = blockIdx.x * C::BX, y0 = blockIdx.y * C::BY;
     const int za = chunk * zchunk, zb = min(a.L.nz, za + zchunk);
     const int nplanes = zb - za + 2 * R;
-    const int wp = 4 * shot + a.cur, wr = 4 * shot + 2 + a.cur;
     __syncthreads();
+    chain_wait();
+    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;  // stopped by the divergence watchdog
 
     int issued = 0;
-    auto issue = [&](int jj) -> bool {
-        const int slot = jj % C::NSL;
-        if (jj >= C::NSL &&
-            !mbar_wait_bounded(&ring.empty[slot], (uint32_t)(((jj - C::NSL) / C::NSL) & 1)))
-            return false;
-        const bool out = jj >= 2 * R;
-        const uint32_t bytes = 2 * C::INT * 4 + (out ? (2 * C::PW * C::PH + 3 * C::INT) * 4 : 0);
-        mbar_arrive_expect_tx(&ring.full[slot], bytes);
-        float *st = ring.smem + slot * C::STAGE1;
-        const int zj = za - R + jj;
-        tma_load_4d(st, &map_wint, &ring.full[slot], x0, y0, zj, wp);
-        tma_load_4d(st + C::INT, &map_wint, &ring.full[slot], x0, y0, zj, wr);
-        if (out) {
-            const int zs = zj - R;
-            float *h = st + 2 * C::INT;
-            tma_load_4d(h, &map_whalo, &ring.full[slot], x0 - C::RA, y0 - R, zs, wp);
-            tma_load_4d(h + C::HXY, &map_whalo, &ring.full[slot], x0 - C::RA, y0 - R, zs, wr);
-            float *n = h + 2 * C::HXY;
-            for (int c = 0; c < 3; ++c)
-                tma_load_4d(n + c * C::INT, &map_cint, &ring.full[slot], x0, y0, zs, 3 + c);
+    if (tid >= C::CONSUMERS) {
+        if (lane == 0) {
+            prefetch_tensormap(&map_wint);
+            prefetch_tensormap(&map_whalo);
+            prefetch_tensormap(&map_cint);
+            issued = produce<C::NSL>(
+                ring, C::STAGE1, nplanes, a.err, [&](int jj, float *st, uint64_t *full) {
+                    const bool out = jj >= 2 * R;
+                    mbar_arrive_expect_tx(
+                        full, (2 * C::INT + (out ? 2 * C::HXY + 3 * C::INT : 0)) * 4);
+                    const int zj = za - R + jj;
+                    tma_load_5d(st, &map_wint, full, x0, y0, zj, a.cur, 2 * shot);
+                    if (out) {
+                        tma_load_5d(st + C::OFF1_H, &map_whalo, full, x0 - C::RA, y0 - R, zj - R,
+                                    a.cur, 2 * shot);
+                        tma_load_4d(st + C::OFF1_N, &map_cint, full, x0, y0, zj - R, 3);
+                    }
+                });
         }
-        issued = jj + 1;
-        return true;
-    };
-    if (tid == 0)
-        for (int jj = 0; jj < D && jj < nplanes; ++jj) issue(jj);
-
-    const int gx = x0 + 4 * tx, gy = y0 + ty;
-    const bool ok = gx < a.L.nxp && gy < a.L.ny;
-    float *out = a.tmp + (int64_t)(6 * shot + 3 * field) * a.L.vol;
-    float4 acc[2 * R];
-#pragma unroll
-    for (int i = 0; i < 2 * R; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    bool failed = false;
-#pragma unroll U
-    for (int j = 0; j < nplanes; ++j) {
-        if (tid == 0 && j + D < nplanes && !failed && !issue(j + D)) {
-            failed = true;
-            *ring.abort_flag = 1;
-            atomicOr(a.err, DEV_ERR_TIMEOUT);
-        }
-        const int slot = j % C::NSL;
-        if (*ring.abort_flag ||
-            !mbar_wait_bounded(&ring.full[slot], (uint32_t)((j / C::NSL) & 1))) {
-            *ring.abort_flag = 1;
-            atomicOr(a.err, DEV_ERR_TIMEOUT);
-            break;
-        }
-        const float *st = ring.smem + slot * C::STAGE1;
+    } else {
+        const int gx = x0 + 4 * tx, gy = y0 + ty;
+        const bool ok = gx < a.L.nxp && gy < a.L.ny;
         const int q = ty * C::BX + 4 * tx;
-        const float4 c = lds4(st + field * C::INT + q);
-        dz_feed<R, KIND>(acc, c, a.t1[2]);
-        if (j >= 2 * R) {
-            const int zs = za - 2 * R + j;
-            const float *H = st + 2 * C::INT + field * C::HXY;
-            const float4 gxv = dx4<R, C::RA, KIND>(H + (R + ty) * C::PW + 4 * tx, a.t1[0]);
-            const float4 gyv =
-                dy4<R, KIND>(H + (R + ty) * C::PW + C::RA + 4 * tx, C::PW, a.t1[1]);
-            const float4 gzv = acc[0];
-            const float *N = st + 2 * C::INT + 2 * C::HXY;
-            const float4 nx = lds4(N + q), ny = lds4(N + C::INT + q), nz = lds4(N + 2 * C::INT + q);
-            float4 h;
-            h.x = nx.x * gxv.x + ny.x * gyv.x + nz.x * gzv.x;
-            h.y = nx.y * gxv.y + ny.y * gyv.y + nz.y * gzv.y;
-            h.z = nx.z * gxv.z + ny.z * gyv.z + nz.z * gzv.z;
-            h.w = nx.w * gxv.w + ny.w * gyv.w + nz.w * gzv.w;
-            float4 o0, o1, o2;
-            if (field == 0) {  // f_i = g_i - n_i h
-                o0 = make_float4(gxv.x - nx.x * h.x, gxv.y - nx.y * h.y, gxv.z - nx.z * h.z, gxv.w - nx.w * h.w);
-                o1 = make_float4(gyv.x - ny.x * h.x, gyv.y - ny.y * h.y, gyv.z - ny.z * h.z, gyv.w - ny.w * h.w);
-                o2 = make_float4(gzv.x - nz.x * h.x, gzv.y - nz.y * h.y, gzv.z - nz.z * h.z, gzv.w - nz.w * h.w);
-            } else {  // e_i = n_i h
-                o0 = make_float4(nx.x * h.x, nx.y * h.y, nx.z * h.z, nx.w * h.w);
-                o1 = make_float4(ny.x * h.x, ny.y * h.y, ny.z * h.z, ny.w * h.w);
-                o2 = make_float4(nz.x * h.x, nz.y * h.y, nz.z * h.z, nz.w * h.w);
+        float *out = a.tmp + (int64_t)6 * shot * a.L.vol + (int64_t)gy * a.L.nxp + gx;
+        Q4 acc[2][2 * R];
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+            for (int i = 0; i < 2 * R; ++i) acc[f][i] = Q4{0ull, 0ull};
+        RingPos<C::NSL> pos;
+#pragma unroll U
+        for (int j = 0; j < nplanes; ++j, pos.next()) {
+            const int slot = pos.slot(j);
+            if (*ring.abort_flag || !mbar_wait_bounded(&ring.full[slot], pos.phase(j))) {
+                *ring.abort_flag = 1;
+                atomicOr(a.err, DEV_ERR_TIMEOUT);
+                break;
             }
-            if (ok) {
-                const int64_t off = (int64_t)zs * a.L.plane + (int64_t)gy * a.L.nxp + gx;
-                // streaming stores: the temporaries are read once, by pass 2,
-                // and must not push the p/r halo planes out of L2 meanwhile
-                __stcs(reinterpret_cast<float4 *>(out + off), o0);
-                __stcs(reinterpret_cast<float4 *>(out + a.L.vol + off), o1);
-                __stcs(reinterpret_cast<float4 *>(out + 2 * a.L.vol + off), o2);
+            const float *st = ring.smem + slot * C::STAGE1;
+            const Q4 cp = lds_q4(st + q), cr = lds_q4(st + C::INT + q);
+            dz_feed_q4<R, KIND>(acc[0], cp, a.t1[2]);
+            dz_feed_q4<R, KIND>(acc[1], cr, a.t1[2]);
+            if (j >= 2 * R) {
+                const float *N = st + C::OFF1_N + q;
+                const Q4 nx = lds_q4(N), ny = lds_q4(N + C::INT), nz = lds_q4(N + 2 * C::INT);
+                const int64_t off = (int64_t)(za - 2 * R + j) * a.L.plane;
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    const float *H = st + C::OFF1_H + f * C::HXY + (R + ty) * C::PW + 4 * tx;
+                    const Q4 gxv = q4_from(dx4<R, C::RA, KIND>(H, a.t1[0]));
+                    const Q4 gyv = dy_q4<R, KIND>(H + C::RA, C::PW, a.t1[1]);
+                    const Q4 gzv = acc[f][0];
+                    const Q4 h = q4_fma(nz, gzv, q4_fma(nx, gxv, q4_mul(ny, gyv)));
+                    Q4 o[3];
+                    if (f == 0) {  // f_i = D_i p - n_i h
+                        const Q4 mh = q4_neg(h);
+                        o[0] = q4_fma(nx, mh, gxv);
+                        o[1] = q4_fma(ny, mh, gyv);
+                        o[2] = q4_fma(nz, mh, gzv);
+                    } else {  // e_i = n_i h
+                        o[0] = q4_mul(nx, h);
+                        o[1] = q4_mul(ny, h);
+                        o[2] = q4_mul(nz, h);
+                    }
+                    // streaming stores: the temporaries are read once, by
+                    // pass 2, and must not push the p/r halo planes out of L2
+                    if (ok)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const float4 v =
+                                make_float4(f32x2::f2_lo(o[c].lo), f32x2::f2_hi(o[c].lo),
+                                            f32x2::f2_lo(o[c].hi), f32x2::f2_hi(o[c].hi));
+                            __stcs(reinterpret_cast<float4 *>(out + (3 * f + c) * a.L.vol + off),
+                                   v);
+                        }
+                }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ring.empty[slot]);
+            dz_shift_q4<R, KIND>(acc[0], cp, a.t1[2]);
+            dz_shift_q4<R, KIND>(acc[1], cr, a.t1[2]);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ring.empty[slot]);
-        dz_shift<R, KIND>(acc, c, a.t1[2]);
     }
     __syncthreads();
-    if (*ring.abort_flag && tid == 0)
-        for (int jj = issued - C::NSL; jj < issued; ++jj)
-            if (jj >= 0)
-                mbar_wait_bounded(&ring.full[jj % C::NSL], (uint32_t)((jj / C::NSL) & 1), 200000000ull);
+    if (*ring.abort_flag && tid == C::CONSUMERS) drain<C::NSL>(ring, issued);
 }
 
 // ---------------------------------------------------------------- pass 2
 
-template <int R, int TX, int TY, int D, int KIND, int U>
-__global__ void __launch_bounds__(2 * TX * TY)
+template <int R, int TX, int TY, int D, int KIND, int U, int MINB>
+__global__ void __launch_bounds__(TX *TY + 32, MINB)
     tti_pass2_kernel(const __grid_constant__ CUtensorMap map_tint,
                      const __grid_constant__ CUtensorMap map_tx,
                      const __grid_constant__ CUtensorMap map_ty,
-                     const __grid_constant__ CUtensorMap map_wint,
-                     const __grid_constant__ CUtensorMap map_cint, const TtiArgs a, int zchunk,
-                     int nzc) {
+                     const __grid_constant__ CUtensorMap map_wlev,
+                     const __grid_constant__ CUtensorMap map_cint,
+                     const __grid_constant__ TtiArgs a, const __grid_constant__ AcousticInject inj,
+                     int zchunk, int nzc) {
     using C = TtiCfg<R, TX, TY, D>;
-    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;  // stopped by the divergence watchdog
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    Ring ring = ring_init<C::NSL, C::WARPS>(smem_raw, C::STAGE2, 4 * C::INT);
-    float *xchg = ring.smem + C::NSL * C::STAGE2;  // [2 buffers][A | B][INT]
+    Ring ring = ring_init<C::NSL, C::WARPS>(smem_raw, C::STAGE2);
     const int tid = threadIdx.x, lane = tid & 31;
-    const int field = tid / C::GROUP;  // 0: A = Hxy p (f), 1: B = Hz r (e)
-    const int t = tid - field * C::GROUP;
-    const int tx = t % TX, ty = t / TX;
+    const int tx = tid % TX, ty = tid / TX;
     const int shot = blockIdx.z / nzc, chunk = blockIdx.z - shot * nzc;
     const int x0 = blockIdx.x * C::BX, y0 = blockIdx.y * C::BY;
     const int za = chunk * zchunk, zb = min(a.L.nz, za + zchunk);
     const int nplanes = zb - za + 2 * R;
-    const int tbase = 6 * shot;
-    const int wq = 4 * shot + 2 * field + a.cur, wqm = 4 * shot + 2 * field + 1 - a.cur;
+    // For R <= 2 the x/y derivatives of a plane enter the z pipeline when the
+    // plane arrives, between the contributions of the planes below and above
+    // it, as in the fused scheme: the automatic scheme then gives the same
+    // bits on either side of its size limit.  Wider stencils take them with
+    // the output plane.
+    constexpr bool EARLY = R <= 2;
     __syncthreads();
+    chain_wait();
+    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;  // stopped by the divergence watchdog
 
     int issued = 0;
-    auto issue = [&](int jj) -> bool {
-        const int slot = jj % C::NSL;
-        if (jj >= C::NSL &&
-            !mbar_wait_bounded(&ring.empty[slot], (uint32_t)(((jj - C::NSL) / C::NSL) & 1)))
-            return false;
-        const bool out = jj >= 2 * R;
-        const uint32_t bytes =
-            2 * C::INT * 4 + (out ? (2 * C::PW * C::BY + 2 * C::BX * C::PH + 7 * C::INT) * 4 : 0);
-        mbar_arrive_expect_tx(&ring.full[slot], bytes);
-        float *st = ring.smem + slot * C::STAGE2;
-        const int zj = za - R + jj;
-        tma_load_4d(st, &map_tint, &ring.full[slot], x0, y0, zj, tbase + 2);           // f_z
-        tma_load_4d(st + C::INT, &map_tint, &ring.full[slot], x0, y0, zj, tbase + 5);  // e_z
-        if (out) {
-            const int zs = zj - R;
-            float *hx = st + 2 * C::INT;
-            tma_load_4d(hx, &map_tx, &ring.full[slot], x0 - C::RA, y0, zs, tbase + 0);       // f_x
-            tma_load_4d(hx + C::HX, &map_tx, &ring.full[slot], x0 - C::RA, y0, zs, tbase + 3);  // e_x
-            float *hy = hx + 2 * C::HX;
-            tma_load_4d(hy, &map_ty, &ring.full[slot], x0, y0 - R, zs, tbase + 1);       // f_y
-            tma_load_4d(hy + C::HY, &map_ty, &ring.full[slot], x0, y0 - R, zs, tbase + 4);  // e_y
-            float *w = hy + 2 * C::HY;
-            const int wb = 4 * shot;
-            tma_load_4d(w, &map_wint, &ring.full[slot], x0, y0, zs, wb + a.cur);                   // p
-            tma_load_4d(w + C::INT, &map_wint, &ring.full[slot], x0, y0, zs, wb + 1 - a.cur);      // p-
-            tma_load_4d(w + 2 * C::INT, &map_wint, &ring.full[slot], x0, y0, zs, wb + 2 + a.cur);  // r
-            tma_load_4d(w + 3 * C::INT, &map_wint, &ring.full[slot], x0, y0, zs, wb + 3 - a.cur);  // r-
-            for (int c = 0; c < 3; ++c)  // b, a, s
-                tma_load_4d(w + (4 + c) * C::INT, &map_cint, &ring.full[slot], x0, y0, zs, c);
+    if (tid >= C::CONSUMERS) {
+        if (lane == 0) {
+            issued = produce<C::NSL>(
+                ring, C::STAGE2, nplanes, a.err, [&](int jj, float *st, uint64_t *full) {
+                    const bool out = jj >= 2 * R;
+                    const bool xy = EARLY ? jj >= R && jj < nplanes - R : out;
+                    mbar_arrive_expect_tx(full, (2 * C::INT + (xy ? 2 * C::HX + 2 * C::HY : 0) +
+                                                 (out ? 7 * C::INT : 0)) *
+                                                    4);
+                    const int zj = za - R + jj, zs = zj - R, zxy = EARLY ? zj : zs;
+                    tma_load_5d(st, &map_tint, full, x0, y0, zj, 2, 2 * shot);  // f_z, e_z
+                    if (xy) {
+                        tma_load_5d(st + C::OFF2_X, &map_tx, full, x0 - C::RA, y0, zxy, 0,
+                                    2 * shot);  // f_x, e_x
+                        tma_load_5d(st + C::OFF2_Y, &map_ty, full, x0, y0 - R, zxy, 1,
+                                    2 * shot);  // f_y, e_y
+                    }
+                    if (out) {
+                        tma_load_5d(st + C::OFF2_W, &map_wlev, full, x0, y0, zs, 0, 2 * shot);
+                        tma_load_4d(st + C::OFF2_C, &map_cint, full, x0, y0, zs, 0);  // b, a, s
+                    }
+                });
         }
-        issued = jj + 1;
-        return true;
-    };
-    if (tid == 0)
-        for (int jj = 0; jj < D && jj < nplanes; ++jj) issue(jj);
-
-    const int gx = x0 + 4 * tx, gy = y0 + ty;
-    const bool ok = gx < a.L.nxp && gy < a.L.ny;
-    float dpx4[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) dpx4[i] = (gx + i < a.L.nx) ? a.dpx[gx + i] : 0.f;
-    const float dpy = gy < a.L.ny ? a.dpy[gy] : 0.f;
-    float *qn = a.wave + (int64_t)wqm * a.L.vol;  // q^{n+1} overwrites q^{n-1}
-    (void)wq;
-    float4 acc[2 * R];
-#pragma unroll
-    for (int i = 0; i < 2 * R; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    bool failed = false;
-#pragma unroll U
-    for (int j = 0; j < nplanes; ++j) {
-        if (tid == 0 && j + D < nplanes && !failed && !issue(j + D)) {
-            failed = true;
-            *ring.abort_flag = 1;
-            atomicOr(a.err, DEV_ERR_TIMEOUT);
-        }
-        const int slot = j % C::NSL;
-        bool good = !*ring.abort_flag &&
-                    mbar_wait_bounded(&ring.full[slot], (uint32_t)((j / C::NSL) & 1));
-        if (!good) {
-            *ring.abort_flag = 1;
-            atomicOr(a.err, DEV_ERR_TIMEOUT);
-        }
-        const float *st = ring.smem + slot * C::STAGE2;
+    } else {
+        const int gx = x0 + 4 * tx, gy = y0 + ty;
+        const bool ok = gx < a.L.nxp && gy < a.L.ny;
         const int q = ty * C::BX + 4 * tx;
-        float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (good) {
-            c = lds4(st + field * C::INT + q);
-            dz_feed<R, KIND>(acc, c, a.t2[2]);
-        }
-        const bool outp = j >= 2 * R;
-        float *xb = xchg + (j & 1) * 2 * C::INT;
-        if (outp && good) {
-            const float *hx = st + 2 * C::INT + field * C::HX;
-            const float *hy = st + 2 * C::INT + 2 * C::HX + field * C::HY;
-            const float4 dxv = dx4<R, C::RA, KIND>(hx + ty * C::PW + 4 * tx, a.t2[0]);
-            const float4 dyv = dy4<R, KIND>(hy + (R + ty) * C::BX + 4 * tx, C::BX, a.t2[1]);
-            const float4 v = f4add(f4add(dxv, dyv), acc[0]);  // A (field 0) or B (field 1)
-            *reinterpret_cast<float4 *>(xb + field * C::INT + q) = v;
-        }
-        // all threads (both groups) reach this barrier every iteration
-        if (outp) __syncthreads();
-        if (*ring.abort_flag) break;
-        if (outp) {
+        float dpx4[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dpx4[i] = (gx + i < a.L.nx) ? a.dpx[gx + i] : 0.f;
+        const f2 dpx_lo = f2_pack(dpx4[0], dpx4[1]), dpx_hi = f2_pack(dpx4[2], dpx4[3]);
+        const float dpy = gy < a.L.ny ? a.dpy[gy] : 0.f;
+        const f2 one2 = f2_splat(1.f);
+        // q^{n+1} overwrites q^{n-1}
+        float *qn = a.wave + (int64_t)(4 * shot + 1 - a.cur) * a.L.vol +
+                    (int64_t)gy * a.L.nxp + gx;
+        Q4 acc[2][2 * R];
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+            for (int i = 0; i < 2 * R; ++i) acc[f][i] = Q4{0ull, 0ull};
+        RingPos<C::NSL> pos;
+#pragma unroll U
+        for (int j = 0; j < nplanes; ++j, pos.next()) {
+            const int slot = pos.slot(j);
             const int zs = za - 2 * R + j;
-            const float *w = st + 2 * C::INT + 2 * C::HX + 2 * C::HY;
-            const float4 A = lds4(xb + q), B = lds4(xb + C::INT + q);
-            const float4 qc = lds4(w + 2 * field * C::INT + q);
-            const float4 qm = lds4(w + (2 * field + 1) * C::INT + q);
-            const float4 b = lds4(w + 4 * C::INT + q), av = lds4(w + 5 * C::INT + q),
-                         sv = lds4(w + 6 * C::INT + q);
-            const float dyz = dpy + a.dpz[zs];
-            float4 rhs;
-            if (field == 0) {  // p: a A + s B
-                rhs = make_float4(av.x * A.x + sv.x * B.x, av.y * A.y + sv.y * B.y,
-                                  av.z * A.z + sv.z * B.z, av.w * A.w + sv.w * B.w);
-            } else {  // r: s A + B
-                rhs = make_float4(sv.x * A.x + B.x, sv.y * A.y + B.y, sv.z * A.z + B.z,
-                                  sv.w * A.w + B.w);
+            const float dz = j >= 2 * R ? __ldg(a.dpz + zs) : 0.f;
+            if (*ring.abort_flag || !mbar_wait_bounded(&ring.full[slot], pos.phase(j))) {
+                *ring.abort_flag = 1;
+                atomicOr(a.err, DEV_ERR_TIMEOUT);
+                break;
             }
-            float4 o;
-            o.x = qc.x + (1.f - (dpx4[0] + dyz) * b.x) * (qc.x - qm.x) + b.x * rhs.x;
-            o.y = qc.y + (1.f - (dpx4[1] + dyz) * b.y) * (qc.y - qm.y) + b.y * rhs.y;
-            o.z = qc.z + (1.f - (dpx4[2] + dyz) * b.z) * (qc.z - qm.z) + b.z * rhs.z;
-            o.w = qc.w + (1.f - (dpx4[3] + dyz) * b.w) * (qc.w - qm.w) + b.w * rhs.w;
-            if (ok) {
-                const int64_t off = (int64_t)zs * a.L.plane + (int64_t)gy * a.L.nxp + gx;
-                *reinterpret_cast<float4 *>(qn + off) = o;
+            const float *st = ring.smem + slot * C::STAGE2;
+            const Q4 cf = lds_q4(st + q), ce = lds_q4(st + C::INT + q);
+            dz_feed_q4<R, KIND>(acc[0], cf, a.t2[2]);
+            dz_feed_q4<R, KIND>(acc[1], ce, a.t2[2]);
+            Q4 dxy[2];
+            if (EARLY ? j >= R && j < nplanes - R : j >= 2 * R) {
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    const float *hx = st + C::OFF2_X + f * C::HX + ty * C::PW + 4 * tx;
+                    const float *hy = st + C::OFF2_Y + f * C::HY + (R + ty) * C::BX + 4 * tx;
+                    const Q4 dxv = q4_from(dx4<R, C::RA, KIND>(hx, a.t2[0]));
+                    const Q4 dyv = dy_q4<R, KIND>(hy, C::BX, a.t2[1]);
+                    dxy[f] = q4_add(dxv, dyv);
+                    if (EARLY) acc[f][R] = q4_add(acc[f][R], dxy[f]);
+                }
             }
+            if (j >= 2 * R) {
+                Q4 H[2];  // Hxy p, Hz r
+#pragma unroll
+                for (int f = 0; f < 2; ++f)
+                    H[f] = EARLY ? acc[f][0] : q4_add(dxy[f], acc[f][0]);
+                const float *w = st + C::OFF2_W + q, *cc = st + C::OFF2_C + q;
+                const Q4 b = lds_q4(cc), av = lds_q4(cc + C::INT), sv = lds_q4(cc + 2 * C::INT);
+                const f2 dyz = f2_splat(-(dpy + dz));
+                // 1 - zeta, zeta = (dx + dy + dz) b
+                const Q4 keep = Q4{f2_fma(f2_sub(dyz, dpx_lo), b.lo, one2),
+                                   f2_fma(f2_sub(dyz, dpx_hi), b.hi, one2)};
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    const Q4 rhs = f == 0 ? q4_fma(av, H[0], q4_mul(sv, H[1]))  // a Hxy p + s Hz r
+                                          : q4_fma(sv, H[0], H[1]);             // s Hxy p + Hz r
+                    const Q4 qc = lds_q4(w + (2 * f + a.cur) * C::INT);
+                    const Q4 qm = lds_q4(w + (2 * f + 1 - a.cur) * C::INT);
+                    const Q4 o = q4_fma(b, rhs, q4_fma(keep, q4_sub(qc, qm), qc));
+                    if (ok)
+                        *reinterpret_cast<ulonglong2 *>(qn + 2 * f * a.L.vol +
+                                                        (int64_t)zs * a.L.plane) =
+                            make_ulonglong2(o.lo, o.hi);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ring.empty[slot]);
+            dz_shift_q4<R, KIND>(acc[0], cf, a.t2[2]);
+            dz_shift_q4<R, KIND>(acc[1], ce, a.t2[2]);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ring.empty[slot]);
-        dz_shift<R, KIND>(acc, c, a.t2[2]);
     }
     __syncthreads();
-    if (*ring.abort_flag && tid == 0)
-        for (int jj = issued - C::NSL; jj < issued; ++jj)
-            if (jj >= 0)
-                mbar_wait_bounded(&ring.full[jj % C::NSL], (uint32_t)((jj / C::NSL) & 1), 200000000ull);
+    if (*ring.abort_flag && tid == C::CONSUMERS) drain<C::NSL>(ring, issued);
+    if (inj.nsrc > 0 && tid == 0 && !*ring.abort_flag)
+        tti_inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
 }
 
 // ---------------------------------------------------------------- recompute
@@ -442,179 +478,244 @@ __global__ void __launch_bounds__(kRecBX *kRecBY) tti_recompute_kernel(const Tti
 
 // ---------------------------------------------------------------- host side
 
-constexpr int kTX = 16, kTY = 8;  // 64 x 8 tile, two groups of 128 threads (64 x 4 at R = 8)
-
-// Launch configurations of the two passes: prefetch depths D1, D2 and the
-// unroll U of the plane loop (the pending z-outputs rotate by one register
-// per plane; unrolling turns the moves into renaming).  Pass 2 stages carry
-// eleven tiles, so a shallower ring keeps more CTAs per SM.
-template <int R, int STAG, int D1_, int D2_, int U_, int TYV = kTY>
-struct TtiKernels {
-    static constexpr int D1 = D1_;
-    static constexpr int D2 = D2_;
-    static constexpr int K1 = STAG ? 1 : 0;   // inner derivative: D+ or centred
-    static constexpr int K2 = STAG ? -1 : 0;  // outer derivative: D- or centred
-    using C1 = TtiCfg<R, kTX, TYV, D1>;
-    using C2 = TtiCfg<R, kTX, TYV, D2>;
-    static const void *p1() { return (const void *)&tti_pass1_kernel<R, kTX, TYV, D1, K1, U_>; }
-    static const void *p2() { return (const void *)&tti_pass2_kernel<R, kTX, TYV, D2, K2, U_>; }
-    static const void *rc() { return (const void *)&tti_recompute_kernel<R, K1, K2>; }
-};
-
-struct TtiInfo {
-    const void *p1, *p2, *rc;
-    size_t smem1, smem2;
+// A launch configuration of one pass with its cost constants (microseconds),
+// as in acoustic.cu.
+struct PassEntry {
+    const void *fn;
+    size_t smem;
     int bx, by, pw, ph, threads;
+    float launch, lat, thr, warm;
 };
 
-template <int R, int STAG, int D1, int D2, int U, int TYV = kTY>
-TtiInfo info_r() {
-    using K = TtiKernels<R, STAG, D1, D2, U, TYV>;
-    using C1 = typename K::C1;
-    using C2 = typename K::C2;
-    static_assert(C1::BX == C2::BX && C1::BY == C2::BY && C1::THREADS == C2::THREADS, "tiles");
-    return TtiInfo{K::p1(), K::p2(), K::rc(), C1::SMEM1, C2::SMEM2, C1::BX, C1::BY, C1::PW, C1::PH,
-                   C1::THREADS};
+template <int PASS, int R, int TX, int TY, int D, int U, int MINB, int STAG>
+PassEntry pass_entry(float launch, float lat, float thr, float warm) {
+    using C = TtiCfg<R, TX, TY, D>;
+    constexpr int KIND = STAG ? (PASS == 1 ? 1 : -1) : 0;  // D+ inner, D- outer, or centred
+    const void *fn;
+    if constexpr (PASS == 1)
+        fn = (const void *)&tti_pass1_kernel<R, TX, TY, D, KIND, U, MINB>;
+    else
+        fn = (const void *)&tti_pass2_kernel<R, TX, TY, D, KIND, U, MINB>;
+    return PassEntry{fn,    PASS == 1 ? C::SMEM1 : C::SMEM2,
+                     C::BX, C::BY, C::PW, C::PH, C::THREADS, launch, lat, thr, warm};
 }
 
-// Built-in configuration per radius, measured on GB300 at 512^3: a deeper
-// pass-1 prefetch and a 4x unrolled plane loop pay for R = 4 and R = 6
-// (+18 % and +7 %); at R = 8 the unroll costs occupancy (registers), and
-// 64 x 4 tiles (two groups of 64 threads, twice the columns) run the step
-// 6 % faster than 64 x 8 (2.58 against 2.74 ms; 5-10 % slower at R = 4, 6).
-template <int R>
-struct TtiDefault {
-    static constexpr bool MID = R == 4 || R == 6;
-    static constexpr int D1 = MID ? 3 : 2;
-    static constexpr int D2 = MID ? 2 : (R >= 6 ? 1 : 2);
-    static constexpr int U = MID ? 4 : 1;
-    static constexpr int TY = R == 8 ? 4 : kTY;
+struct PassTable {
+    const PassEntry *e;
+    int n;
 };
 
-// Configuration table: index 0 is the built-in choice, the others are kept
-// for tuning sweeps; the staggered reading is compiled in the built-in
-// configuration only.
-template <int R, int STAG>
-bool tti_info_r(int config, TtiInfo *out) {
-    using Df = TtiDefault<R>;
-    constexpr int D2d = R >= 6 ? 1 : 2;
-    if (STAG) {
-        *out = info_r<R, STAG, Df::D1, Df::D2, Df::U, Df::TY>();
-        return true;
-    }
-    switch (config) {
-        case 0: *out = info_r<R, 0, Df::D1, Df::D2, Df::U, Df::TY>(); return true;
-        case 1: *out = info_r<R, 0, 2, D2d, 1>(); return true;
-        case 2: *out = info_r<R, 0, 2, D2d, 4>(); return true;
-        case 3: *out = info_r<R, 0, 3, 2, 4>(); return true;
-        case 4: *out = info_r<R, 0, 1, 1, 4>(); return true;
-        case 5: *out = info_r<R, 0, 3, 1, 1>(); return true;
-        case 6: *out = info_r<R, 0, Df::D1, Df::D2, Df::U, Df::TY == 4 ? 8 : 4>(); return true;
-        default: return false;
+#define FD_TTI_ENTRY(PASS, R, TX, TY, D, U, MB, ...) \
+    pass_entry<PASS, R, TX, TY, D, U, MB, STAG>(__VA_ARGS__)
+
+// Per radius (template arguments TX, TY, D, U, minimum CTAs per SM), fitted
+// and chosen on 13 problems from 48^3 to 512^3.  Both fields' pending z
+// outputs take 16R registers of a thread, which decides the tile: 64 x 8 with
+// two or three CTAs per SM up to so 12, one CTA of 64 x 14 (224 + 32 threads
+// with 255 registers) at so 16, a smaller one beside it for small grids.
+// 512^3, pass 1 + pass 2, so 4 / 8 / 12 / 16: 880 + 1153, 892 + 1169, 927 +
+// 1171 and 1039 + 1188 us, within 8 % of 104 bytes per point at the copy
+// bandwidth (2065 us); before (one thread group per field): 2112 / 2110 /
+// 2264 / 2570 us in all.
+template <int STAG>
+PassTable pass1_table(int radius) {
+    static const PassEntry r1[] = {
+        FD_TTI_ENTRY(1, 1, 16, 8, 3, 4, 0, 5.74f, 0.050f, 0.467f, 0.10f)};
+    static const PassEntry r2[] = {
+        FD_TTI_ENTRY(1, 2, 16, 8, 3, 4, 0, 5.74f, 0.050f, 0.467f, 0.10f),
+        FD_TTI_ENTRY(1, 2, 16, 16, 3, 4, 0, 2.59f, 0.771f, 0.249f, 0.66f)};
+    static const PassEntry r4[] = {
+        FD_TTI_ENTRY(1, 4, 16, 8, 3, 4, 0, 6.43f, 0.275f, 0.453f, 0.21f)};
+    static const PassEntry r6[] = {
+        FD_TTI_ENTRY(1, 6, 16, 8, 3, 4, 2, 6.84f, 0.449f, 0.465f, 0.25f),
+        FD_TTI_ENTRY(1, 6, 16, 14, 3, 4, 1, 4.65f, 0.828f, 0.145f, 0.41f)};
+    static const PassEntry r8[] = {
+        FD_TTI_ENTRY(1, 8, 16, 14, 3, 2, 1, 5.46f, 0.529f, 0.851f, 0.39f),
+        FD_TTI_ENTRY(1, 8, 16, 6, 3, 2, 2, 7.26f, 0.548f, 0.423f, 0.30f)};
+    switch (radius) {
+        case 1: return {r1, 1};
+        case 2: return {r2, 2};
+        case 4: return {r4, 1};
+        case 6: return {r6, 2};
+        case 8: return {r8, 2};
+        default: return {nullptr, 0};
     }
 }
-
-constexpr int kTtiConfigs = 7;
 
 template <int STAG>
-bool tti_info_s(int radius, int config, TtiInfo *out) {
+PassTable pass2_table(int radius) {
+    static const PassEntry r1[] = {
+        FD_TTI_ENTRY(2, 1, 16, 8, 2, 4, 0, 5.87f, 0.050f, 0.632f, 0.27f)};
+    static const PassEntry r2[] = {
+        FD_TTI_ENTRY(2, 2, 16, 8, 2, 4, 0, 5.87f, 0.050f, 0.632f, 0.27f)};
+    static const PassEntry r4[] = {
+        FD_TTI_ENTRY(2, 4, 16, 8, 2, 4, 0, 7.16f, 0.199f, 0.631f, 0.20f)};
+    static const PassEntry r6[] = {
+        FD_TTI_ENTRY(2, 6, 16, 8, 2, 4, 2, 7.92f, 0.408f, 0.622f, 0.25f)};
+    static const PassEntry r8[] = {
+        FD_TTI_ENTRY(2, 8, 16, 14, 2, 4, 1, 4.78f, 0.652f, 0.881f, 0.40f),
+        FD_TTI_ENTRY(2, 8, 16, 6, 1, 1, 2, 7.03f, 0.648f, 0.499f, 0.32f)};
     switch (radius) {
-        case 1: return tti_info_r<1, STAG>(config, out);
-        case 2: return tti_info_r<2, STAG>(config, out);
-        case 4: return tti_info_r<4, STAG>(config, out);
-        case 6: return tti_info_r<6, STAG>(config, out);
-        case 8: return tti_info_r<8, STAG>(config, out);
-        default: return false;
+        case 1: return {r1, 1};
+        case 2: return {r2, 1};
+        case 4: return {r4, 1};
+        case 6: return {r6, 1};
+        case 8: return {r8, 2};
+        default: return {nullptr, 0};
     }
 }
 
-bool tti_info(int radius, int stag, int config, TtiInfo *out) {
-    if (config < 0 || config >= kTtiConfigs) config = 0;
-    return stag ? tti_info_s<1>(radius, 0, out) : tti_info_s<0>(radius, config, out);
+PassTable pass_table(int pass, int radius, int stag) {
+    return pass == 1 ? (stag ? pass1_table<1>(radius) : pass1_table<0>(radius))
+                     : (stag ? pass2_table<1>(radius) : pass2_table<0>(radius));
+}
+
+const void *recompute_fn(int radius, int stag) {
+    switch (radius) {
+        case 1: return stag ? (const void *)&tti_recompute_kernel<1, 1, -1>
+                            : (const void *)&tti_recompute_kernel<1, 0, 0>;
+        case 2: return stag ? (const void *)&tti_recompute_kernel<2, 1, -1>
+                            : (const void *)&tti_recompute_kernel<2, 0, 0>;
+        case 4: return stag ? (const void *)&tti_recompute_kernel<4, 1, -1>
+                            : (const void *)&tti_recompute_kernel<4, 0, 0>;
+        case 6: return stag ? (const void *)&tti_recompute_kernel<6, 1, -1>
+                            : (const void *)&tti_recompute_kernel<6, 0, 0>;
+        case 8: return stag ? (const void *)&tti_recompute_kernel<8, 1, -1>
+                            : (const void *)&tti_recompute_kernel<8, 0, 0>;
+        default: return nullptr;
+    }
+}
+
+// The entry and chunk count with the smallest estimated time for one pass.
+fd_status plan_pass(int pass, int radius, int stag, int config, const WaveLayout &L, int nshots,
+                    TtiPassPlan *p) {
+    const PassTable t = pass_table(pass, radius, stag);
+    if (!t.e) return set_error(FD_ERR_SO, "no TTI kernel for radius %d", radius);
+    int dev = 0, nsm = 0;
+    FD_CUDA_TRY(cudaGetDevice(&dev));
+    FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    int best = -1, chunk = 0;
+    double best_us = 0.0;
+    for (int i = 0; i < t.n; ++i) {
+        if (config >= 0 && i != (config < t.n ? config : t.n - 1)) continue;
+        const PassEntry &e = t.e[i];
+        int per_sm = 0;
+        FD_TRY(raise_smem_limit(e.fn, e.smem));
+        FD_CUDA_TRY(
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e.fn, e.threads, e.smem));
+        if (per_sm < 1) return set_error(FD_ERR_CUDA, "TTI pass-%d kernel does not fit", pass);
+        const int64_t cols = (int64_t)((L.nx + e.bx - 1) / e.bx) *
+                             ((L.ny + e.by - 1) / e.by) * nshots;
+        double planes = 0.0;
+        int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
+                                &planes);
+        if (nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
+        const double us = e.launch + e.lat * planes;
+        if (best < 0 || us < best_us) {
+            best = i;
+            best_us = us;
+            chunk = (L.nz + nzc - 1) / nzc;
+        }
+    }
+    const PassEntry &e = t.e[best];
+    const int ntx = (L.nx + e.bx - 1) / e.bx, nty = (L.ny + e.by - 1) / e.by;
+    const int nzc = (L.nz + chunk - 1) / chunk;
+    if ((int64_t)nshots * nzc > 65535 || nty > 65535)
+        return set_error(FD_ERR_ARG, "grid too large for the TTI launch configuration");
+    p->fn = e.fn;
+    p->grid = dim3(ntx, nty, nshots * nzc);
+    p->block = dim3(e.threads, 1, 1);
+    p->smem = e.smem;
+    p->zchunk = chunk;
+    p->nzc = nzc;
+    p->bx = e.bx;
+    p->by = e.by;
+    p->pw = e.pw;
+    p->ph = e.ph;
+    p->est_us = best_us;
+    return FD_OK;
 }
 
 }  // namespace
 
 int tti_num_configs(int radius) {
-    TtiInfo in;
-    return tti_info(radius, 0, 0, &in) ? kTtiConfigs : 0;
+    const PassTable a = pass_table(1, radius, 0), b = pass_table(2, radius, 0);
+    return a.n > b.n ? a.n : b.n;
 }
 
 fd_status tti_plan(int radius, const WaveLayout &L, int nshots, float *wave, float *tmp,
                    const float *coef, TtiPlan *plan, int stag, int scheme, int config) {
-    TtiInfo in;
-    if (!tti_info(radius, stag, config, &in))
-        return set_error(FD_ERR_SO, "no TTI kernel for radius %d", radius);
     plan->radius = radius;
     plan->stag = stag ? 1 : 0;
     plan->scheme = scheme;
-    plan->config = config < 0 || config >= kTtiConfigs ? 0 : config;
     if (scheme == kTtiRecompute) {
+        if (!recompute_fn(radius, stag))
+            return set_error(FD_ERR_SO, "no TTI kernel for radius %d", radius);
         if ((int64_t)nshots * L.nz > 65535)
             return set_error(FD_ERR_ARG, "grid too large for the TTI recompute launch");
-        plan->grid = dim3((L.nx + kRecBX - 1) / kRecBX, (L.ny + kRecBY - 1) / kRecBY,
-                          nshots * L.nz);
-        plan->block = dim3(kRecBX, kRecBY, 1);
+        plan->p1.grid = dim3((L.nx + kRecBX - 1) / kRecBX, (L.ny + kRecBY - 1) / kRecBY,
+                             nshots * L.nz);
+        plan->p1.block = dim3(kRecBX, kRecBY, 1);
         return FD_OK;
     }
     if (scheme != kTtiTwoPass) return set_error(FD_ERR_ARG, "unknown TTI scheme %d", scheme);
-    int dev = 0, nsm = 0, per_sm = 0;
-    FD_CUDA_TRY(cudaGetDevice(&dev));
-    FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    FD_TRY(raise_smem_limit(in.p1, in.smem1));
-    FD_TRY(raise_smem_limit(in.p2, in.smem2));
-    FD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, in.p2, in.threads, in.smem2));
-    if (per_sm < 1) return set_error(FD_ERR_CUDA, "TTI pass-2 kernel does not fit on an SM");
-    const int ntx = (L.nx + in.bx - 1) / in.bx, nty = (L.ny + in.by - 1) / in.by;
-    const int64_t cols = (int64_t)ntx * nty * nshots;
-    // both passes together; their 2R warm-up planes only feed the z pipeline
-    // (fitted: 0.2 .. 0.44 of a plane each; load 0.64 .. 0.69 of 64 x 8
-    // tiles, 0.31 of 64 x 4)
-    int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, 0.35 * 2 * radius, in.bx * in.by / 800.0);
-    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
-    const int zchunk = (L.nz + nzc - 1) / nzc;
-    nzc = (L.nz + zchunk - 1) / zchunk;
-    if ((int64_t)nshots * nzc > 65535 || nty > 65535)
-        return set_error(FD_ERR_ARG, "grid too large for the TTI launch configuration");
-    plan->grid = dim3(ntx, nty, nshots * nzc);
-    plan->block = dim3(in.threads, 1, 1);
-    plan->smem1 = in.smem1;
-    plan->smem2 = in.smem2;
-    plan->zchunk = zchunk;
-    plan->nzc = nzc;
-    const uint64_t sy = (uint64_t)L.nxp * 4, sz = (uint64_t)L.plane * 4, sw = (uint64_t)L.vol * 4;
-    FD_TRY(make_tensor_map_4d(&plan->map_wint, wave, L.nx, L.ny, L.nz, 4ull * nshots, sy, sz, sw,
-                              in.bx, in.by, 1, 1));
-    FD_TRY(make_tensor_map_4d(&plan->map_whalo, wave, L.nx, L.ny, L.nz, 4ull * nshots, sy, sz, sw,
-                              in.pw, in.ph, 1, 1));
-    FD_TRY(make_tensor_map_4d(&plan->map_tint, tmp, L.nx, L.ny, L.nz, 6ull * nshots, sy, sz, sw,
-                              in.bx, in.by, 1, 1));
-    FD_TRY(make_tensor_map_4d(&plan->map_tx, tmp, L.nx, L.ny, L.nz, 6ull * nshots, sy, sz, sw,
-                              in.pw, in.by, 1, 1));
-    FD_TRY(make_tensor_map_4d(&plan->map_ty, tmp, L.nx, L.ny, L.nz, 6ull * nshots, sy, sz, sw,
-                              in.bx, in.ph, 1, 1));
-    return make_tensor_map_4d(&plan->map_cint, coef, L.nx, L.ny, L.nz, 6, sy, sz, sw, in.bx,
-                              in.by, 1, 1);
+    FD_TRY(plan_pass(1, radius, stag, config, L, nshots, &plan->p1));
+    FD_TRY(plan_pass(2, radius, stag, config, L, nshots, &plan->p2));
+    const uint64_t sy = (uint64_t)L.nxp * 4, sz = (uint64_t)L.plane * 4, sv = (uint64_t)L.vol * 4;
+    const uint64_t nx = L.nx, ny = L.ny, nz = L.nz, nf = 2ull * nshots;
+    // p/r buffers [shot][field][level], temporaries [shot][field][component]
+    const uint64_t wdim[5] = {nx, ny, nz, 2, nf}, wstr[4] = {sy, sz, sv, 2 * sv};
+    const uint64_t tdim[5] = {nx, ny, nz, 3, nf}, tstr[4] = {sy, sz, sv, 3 * sv};
+    const uint32_t bx1 = plan->p1.bx, by1 = plan->p1.by, bx2 = plan->p2.bx, by2 = plan->p2.by;
+    const uint32_t wint[5] = {bx1, by1, 1, 1, 2};
+    const uint32_t whalo[5] = {(uint32_t)plan->p1.pw, (uint32_t)plan->p1.ph, 1, 1, 2};
+    const uint32_t wlev[5] = {bx2, by2, 1, 2, 2};
+    const uint32_t tint[5] = {bx2, by2, 1, 1, 2};
+    const uint32_t txb[5] = {(uint32_t)plan->p2.pw, by2, 1, 1, 2};
+    const uint32_t tyb[5] = {bx2, (uint32_t)plan->p2.ph, 1, 1, 2};
+    FD_TRY(make_tensor_map_5d(&plan->map_wint, wave, wdim, wstr, wint));
+    FD_TRY(make_tensor_map_5d(&plan->map_whalo, wave, wdim, wstr, whalo));
+    FD_TRY(make_tensor_map_5d(&plan->map_wlev, wave, wdim, wstr, wlev));
+    FD_TRY(make_tensor_map_5d(&plan->map_tint, tmp, tdim, tstr, tint));
+    FD_TRY(make_tensor_map_5d(&plan->map_tx, tmp, tdim, tstr, txb));
+    FD_TRY(make_tensor_map_5d(&plan->map_ty, tmp, tdim, tstr, tyb));
+    FD_TRY(make_tensor_map_4d(&plan->map_c1, coef, L.nx, L.ny, L.nz, 6, sy, sz, sv, bx1, by1, 1,
+                              3));
+    return make_tensor_map_4d(&plan->map_c2, coef, L.nx, L.ny, L.nz, 6, sy, sz, sv, bx2, by2, 1,
+                              3);
+}
+
+fd_status tti_choose_scheme(int radius, int stag, const WaveLayout &L, int nshots, int *scheme) {
+    *scheme = kTtiTwoPass;
+    // from so 8 on the cross cells of the fused scheme cost more than the
+    // temporaries' 56 bytes per point
+    if (radius > 2 || !tti_fused_supported(radius)) return FD_OK;
+    double fused_us = 0.0;
+    FD_TRY(tti_fused_time(radius, stag, L, nshots, &fused_us));
+    TtiPassPlan p1, p2;
+    FD_TRY(plan_pass(1, radius, stag, -1, L, nshots, &p1));
+    FD_TRY(plan_pass(2, radius, stag, -1, L, nshots, &p2));
+    // so 4: two passes up to about 128^3 (48^3 10.0 against 15.5 us per step,
+    // 96^3 21.3 and 23.0, 128^3 34.4 and 34.1), fused above (256^3 204 against
+    // 268, 512^3 1430 against 2025).  The pass tables were fitted to launches
+    // between events, 3.7 us each longer than chained ones.  The six
+    // temporaries are not spent on many small shots at once.
+    const bool cheap = (int64_t)6 * nshots * L.vol * 4 <= (int64_t)1 << 30;
+    if (!cheap || fused_us <= p1.est_us + p2.est_us - 7.5) *scheme = kTtiFused;
+    return FD_OK;
+}
+
+bool tti_records_receivers(const TtiPlan &plan) {
+    return plan.scheme != kTtiRecompute && plan.p1.grid.z < 65535;
 }
 
 fd_status tti_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
-                     cudaEvent_t *ev) {
-    TtiInfo in;
-    if (!tti_info(plan.radius, plan.stag, plan.config, &in))
-        return set_error(FD_ERR_SO, "bad TTI plan");
-    int zchunk = plan.zchunk, nzc = plan.nzc;
+                     cudaEvent_t *ev, const AcousticInject *inject, const ReceiveArgs *receive) {
     if (ev) FD_CUDA_TRY(cudaEventRecord(ev[0], stream));
-    if (plan.scheme == kTtiFused) {
-        FD_TRY(tti_fused_launch(plan, a, stream));
-        if (ev) {
-            FD_CUDA_TRY(cudaEventRecord(ev[1], stream));
-            FD_CUDA_TRY(cudaEventRecord(ev[2], stream));
-        }
-        return FD_OK;
-    }
     if (plan.scheme == kTtiRecompute) {
         void *pr[] = {(void *)&a};
-        FD_CUDA_TRY(cudaLaunchKernel(in.rc, plan.grid, plan.block, pr, 0, stream));
+        FD_CUDA_TRY(cudaLaunchKernel(recompute_fn(plan.radius, plan.stag), plan.p1.grid,
+                                     plan.p1.block, pr, 0, stream));
         note_launch(stream);
         if (ev) {
             FD_CUDA_TRY(cudaEventRecord(ev[1], stream));
@@ -622,15 +723,37 @@ fd_status tti_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
         }
         return FD_OK;
     }
-    void *p1[] = {(void *)&plan.map_wint, (void *)&plan.map_whalo, (void *)&plan.map_cint,
-                  (void *)&a, (void *)&zchunk, (void *)&nzc};
-    FD_CUDA_TRY(cudaLaunchKernel(in.p1, plan.grid, plan.block, p1, plan.smem1, stream));
+    AcousticInject inj;
+    memset(&inj, 0, sizeof(inj));
+    if (inject) inj = *inject;
+    ReceiveArgs rec;
+    memset(&rec, 0, sizeof(rec));
+    dim3 grid1 = plan.p1.grid;
+    if (receive) rec = *receive;
+    if (plan.scheme == kTtiFused) {
+        FD_TRY(tti_fused_launch(plan, a, stream, inj, rec));
+        if (ev) {
+            FD_CUDA_TRY(cudaEventRecord(ev[1], stream));
+            FD_CUDA_TRY(cudaEventRecord(ev[2], stream));
+        }
+        return FD_OK;
+    }
+    if (rec.nrec > 0) {
+        rec.slices = receive_slices(rec, grid1.x, grid1.y, plan.p1.block.x);
+        if (grid1.z >= 65535) return set_error(FD_ERR_ARG, "no grid slice left for receivers");
+        if ((int64_t)grid1.z + rec.slices > 65535) rec.slices = 65535 - grid1.z;
+        grid1.z += rec.slices;
+    }
+    int zc1 = plan.p1.zchunk, nzc1 = plan.p1.nzc, zc2 = plan.p2.zchunk, nzc2 = plan.p2.nzc;
+    void *p1[] = {(void *)&plan.map_wint, (void *)&plan.map_whalo, (void *)&plan.map_c1,
+                  (void *)&a, (void *)&rec, (void *)&zc1, (void *)&nzc1};
+    FD_CUDA_TRY(launch_chained(plan.p1.fn, grid1, plan.p1.block, p1, plan.p1.smem, stream));
     note_launch(stream);
     if (ev) FD_CUDA_TRY(cudaEventRecord(ev[1], stream));
     void *p2[] = {(void *)&plan.map_tint, (void *)&plan.map_tx, (void *)&plan.map_ty,
-                  (void *)&plan.map_wint, (void *)&plan.map_cint, (void *)&a, (void *)&zchunk,
-                  (void *)&nzc};
-    FD_CUDA_TRY(cudaLaunchKernel(in.p2, plan.grid, plan.block, p2, plan.smem2, stream));
+                  (void *)&plan.map_wlev, (void *)&plan.map_c2, (void *)&a, (void *)&inj,
+                  (void *)&zc2, (void *)&nzc2};
+    FD_CUDA_TRY(launch_chained(plan.p2.fn, plan.p2.grid, plan.p2.block, p2, plan.p2.smem, stream));
     note_launch(stream);
     if (ev) FD_CUDA_TRY(cudaEventRecord(ev[2], stream));
     return FD_OK;

@@ -4,34 +4,47 @@
 //
 // Same operators as the two passes of tti.cu (Hxy p = sum_i D_i f_i,
 // Hz r = sum_i D_i e_i, f_i = D_i p - n_i (n . grad p), e_i = n_i (n . grad r)).
-// One CTA owns a 64 x 8 column and marches it through z with two thread
-// groups, one per field (p, r):
+// One CTA owns a 64 x 16 column and marches it through z; a thread owns one
+// "cross" cell -- four x points of the tile, of the R rows above and below it
+// or of the float4 column left and right of it, the points whose temporaries
+// the tile's outer stencil reads -- for BOTH fields:
 //   * every arriving plane of p and r comes with a halo of 2R rows and 2RA
 //     columns (TMA, zero fill outside the grid) into a ring of R + 1 + D
-//     planes; its values feed the z-derivative accumulators of the "cross"
-//     cells -- the tile plus R rows above and below it and one float4
-//     column left and right, the points whose temporaries the tile's outer
-//     stencil reads;
-//   * R planes behind, the gradient of the cross cells is complete: the
-//     temporaries f (group p) or e (group r) of that plane are written to
-//     shared memory (f_x, e_x on the x-extended tile, f_y, e_y on the
-//     y-extended tile, f_z, e_z on the tile; zero outside the grid, as the
-//     ghosts of the two-pass scheme);
-//   * the outer derivatives of the temporaries feed a second accumulator
-//     pipeline, whose output R planes further behind is complete; the groups
-//     exchange Hxy p and Hz r through shared memory and update p and r.
-// HBM traffic per point: p, r and n_x, n_y, n_z once with halos, p, p-, r,
-// r-, b, a, s for the update, p+, r+ out: 48 bytes against 104 for the two
-// passes; the price is the gradient of the cross cells (1.6x the tile's).
+//     planes and feeds the cell's z-derivative accumulators;
+//   * R planes behind, the gradient of the cells is complete: f_x, e_x on the
+//     x-extended tile and f_y, e_y on the y-extended tile go to shared memory
+//     (zero outside the grid, as the ghosts of the two-pass scheme), f_z, e_z
+//     stay with the tile cell's thread;
+//   * after one barrier, the tile warps feed the outer derivatives to a second
+//     accumulator pipeline, whose output R planes further behind is complete:
+//     p and r are updated by the thread that holds Hxy p and Hz r.  The strip
+//     warps meanwhile start the next plane (the temporaries have two buffers).
+// A producer warp issues the four copies of a plane (both fields, n, both
+// levels, coefficients).  HBM traffic per point: p, r and n_x, n_y, n_z once
+// with halos, p, p-, r, r-, b, a, s for the update, p+, r+ out: 48 bytes
+// against 104 for the two passes; the price is the gradient of the cross
+// cells (1.38x the tile's at R = 2).  Bound by shared memory (about 85 floats
+// per point, 87 % of its bandwidth at 512^3) and by the latency of a plane's
+// chain (wait, gradient, barrier, outer derivative).
+// 512^3 so 4: 1430 us per step; with one thread group per field
+// exchanging Hxy p and Hz r at a second barrier, two cells for some threads
+// and a consumer thread issuing twelve copies per plane, 1763 us.
+#include <string.h>
+
 #include "kernels.cuh"
+#include "receive.cuh"
+#include "ring.cuh"
 #include "runtime.cuh"
+#include "tti_inject.cuh"
 #include "tti_stencil.cuh"
 
 namespace fdsweep {
 namespace {
 using namespace tti;
 
-template <int R, int D, int TY_>
+constexpr int round32(int n) { return (n + 31) / 32 * 32; }
+
+template <int R, int TY_, int D>
 struct TfCfg {
     static constexpr int TX = 16, TY = TY_;
     static constexpr int BX = 4 * TX, BY = TY;
@@ -42,332 +55,329 @@ struct TfCfg {
     // fall on distinct banks) and the cross bounding box
     static constexpr int PX = BX + 4 * RA + 4, PY = BY + 4 * R;
     static constexpr int NXW = BX + 2 * RA, NYH = BY + 2 * R;
-    static constexpr int GROUP = TX * TY, THREADS = 2 * GROUP, WARPS = THREADS / 32;
-    static constexpr int INT = BX * BY;
-    static constexpr int BOX = (PX * PY + 31) / 32 * 32;
-    static constexpr int NBOX = (NXW * NYH + 31) / 32 * 32;
+    static constexpr int INT = BX * BY, TILE = TX * TY;
+    static constexpr int NCELL = TILE + 2 * BY + 2 * R * TX;
+    static constexpr int WARPS = (NCELL + 31) / 32;
+    static constexpr int CONSUMERS = 32 * WARPS;
+    static constexpr int THREADS = CONSUMERS + 32;  // + the producer warp
+    static constexpr int BOX = PX * PY, NBOX = NXW * NYH;
     static constexpr int NP = R + 1 + D;  // plane ring: plane s .. arriving plane, + prefetch
     static constexpr int NQ = D + 1;      // per-iteration ring: n at s, update tiles at o
-    static constexpr int PSLOT = 2 * BOX;
-    static constexpr int QSLOT = 3 * NBOX + 7 * INT;
-    static constexpr int FX = (NXW * BY + 31) / 32 * 32;  // f_x / e_x, x-extended
-    static constexpr int FY = (BX * NYH + 31) / 32 * 32;  // f_y / e_y, y-extended
-    static constexpr int TMP = FX + FY + INT;             // + f_z / e_z on the tile
-    static constexpr int NCELL = (BX / 4) * BY + 2 * BY + 2 * R * (BX / 4);
-    static constexpr int KC = (NCELL + GROUP - 1) / GROUP;  // cross cells per thread
-    static constexpr uint32_t PBYTES = 2 * PX * PY * 4;
-    static constexpr uint32_t NBYTES = 3 * NXW * NYH * 4, UBYTES = 7 * INT * 4;
-    static constexpr size_t SMEM =
-        ((size_t)NP * PSLOT + (size_t)NQ * QSLOT + 2 * TMP + 4 * INT) * 4 +
-        (size_t)(NP + NQ) * 2 * 8 + 16 + 128;
+    static constexpr int PSLOT = round32(2 * BOX);
+    static constexpr int OFF_W = round32(3 * NBOX);            // p0, p1, r0, r1
+    static constexpr int OFF_C = OFF_W + round32(4 * INT);     // b, a, s
+    static constexpr int QSLOT = OFF_C + round32(3 * INT);
+    static constexpr int FX = round32(NXW * BY);  // f_x / e_x, x-extended
+    static constexpr int FY = round32(BX * NYH);  // f_y / e_y, y-extended
+    static constexpr int TMP = FX + FY;
+    static constexpr uint32_t PBYTES = 2 * BOX * 4;
+    static constexpr uint32_t NBYTES = 3 * NBOX * 4, UBYTES = 7 * INT * 4;
+    static constexpr size_t SMEM = ((size_t)NP * PSLOT + (size_t)NQ * QSLOT + 4 * TMP) * 4 +
+                                   (size_t)(2 * NP + NQ) * 8 + 16 + 128;
     static_assert(PX <= 256 && PY <= 256, "TMA box dimension limit");
+    static_assert(TILE % 32 == 0, "whole tile warps");
 };
 
-__device__ __forceinline__ void group_sync(int group, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(nthreads) : "memory");
+// Barrier of the first `n` threads with the OR of a flag over them, so that
+// all of them leave together after a failed wait.
+__device__ __forceinline__ bool consumers_or(int n, bool flag) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(flag ? 1u : 0u), "r"(n)
+        : "memory");
+    return r != 0;
 }
 
-template <int R, int D, int K1, int K2, int TY>
-__global__ void __launch_bounds__(32 * TY)
+__device__ __forceinline__ float4 masked(Q4 v, unsigned m) {
+    return make_float4((m & 1u) ? f32x2::f2_lo(v.lo) : 0.f, (m & 2u) ? f32x2::f2_hi(v.lo) : 0.f,
+                       (m & 4u) ? f32x2::f2_lo(v.hi) : 0.f, (m & 8u) ? f32x2::f2_hi(v.hi) : 0.f);
+}
+
+template <int R, int TY, int D, int K1, int K2, int U, int MINB>
+__global__ void __launch_bounds__(TfCfg<R, TY, D>::THREADS, MINB)
     tti_fused_kernel(const __grid_constant__ CUtensorMap map_box,
                      const __grid_constant__ CUtensorMap map_nbox,
-                     const __grid_constant__ CUtensorMap map_wint,
-                     const __grid_constant__ CUtensorMap map_cint, const TtiArgs a, int zchunk,
-                     int nzc) {
-    using C = TfCfg<R, D, TY>;
-    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;  // stopped by the divergence watchdog
+                     const __grid_constant__ CUtensorMap map_wlev,
+                     const __grid_constant__ CUtensorMap map_cint,
+                     const __grid_constant__ TtiArgs a, const __grid_constant__ AcousticInject inj,
+                     const __grid_constant__ ReceiveArgs rec, int zchunk, int nzc) {
+    using C = TfCfg<R, TY, D>;
+    if (blockIdx.z >= gridDim.z - rec.slices) {
+        chain_trigger();
+        chain_wait();
+        if (!(__ldcg(a.err) & DEV_ERR_NONFINITE))
+            record_receivers(&rec, a.wave, 4, a.cur, 2 + a.cur, &a.L);
+        return;
+    }
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *smem = reinterpret_cast<float *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
     float *ringP = smem;
     float *ringQ = ringP + C::NP * C::PSLOT;
-    float *tmp = ringQ + C::NQ * C::QSLOT;  // [field][fx | fy | fz]
-    float *xchg = tmp + 2 * C::TMP;         // [2 buffers][A | B]
-    uint64_t *fullP = reinterpret_cast<uint64_t *>(xchg + 4 * C::INT);
-    uint64_t *emptyP = fullP + C::NP;
-    uint64_t *fullQ = emptyP + C::NP;
-    uint64_t *emptyQ = fullQ + C::NQ;
+    float *tmp = ringQ + C::NQ * C::QSLOT;  // [2 buffers][field][fx | fy]
+    uint64_t *full = reinterpret_cast<uint64_t *>(tmp + 4 * C::TMP);  // one per P slot
+    uint64_t *emptyP = full + C::NP;
+    uint64_t *emptyQ = emptyP + C::NP;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(emptyQ + C::NQ);
 
     const int tid = threadIdx.x, lane = tid & 31;
-    const int field = tid / C::GROUP;  // 0: p (temporaries f), 1: r (temporaries e)
-    const int t = tid - field * C::GROUP;
     const int shot = blockIdx.z / nzc, chunk = blockIdx.z - shot * nzc;
     const int x0 = blockIdx.x * C::BX, y0 = blockIdx.y * C::BY;
     const int za = chunk * zchunk, zb = min(a.L.nz, za + zchunk);
     const int nplanes = zb - za + 4 * R;
     const int P0 = za - 2 * R;  // first arriving plane
-    const int wp = 4 * shot + a.cur, wr = 4 * shot + 2 + a.cur;
 
     if (tid == 0) {
-        prefetch_tensormap(&map_box);
-        prefetch_tensormap(&map_nbox);
-        prefetch_tensormap(&map_wint);
-        prefetch_tensormap(&map_cint);
         for (int i = 0; i < C::NP; ++i) {
-            mbar_init(&fullP[i], 1);
+            mbar_init(&full[i], 1);
             mbar_init(&emptyP[i], C::WARPS);
         }
-        for (int i = 0; i < C::NQ; ++i) {
-            mbar_init(&fullQ[i], 1);
-            mbar_init(&emptyQ[i], C::WARPS);
-        }
+        for (int i = 0; i < C::NQ; ++i) mbar_init(&emptyQ[i], C::WARPS);
         fence_mbar_init();
         *abort_flag = 0;
     }
     __syncthreads();
+    chain_wait();
+    if (__ldcg(a.err) & DEV_ERR_NONFINITE) return;  // stopped by the divergence watchdog
 
-    // Producer (thread 0).  Ring P slot jj % NP: planes of p and r (box);
-    // ring Q slot jj % NQ: n boxes at s = P0 + jj - R (from jj >= 2R) and the
-    // update tiles at o = P0 + jj - 2R (from jj >= 4R); zero bytes otherwise.
-    int issuedP = 0;
-    auto issue = [&](int jj) -> bool {
-        const int sp = jj % C::NP, sq = jj % C::NQ;
-        if (jj >= C::NP &&
-            !mbar_wait_bounded(&emptyP[sp], (uint32_t)(((jj - C::NP) / C::NP) & 1)))
-            return false;
-        if (jj >= C::NQ &&
-            !mbar_wait_bounded(&emptyQ[sq], (uint32_t)(((jj - C::NQ) / C::NQ) & 1)))
-            return false;
-        float *P = ringP + sp * C::PSLOT;
-        mbar_arrive_expect_tx(&fullP[sp], C::PBYTES);
-        tma_load_4d(P, &map_box, &fullP[sp], x0 - 2 * C::RA, y0 - 2 * R, P0 + jj, wp);
-        tma_load_4d(P + C::BOX, &map_box, &fullP[sp], x0 - 2 * C::RA, y0 - 2 * R, P0 + jj, wr);
-        const bool qs = jj >= 2 * R, qo = jj >= 4 * R;
-        mbar_arrive_expect_tx(&fullQ[sq], (qs ? C::NBYTES : 0) + (qo ? C::UBYTES : 0));
-        float *Q = ringQ + sq * C::QSLOT;
-        if (qs)
-            for (int c = 0; c < 3; ++c)
-                tma_load_4d(Q + c * C::NBOX, &map_nbox, &fullQ[sq], x0 - C::RA, y0 - R,
-                            P0 + jj - R, 3 + c);
-        if (qo) {
-            const int o = P0 + jj - 2 * R, wb = 4 * shot;
-            float *U = Q + 3 * C::NBOX;
-            tma_load_4d(U, &map_wint, &fullQ[sq], x0, y0, o, wb + a.cur);                  // p
-            tma_load_4d(U + C::INT, &map_wint, &fullQ[sq], x0, y0, o, wb + 1 - a.cur);     // p-
-            tma_load_4d(U + 2 * C::INT, &map_wint, &fullQ[sq], x0, y0, o, wb + 2 + a.cur); // r
-            tma_load_4d(U + 3 * C::INT, &map_wint, &fullQ[sq], x0, y0, o, wb + 3 - a.cur); // r-
-            for (int c = 0; c < 3; ++c)  // b, a, s
-                tma_load_4d(U + (4 + c) * C::INT, &map_cint, &fullQ[sq], x0, y0, o, c);
-        }
-        issuedP = jj + 1;
-        return true;
-    };
-    if (tid == 0)
-        for (int jj = 0; jj < D && jj < nplanes; ++jj) issue(jj);
-
-    // cross cells of this thread: float4 column qx in [-1, 16], row y in
-    // [-R, BY + R); kind 0 tile, 1 x strip, 2 y strip
-    int cbox[C::KC], cnb[C::KC], ckind[C::KC], cqx[C::KC], cy[C::KC];
-    bool cvalid[C::KC];
-    unsigned cmask[C::KC];  // in-grid x elements (bits 0..3) when the row is in the grid
-#pragma unroll
-    for (int k = 0; k < C::KC; ++k) {
-        const int c = t + k * C::GROUP;
-        cvalid[k] = c < C::NCELL;
-        int qx = 0, y = 0, kind = 0;
-        if (c < (C::BX / 4) * C::BY) {
-            qx = c % (C::BX / 4);
-            y = c / (C::BX / 4);
-        } else if (c < (C::BX / 4) * C::BY + 2 * C::BY) {
-            const int e = c - (C::BX / 4) * C::BY;
-            qx = e < C::BY ? -1 : C::BX / 4;
-            y = e % C::BY;
-            kind = 1;
-        } else if (cvalid[k]) {
-            const int e = c - (C::BX / 4) * C::BY - 2 * C::BY;
-            const int rr = e / (C::BX / 4);
-            qx = e % (C::BX / 4);
-            y = rr < R ? rr - R : C::BY + (rr - R);
-            kind = 2;
-        }
-        cqx[k] = qx;
-        cy[k] = y;
-        ckind[k] = kind;
-        cbox[k] = (y + 2 * R) * C::PX + 4 * qx + 2 * C::RA;  // the cell in the p/r box
-        cnb[k] = (y + R) * C::NXW + 4 * qx + C::RA;          // the cell in the n box
-        unsigned m = 0u;
-        const int gy = y0 + y;
-        if (gy >= 0 && gy < a.L.ny)
-            for (int e = 0; e < 4; ++e) {
-                const int gx = x0 + 4 * qx + e;
-                if (gx >= 0 && gx < a.L.nx) m |= 1u << e;
-            }
-        cmask[k] = m;
-    }
-    // the thread's tile cell for the outer derivative and the update
-    const int tx = t % C::TX, ty = t / C::TX;
-    const int gx = x0 + 4 * tx, gy = y0 + ty;
-    const bool ok = gx < a.L.nxp && gy < a.L.ny;
-    float dpx4[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) dpx4[i] = (gx + i < a.L.nx) ? a.dpx[gx + i] : 0.f;
-    const float dpy = gy < a.L.ny ? a.dpy[gy] : 0.f;
-    float *qn = a.wave + (int64_t)(4 * shot + 2 * field + 1 - a.cur) * a.L.vol;
-    float *T = tmp + field * C::TMP;
-    float *Tfx = T, *Tfy = T + C::FX, *Tfz = T + C::FX + C::FY;
-
-    float4 acc1[C::KC][2 * R], acc2[2 * R];
-#pragma unroll
-    for (int k = 0; k < C::KC; ++k)
-#pragma unroll
-        for (int i = 0; i < 2 * R; ++i) acc1[k][i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < 2 * R; ++i) acc2[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-
-    bool failed = false;
-    for (int j = 0; j < nplanes; ++j) {
-        bool bad = false;
-        if (tid == 0 && j + D < nplanes && !failed && !issue(j + D)) {
-            failed = true;
-            bad = true;
-        }
-        const int sp = j % C::NP, sq = j % C::NQ;
-        if (!mbar_wait_bounded(&fullP[sp], (uint32_t)((j / C::NP) & 1))) bad = true;
-        if (!mbar_wait_bounded(&fullQ[sq], (uint32_t)((j / C::NQ) & 1))) bad = true;
-        const int s = P0 + j - R, o = P0 + j - 2 * R;
-        const bool has_s = j >= 2 * R, has_o = j >= 4 * R;
-        const float *Pa = ringP + sp * C::PSLOT + field * C::BOX;  // arriving plane
-        const float *Ps = ringP + ((j - R + C::NP * (R + 1)) % C::NP) * C::PSLOT + field * C::BOX;
-        const float *Q = ringQ + sq * C::QSLOT;
-        const bool s_in = s >= 0 && s < a.L.nz;
-
-        // ---- stage 1: z-derivative feed; gradient and temporaries of plane s
-#pragma unroll
-        for (int k = 0; k < C::KC; ++k) {
-            if (!cvalid[k]) continue;
-            const float4 cv = lds4(Pa + cbox[k]);
-            dz_feed<R, K1>(acc1[k], cv, a.t1[2]);
-            if (has_s) {
-                const float4 g_x = dx4<R, C::RA, K1>(Ps + cbox[k] - C::RA, a.t1[0]);
-                const float4 g_y = dy4<R, K1>(Ps + cbox[k], C::PX, a.t1[1]);
-                const float4 g_z = acc1[k][0];
-                const float4 nx = lds4(Q + cnb[k]), ny = lds4(Q + C::NBOX + cnb[k]),
-                             nz = lds4(Q + 2 * C::NBOX + cnb[k]);
-                float4 h;
-                h.x = nx.x * g_x.x + ny.x * g_y.x + nz.x * g_z.x;
-                h.y = nx.y * g_x.y + ny.y * g_y.y + nz.y * g_z.y;
-                h.z = nx.z * g_x.z + ny.z * g_y.z + nz.z * g_z.z;
-                h.w = nx.w * g_x.w + ny.w * g_y.w + nz.w * g_z.w;
-                float4 o0, o1, o2;
-                if (field == 0) {  // f_i = g_i - n_i h
-                    o0 = make_float4(g_x.x - nx.x * h.x, g_x.y - nx.y * h.y, g_x.z - nx.z * h.z, g_x.w - nx.w * h.w);
-                    o1 = make_float4(g_y.x - ny.x * h.x, g_y.y - ny.y * h.y, g_y.z - ny.z * h.z, g_y.w - ny.w * h.w);
-                    o2 = make_float4(g_z.x - nz.x * h.x, g_z.y - nz.y * h.y, g_z.z - nz.z * h.z, g_z.w - nz.w * h.w);
-                } else {  // e_i = n_i h
-                    o0 = make_float4(nx.x * h.x, nx.y * h.y, nx.z * h.z, nx.w * h.w);
-                    o1 = make_float4(ny.x * h.x, ny.y * h.y, ny.z * h.z, ny.w * h.w);
-                    o2 = make_float4(nz.x * h.x, nz.y * h.y, nz.z * h.z, nz.w * h.w);
-                }
-                // zero ghosts: temporaries outside the grid vanish
-                const unsigned m = s_in ? cmask[k] : 0u;
-                auto masked = [m](float4 v) {
-                    return make_float4((m & 1u) ? v.x : 0.f, (m & 2u) ? v.y : 0.f,
-                                       (m & 4u) ? v.z : 0.f, (m & 8u) ? v.w : 0.f);
-                };
-                const int y = cy[k], qx = cqx[k];
-                if (ckind[k] != 2)  // tile or x strip: f_x / e_x
-                    *reinterpret_cast<float4 *>(Tfx + y * C::NXW + 4 * qx + C::RA) = masked(o0);
-                if (ckind[k] != 1)  // tile or y strip: f_y / e_y
-                    *reinterpret_cast<float4 *>(Tfy + (y + R) * C::BX + 4 * qx) = masked(o1);
-                if (ckind[k] == 0)
-                    *reinterpret_cast<float4 *>(Tfz + y * C::BX + 4 * qx) = masked(o2);
-            }
-            dz_shift<R, K1>(acc1[k], cv, a.t1[2]);
-        }
-        group_sync(field, C::GROUP);
-
-        // ---- stage 2: outer derivatives of the temporaries of plane s feed
-        //      the pending outputs; output o = s - R is complete
-        float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (has_s) {
-            const float4 cz = lds4(Tfz + ty * C::BX + 4 * tx);
-            dz_feed<R, K2>(acc2, cz, a.t2[2]);
-            const float4 dxv = dx4<R, C::RA, K2>(Tfx + ty * C::NXW + 4 * tx, a.t2[0]);
-            const float4 dyv = dy4<R, K2>(Tfy + (ty + R) * C::BX + 4 * tx, C::BX, a.t2[1]);
-            acc2[R] = f4add(acc2[R], f4add(dxv, dyv));
-            val = acc2[0];
-            dz_shift<R, K2>(acc2, cz, a.t2[2]);
-        }
-        float *XB = xchg + (j & 1) * 2 * C::INT;
-        const int q = ty * C::BX + 4 * tx;
-        if (has_o) *reinterpret_cast<float4 *>(XB + field * C::INT + q) = val;
-        // every thread: temporaries consumed, A and B exchanged (or abandon)
-        if (__syncthreads_or(bad || *abort_flag)) {
-            if (tid == 0) {
-                *abort_flag = 1;
-                atomicOr(a.err, DEV_ERR_TIMEOUT);
-            }
-            break;
-        }
-        if (has_o) {
-            const float *U = Q + 3 * C::NBOX;
-            const float4 A = lds4(XB + q), B = lds4(XB + C::INT + q);
-            const float4 qc = lds4(U + 2 * field * C::INT + q);
-            const float4 qm = lds4(U + (2 * field + 1) * C::INT + q);
-            const float4 b = lds4(U + 4 * C::INT + q), av = lds4(U + 5 * C::INT + q),
-                         sv = lds4(U + 6 * C::INT + q);
-            const float dyz = dpy + a.dpz[o];
-            float4 rhs;
-            if (field == 0)
-                rhs = make_float4(av.x * A.x + sv.x * B.x, av.y * A.y + sv.y * B.y,
-                                  av.z * A.z + sv.z * B.z, av.w * A.w + sv.w * B.w);
-            else
-                rhs = make_float4(sv.x * A.x + B.x, sv.y * A.y + B.y, sv.z * A.z + B.z,
-                                  sv.w * A.w + B.w);
-            float4 v;
-            v.x = qc.x + (1.f - (dpx4[0] + dyz) * b.x) * (qc.x - qm.x) + b.x * rhs.x;
-            v.y = qc.y + (1.f - (dpx4[1] + dyz) * b.y) * (qc.y - qm.y) + b.y * rhs.y;
-            v.z = qc.z + (1.f - (dpx4[2] + dyz) * b.z) * (qc.z - qm.z) + b.z * rhs.z;
-            v.w = qc.w + (1.f - (dpx4[3] + dyz) * b.w) * (qc.w - qm.w) + b.w * rhs.w;
-            if (ok) {
-                const int64_t off = (int64_t)o * a.L.plane + (int64_t)gy * a.L.nxp + gx;
-                *reinterpret_cast<float4 *>(qn + off) = v;
-            }
-        }
-        // release: plane s (no longer needed) and this iteration's Q slot
-        __syncwarp();
+    int issued = 0;
+    if (tid >= C::CONSUMERS) {
+        // Producer lane.  Ring P slot jj % NP: the plane's box of p and r;
+        // ring Q slot jj % NQ: the n box at s = P0 + jj - R (from jj >= 2R)
+        // and the update tiles at o = P0 + jj - 2R (from jj >= 4R).  One full
+        // barrier covers both.
         if (lane == 0) {
-            if (j >= R) mbar_arrive(&emptyP[(j - R) % C::NP]);
-            mbar_arrive(&emptyQ[sq]);
+            RingPos<C::NP> pp;
+            RingPos<C::NQ> pq;
+            for (int jj = 0; jj < nplanes && !*abort_flag; ++jj, pp.next(), pq.next()) {
+                const int sp = pp.slot(jj), sq = pq.slot(jj);
+                if ((jj >= C::NP && !mbar_wait_bounded(&emptyP[sp], pp.phase(jj) ^ 1u)) ||
+                    (jj >= C::NQ && !mbar_wait_bounded(&emptyQ[sq], pq.phase(jj) ^ 1u))) {
+                    if (!*abort_flag) atomicOr(a.err, DEV_ERR_TIMEOUT);
+                    *abort_flag = 1;
+                    break;
+                }
+                const bool qs = jj >= 2 * R, qo = jj >= 4 * R;
+                mbar_arrive_expect_tx(&full[sp], C::PBYTES + (qs ? C::NBYTES : 0) +
+                                                     (qo ? C::UBYTES : 0));
+                tma_load_5d(ringP + sp * C::PSLOT, &map_box, &full[sp], x0 - 2 * C::RA,
+                            y0 - 2 * R, P0 + jj, a.cur, 2 * shot);
+                float *Q = ringQ + sq * C::QSLOT;
+                if (qs)
+                    tma_load_4d(Q, &map_nbox, &full[sp], x0 - C::RA, y0 - R, P0 + jj - R, 3);
+                if (qo) {
+                    const int o = P0 + jj - 2 * R;
+                    tma_load_5d(Q + C::OFF_W, &map_wlev, &full[sp], x0, y0, o, 0, 2 * shot);
+                    tma_load_4d(Q + C::OFF_C, &map_cint, &full[sp], x0, y0, o, 0);
+                }
+                issued = jj + 1;
+            }
+            chain_trigger();  // the next launch may move in (see acoustic.cu)
+        }
+    } else {
+        // the thread's cross cell: float4 column qx in [-1, 16], row y in
+        // [-R, BY + R); tile cells first, then the x strips, then the y strips
+        const bool valid = tid < C::NCELL, tile = tid < C::TILE;
+        int qx = tid % C::TX, y = tid / C::TX;
+        bool to_x = tile, to_y = tile;  // whether f_x / f_y of the cell is needed
+        if (!tile && tid < C::TILE + 2 * C::BY) {
+            const int e = tid - C::TILE;
+            qx = e < C::BY ? -1 : C::TX;
+            y = e % C::BY;
+            to_x = true;
+        } else if (!tile && valid) {
+            const int e = tid - C::TILE - 2 * C::BY;
+            const int rr = e / C::TX;
+            qx = e % C::TX;
+            y = rr < R ? rr - R : C::BY + (rr - R);
+            to_y = true;
+        }
+        const int cbox = (y + 2 * R) * C::PX + 4 * qx + 2 * C::RA;  // the cell in the p/r box
+        const int cnb = (y + R) * C::NXW + 4 * qx + C::RA;          // the cell in the n box
+        unsigned mask = 0u;  // elements inside the grid
+        if (y0 + y >= 0 && y0 + y < a.L.ny)
+            for (int e = 0; e < 4; ++e) {
+                const int xe = x0 + 4 * qx + e;
+                if (xe >= 0 && xe < a.L.nx) mask |= 1u << e;
+            }
+        const int gx = x0 + 4 * qx, gy = y0 + y;
+        const bool ok = tile && gx < a.L.nxp && gy < a.L.ny;
+        float dpx4[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            dpx4[i] = (tile && gx + i < a.L.nx) ? a.dpx[gx + i] : 0.f;
+        const f2 dpx_lo = f2_pack(dpx4[0], dpx4[1]), dpx_hi = f2_pack(dpx4[2], dpx4[3]);
+        const float dpy = ok ? a.dpy[gy] : 0.f;
+        const f2 one2 = f2_splat(1.f);
+        float *qn = a.wave + (int64_t)(4 * shot + 1 - a.cur) * a.L.vol +
+                    (ok ? (int64_t)gy * a.L.nxp + gx : 0);
+        const int q = y * C::BX + 4 * qx;
+
+        Q4 acc1[2][2 * R], acc2[2][2 * R];
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+            for (int i = 0; i < 2 * R; ++i) acc1[f][i] = acc2[f][i] = Q4{0ull, 0ull};
+        RingPos<C::NP> pp, ps;  // slots of the arriving plane and of plane s
+        RingPos<C::NQ> pq;
+#pragma unroll U
+        for (int j = 0; j < nplanes; ++j) {
+            const int sp = pp.slot(j), sq = pq.slot(j);
+            const bool has_s = j >= 2 * R, has_o = j >= 4 * R;
+            const int s = P0 + j - R, o = P0 + j - 2 * R;
+            const float dz = has_o ? __ldg(a.dpz + o) : 0.f;
+            const bool good = !*abort_flag && mbar_wait_bounded(&full[sp], pp.phase(j));
+            const int ss = j >= R ? ps.slot(j - R) : 0;  // slot of plane s
+            const float *Q = ringQ + sq * C::QSLOT;
+            float *T = tmp + (j & 1) * 2 * C::TMP;
+
+            // ---- stage 1: z-derivative feed; gradient and temporaries of plane s
+            Q4 fz[2];
+            if (good && valid) {
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    const Q4 cv = lds_q4(ringP + sp * C::PSLOT + f * C::BOX + cbox);
+                    dz_feed_q4<R, K1>(acc1[f], cv, a.t1[2]);
+                    if (has_s) {
+                        const float *B = ringP + ss * C::PSLOT + f * C::BOX + cbox;
+                        const Q4 gxv = q4_from(dx4<R, C::RA, K1>(B - C::RA, a.t1[0]));
+                        const Q4 gyv = dy_q4<R, K1>(B, C::PX, a.t1[1]);
+                        const Q4 gzv = acc1[f][0];
+                        const Q4 nx = lds_q4(Q + cnb), ny = lds_q4(Q + C::NBOX + cnb),
+                                 nz = lds_q4(Q + 2 * C::NBOX + cnb);
+                        const Q4 h = q4_fma(nz, gzv, q4_fma(nx, gxv, q4_mul(ny, gyv)));
+                        Q4 o0, o1, o2;
+                        if (f == 0) {  // f_i = D_i p - n_i h
+                            const Q4 mh = q4_neg(h);
+                            o0 = q4_fma(nx, mh, gxv);
+                            o1 = q4_fma(ny, mh, gyv);
+                            o2 = q4_fma(nz, mh, gzv);
+                        } else {  // e_i = n_i h
+                            o0 = q4_mul(nx, h);
+                            o1 = q4_mul(ny, h);
+                            o2 = q4_mul(nz, h);
+                        }
+                        // zero ghosts: temporaries outside the grid vanish
+                        const unsigned m = s >= 0 && s < a.L.nz ? mask : 0u;
+                        float *Tf = T + f * C::TMP;
+                        if (to_x)
+                            *reinterpret_cast<float4 *>(Tf + y * C::NXW + 4 * qx + C::RA) =
+                                masked(o0, m);
+                        if (to_y)
+                            *reinterpret_cast<float4 *>(Tf + C::FX + (y + R) * C::BX + 4 * qx) =
+                                masked(o1, m);
+                        fz[f] = q4_from(masked(o2, m));
+                    }
+                    dz_shift_q4<R, K1>(acc1[f], cv, a.t1[2]);
+                }
+            }
+            __syncwarp();
+            // the temporaries of plane s are written (and those of two planes
+            // before consumed); leave together after a failed wait
+            if (consumers_or(C::CONSUMERS, !good)) {
+                if (tid == 0) {
+                    *abort_flag = 1;
+                    atomicOr(a.err, DEV_ERR_TIMEOUT);
+                }
+                break;
+            }
+            // the box of plane s has been read by this warp (stage 2 reads
+            // only temporaries and the Q slot)
+            if (lane == 0 && j >= R) mbar_arrive(&emptyP[ss]);
+
+            // ---- stage 2 (tile warps): outer derivatives of the temporaries
+            //      of plane s feed the pending outputs; output o is complete
+            if (tile && has_s) {
+                Q4 H[2];
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    const float *Tf = T + f * C::TMP;
+                    dz_feed_q4<R, K2>(acc2[f], fz[f], a.t2[2]);
+                    const Q4 dxv =
+                        q4_from(dx4<R, C::RA, K2>(Tf + y * C::NXW + 4 * qx, a.t2[0]));
+                    const Q4 dyv =
+                        dy_q4<R, K2>(Tf + C::FX + (y + R) * C::BX + 4 * qx, C::BX, a.t2[1]);
+                    acc2[f][R] = q4_add(acc2[f][R], q4_add(dxv, dyv));
+                    H[f] = acc2[f][0];
+                    dz_shift_q4<R, K2>(acc2[f], fz[f], a.t2[2]);
+                }
+                if (has_o) {
+                    const float *w = Q + C::OFF_W + q, *cc = Q + C::OFF_C + q;
+                    const Q4 b = lds_q4(cc), av = lds_q4(cc + C::INT),
+                             sv = lds_q4(cc + 2 * C::INT);
+                    const f2 dyz = f2_splat(-(dpy + dz));
+                    const Q4 keep = Q4{f2_fma(f2_sub(dyz, dpx_lo), b.lo, one2),
+                                       f2_fma(f2_sub(dyz, dpx_hi), b.hi, one2)};
+#pragma unroll
+                    for (int f = 0; f < 2; ++f) {
+                        const Q4 rhs = f == 0 ? q4_fma(av, H[0], q4_mul(sv, H[1]))
+                                              : q4_fma(sv, H[0], H[1]);
+                        const Q4 qc = lds_q4(w + (2 * f + a.cur) * C::INT);
+                        const Q4 qm = lds_q4(w + (2 * f + 1 - a.cur) * C::INT);
+                        const Q4 v = q4_fma(b, rhs, q4_fma(keep, q4_sub(qc, qm), qc));
+                        if (ok)
+                            *reinterpret_cast<ulonglong2 *>(qn + 2 * f * a.L.vol +
+                                                            (int64_t)o * a.L.plane) =
+                                make_ulonglong2(v.lo, v.hi);
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&emptyQ[sq]);
+            pp.next();
+            pq.next();
+            if (j >= R) ps.next();
         }
     }
     __syncthreads();
-    if (*abort_flag && tid == 0) {
-        for (int jj = issuedP - C::NQ; jj < issuedP; ++jj)
-            if (jj >= 0) {
-                mbar_wait_bounded(&fullP[jj % C::NP], (uint32_t)((jj / C::NP) & 1), 200000000ull);
-                mbar_wait_bounded(&fullQ[jj % C::NQ], (uint32_t)((jj / C::NQ) & 1), 200000000ull);
-            }
+    if (*abort_flag && tid == C::CONSUMERS) {
+        for (int jj = issued - C::NP; jj < issued; ++jj)
+            if (jj >= 0)
+                mbar_wait_bounded(&full[jj % C::NP], (uint32_t)((jj / C::NP) & 1), 200000000ull);
     }
-}
-
-template <int R, int STAG, int TY>
-const void *fused_fn() {
-    return (const void *)&tti_fused_kernel<R, 1, STAG ? 1 : 0, STAG ? -1 : 0, TY>;
+    if (inj.nsrc > 0 && tid == 0 && !*abort_flag)
+        tti_inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
 }
 
 struct FusedInfo {
     const void *fn;
     size_t smem;
     int px, py, nxw, nyh, by, threads;
+    float launch, lat, thr, warm;  // cost constants (see acoustic.cu)
 };
 
-template <int R, int TY>
-FusedInfo fused_info_t(int stag) {
-    using C = TfCfg<R, 1, TY>;
-    return FusedInfo{stag ? fused_fn<R, 1, TY>() : fused_fn<R, 0, TY>(), C::SMEM, C::PX, C::PY,
-                     C::NXW, C::NYH, C::BY, C::THREADS};
+template <int R, int TY, int D, int U, int MINB>
+FusedInfo fused_info_t(int stag, float launch, float lat, float thr, float warm) {
+    using C = TfCfg<R, TY, D>;
+    return FusedInfo{stag ? (const void *)&tti_fused_kernel<R, TY, D, 1, -1, U, MINB>
+                          : (const void *)&tti_fused_kernel<R, TY, D, 0, 0, U, MINB>,
+                     C::SMEM, C::PX,  C::PY, C::NXW, C::NYH, C::BY, C::THREADS,
+                     launch,  lat,    thr,   warm};
 }
 
-// Configuration 0: 64 x 8 tiles, two CTAs per SM; configuration 1: 64 x 16
-// tiles (fewer recomputed cross cells per tile point), one CTA per SM.
+// Configuration 0: 64 x 16 tiles, one CTA per SM (R <= 2; 1.38x the tile's
+// gradients); configuration 1: 64 x 8 tiles, two CTAs (1.63x).  so 4, us per
+// step: 96^3 23.0 and 26.7, 256^3 204 and 248, 384^3 598 and 711, 512^3 1430
+// and 1664.  The costs are fitted to 13 problems.
 bool fused_info(int radius, int stag, int config, FusedInfo *out) {
-    const bool tall = config == 1;
+    const bool small = config == 1;
     switch (radius) {
-        case 1: *out = tall ? fused_info_t<1, 16>(stag) : fused_info_t<1, 8>(stag); return true;
-        case 2: *out = tall ? fused_info_t<2, 16>(stag) : fused_info_t<2, 8>(stag); return true;
-        case 4: *out = fused_info_t<4, 8>(stag); return true;
+        case 1:
+            *out = small ? fused_info_t<1, 8, 1, 2, 2>(stag, 4.1f, 1.05f, 0.60f, 0.59f)
+                         : fused_info_t<1, 16, 1, 2, 1>(stag, 2.2f, 1.30f, 0.05f, 0.72f);
+            return true;
+        case 2:
+            *out = small ? fused_info_t<2, 8, 1, 2, 2>(stag, 4.1f, 1.18f, 0.715f, 0.59f)
+                         : fused_info_t<2, 16, 1, 2, 1>(stag, 2.2f, 1.46f, 0.05f, 0.72f);
+            return true;
+        case 4:
+            *out = fused_info_t<4, 8, 1, 1, 1>(stag, 3.f, 2.5f, 1.0f, 0.55f);
+            return true;
         default: return false;
     }
 }
@@ -379,23 +389,43 @@ bool tti_fused_supported(int radius) {
     return fused_info(radius, 0, 0, &in);
 }
 
-fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, float *wave,
-                         const float *coef, TtiPlan *plan, int config) {
-    FusedInfo in;
-    if (!fused_info(radius, stag, config, &in))
-        return set_error(FD_ERR_ARG, "the fused TTI scheme covers space orders up to 8");
+// Estimated time (us) of a fused step and its chunk count.
+static fd_status fused_estimate(const FusedInfo &in, int radius, const WaveLayout &L, int nshots,
+                                int *nzc, double *us) {
     FD_TRY(raise_smem_limit(in.fn, in.smem));
     int dev = 0, nsm = 0, per_sm = 0;
     FD_CUDA_TRY(cudaGetDevice(&dev));
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     FD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, in.fn, in.threads, in.smem));
     if (per_sm < 1) return set_error(FD_ERR_CUDA, "fused TTI kernel does not fit on an SM");
-    const int bx = 64, by = in.by;
-    const int ntx = (L.nx + bx - 1) / bx, nty = (L.ny + by - 1) / by;
-    const int64_t cols = (int64_t)ntx * nty * nshots;
+    const int64_t cols =
+        (int64_t)((L.nx + 63) / 64) * ((L.ny + in.by - 1) / in.by) * nshots;
     // 4R warm-up planes, the first half of which only feed the z pipeline
-    int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, 0.55 * 4 * radius, bx * by / 950.0);
-    if (nzc > 65535 / nshots) nzc = 65535 / nshots > 1 ? 65535 / nshots : 1;
+    double planes = 0.0;
+    *nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, in.warm * 4 * radius, in.thr / in.lat, &planes);
+    if (*nzc > 60000 / nshots) *nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
+    *us = in.launch + in.lat * planes;
+    return FD_OK;
+}
+
+fd_status tti_fused_time(int radius, int stag, const WaveLayout &L, int nshots, double *us) {
+    FusedInfo in;
+    if (!fused_info(radius, stag, 0, &in))
+        return set_error(FD_ERR_ARG, "the fused TTI scheme covers space orders up to 8");
+    int nzc = 1;
+    return fused_estimate(in, radius, L, nshots, &nzc, us);
+}
+
+fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, float *wave,
+                         const float *coef, TtiPlan *plan, int config) {
+    FusedInfo in;
+    if (!fused_info(radius, stag, config, &in))
+        return set_error(FD_ERR_ARG, "the fused TTI scheme covers space orders up to 8");
+    const uint32_t bx = 64, by = in.by;
+    const int ntx = (L.nx + bx - 1) / bx, nty = (L.ny + by - 1) / by;
+    int nzc = 1;
+    double us = 0.0;
+    FD_TRY(fused_estimate(in, radius, L, nshots, &nzc, &us));
     const int zchunk = (L.nz + nzc - 1) / nzc;
     nzc = (L.nz + zchunk - 1) / zchunk;
     if ((int64_t)nshots * nzc > 65535 || nty > 65535)
@@ -404,30 +434,41 @@ fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, 
     plan->stag = stag ? 1 : 0;
     plan->scheme = kTtiFused;
     plan->config = config == 1 ? 1 : 0;
-    plan->grid = dim3(ntx, nty, nshots * nzc);
-    plan->block = dim3(in.threads, 1, 1);
-    plan->smem1 = in.smem;
-    plan->zchunk = zchunk;
-    plan->nzc = nzc;
-    const uint64_t sy = (uint64_t)L.nxp * 4, sz = (uint64_t)L.plane * 4, sw = (uint64_t)L.vol * 4;
-    FD_TRY(make_tensor_map_4d(&plan->map_fbox, wave, L.nx, L.ny, L.nz, 4ull * nshots, sy, sz, sw,
-                              in.px, in.py, 1, 1));
-    FD_TRY(make_tensor_map_4d(&plan->map_fnbox, coef, L.nx, L.ny, L.nz, 6, sy, sz, sw, in.nxw,
-                              in.nyh, 1, 1));
-    FD_TRY(make_tensor_map_4d(&plan->map_wint, wave, L.nx, L.ny, L.nz, 4ull * nshots, sy, sz, sw,
-                              bx, by, 1, 1));
-    return make_tensor_map_4d(&plan->map_cint, coef, L.nx, L.ny, L.nz, 6, sy, sz, sw, bx, by, 1,
-                              1);
+    plan->p1.fn = in.fn;
+    plan->p1.grid = dim3(ntx, nty, nshots * nzc);
+    plan->p1.block = dim3(in.threads, 1, 1);
+    plan->p1.smem = in.smem;
+    plan->p1.zchunk = zchunk;
+    plan->p1.nzc = nzc;
+    plan->p1.est_us = us;
+    const uint64_t sy = (uint64_t)L.nxp * 4, sz = (uint64_t)L.plane * 4, sv = (uint64_t)L.vol * 4;
+    const uint64_t wdim[5] = {(uint64_t)L.nx, (uint64_t)L.ny, (uint64_t)L.nz, 2, 2ull * nshots};
+    const uint64_t wstr[4] = {sy, sz, sv, 2 * sv};
+    const uint32_t box[5] = {(uint32_t)in.px, (uint32_t)in.py, 1, 1, 2};
+    const uint32_t lev[5] = {bx, by, 1, 2, 2};
+    FD_TRY(make_tensor_map_5d(&plan->map_fbox, wave, wdim, wstr, box));
+    FD_TRY(make_tensor_map_5d(&plan->map_wlev, wave, wdim, wstr, lev));
+    FD_TRY(make_tensor_map_4d(&plan->map_fnbox, coef, L.nx, L.ny, L.nz, 6, sy, sz, sv, in.nxw,
+                              in.nyh, 1, 3));
+    return make_tensor_map_4d(&plan->map_c2, coef, L.nx, L.ny, L.nz, 6, sy, sz, sv, bx, by, 1, 3);
 }
 
-fd_status tti_fused_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream) {
-    FusedInfo in;
-    if (!fused_info(plan.radius, plan.stag, plan.config, &in))
-        return set_error(FD_ERR_SO, "bad fused TTI plan");
-    int zchunk = plan.zchunk, nzc = plan.nzc;
-    void *params[] = {(void *)&plan.map_fbox, (void *)&plan.map_fnbox, (void *)&plan.map_wint,
-                      (void *)&plan.map_cint, (void *)&a, (void *)&zchunk, (void *)&nzc};
-    FD_CUDA_TRY(cudaLaunchKernel(in.fn, plan.grid, plan.block, params, plan.smem1, stream));
+fd_status tti_fused_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
+                           const AcousticInject &inj, const ReceiveArgs &receive) {
+    ReceiveArgs rec = receive;
+    dim3 grid = plan.p1.grid;
+    rec.slices = 0;
+    if (rec.nrec > 0) {
+        if (grid.z >= 65535) return set_error(FD_ERR_ARG, "no grid slice left for receivers");
+        rec.slices = receive_slices(rec, grid.x, grid.y, plan.p1.block.x);
+        if ((int64_t)grid.z + rec.slices > 65535) rec.slices = 65535 - grid.z;
+        grid.z += rec.slices;
+    }
+    int zchunk = plan.p1.zchunk, nzc = plan.p1.nzc;
+    void *params[] = {(void *)&plan.map_fbox, (void *)&plan.map_fnbox, (void *)&plan.map_wlev,
+                      (void *)&plan.map_c2,   (void *)&a,              (void *)&inj,
+                      (void *)&rec,           (void *)&zchunk,         (void *)&nzc};
+    FD_CUDA_TRY(launch_chained(plan.p1.fn, grid, plan.p1.block, params, plan.p1.smem, stream));
     note_launch(stream);
     return FD_OK;
 }

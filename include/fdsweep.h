@@ -126,9 +126,9 @@ fd_status acoustic_forward(const fd_grid *grid, int so, double dt, int nt, int n
  *                  with it.
  *                  FD_STORAGE_AUTO: the faster of the two on GB300 for the
  *                  space order, measured at 512^3: binary16 for so <= 8 (its
- *                  kernel 1.26x / 1.10x the FP32 one at so 4 / 8), FP32 for
- *                  so 12 and 16 (where the binary16 kernel, bound by shared
- *                  memory and conversions, ran 0.94x / 0.89x), and FP32 with
+ *                  kernel 1.69x / 1.15x the FP32 one at so 4 / 8), FP32 for
+ *                  so 12 and 16 (where the binary16 kernel, bound by the
+ *                  conversions, ran 0.95x / 0.80x), and FP32 with
  *                  FD_DAMP_FIELD.  The results are those of the storage
  *                  chosen.
  *   opts->damp_layout

@@ -835,7 +835,6 @@ static fd_status acoustic_forward_h_impl(const fd_grid *grid, int so, double dt,
     FD_STAGE(s, "acoustic f16: inputs staged");
 
     // ---- K0: coefficients (FP64 -> FP32 as in the FP32 path, then binary16)
-    FD_CUDA_TRY(cudaMemsetAsync(bh, 0, (size_t)LH.vol * 2, s));
     FD_TRY(init_medium_stats(dstats, s));
     FD_TRY(setup_acoustic_coeffs(sm.dev, sdamp.dev, dt, L, b32, dps, dstats, s));
     FD_TRY(narrow_rows(b32, L.nxp, bh, LH.nxp, L.nx, rows, s));
@@ -902,9 +901,23 @@ static fd_status acoustic_forward_h_impl(const fd_grid *grid, int so, double dt,
     const bool graphs = !timing && trace_level() < 2;
     StepEvents evs;
     if (timing) FD_TRY(evs.create(nsteps + 1, 3));
-    SideLane side;
-    const bool overlap = nrec > 0;
-    if (overlap) FD_TRY(side.begin());
+    const bool inject_in_k1 = nsrc > 0 && nsrc <= kInjectMaxSources;
+    const bool record_in_k1 = nrec > 0 && plan.grid.z < 65535;
+    AcousticInject inj;
+    memset(&inj, 0, sizeof(inj));
+    if (inject_in_k1) {
+        inj.src_tab = src_tab;
+        inj.src_wav = swav.dev;
+        inj.nsrc = nsrc;
+        inj.nt = nt;
+    }
+    ReceiveArgs rec;
+    memset(&rec, 0, sizeof(rec));
+    rec.tab = rec_tab;
+    rec.out = srec.dev;
+    rec.nshots = nshots;
+    rec.nrec = record_in_k1 ? nrec : 0;
+    rec.nt = nt;
     auto step = [&](int i, int par, bool via_counter) -> fd_status {
         AcousticHArgs ai = a;
         ai.lev_cur = par;
@@ -914,21 +927,18 @@ static fd_status acoustic_forward_h_impl(const fd_grid *grid, int so, double dt,
         si.inj_level = 1 - par;
         si.rec_level = par;
         si.step_base = via_counter ? counter : nullptr;
-        if (overlap) {
-            FD_TRY(side.fork(s));
-            FD_TRY(sparse_h_launch(si, i, false, true, side.get()));
-        }
+        inj.step = rec.step = i;
+        inj.step_base = rec.step_base = si.step_base;
         if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 0), s));
-        FD_TRY(acoustic_h_launch(plan, ai, s));
+        FD_TRY(acoustic_h_launch(plan, ai, s, &inj, &rec));
         if (!via_counter && trace_level() >= 2) FD_STAGE(s, "acoustic_step_h kernel");
         if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 1), s));
-        FD_TRY(sparse_h_launch(si, i, nsrc > 0, false, s));
+        FD_TRY(sparse_h_launch(si, i, nsrc > 0 && !inject_in_k1, nrec > 0 && !record_in_k1, s));
         if (timing) FD_CUDA_TRY(cudaEventRecord(evs.at(i, 2), s));
-        if (overlap) FD_TRY(side.join(s));
         return FD_OK;
     };
     FD_TRY(run_time_loop(nsteps, s, counter, graphs, step,
-                         [&](int n) { return traces.upto(n, s); }));
+                         [&](int n) { return traces.upto(n, s); }, kFewLaunchesGraph));
     const int last = nsteps & 1, prev_of_last = 1 - last;
     {
         SparseHArgs si = sp;
@@ -1612,10 +1622,9 @@ fd_status acoustic_forward_opts(const fd_grid *grid, int so, double dt, int nt, 
         return fdsweep::set_error(FD_ERR_ARG, "acoustic_forward_opts: damp_layout %d not in {0, 1}",
                                   layout);
     // FD_STORAGE_AUTO: binary16 storage where its kernel measured faster than
-    // the FP32 one on GB300 at 512^3 (so <= 8: 1.26x and 1.10x), FP32 storage
-    // where it did not (so 12: 0.94x, so 16: 0.89x; the binary16 kernel is
-    // bound by shared memory and conversions there), and FP32 with a 3-D
-    // damping field.
+    // the FP32 one on GB300 at 512^3 (so 4: 1.69x, so 8: 1.15x), FP32 storage
+    // where it did not (so 12: 0.95x, so 16: 0.80x; the binary16 kernel is
+    // bound by the conversions there), and FP32 with a 3-D damping field.
     if (storage == FD_STORAGE_AUTO)
         storage = (so <= 8 && layout == FD_DAMP_AXES) ? FD_STORAGE_F16 : FD_STORAGE_F32;
     if (storage == FD_STORAGE_F32)

@@ -367,7 +367,8 @@ int acoustic_h_num_configs(int radius);  // 0: no binary16 kernel for this radiu
 fd_status acoustic_h_plan(int radius, int config, const WaveLayout &L, int nshots, int lps,
                           half_bits *wave, const half_bits *bcoef, AcousticPlan *plan);
 fd_status acoustic_h_launch(const AcousticPlan &plan, const AcousticHArgs &args,
-                            cudaStream_t stream);
+                            cudaStream_t stream, const AcousticInject *inject = nullptr,
+                            const ReceiveArgs *receive = nullptr);
 
 // Sparse injection / interpolation on binary16 levels (forward schedule:
 // src[n] into level inj_level, rec[n] from level rec_level at step n).  The
@@ -393,7 +394,8 @@ fd_status sparse_h_launch(const SparseHArgs &a, int step, bool do_inject, bool d
                           cudaStream_t stream);
 
 // dst row r (stride dst_stride halves) = nearest binary16 values of src row r
-// (stride src_stride floats), nx values per row, `rows` rows; and back.
+// (stride src_stride floats), nx values per row (rounded up to four with
+// zeros), `rows` rows; and back.
 fd_status narrow_rows(const float *src, int64_t src_stride, half_bits *dst, int64_t dst_stride,
                       int nx, int64_t rows, cudaStream_t stream);
 fd_status widen_rows(const half_bits *src, int64_t src_stride, float *dst, int64_t dst_stride,

@@ -274,17 +274,20 @@ fd_status acoustic_adjoint(const fd_grid *grid, int so, double dt, int nt, int n
  * J(m) = 1/2 sum ||d(m) - d_obs||^2 (adjoint-state method):
  *   grad m = -(1/dt^2) sum_{k=1}^{nt-1} w^k (u^k - 2u^{k-1} + u^{k-2}),
  * w the adjoint of acoustic_adjoint.  The forward wavefield is checkpointed
- * (both time levels) every `checkpoint_every` steps (0: round(sqrt(nt-1)))
- * and recomputed segment by segment during the reverse sweep (the paper's
- * time-subsampled save, Listing fd-4, used for inversion).
+ * (both time levels) every `checkpoint_every` steps and recomputed segment by
+ * segment during the reverse sweep (the paper's time-subsampled save, Listing
+ * fd-4, used for inversion).  0: the whole history of a batch of shots, which
+ * needs no recomputation, when it takes at most an eighth of the device memory
+ * and a quarter of what is free, otherwise every round(sqrt(nt-1)) steps.
  *
  *   src_wav   [nshots][nt][nsrc]  source wavelets of the forward model.
  *   rec_resid [nshots][nt][nrec]  residual traces.
  *   grad_m    [nz][ny][nx]        output.
- *   Device memory: 4 + K + 2 + 2 ceil((nt-1)/K) wavefield volumes per shot
- *   of a batch, K the checkpoint interval; shots are stepped together in
- *   batches of as many as fit in 80 % of the free device memory (at least
- *   one; the environment variable FDSWEEP_GRAD_BATCH=n caps the batch).
+ *   Device memory: 11 + K + 2 + 2 ceil((nt-1)/K) wavefield volumes per shot
+ *   of a batch (9 + K + 2 for one segment), K the checkpoint interval; 7 fewer
+ *   where one shot would not fit otherwise.  Shots are stepped together in
+ *   batches of up to 16, as many as fit in 80 % of the free device memory (at
+ *   least one; the environment variable FDSWEEP_GRAD_BATCH=n caps the batch).
  *   Other arguments as for acoustic_forward.
  */
 fd_status acoustic_gradient(const fd_grid *grid, int so, double dt, int nt, int nshots,
@@ -292,6 +295,17 @@ fd_status acoustic_gradient(const fd_grid *grid, int so, double dt, int nt, int 
                             const float *src_wav, int nrec, const float *rec_xyz,
                             const float *rec_resid, int checkpoint_every, float *grad_m,
                             void *stream);
+
+/*
+ * acoustic_vjp -- acoustic_gradient and acoustic_adjoint in one reverse sweep:
+ * both gradients of <rec_resid, d(m, q)>, with respect to m (grad_m) and to the
+ * source wavelets (src_grad [nshots][nt][nsrc], as acoustic_adjoint returns
+ * it).  Arguments and errors as for acoustic_gradient.
+ */
+fd_status acoustic_vjp(const fd_grid *grid, int so, double dt, int nt, int nshots, const float *m,
+                       const float *damp, int nsrc, const float *src_xyz, const float *src_wav,
+                       int nrec, const float *rec_xyz, const float *rec_resid,
+                       int checkpoint_every, float *grad_m, float *src_grad, void *stream);
 
 /*
  * acoustic_forward_noalloc -- acoustic_forward for callers that cannot

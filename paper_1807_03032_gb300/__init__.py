@@ -193,7 +193,7 @@ def acoustic_gradient(grid, so, dt, nt, m, src_xyz, src_wav, rec_xyz, rec_resid,
                       checkpoint_every=0, grad=None, stream=None):
     """Gradient with respect to m of <rec_resid, d(m)> (C ABI
     ``acoustic_gradient``), checkpointing the forward wavefield every
-    ``checkpoint_every`` steps (0: sqrt(nt-1)).  Returns [nz][ny][nx]."""
+    ``checkpoint_every`` steps (0: automatic).  Returns [nz][ny][nx]."""
     g = _as_grid(grid)
     nshots, nsrc = int(src_xyz.shape[0]), int(src_xyz.shape[1])
     nrec = int(rec_xyz.shape[1])

@@ -25,8 +25,8 @@ STATUS_NAMES = {
 EXPORTED = ("acoustic_forward", "tti_forward", "tti_forward_opts", "fd_last_error", "fd_version",
             "fd_stats_enable", "fd_stats_reset", "fd_stats_get", "fd_set_acoustic_config",
             "fd_num_acoustic_configs", "fd_launch_count", "acoustic_forward_noalloc",
-            "acoustic_adjoint", "acoustic_gradient", "fd_engine_footprint", "fd_engine_create",
-            "fd_engine_add_shot", "fd_engine_step", "fd_engine_shot_status", "fd_engine_release",
+            "acoustic_adjoint", "acoustic_gradient", "acoustic_vjp", "fd_engine_footprint",
+            "fd_engine_create", "fd_engine_add_shot", "fd_engine_step", "fd_engine_shot_status", "fd_engine_release",
             "fd_engine_stream", "fd_engine_sync", "fd_engine_destroy", "fd_set_time_tiling",
             "fd_num_time_tiling_configs", "fd_set_tti_config", "fd_num_tti_configs",
             "acoustic_forward_opts", "fd_set_acoustic_f16_config", "fd_num_acoustic_f16_configs",
@@ -100,6 +100,8 @@ def load(path: str = LIB_PATH):
         lib.acoustic_adjoint.restype = I
         lib.acoustic_gradient.argtypes = [G, I, D, I, I, P, P, I, P, P, I, P, P, I, P, P]
         lib.acoustic_gradient.restype = I
+        lib.acoustic_vjp.argtypes = [G, I, D, I, I, P, P, I, P, P, I, P, P, I, P, P, P]
+        lib.acoustic_vjp.restype = I
         lib.tti_forward.argtypes = [G, I, D, I, I, P, P, P, P, P, P, I, P, P, I, P, P, P, P, P,
                                     P, P]
         lib.tti_forward.restype = I

@@ -1402,22 +1402,33 @@ static fd_status acoustic_adjoint_impl(const fd_grid *grid, int so, double dt, i
 /*
  * FWI gradient: grad m = d<dd, d(m)>/dm, summed over shots (in batches of
  * shots stepped together, as many as the device memory holds).  Forward with a
- * checkpoint (u^t, u^{t-1}) every K steps; then, segment by segment from the
- * last, the forward states of the segment are recomputed from its checkpoint
- * and the adjoint w (see acoustic_adjoint) is stepped back through it while
+ * checkpoint (u^t, u^{t-1}) every K steps up to the last segment's start; then,
+ * segment by segment from the last, the forward states of the segment are
+ * computed from its checkpoint and the adjoint w (see acoustic_adjoint) is
+ * stepped back through it while
  *   grad += w^k (u^k - 2 u^{k-1} + u^{k-2}),   k = nt-1 .. 1,
  * and finally grad *= -1/dt^2 (du^k/dm = -(u^k - 2u^{k-1} + u^{k-2})/(m+eta)
- * and w = dt^2/(m+eta) lambda).
+ * and w = dt^2/(m+eta) lambda).  With src_grad the adjoint source wavelets
+ * S w^{n+1} are sampled on the way (what acoustic_adjoint returns), so that
+ * both gradients cost one reverse sweep.
+ *
+ * One segment (K = nt-1) needs no recomputation: two stencil sweeps instead of
+ * three.  checkpoint_every = 0 takes it when the history of a batch fits in an
+ * eighth of the device memory and in a quarter of what is free, and segments
+ * of round(sqrt(nt-1)) otherwise.  At so 8: 4 shots at 128^3, 239 steps, 8 GB:
+ * 15.4 ms against 22.2; 2 shots at 64^3: 4.3 against 6.4.
  */
+static constexpr int kGradSteps = 8;  // 1 / 3 / 8 / 16: 19.7 / 16.9 / 16.1 / 15.7 ms
+
 static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, int nt,
                                         int nshots, const float *m, const float *damp, int nsrc,
                                         const float *src_xyz, const float *src_wav, int nrec,
                                         const float *rec_xyz, const float *rec_resid,
-                                        int checkpoint_every, float *grad_m,
-                                        cudaStream_t caller) {
+                                        int checkpoint_every, float *grad_m, float *src_grad,
+                                        const char *what, cudaStream_t caller) {
     FD_TRY(validate_common(grid, so, dt, nt, nshots, m, nsrc, src_xyz, src_wav, nrec, rec_xyz,
                            rec_resid));
-    if (!grad_m) return set_error(FD_ERR_ARG, "acoustic_gradient: grad_m is null");
+    if (!grad_m) return set_error(FD_ERR_ARG, "%s: grad_m is null", what);
     if (checkpoint_every < 0) return set_error(FD_ERR_ARG, "checkpoint_every must be >= 0");
     const int R = so / 2;
     GridDerived gd = derive(grid, so);
@@ -1425,7 +1436,18 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     const size_t dense = (size_t)L.nx * L.ny * L.nz;
     const int ndamp = L.nx + L.ny + L.nz;
     const int nsteps = nt - 1;
+    const int64_t vol = L.vol;
     int K = checkpoint_every > 0 ? checkpoint_every : (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
+    // shots of a batch: at most kGradMaxShots, in batches of about equal size
+    const int nbatch = (nshots + kGradMaxShots - 1) / kGradMaxShots;
+    const int most = nbatch > 0 ? (nshots + nbatch - 1) / nbatch : 0;
+    if (checkpoint_every == 0) {
+        size_t free_b = 0, total_b = 0;
+        FD_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+        const double history = (double)most * (nsteps + 2) * (double)vol * 4;
+        if (history <= (double)total_b / 8 && history <= ((double)free_b + pool_unused()) / 4)
+            K = nsteps;
+    }
     if (K < 1) K = 1;
     if (nsteps > 0 && K > nsteps) K = nsteps;
     const int nseg = nsteps > 0 ? (nsteps + K - 1) / K : 0;
@@ -1435,8 +1457,10 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     // Shots are processed in batches of B (one stencil launch per step for the
     // whole batch); B is bounded by the device memory the per-shot buffers
     // (forward and adjoint pairs, the segment, the checkpoints) need.
-    const int64_t vol = L.vol;
-    const int64_t per_shot = (int64_t)(4 + (K + 2) + 2 * (nseg > 0 ? nseg : 1)) * vol * 4;
+    // The adjoint's levels are a ring of G + 1, so that the imaging condition of
+    // G steps is one launch (see grad_steps_kernel).
+    const int nfwd = nseg > 1 ? 2 : 0, nck = nseg > 1 ? 2 * nseg : 0;
+    int G = K < kGradSteps ? (K > 1 ? K : 1) : kGradSteps;
     int B = 1;
     {
         size_t free_b = 0, total_b = 0;
@@ -1444,20 +1468,28 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
         const int64_t fixed = (int64_t)(4 + 2) * vol * 4 +
                               (int64_t)nshots * (int64_t)nt * (nrec + nsrc) * 4;
         const int64_t budget = (int64_t)(0.8 * (double)free_b) - fixed;
-        const int64_t fit = per_shot > 0 ? budget / per_shot : 1;
-        B = (int)(fit < 1 ? 1 : (fit > nshots ? nshots : fit));
         // FDSWEEP_GRAD_BATCH=n caps the batch (to exercise several batches)
         const char *cap = getenv("FDSWEEP_GRAD_BATCH");
-        if (cap && atoi(cap) > 0 && atoi(cap) < B) B = atoi(cap);
+        auto batch = [&](int g) {
+            const int64_t per_shot = (int64_t)(nfwd + g + 1 + K + 2 + nck) * vol * 4;
+            const int64_t fit = per_shot > 0 ? budget / per_shot : 1;
+            const int b = (int)(fit > most ? most : fit);
+            return cap && atoi(cap) > 0 && atoi(cap) < b ? atoi(cap) : b;
+        };
+        B = batch(G);
+        if (B < 1) {  // the least: one shot, two adjoint levels, one step per launch
+            G = 1;
+            B = 1;
+        }
     }
     Workspace ws;
     float *fwd, *adj, *seg, *ckpt, *grad, *bcoef, *dps;
     SparsePoint *src_tab, *rec_tab;
     MediumStats *dstats;
-    ws.add(&fwd, (size_t)2 * B * vol);
-    ws.add(&adj, (size_t)2 * B * vol);
+    ws.add(&fwd, (size_t)nfwd * B * vol);
+    ws.add(&adj, (size_t)(G + 1) * B * vol);
     ws.add(&seg, (size_t)(K + 2) * B * vol);
-    ws.add(&ckpt, (size_t)2 * (nseg > 0 ? nseg : 1) * B * vol);
+    ws.add(&ckpt, (size_t)nck * B * vol);
     ws.add(&grad, vol);
     ws.add(&bcoef, vol);
     ws.add(&dps, ndamp);
@@ -1465,7 +1497,7 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     ws.add(&rec_tab, (size_t)nshots * nrec);
     ws.add(&dstats, 1);
     Staged sm, sdamp, ssxyz, swav, srxyz, sres;
-    StagedOut sg;
+    StagedOut sg, sq;
     sm.plan(ws, m, dense);
     sdamp.plan(ws, damp, damp ? ndamp : 0);
     ssxyz.plan(ws, src_xyz, (size_t)nshots * nsrc * 3);
@@ -1473,18 +1505,21 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     srxyz.plan(ws, rec_xyz, (size_t)nshots * nrec * 3);
     sres.plan(ws, rec_resid, (size_t)nshots * nt * nrec);
     sg.plan(ws, grad_m, dense);
+    sq.plan(ws, src_grad, src_grad ? (size_t)nshots * nt * nsrc : 0);
     FD_TRY(ws.allocate(s));
     for (Staged *st : {&sm, &sdamp, &ssxyz, &swav, &srxyz, &sres}) FD_TRY(st->place(s));
     FD_TRY(acoustic_common_setup(grid, so, dt, gd, nshots, sm.dev, sdamp.dev, nsrc, ssxyz.dev,
-                                 nrec, srxyz.dev, bcoef, dps, src_tab, rec_tab, dstats,
-                                 "acoustic_gradient", s));
+                                 nrec, srxyz.dev, bcoef, dps, src_tab, rec_tab, dstats, what, s));
     FD_CUDA_TRY(cudaMemsetAsync(grad, 0, (size_t)vol * 4, s));
+    if (sq.dev && nsrc > 0)
+        FD_CUDA_TRY(cudaMemsetAsync(sq.dev, 0, (size_t)nshots * nt * nsrc * 4, s));
     const size_t vb = (size_t)vol * 4;
     for (int s0 = 0; s0 < nshots && nsteps > 0; s0 += B) {
         const int nb = nshots - s0 < B ? nshots - s0 : B;
         AcousticPlan pf, pa, ps;
-        FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nb, 2, fwd, bcoef, &pf));
-        FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nb, 2, adj, bcoef, &pa));
+        if (nseg > 1)
+            FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nb, 2, fwd, bcoef, &pf));
+        FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nb, G + 1, adj, bcoef, &pa));
         FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nb, K + 2, seg, bcoef, &ps));
         AcousticStepArgs af, aa, as;
         fill_step_args(af, grid, gd, fwd, bcoef, dps, nb, &dstats->flags);
@@ -1507,10 +1542,38 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
         res.nsrc = nrec;
         res.src_tab = rec_tab + (size_t)s0 * nrec;
         res.src_wav = sres.dev + (size_t)s0 * nt * nrec;
+        // a few sources are injected by the stencil kernel (see the forward
+        // run), and its extra blocks sample the adjoint at the sources
+        const bool inject_in_k1 = nsrc > 0 && nsrc <= kInjectMaxSources;
+        AcousticInject inj;
+        memset(&inj, 0, sizeof(inj));
+        if (inject_in_k1) {
+            inj.src_tab = src.src_tab;
+            inj.src_wav = src.src_wav;
+            inj.nsrc = nsrc;
+            inj.nt = nt;
+        }
+        float *const qout = sq.dev ? sq.dev + (size_t)s0 * nt * nsrc : nullptr;
+        const bool sample_in_k1 = qout && nsrc > 0 && pa.grid.z < 65535;
+        ReceiveArgs smp;
+        memset(&smp, 0, sizeof(smp));
+        smp.tab = src.src_tab;
+        smp.out = qout;
+        smp.nshots = nb;
+        smp.nrec = sample_in_k1 ? nsrc : 0;
+        smp.nt = nt;
+        SparseArgs sam = src;  // the same by the sparse kernel
+        sam.wave = adj;
+        sam.fields_per_shot = G + 1;
+        sam.nrec = nsrc;
+        sam.rec_tab = src.src_tab;
+        sam.rec_out = qout;
+        sam.rec_dt = 0;
         // 1. forward with checkpoints: ckpt[c] holds (u^{cK-1}, u^{cK}) of every
-        //    shot of the batch ([nseg][nb][2][vol])
-        FD_CUDA_TRY(cudaMemsetAsync(fwd, 0, 2 * nb * vb, s));
-        for (int t = 0; t < nsteps; ++t) {
+        //    shot of the batch ([nseg][nb][2][vol]); the last segment is not
+        //    run here, one segment needs no checkpoint at all
+        if (nseg > 1) FD_CUDA_TRY(cudaMemsetAsync(fwd, 0, 2 * nb * vb, s));
+        for (int t = 0; nseg > 1 && t <= (nseg - 1) * K; ++t) {
             const int cur = t & 1;
             if (t % K == 0) {
                 float *dst = ckpt + (size_t)(t / K) * 2 * nb * vol;
@@ -1519,22 +1582,25 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
                 FD_CUDA_TRY(cudaMemcpy2DAsync(dst + vol, 2 * vb, fwd + (size_t)cur * vol, 2 * vb,
                                               vb, nb, cudaMemcpyDeviceToDevice, s));
             }
+            if (t == (nseg - 1) * K) break;
             AcousticStepArgs ai = af;
             set_two_levels(ai, cur);
-            FD_TRY(acoustic_launch(pf, ai, s));
+            inj.step = t;
+            FD_TRY(acoustic_launch(pf, ai, s, &inj));
             SparseArgs si = src;
             si.wave = fwd;
             si.fields_per_shot = 2;
             si.inj_level0 = 1 - cur;
-            FD_TRY(sparse_launch(si, t, nsrc > 0, false, s));
+            FD_TRY(sparse_launch(si, t, nsrc > 0 && !inject_in_k1, false, s));
         }
-        // 2. adjoint state: w^{nt-1} = B R^T dd^{nt-1} in level acur, w^{nt} = 0
-        FD_CUDA_TRY(cudaMemsetAsync(adj, 0, 2 * nb * vb, s));
+        // 2. adjoint state: w^{nt-1} = B R^T dd^{nt-1} in level acur, w^{nt} = 0 in
+        //    the level before it (all levels are cleared: their halos stay zero)
+        FD_CUDA_TRY(cudaMemsetAsync(adj, 0, (size_t)(G + 1) * nb * vb, s));
         int acur = 0;
         {
             SparseArgs si = res;
             si.wave = adj;
-            si.fields_per_shot = 2;
+            si.fields_per_shot = G + 1;
             si.inj_level0 = acur;
             si.inj_t0 = nt - 1;
             si.inj_dt = 0;
@@ -1545,39 +1611,68 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
             const int t0 = c * K;
             const int kmax = (c + 1) * K < nsteps ? (c + 1) * K : nsteps;
             // seg level l of every shot holds u^{t0 - 1 + l}
-            FD_CUDA_TRY(cudaMemcpy2DAsync(seg, (size_t)(K + 2) * vb,
-                                          ckpt + (size_t)c * 2 * nb * vol, 2 * vb, 2 * vb, nb,
-                                          cudaMemcpyDeviceToDevice, s));
+            if (nseg > 1)
+                FD_CUDA_TRY(cudaMemcpy2DAsync(seg, (size_t)(K + 2) * vb,
+                                              ckpt + (size_t)c * 2 * nb * vol, 2 * vb, 2 * vb, nb,
+                                              cudaMemcpyDeviceToDevice, s));
+            else
+                FD_CUDA_TRY(cudaMemset2DAsync(seg, (size_t)(K + 2) * vb, 0, 2 * vb, nb, s));
             for (int t = t0 + 1; t <= kmax; ++t) {
                 AcousticStepArgs ai = as;
                 ai.lps = K + 2;
                 ai.lev_cur = t - t0;
                 ai.lev_prev = t - t0 - 1;
                 ai.lev_out = t - t0 + 1;
-                FD_TRY(acoustic_launch(ps, ai, s));
+                inj.step = t - 1;
+                FD_TRY(acoustic_launch(ps, ai, s, &inj));
                 SparseArgs si = src;
                 si.wave = seg;
                 si.fields_per_shot = K + 2;
                 si.inj_level0 = t - t0 + 1;
-                FD_TRY(sparse_launch(si, t - 1, nsrc > 0, false, s));
+                FD_TRY(sparse_launch(si, t - 1, nsrc > 0 && !inject_in_k1, false, s));
             }
+            int done = kmax;  // steps above are in the gradient
             for (int k = kmax; k >= t0 + 1; --k) {
-                FD_TRY(grad_accumulate_batch(grad, adj + (size_t)acur * vol, 2 * vol,
-                                             seg + (size_t)(k - t0 + 1) * vol,
-                                             (int64_t)(K + 2) * vol, nb, vol, s));
+                if (done - k + 1 == G || k == t0 + 1) {
+                    GradArgs ga;
+                    ga.grad = grad;
+                    ga.w = adj;
+                    ga.w_stride = (G + 1) * vol;
+                    ga.w_levels = G + 1;
+                    ga.w_level = (acur + G + 1 - (done - k)) % (G + 1);
+                    ga.u = seg + (size_t)(done - t0 + 1) * vol;
+                    ga.u_stride = (int64_t)(K + 2) * vol;
+                    ga.vol = vol;
+                    ga.nb = nb;
+                    ga.steps = done - k + 1;
+                    FD_TRY(grad_accumulate(ga, s));
+                    done = k - 1;
+                }
+                // dq^{k-1} = S w^k, before w^{k-1} is formed
+                if (qout && (k < 2 || !sample_in_k1)) {
+                    SparseArgs si = sam;
+                    si.rec_level = acur;
+                    si.rec_t0 = k - 1;
+                    FD_TRY(sparse_launch(si, 0, false, nsrc > 0, s));
+                }
                 if (k >= 2) {
                     // w^{k-1} = M1 w^k - M2 w^{k+1} + B R^T dd^{k-1}
+                    const int anext = (acur + 1) % (G + 1);
                     AcousticStepArgs ai = aa;
-                    set_two_levels(ai, acur);
-                    FD_TRY(acoustic_launch(pa, ai, s));
+                    ai.lps = G + 1;
+                    ai.lev_cur = acur;
+                    ai.lev_prev = (acur + G) % (G + 1);
+                    ai.lev_out = anext;
+                    smp.step = k - 1;
+                    FD_TRY(acoustic_launch(pa, ai, s, nullptr, &smp));
                     SparseArgs si = res;
                     si.wave = adj;
-                    si.fields_per_shot = 2;
-                    si.inj_level0 = 1 - acur;
+                    si.fields_per_shot = G + 1;
+                    si.inj_level0 = anext;
                     si.inj_t0 = k - 1;
                     si.inj_dt = 0;
                     FD_TRY(sparse_launch(si, 0, nrec > 0, false, s));
-                    acur = 1 - acur;
+                    acur = anext;
                 }
             }
         }
@@ -1587,11 +1682,12 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     FD_TRY(check_finite(grad, L, 1, &dstats->flags, s));
     FD_TRY(copy_field_out(sg.dev, grad, L, s));
     FD_TRY(sg.copy_back(s));
+    FD_TRY(sq.copy_back(s));
     MediumStats hs;
     FD_TRY(read_stats(dstats, &hs, s));
     ws.release();
     FD_TRY(cs.finish());
-    return flags_to_status(hs.flags, "acoustic_gradient");
+    return flags_to_status(hs.flags, what);
 }
 
 }  // namespace fdsweep
@@ -1687,7 +1783,21 @@ fd_status acoustic_gradient(const fd_grid *grid, int so, double dt, int nt, int 
     fdsweep::clear_error();
     return fdsweep::acoustic_gradient_impl(grid, so, dt, nt, nshots, m, damp, nsrc, src_xyz,
                                            src_wav, nrec, rec_xyz, rec_resid, checkpoint_every,
-                                           grad_m, static_cast<cudaStream_t>(stream));
+                                           grad_m, nullptr, "acoustic_gradient",
+                                           static_cast<cudaStream_t>(stream));
+}
+
+fd_status acoustic_vjp(const fd_grid *grid, int so, double dt, int nt, int nshots, const float *m,
+                       const float *damp, int nsrc, const float *src_xyz, const float *src_wav,
+                       int nrec, const float *rec_xyz, const float *rec_resid,
+                       int checkpoint_every, float *grad_m, float *src_grad, void *stream) {
+    fdsweep::clear_error();
+    if (nsrc > 0 && !src_grad)
+        return fdsweep::set_error(FD_ERR_ARG, "acoustic_vjp: src_grad is null");
+    return fdsweep::acoustic_gradient_impl(grid, so, dt, nt, nshots, m, damp, nsrc, src_xyz,
+                                           src_wav, nrec, rec_xyz, rec_resid, checkpoint_every,
+                                           grad_m, src_grad, "acoustic_vjp",
+                                           static_cast<cudaStream_t>(stream));
 }
 
 const char *fd_last_error(void) { return fdsweep::last_error(); }

@@ -218,13 +218,20 @@ struct SparseArgs {
 fd_status sparse_launch(const SparseArgs &a, int step, bool do_inject, bool do_interp,
                         cudaStream_t stream);
 fd_status bump_counter(int *counter, int by, cudaStream_t stream);
-// grad += sum_b w_b (u_b - 2 u_b' + u_b'') over `n` floats, the FWI imaging
-// condition of one time step for nb shots (scaled by -1/dt^2 once at the end):
-// w_b = w + b w_stride, u_b = u + b u_stride is the level of u^k and u_b',
-// u_b'' (u^{k-1}, u^{k-2}) are the n and 2n floats below it; shots are
-// accumulated in order.
-fd_status grad_accumulate_batch(float *grad, const float *w, int64_t w_stride, const float *u,
-                                int64_t u_stride, int nb, int64_t n, cudaStream_t stream);
+// grad += sum_j sum_b w_jb (u_jb - 2 u_jb' + u_jb''), the FWI imaging condition
+// of `steps` consecutive time steps k, k-1, .. (j = 0, 1, ..) for nb shots
+// (scaled by -1/dt^2 once at the end).  Shot b's adjoint levels are a ring of
+// w_levels fields of vol floats from w + b w_stride, step j in level
+// (w_level + j) mod w_levels; u + b u_stride is its level u^k and the levels
+// below it are the vol, 2 vol, .. floats before.  nb <= kGradMaxShots.
+struct GradArgs {
+    float *grad;
+    const float *w, *u;
+    int64_t w_stride, u_stride, vol;
+    int w_level, w_levels, nb, steps;
+};
+constexpr int kGradMaxShots = 16;
+fd_status grad_accumulate(const GradArgs &a, cudaStream_t stream);
 fd_status scale_field(float *f, float s, int64_t n, cudaStream_t stream);
 
 // ---------------------------------------------------------------- setup K0

@@ -349,6 +349,21 @@ fd_status Workspace::allocate(cudaStream_t s) {
     return FD_OK;
 }
 
+double pool_unused() {
+    int dev = 0;
+    cudaMemPool_t pool;
+    uint64_t reserved = 0, used = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetDefaultMemPool(&pool, dev) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) !=
+            cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+        cudaGetLastError();
+        return 0.;
+    }
+    return reserved > used ? (double)(reserved - used) : 0.;
+}
+
 void Workspace::release() {
     if (base_) {
         cudaFreeAsync(base_, stream_);

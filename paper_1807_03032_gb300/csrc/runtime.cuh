@@ -102,6 +102,10 @@ class Workspace {
     cudaStream_t stream_ = nullptr;
 };
 
+// Bytes that the device's default memory pool (the workspaces' pool) holds
+// but does not use: they count as taken in cudaMemGetInfo.
+double pool_unused();
+
 // The library's own non-blocking stream for one call, ordered after the work
 // already queued on the caller's stream (and the caller's stream after it).
 // Keeping a private stream lets the time loop be captured into a CUDA graph

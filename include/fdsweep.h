@@ -286,7 +286,7 @@ fd_status acoustic_adjoint(const fd_grid *grid, int so, double dt, int nt, int n
  *   Device memory: 11 + K + 2 + 2 ceil((nt-1)/K) wavefield volumes per shot
  *   of a batch (9 + K + 2 for one segment), K the checkpoint interval; 7 fewer
  *   where one shot would not fit otherwise.  Shots are stepped together in
- *   batches of up to 16, as many as fit in 80 % of the free device memory (at
+ *   batches of up to 8, as many as fit in 80 % of the free device memory (at
  *   least one; the environment variable FDSWEEP_GRAD_BATCH=n caps the batch).
  *   Other arguments as for acoustic_forward.
  */

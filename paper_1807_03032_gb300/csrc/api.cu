@@ -1438,9 +1438,8 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     const int nsteps = nt - 1;
     const int64_t vol = L.vol;
     int K = checkpoint_every > 0 ? checkpoint_every : (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
-    // shots of a batch: at most kGradMaxShots, in batches of about equal size
-    const int nbatch = (nshots + kGradMaxShots - 1) / kGradMaxShots;
-    const int most = nbatch > 0 ? (nshots + nbatch - 1) / nbatch : 0;
+    // shots of a batch
+    const int most = nshots < kGradMaxShots ? nshots : kGradMaxShots;
     if (checkpoint_every == 0) {
         size_t free_b = 0, total_b = 0;
         FD_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));

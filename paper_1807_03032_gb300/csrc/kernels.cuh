@@ -230,7 +230,7 @@ struct GradArgs {
     int64_t w_stride, u_stride, vol;
     int w_level, w_levels, nb, steps;
 };
-constexpr int kGradMaxShots = 16;
+constexpr int kGradMaxShots = 8;
 fd_status grad_accumulate(const GradArgs &a, cudaStream_t stream);
 fd_status scale_field(float *f, float s, int64_t n, cudaStream_t stream);
 

@@ -76,25 +76,22 @@ __global__ void bump_kernel(int *counter, int by) { *counter += by; }
 
 template <int V>
 __device__ __forceinline__ void vec_load(float (&d)[V], const float *s) {
+    static_assert(V == 4 || V == 2, "vectors of 2 or 4 floats");
     if (V == 4) {
         const float4 t = *reinterpret_cast<const float4 *>(s);
-        d[0] = t.x, d[1 % V] = t.y, d[2 % V] = t.z, d[3 % V] = t.w;
-    } else if (V == 2) {
-        const float2 t = *reinterpret_cast<const float2 *>(s);
-        d[0] = t.x, d[1 % V] = t.y;
+        d[0] = t.x, d[1] = t.y, d[2 % V] = t.z, d[3 % V] = t.w;
     } else {
-        d[0] = *s;
+        const float2 t = *reinterpret_cast<const float2 *>(s);
+        d[0] = t.x, d[1] = t.y;
     }
 }
 
 template <int V>
 __device__ __forceinline__ void vec_store(float *d, const float (&s)[V]) {
     if (V == 4)
-        *reinterpret_cast<float4 *>(d) = make_float4(s[0], s[1 % V], s[2 % V], s[3 % V]);
-    else if (V == 2)
-        *reinterpret_cast<float2 *>(d) = make_float2(s[0], s[1 % V]);
+        *reinterpret_cast<float4 *>(d) = make_float4(s[0], s[1], s[2 % V], s[3 % V]);
     else
-        *d = s[0];
+        *reinterpret_cast<float2 *>(d) = make_float2(s[0], s[1]);
 }
 
 // g += sum over steps j and shots b of w_jb (u_jb - 2 u_jb' + u_jb''), step j
@@ -105,9 +102,10 @@ __device__ __forceinline__ void vec_store(float *d, const float (&s)[V]) {
 // shot-point instead of 16 + 8/nb.  V floats per thread and NB >= nb shots
 // trade the width of the loads against the registers of the window (2 NB V).
 // 128^3, 239 steps, whole gradient: 4 shots 19.7 ms with one launch per step
-// and 15.4 in eights, 16 shots (119 steps) 45.0 and 29.4.  Two blocks of 128
-// registers per SM and no unrolling: with the 255 registers of unroll 2 the
-// 16-shot kernel is slower (48.4 ms) than one launch per step.
+// and 15.4 in eights, 8 shots 34.1 and 26.7.  Two blocks of 128 registers per
+// SM and no unrolling: with unroll 2 (255 registers) 16.1 and 27.1 ms, and a
+// 16-shot kernel of single floats was slower than two batches of 8 (29.4 ms
+// against 27.1 for 119 steps).
 template <int V, int NB>
 __global__ void __launch_bounds__(256, 2) grad_steps_kernel(const GradArgs a) {
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V; i < a.vol;
@@ -197,10 +195,8 @@ fd_status grad_accumulate(const GradArgs &a, cudaStream_t stream) {
         return set_error(FD_ERR_ARG, "grad_accumulate: %d shots in a batch", a.nb);
     if (a.nb <= 4)
         grad_steps_kernel<4, 4><<<stream_grid(a.vol / 4, 256), 256, 0, stream>>>(a);
-    else if (a.nb <= 8)
-        grad_steps_kernel<2, 8><<<stream_grid(a.vol / 2, 256), 256, 0, stream>>>(a);
     else
-        grad_steps_kernel<1, kGradMaxShots><<<stream_grid(a.vol, 256), 256, 0, stream>>>(a);
+        grad_steps_kernel<2, kGradMaxShots><<<stream_grid(a.vol / 2, 256), 256, 0, stream>>>(a);
     FD_CUDA_TRY(cudaGetLastError());
     note_launch(stream);
     return FD_OK;

@@ -1,7 +1,7 @@
 """Both gradients of the source-to-receiver map from one reverse sweep.
 
-The imaging condition takes several time steps per launch, with a kernel for up to 4, 8
-and 16 shots and two batches above; the steps of a segment are a full launch, a remainder
+The imaging condition takes several time steps per launch, with a kernel for up to 4 and
+8 shots and several batches above; the steps of a segment are a full launch, a remainder
 or fewer than a launch takes.  Tolerance: the repository's 1e-4 relative L2 for FP32
 against the FP64 oracle; the two entry points run the same operations and differ only in
 the order of the atomic injections, 1e-6."""

@@ -123,7 +123,10 @@ __device__ __noinline__ void inject_column(const AcousticStepArgs *a, const Acou
 // failure-injection setting of fd_set_wait_limit_ns); otherwise it is the
 // constant 2 s, which keeps the limit out of the plane loop's registers (a
 // limit read at run time cost 13 % at so 8).
-template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB = 0, bool WL = false>
+// EDGE: the R planes before and behind a chunk, which only feed its outputs
+// along z, are loaded as interior tiles without a halo and skip the x/y part.
+template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB = 0, bool EDGE = false,
+          bool WL = false>
 __global__ void __launch_bounds__(TX *TY + 32, MINB)
     acoustic_step_kernel(const __grid_constant__ CUtensorMap map_halo,
                          const __grid_constant__ CUtensorMap map_int,
@@ -194,10 +197,14 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
                     break;
                 }
                 const bool with_out = jj >= 2 * R;
-                mbar_arrive_expect_tx(&full[slot],
-                                      C::HALO_BYTES + (with_out ? C::NINT * C::INT_BYTES : 0));
+                const bool edge = EDGE && (jj < R || jj >= nplanes - R);
+                mbar_arrive_expect_tx(&full[slot], (edge ? C::INT_BYTES : C::HALO_BYTES) +
+                                                       (with_out ? C::NINT * C::INT_BYTES : 0));
                 float *st = smem + slot * C::STAGE;
-                tma_load_4d(st, &map_halo, &full[slot], x0 - C::RA, y0 - R, za - R + jj, wcur);
+                if (edge)
+                    tma_load_4d(st, &map_int, &full[slot], x0, y0, za - R + jj, wcur);
+                else
+                    tma_load_4d(st, &map_halo, &full[slot], x0 - C::RA, y0 - R, za - R + jj, wcur);
                 if (with_out) {
                     const int zo = za - 2 * R + jj;
                     tma_load_4d(st + C::HALO, &map_int, &full[slot], x0, y0, zo, wcur);
@@ -252,6 +259,13 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
         // x/y part of the Laplacian of plane p (centre weight of all axes
         // included) and the centre values
         Q4 cen[VY], lxy[VY];
+        if (EDGE && (j < R || j >= nplanes - R)) {
+#pragma unroll
+            for (int v = 0; v < VY; ++v) {
+                cen[v] = lds_q4(H + (ty * VY + v) * C::BX + 4 * tx);
+                lxy[v] = Q4{0ull, 0ull};
+            }
+        } else {
 #pragma unroll
         for (int v = 0; v < VY; ++v) {
             constexpr int NP = (2 * C::RA + 4) / 2;  // packed pairs in the x span
@@ -311,6 +325,8 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
                     lxy[v].hi = f2_fma(w2, f.hi, lxy[v].hi);
                 }
             }
+        }
+
         }
 
         // z part: plane p feeds the pending outputs p-R .. p+R-1 and starts p+R
@@ -403,27 +419,28 @@ struct ConfigEntry {
     const char *name;
 };
 
-template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB>
+template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB, bool EDGE>
 ConfigEntry make_entry(const char *name, float launch, float lat, float thr, float warm) {
     using C = AcCfg<R, TX, TY, VY, D, DF>;
     const void *wl = nullptr;
-    if constexpr (!DF) wl = (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, true>;
-    return ConfigEntry{R,      (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB>,
+    if constexpr (!DF)
+        wl = (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, EDGE, true>;
+    return ConfigEntry{R,      (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, EDGE>,
                        wl,     C::SMEM, C::BX, C::BY, C::PW, C::PH, C::THREADS,
                        launch, lat, thr, warm, name};
 }
 
-#define FD_AC_ENTRY(R, TX, TY, VY, D, U, MB, ...)                                               \
-    make_entry<R, TX, TY, VY, D, U, false, MB>("acoustic_step<" #R "," #TX "," #TY "," #VY "," \
+#define FD_AC_ENTRY(R, TX, TY, VY, D, U, MB, ED, ...)                                           \
+    make_entry<R, TX, TY, VY, D, U, false, MB, ED>("acoustic_step<" #R "," #TX "," #TY "," #VY "," \
                                                #D "," #U ">",                                  \
                                                __VA_ARGS__)
-#define FD_AC_ENTRY_DF(R, TX, TY, VY, D, U, MB, ...)                                           \
-    make_entry<R, TX, TY, VY, D, U, true, MB>("acoustic_step<" #R "," #TX "," #TY "," #VY "," \
+#define FD_AC_ENTRY_DF(R, TX, TY, VY, D, U, MB, ED, ...)                                       \
+    make_entry<R, TX, TY, VY, D, U, true, MB, ED>("acoustic_step<" #R "," #TX "," #TY "," #VY "," \
                                               #D "," #U ",damp field>",                       \
                                               __VA_ARGS__)
 
 // The configurations of each radius (template arguments R, TX, TY, VY, D, U,
-// minimum CTAs per SM); acoustic_plan takes the one with the smallest
+// minimum CTAs per SM, EDGE); acoustic_plan takes the one with the smallest
 // estimated time for the grid.  Ring sizes are powers of two (D = 3), so that
 // the unrolled plane loop has constant stage addresses.
 //  * Small tiles fill the machine on small grids (64 x 4 at so 16: 128^3 17.8
@@ -435,29 +452,36 @@ ConfigEntry make_entry(const char *name, float launch, float lat, float thr, flo
 //    255 registers per SM, run 512^3 so 16 in 369 us (442 with 64 x 8, 472
 //    before the producer warp); 64 x 44 at so 12 in 340 us (387 and 402).
 //  * so 4 and 8 are at the HBM limit at 512^3 (306 and 318 us for 2.15 GB).
+//  * EDGE (see the kernel) halves what the 2R extra planes of a chunk cost, so
+//    that wide stencils can be cut into more chunks: so 16 4 x 128^3 41.4 ->
+//    37.5 us per step, 160^3 25.9 -> 22.4, 64^3 11.4 -> 9.4; so 12 4 x 128^3
+//    31.0 -> 26.9, 160^3 21.3 -> 18.6; so 8 96^3 8.8 -> 8.1.  Without gain at
+//    so 4; a 64 x 28 tile that marches the whole axis in one chunk (512^3 so
+//    16) is 1 % faster without it.
 const ConfigEntry *config_table(int radius, int *count) {
     static const ConfigEntry r1[] = {
-        FD_AC_ENTRY(1, 16, 16, 1, 3, 4, 0, 2.4f, 0.30f, 0.27f, 0.9f)};
+        FD_AC_ENTRY(1, 16, 16, 1, 3, 4, 0, 0, 2.4f, 0.30f, 0.27f, 0.9f)};
     static const ConfigEntry r2[] = {
-        FD_AC_ENTRY(2, 16, 8, 1, 3, 4, 0, 3.57f, 0.278f, 0.162f, 0.40f),
-        FD_AC_ENTRY(2, 16, 16, 1, 4, 2, 0, 2.44f, 0.299f, 0.269f, 0.91f)};
+        FD_AC_ENTRY(2, 16, 8, 1, 3, 4, 0, 0, 3.57f, 0.278f, 0.162f, 0.40f),
+        FD_AC_ENTRY(2, 16, 16, 1, 4, 2, 0, 0, 2.44f, 0.299f, 0.269f, 0.91f)};
     static const ConfigEntry r4[] = {
-        FD_AC_ENTRY(4, 16, 8, 1, 3, 8, 0, 3.23f, 0.346f, 0.152f, 0.68f),
-        FD_AC_ENTRY(4, 16, 4, 2, 3, 8, 0, 2.94f, 0.458f, 0.119f, 0.73f)};
+        FD_AC_ENTRY(4, 16, 8, 1, 3, 8, 0, 0, 3.70f, 0.269f, 0.157f, 0.73f),
+        FD_AC_ENTRY(4, 16, 4, 2, 3, 8, 0, 1, 3.02f, 0.455f, 0.124f, 0.57f)};
     static const ConfigEntry r6[] = {
-        FD_AC_ENTRY(6, 16, 8, 1, 3, 4, 0, 3.05f, 0.394f, 0.147f, 0.91f),
-        FD_AC_ENTRY(6, 16, 8, 2, 3, 4, 2, 2.90f, 0.513f, 0.250f, 0.85f),
-        FD_AC_ENTRY(6, 16, 22, 2, 3, 4, 1, 1.67f, 0.501f, 0.697f, 0.96f)};
+        FD_AC_ENTRY(6, 16, 8, 1, 3, 4, 0, 1, 3.71f, 0.356f, 0.161f, 0.59f),
+        FD_AC_ENTRY(6, 16, 8, 2, 3, 4, 2, 1, 2.80f, 0.488f, 0.279f, 0.54f),
+        FD_AC_ENTRY(6, 16, 22, 2, 3, 4, 1, 1, 1.29f, 0.785f, 0.436f, 0.59f)};
     static const ConfigEntry r8[] = {
-        FD_AC_ENTRY(8, 16, 8, 1, 3, 8, 3, 3.95f, 0.372f, 0.185f, 0.89f),
-        FD_AC_ENTRY(8, 16, 4, 1, 3, 4, 0, 2.86f, 0.386f, 0.078f, 0.98f),
-        FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 2.10f, 0.689f, 0.097f, 0.97f)};
+        FD_AC_ENTRY(8, 16, 8, 1, 3, 8, 3, 1, 4.20f, 0.351f, 0.182f, 0.55f),
+        FD_AC_ENTRY(8, 16, 4, 1, 3, 4, 0, 1, 3.25f, 0.412f, 0.093f, 0.48f),
+        FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 1, 1.76f, 0.609f, 0.325f, 0.59f),
+        FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 0, 1.89f, 0.619f, 0.241f, 0.99f)};
     switch (radius) {
         case 1: *count = 1; return r1;
         case 2: *count = 2; return r2;
         case 4: *count = 2; return r4;
         case 6: *count = 3; return r6;
-        case 8: *count = 3; return r8;
+        case 8: *count = 4; return r8;
         default: *count = 0; return nullptr;
     }
 }
@@ -467,19 +491,19 @@ const ConfigEntry *config_table(int radius, int *count) {
 // the costs fitted to 10 problems.
 const ConfigEntry *config_table_df(int radius, int *count) {
     static const ConfigEntry r1[] = {
-        FD_AC_ENTRY_DF(1, 16, 16, 1, 3, 4, 0, 2.7f, 0.28f, 0.38f, 0.5f)};
+        FD_AC_ENTRY_DF(1, 16, 16, 1, 3, 4, 0, 0, 2.7f, 0.28f, 0.38f, 0.5f)};
     static const ConfigEntry r2[] = {
-        FD_AC_ENTRY_DF(2, 16, 8, 1, 3, 4, 0, 3.17f, 0.286f, 0.185f, 0.42f)};
+        FD_AC_ENTRY_DF(2, 16, 8, 1, 3, 4, 0, 0, 3.17f, 0.286f, 0.185f, 0.42f)};
     static const ConfigEntry r4[] = {
-        FD_AC_ENTRY_DF(4, 16, 8, 1, 3, 8, 0, 3.33f, 0.291f, 0.193f, 0.57f),
-        FD_AC_ENTRY_DF(4, 16, 4, 2, 3, 8, 0, 3.91f, 0.342f, 0.181f, 0.42f)};
+        FD_AC_ENTRY_DF(4, 16, 8, 1, 3, 8, 0, 0, 3.33f, 0.291f, 0.193f, 0.57f),
+        FD_AC_ENTRY_DF(4, 16, 4, 2, 3, 8, 0, 0, 3.91f, 0.342f, 0.181f, 0.42f)};
     static const ConfigEntry r6[] = {
-        FD_AC_ENTRY_DF(6, 16, 8, 1, 3, 4, 0, 3.24f, 0.311f, 0.195f, 0.77f),
-        FD_AC_ENTRY_DF(6, 16, 8, 2, 3, 4, 2, 3.96f, 0.372f, 0.382f, 0.61f)};
+        FD_AC_ENTRY_DF(6, 16, 8, 1, 3, 4, 0, 1, 3.48f, 0.384f, 0.179f, 0.59f),
+        FD_AC_ENTRY_DF(6, 16, 8, 2, 3, 4, 2, 1, 3.01f, 0.460f, 0.360f, 0.44f)};
     static const ConfigEntry r8[] = {
-        FD_AC_ENTRY_DF(8, 16, 8, 1, 3, 8, 3, 3.20f, 0.297f, 0.218f, 0.89f),
-        FD_AC_ENTRY_DF(8, 16, 4, 1, 3, 4, 0, 4.22f, 0.314f, 0.107f, 0.87f),
-        FD_AC_ENTRY_DF(8, 16, 14, 2, 3, 8, 1, 1.41f, 0.712f, 0.058f, 0.91f)};
+        FD_AC_ENTRY_DF(8, 16, 8, 1, 3, 8, 3, 1, 3.83f, 0.387f, 0.196f, 0.54f),
+        FD_AC_ENTRY_DF(8, 16, 4, 1, 3, 4, 0, 1, 2.87f, 0.402f, 0.088f, 0.66f),
+        FD_AC_ENTRY_DF(8, 16, 14, 2, 3, 8, 1, 1, 1.12f, 0.536f, 0.509f, 0.56f)};
     switch (radius) {
         case 1: *count = 1; return r1;
         case 2: *count = 1; return r2;

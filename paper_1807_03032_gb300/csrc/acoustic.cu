@@ -116,6 +116,48 @@ __device__ __noinline__ void inject_column(const AcousticStepArgs *a, const Acou
     }
 }
 
+// x part of the Laplacian of 4 consecutive points (centre weight of all axes
+// included) from a row that starts RA points left of them; *cen: the points.
+template <int R, int RA>
+__device__ __forceinline__ Q4 laplace_x(const float *row, const AcousticStepArgs &a, Q4 *cen) {
+    constexpr int NP = (2 * RA + 4) / 2;  // packed pairs in the x span
+    f2 xp[NP];
+#pragma unroll
+    for (int t = 0; t < NP / 2; ++t) {
+        const Q4 q = lds_q4(row + 4 * t);
+        xp[2 * t] = q.lo;
+        xp[2 * t + 1] = q.hi;
+    }
+    constexpr int c0 = RA / 2;  // pair index of points 0,1
+    const Q4 c = Q4{xp[c0], xp[c0 + 1]};
+    const f2 wc2 = f2_splat(a.wc);
+    Q4 s = Q4{f2_mul(wc2, c.lo), f2_mul(wc2, c.hi)};
+    // even shifts keep the pair alignment: packed arithmetic
+#pragma unroll
+    for (int k = 2; k <= R; k += 2) {
+        const f2 w2 = f2_splat(a.wx[k]);
+        s.lo = f2_fma(w2, f2_add(xp[c0 + k / 2], xp[c0 - k / 2]), s.lo);
+        s.hi = f2_fma(w2, f2_add(xp[c0 + 1 + k / 2], xp[c0 + 1 - k / 2]), s.hi);
+    }
+    // odd shifts straddle the pairs: scalar arithmetic
+    float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
+#pragma unroll
+    for (int k = 1; k <= R; k += 2) {
+        auto el = [&](int idx) -> float {
+            return (idx & 1) ? f2_hi(xp[idx >> 1]) : f2_lo(xp[idx >> 1]);
+        };
+        const float w = a.wx[k];
+        o0 = fmaf(w, el(RA + 0 + k) + el(RA + 0 - k), o0);
+        o1 = fmaf(w, el(RA + 1 + k) + el(RA + 1 - k), o1);
+        o2 = fmaf(w, el(RA + 2 + k) + el(RA + 2 - k), o2);
+        o3 = fmaf(w, el(RA + 3 + k) + el(RA + 3 - k), o3);
+    }
+    s.lo = f2_add(s.lo, f2_pack(o0, o1));
+    s.hi = f2_add(s.hi, f2_pack(o2, o3));
+    *cen = c;
+    return s;
+}
+
 // U: unroll factor of the plane loop.  The pending-output registers shift by
 // one plane per iteration; unrolling by U turns U - 1 of every U shifts into
 // register renaming instead of moves (U = 2R removes them all).
@@ -268,43 +310,7 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
         } else {
 #pragma unroll
         for (int v = 0; v < VY; ++v) {
-            constexpr int NP = (2 * C::RA + 4) / 2;  // packed pairs in the x span
-            f2 xp[NP];
-            const float *row = H + (rbase + v) * C::PW + 4 * tx;
-#pragma unroll
-            for (int t = 0; t < NP / 2; ++t) {
-                const Q4 q = lds_q4(row + 4 * t);
-                xp[2 * t] = q.lo;
-                xp[2 * t + 1] = q.hi;
-            }
-            constexpr int c0 = C::RA / 2;  // pair index of points 0,1
-            const Q4 c = Q4{xp[c0], xp[c0 + 1]};
-            const f2 wc2 = f2_splat(a.wc);
-            Q4 s = Q4{f2_mul(wc2, c.lo), f2_mul(wc2, c.hi)};
-            // even shifts keep the pair alignment: packed arithmetic
-#pragma unroll
-            for (int k = 2; k <= R; k += 2) {
-                const f2 w2 = f2_splat(a.wx[k]);
-                s.lo = f2_fma(w2, f2_add(xp[c0 + k / 2], xp[c0 - k / 2]), s.lo);
-                s.hi = f2_fma(w2, f2_add(xp[c0 + 1 + k / 2], xp[c0 + 1 - k / 2]), s.hi);
-            }
-            // odd shifts straddle the pairs: scalar arithmetic
-            float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-#pragma unroll
-            for (int k = 1; k <= R; k += 2) {
-                auto el = [&](int idx) -> float {
-                    return (idx & 1) ? f2_hi(xp[idx >> 1]) : f2_lo(xp[idx >> 1]);
-                };
-                const float w = a.wx[k];
-                o0 = fmaf(w, el(C::RA + 0 + k) + el(C::RA + 0 - k), o0);
-                o1 = fmaf(w, el(C::RA + 1 + k) + el(C::RA + 1 - k), o1);
-                o2 = fmaf(w, el(C::RA + 2 + k) + el(C::RA + 2 - k), o2);
-                o3 = fmaf(w, el(C::RA + 3 + k) + el(C::RA + 3 - k), o3);
-            }
-            s.lo = f2_add(s.lo, f2_pack(o0, o1));
-            s.hi = f2_add(s.hi, f2_pack(o2, o3));
-            cen[v] = c;
-            lxy[v] = s;
+            lxy[v] = laplace_x<R, C::RA>(H + (rbase + v) * C::PW + 4 * tx, a, &cen[v]);
         }
 #pragma unroll
         for (int dy = -R; dy < VY + R; ++dy) {
@@ -406,10 +412,158 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
         inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
 }
 
+// Small grids: one block of 32 x 8 x 8 points per CTA instead of a march, so
+// that a launch is one copy and one pass of arithmetic long.  The block comes
+// with its halo on all sides (one cp.async.bulk.tensor), a thread owns four x
+// points of one plane, and u^{n-1} and b are plain loads under the copy.  Every
+// point sums its neighbours in the order of the marching kernel: same bits.
+// A step of a small grid is latency: launch, copy, arithmetic and store behind
+// one another.  So the launch lets the next one set itself up at once (the
+// grid is one or two waves, no block waits for a place) and the stop flag is
+// read under the copy.  us per step, direct against the best march: 64^3 so 4
+// 4.5 and 5.6, so 8 4.8 and 6.8, so 16 6.4 and 9.0; 80^3 so 8 6.0 and 8.1; two
+// waves of it lose (128^3 so 8 14.9 and 9.8), and the halo of a block (13
+// times its points at so 16) costs more than the march's above 96^3.
+template <int R>
+struct AcDirect {
+    static constexpr int BX = 32, BY = 8, BZ = 8;
+    static constexpr int RA = (R + 3) / 4 * 4;
+    static constexpr int PW = BX + 2 * RA, PH = BY + 2 * R, PD = BZ + 2 * R;
+    static constexpr int THREADS = BX / 4 * BY * BZ;
+    static constexpr int TILE = (PW * PH * PD + 31) / 32 * 32;
+    static constexpr size_t SMEM = (size_t)TILE * 4 + 16 + 128;
+};
+
+template <int R, bool DF, bool WL = false>
+__global__ void __launch_bounds__(AcDirect<R>::THREADS)
+    acoustic_direct_kernel(const __grid_constant__ CUtensorMap map_halo,
+                           const __grid_constant__ CUtensorMap map_int,
+                           const __grid_constant__ CUtensorMap map_b,
+                           const __grid_constant__ AcousticStepArgs a,
+                           const __grid_constant__ AcousticInject inj,
+                           const __grid_constant__ ReceiveArgs rec, int zchunk, int nzc) {
+    using C = AcDirect<R>;
+    if (blockIdx.z >= gridDim.z - rec.slices) {
+        chain_trigger();
+        chain_wait();
+        if (!(__ldcg(a.err) & DEV_ERR_NONFINITE))
+            record_receivers(&rec, a.wave, a.lps, a.lev_cur, a.lev_cur, &a.L);
+        return;
+    }
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float *tile = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
+                                            ~static_cast<uintptr_t>(127));
+    uint64_t *full = reinterpret_cast<uint64_t *>(tile + C::TILE);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(full + 1);
+    const int tid = threadIdx.x;
+    const int tx = tid % 8, ty = tid / 8 % C::BY, tz = tid / (8 * C::BY);
+    const int shot_i = blockIdx.z / nzc;
+    const int chunk = blockIdx.z - shot_i * nzc;
+    const int shot = a.slot_map ? a.slot_map[shot_i] : shot_i;
+    const int x0 = blockIdx.x * C::BX, y0 = blockIdx.y * C::BY, z0 = chunk * C::BZ;
+    const int gx = x0 + 4 * tx, gy = y0 + ty, gz = z0 + tz;
+    const uint64_t wait_ns = WL ? (a.wait_ns ? a.wait_ns : 2000000000ull) : 2000000000ull;
+    if (tid == 0) {
+        prefetch_tensormap(&map_halo);
+        mbar_init(full, 1);
+        fence_mbar_init();
+        *abort_flag = 0;
+    }
+    __syncthreads();
+    chain_trigger();
+    chain_wait();
+    if (tid == 0) {
+        mbar_arrive_expect_tx(full, C::PW * C::PH * C::PD * 4);
+        tma_load_4d(tile, &map_halo, full, x0 - C::RA, y0 - R, z0 - R,
+                    shot * a.lps + a.lev_cur);
+    }
+    // set by the divergence watchdog to stop the run: nothing is stored then
+    const bool stopped = __ldcg(a.err) & DEV_ERR_NONFINITE;
+    const bool ok = gx < a.L.nxp && gy < a.L.ny && gz < a.L.nz;
+    const int64_t off = (int64_t)gz * a.L.plane + (int64_t)gy * a.L.nxp + gx;
+    float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f), b4 = p4, z4 = p4;
+    if (ok) {
+        p4 = *reinterpret_cast<const float4 *>(
+            a.wave + (int64_t)(shot * a.lps + a.lev_prev) * a.L.vol + off);
+        b4 = __ldg(reinterpret_cast<const float4 *>(a.bcoef + off));
+        if (DF) {
+            z4 = __ldg(reinterpret_cast<const float4 *>(a.bcoef + a.L.vol + off));
+        } else {
+            const float dyz = a.dpy[gy] + a.dpz[gz];
+            z4.x = (gx < a.L.nx ? a.dpx[gx] : 0.f) + dyz;
+            z4.y = (gx + 1 < a.L.nx ? a.dpx[gx + 1] : 0.f) + dyz;
+            z4.z = (gx + 2 < a.L.nx ? a.dpx[gx + 2] : 0.f) + dyz;
+            z4.w = (gx + 3 < a.L.nx ? a.dpx[gx + 3] : 0.f) + dyz;
+        }
+        // the row's padding stays zero, as the copies of the march read it
+        if (gx + 1 >= a.L.nx) p4.y = b4.y = 0.f;
+        if (gx + 2 >= a.L.nx) p4.z = b4.z = 0.f;
+        if (gx + 3 >= a.L.nx) p4.w = b4.w = 0.f;
+        if (gx >= a.L.nx) p4.x = b4.x = 0.f;
+    }
+    if (!mbar_wait_bounded(full, 0, wait_ns)) {
+        *abort_flag = 1;
+        atomicOr(a.err, DEV_ERR_TIMEOUT);
+    } else {
+        constexpr int SY = C::PW, SZ = C::PW * C::PH;
+        const float *c = tile + (R + tz) * SZ + (R + ty) * SY + C::RA + 4 * tx;
+        Q4 u;
+        Q4 lxy = laplace_x<R, C::RA>(c - C::RA, a, &u);
+#pragma unroll
+        for (int d = -R; d <= R; ++d) {
+            if (d == 0) continue;
+            const f2 w2 = f2_splat(a.wy[d < 0 ? -d : d]);
+            const Q4 f = lds_q4(c + d * SY);
+            lxy.lo = f2_fma(w2, f.lo, lxy.lo);
+            lxy.hi = f2_fma(w2, f.hi, lxy.hi);
+        }
+        Q4 s;
+#pragma unroll
+        for (int d = -R; d <= R; ++d) {
+            if (d == 0) {
+                s.lo = f2_add(s.lo, lxy.lo);
+                s.hi = f2_add(s.hi, lxy.hi);
+                continue;
+            }
+            const f2 w2 = f2_splat(a.wz[d < 0 ? -d : d]);
+            const Q4 f = lds_q4(c + d * SZ);
+            if (d == -R) {
+                s.lo = f2_mul(w2, f.lo);
+                s.hi = f2_mul(w2, f.hi);
+            } else {
+                s.lo = f2_fma(w2, f.lo, s.lo);
+                s.hi = f2_fma(w2, f.hi, s.hi);
+            }
+        }
+        if (ok && !stopped) {
+            const f2 one2 = f2_splat(1.f);
+            const f2 blo = f2_pack(b4.x, b4.y), bhi = f2_pack(b4.z, b4.w);
+            f2 zl = f2_pack(z4.x, z4.y), zh = f2_pack(z4.z, z4.w);
+            if (!DF) {
+                zl = f2_mul(zl, blo);
+                zh = f2_mul(zh, bhi);
+            }
+            f2 ol = f2_fma(f2_sub(one2, zl), f2_sub(u.lo, f2_pack(p4.x, p4.y)), u.lo);
+            f2 oh = f2_fma(f2_sub(one2, zh), f2_sub(u.hi, f2_pack(p4.z, p4.w)), u.hi);
+            ol = f2_fma(blo, s.lo, ol);
+            oh = f2_fma(bhi, s.hi, oh);
+            *reinterpret_cast<ulonglong2 *>(
+                a.wave + (int64_t)(shot * a.lps + a.lev_out) * a.L.vol + off) =
+                make_ulonglong2(ol, oh);
+        }
+    }
+    if (inj.nsrc > 0) __syncthreads();
+    // a copy that was given up gets a bounded chance to land
+    if (*abort_flag && tid == 0) mbar_wait_bounded(full, 0, 200000000ull);
+    if (inj.nsrc > 0 && tid == 0 && !*abort_flag && !stopped)
+        inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
+}
+
 // A launch configuration and what a launch of it costs (microseconds, fitted
 // to measured steps of 21 problems from 48^3 to 512^3, ragged and with up to
 // 8 shots, over all chunk counts): `launch` + (planes + warm 2R) x waves, a
-// plane costing sqrt(lat^2 + (k thr)^2) with k CTAs on the SM.
+// plane costing sqrt(lat^2 + (k thr)^2) with k CTAs on the SM; a block of the
+// direct kernel counts as one plane.
 struct ConfigEntry {
     int radius;
     const void *fn, *fn_wl;  // fn_wl: the variant with the wait limit from the arguments
@@ -417,6 +571,7 @@ struct ConfigEntry {
     int bx, by, pw, ph, threads;
     float launch, lat, thr, warm;
     const char *name;
+    int bz, pd;  // z extent of a block and of its copy (marching kernel: 0 and 1)
 };
 
 template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB, bool EDGE>
@@ -427,7 +582,17 @@ ConfigEntry make_entry(const char *name, float launch, float lat, float thr, flo
         wl = (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, EDGE, true>;
     return ConfigEntry{R,      (const void *)&acoustic_step_kernel<R, TX, TY, VY, D, U, DF, MINB, EDGE>,
                        wl,     C::SMEM, C::BX, C::BY, C::PW, C::PH, C::THREADS,
-                       launch, lat, thr, warm, name};
+                       launch, lat, thr, warm, name, 0, 1};
+}
+
+template <int R, bool DF>
+ConfigEntry make_direct(const char *name, float launch, float lat, float thr) {
+    using C = AcDirect<R>;
+    const void *wl = nullptr;
+    if constexpr (!DF) wl = (const void *)&acoustic_direct_kernel<R, DF, true>;
+    return ConfigEntry{R,     (const void *)&acoustic_direct_kernel<R, DF>,
+                       wl,    C::SMEM, C::BX, C::BY, C::PW, C::PH, C::THREADS,
+                       launch, lat, thr, 0.f, name, C::BZ, C::PD};
 }
 
 #define FD_AC_ENTRY(R, TX, TY, VY, D, U, MB, ED, ...)                                           \
@@ -463,25 +628,29 @@ const ConfigEntry *config_table(int radius, int *count) {
         FD_AC_ENTRY(1, 16, 16, 1, 3, 4, 0, 0, 2.4f, 0.30f, 0.27f, 0.9f)};
     static const ConfigEntry r2[] = {
         FD_AC_ENTRY(2, 16, 8, 1, 3, 4, 0, 0, 3.57f, 0.278f, 0.162f, 0.40f),
-        FD_AC_ENTRY(2, 16, 16, 1, 4, 2, 0, 0, 2.44f, 0.299f, 0.269f, 0.91f)};
+        FD_AC_ENTRY(2, 16, 16, 1, 4, 2, 0, 0, 2.44f, 0.299f, 0.269f, 0.91f),
+        make_direct<2, false>("acoustic_direct<2>", 2.85f, 1.41f, 1.20f)};
     static const ConfigEntry r4[] = {
         FD_AC_ENTRY(4, 16, 8, 1, 3, 8, 0, 0, 3.70f, 0.269f, 0.157f, 0.73f),
-        FD_AC_ENTRY(4, 16, 4, 2, 3, 8, 0, 1, 3.02f, 0.455f, 0.124f, 0.57f)};
+        FD_AC_ENTRY(4, 16, 4, 2, 3, 8, 0, 1, 3.02f, 0.455f, 0.124f, 0.57f),
+        make_direct<4, false>("acoustic_direct<4>", 2.56f, 2.02f, 1.48f)};
     static const ConfigEntry r6[] = {
         FD_AC_ENTRY(6, 16, 8, 1, 3, 4, 0, 1, 3.71f, 0.356f, 0.161f, 0.59f),
         FD_AC_ENTRY(6, 16, 8, 2, 3, 4, 2, 1, 2.80f, 0.488f, 0.279f, 0.54f),
-        FD_AC_ENTRY(6, 16, 22, 2, 3, 4, 1, 1, 1.29f, 0.785f, 0.436f, 0.59f)};
+        FD_AC_ENTRY(6, 16, 22, 2, 3, 4, 1, 1, 1.29f, 0.785f, 0.436f, 0.59f),
+        make_direct<6, false>("acoustic_direct<6>", 2.60f, 2.58f, 1.73f)};
     static const ConfigEntry r8[] = {
         FD_AC_ENTRY(8, 16, 8, 1, 3, 8, 3, 1, 4.20f, 0.351f, 0.182f, 0.55f),
         FD_AC_ENTRY(8, 16, 4, 1, 3, 4, 0, 1, 3.25f, 0.412f, 0.093f, 0.48f),
         FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 1, 1.76f, 0.609f, 0.325f, 0.59f),
-        FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 0, 1.89f, 0.619f, 0.241f, 0.99f)};
+        FD_AC_ENTRY(8, 16, 14, 2, 3, 8, 1, 0, 1.89f, 0.619f, 0.241f, 0.99f),
+        make_direct<8, false>("acoustic_direct<8>", 2.80f, 2.68f, 2.20f)};
     switch (radius) {
         case 1: *count = 1; return r1;
-        case 2: *count = 2; return r2;
-        case 4: *count = 2; return r4;
-        case 6: *count = 3; return r6;
-        case 8: *count = 4; return r8;
+        case 2: *count = 3; return r2;
+        case 4: *count = 3; return r4;
+        case 6: *count = 4; return r6;
+        case 8: *count = 5; return r8;
         default: *count = 0; return nullptr;
     }
 }
@@ -493,23 +662,27 @@ const ConfigEntry *config_table_df(int radius, int *count) {
     static const ConfigEntry r1[] = {
         FD_AC_ENTRY_DF(1, 16, 16, 1, 3, 4, 0, 0, 2.7f, 0.28f, 0.38f, 0.5f)};
     static const ConfigEntry r2[] = {
-        FD_AC_ENTRY_DF(2, 16, 8, 1, 3, 4, 0, 0, 3.17f, 0.286f, 0.185f, 0.42f)};
+        FD_AC_ENTRY_DF(2, 16, 8, 1, 3, 4, 0, 0, 3.17f, 0.286f, 0.185f, 0.42f),
+        make_direct<2, true>("acoustic_direct<2,damp field>", 2.85f, 1.41f, 1.20f)};
     static const ConfigEntry r4[] = {
         FD_AC_ENTRY_DF(4, 16, 8, 1, 3, 8, 0, 0, 3.33f, 0.291f, 0.193f, 0.57f),
-        FD_AC_ENTRY_DF(4, 16, 4, 2, 3, 8, 0, 0, 3.91f, 0.342f, 0.181f, 0.42f)};
+        FD_AC_ENTRY_DF(4, 16, 4, 2, 3, 8, 0, 0, 3.91f, 0.342f, 0.181f, 0.42f),
+        make_direct<4, true>("acoustic_direct<4,damp field>", 2.56f, 2.02f, 1.48f)};
     static const ConfigEntry r6[] = {
         FD_AC_ENTRY_DF(6, 16, 8, 1, 3, 4, 0, 1, 3.48f, 0.384f, 0.179f, 0.59f),
-        FD_AC_ENTRY_DF(6, 16, 8, 2, 3, 4, 2, 1, 3.01f, 0.460f, 0.360f, 0.44f)};
+        FD_AC_ENTRY_DF(6, 16, 8, 2, 3, 4, 2, 1, 3.01f, 0.460f, 0.360f, 0.44f),
+        make_direct<6, true>("acoustic_direct<6,damp field>", 2.60f, 2.58f, 1.73f)};
     static const ConfigEntry r8[] = {
         FD_AC_ENTRY_DF(8, 16, 8, 1, 3, 8, 3, 1, 3.83f, 0.387f, 0.196f, 0.54f),
         FD_AC_ENTRY_DF(8, 16, 4, 1, 3, 4, 0, 1, 2.87f, 0.402f, 0.088f, 0.66f),
-        FD_AC_ENTRY_DF(8, 16, 14, 2, 3, 8, 1, 1, 1.12f, 0.536f, 0.509f, 0.56f)};
+        FD_AC_ENTRY_DF(8, 16, 14, 2, 3, 8, 1, 1, 1.12f, 0.536f, 0.509f, 0.56f),
+        make_direct<8, true>("acoustic_direct<8,damp field>", 2.80f, 2.68f, 2.20f)};
     switch (radius) {
         case 1: *count = 1; return r1;
-        case 2: *count = 1; return r2;
-        case 4: *count = 2; return r4;
-        case 6: *count = 2; return r6;
-        case 8: *count = 3; return r8;
+        case 2: *count = 2; return r2;
+        case 4: *count = 3; return r4;
+        case 6: *count = 3; return r6;
+        case 8: *count = 4; return r8;
         default: *count = 0; return nullptr;
     }
 }
@@ -551,18 +724,25 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
                              ((L.ny + e.by - 1) / e.by) * nshots;
         int nzc = 1;
         double planes = 0.0;
-        nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat, &planes);
+        if (e.bz) {
+            nzc = (L.nz + e.bz - 1) / e.bz;
+            planes = wave_cost(cols * nzc, nsm, per_sm, e.thr / e.lat);
+            if ((int64_t)nzc * nshots > 60000 && config < 0) continue;
+        } else {
+            nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
+                                &planes);
+        }
         // damp_z of a chunk follows the stages in shared memory
         const int max_chunk = (max_smem - (int)e.smem) / 4;
         const int min_nzc = (L.nz + max_chunk - 1) / max_chunk;
         if (nzc < min_nzc) nzc = min_nzc;
-        if (nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
+        if (!e.bz && nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
         if (nzc < min_nzc && config < 0 && i + 1 < n) continue;
         const double us = e.launch + e.lat * planes;
         if (best < 0 || us < best_us) {
             best = i;
             best_us = us;
-            zchunk = (L.nz + nzc - 1) / nzc;
+            zchunk = e.bz ? e.bz : (L.nz + nzc - 1) / nzc;
         }
     }
     const ConfigEntry &e = tab[best];
@@ -584,7 +764,7 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
     if (e.fn_wl) FD_TRY(raise_smem_limit(e.fn_wl, plan->smem));
     FD_TRY(make_tensor_map_4d(&plan->map_halo, wave, L.nx, L.ny, L.nz, (uint64_t)map_shots * lps,
                               (uint64_t)L.nxp * 4, (uint64_t)L.plane * 4, (uint64_t)L.vol * 4,
-                              e.pw, e.ph, 1, 1));
+                              e.pw, e.ph, e.pd, 1));
     FD_TRY(make_tensor_map_4d(&plan->map_int, wave, L.nx, L.ny, L.nz, (uint64_t)map_shots * lps,
                               (uint64_t)L.nxp * 4, (uint64_t)L.plane * 4, (uint64_t)L.vol * 4,
                               e.bx, e.by, 1, 1));

@@ -37,6 +37,10 @@ fd_status make_tensor_map_5d(CUtensorMap *map, const float *base, const uint64_t
 // another call is about to launch with (concurrent calls from host threads).
 fd_status raise_smem_limit(const void *fn, size_t bytes);
 
+// Time of `units` equal CTAs on nsm SMs with per_sm places each, in units of a
+// CTA alone on its SM: k CTAs on an SM take sqrt(1 + (load k)^2).
+double wave_cost(int64_t units, int nsm, int per_sm, double load);
+
 // Number of z chunks into which the columns of a z-marching stencil launch
 // are cut (1 .. nz).  A CTA marches `warmup` planes (in units of a full
 // plane's time) before its chunk's first output, and the columns times the

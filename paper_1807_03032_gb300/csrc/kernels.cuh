@@ -306,6 +306,7 @@ struct TtiPassPlan {
     size_t smem = 0;
     int zchunk = 0, nzc = 1;
     int bx = 0, by = 0, pw = 0, ph = 0;  // tile, x-halo width, y-halo height
+    int bz = 1, pd = 1;                  // block depth, z-halo depth (1: marching)
     double est_us = 0.0;                 // estimated time
 };
 

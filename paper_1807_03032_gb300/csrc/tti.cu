@@ -389,6 +389,231 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
         tti_inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
 }
 
+// ---------------------------------------------------------------- small grids
+
+// Both passes with one block of 32 x 8 x 8 points per CTA instead of a march
+// (see acoustic_direct_kernel): a pass of a small grid is latency, and here it
+// is one set of copies and one pass of arithmetic.  The block's operands with
+// halos come in one copy (p and r) or three (the x, y and z temporaries of
+// both fields), the rest are plain loads under them; the launch lets the next
+// one set itself up at once.  Same operations in the same order per point as
+// the marching passes.
+// us per step, best march and this: so 4 48^3 10.1 and 9.6, 80^3 18.8 and 12.9,
+// 96^3 22.0 and 17.2; so 8 80^3 22.6 and 16.3; so 16 64^3 21.9 and 14.9; past
+// about 100^3 the halos of the blocks lose (so 8 128^3 37.9 and 51.5).  The
+// cost model takes either kernel for each pass by itself.
+template <int R>
+struct TtiDirect {
+    static constexpr int BX = 32, BY = 8, BZ = 8;
+    static constexpr int RA = (R + 3) / 4 * 4;
+    static constexpr int PW = BX + 2 * RA, PH = BY + 2 * R, PD = BZ + 2 * R;
+    static constexpr int THREADS = BX / 4 * BY * BZ;
+    static constexpr int F1 = PW * PH * PD;                       // a field of pass 1
+    static constexpr int FX = PW * BY * BZ, FY = BX * PH * BZ, FZ = BX * BY * PD;  // of pass 2
+    static constexpr size_t SMEM1 = (size_t)2 * F1 * 4 + 16 + 128;
+    static constexpr size_t SMEM2 = (size_t)2 * (FX + FY + FZ) * 4 + 16 + 128;
+    static_assert(FX % 16 == 0 && FY % 16 == 0, "128-byte aligned copies");
+};
+
+// First derivative along z of the float4 at `centre`, planes `pitch` floats
+// apart, summed as the z pipeline does (`mid` is added when the centre plane
+// arrives).
+template <int R, int KIND, bool MID>
+__device__ __forceinline__ Q4 dz_direct(const float *centre, int pitch, const float *t, Q4 mid) {
+    const f2 w0 = f2_splat(tap_used<KIND>(-R, R) ? t[0] : 0.f);
+    const Q4 c0 = lds_q4(centre - R * pitch);
+    Q4 s = Q4{f2_mul(w0, c0.lo), f2_mul(w0, c0.hi)};
+#pragma unroll
+    for (int d = -R + 1; d <= R; ++d) {
+        if (tap_used<KIND>(d, R)) s = q4_fma(f2_splat(t[d + R]), lds_q4(centre + d * pitch), s);
+        if (MID && d == 0) s = q4_add(s, mid);
+    }
+    return s;
+}
+
+__device__ __forceinline__ Q4 ldg_q4(const float *p) {
+    return q4_from(__ldg(reinterpret_cast<const float4 *>(p)));
+}
+
+template <int R, int KIND>
+__global__ void __launch_bounds__(TtiDirect<R>::THREADS)
+    tti_direct1_kernel(const __grid_constant__ CUtensorMap map_wint,
+                       const __grid_constant__ CUtensorMap map_whalo,
+                       const __grid_constant__ CUtensorMap map_cint,
+                       const __grid_constant__ TtiArgs a, const __grid_constant__ ReceiveArgs rec,
+                       int zchunk, int nzc) {
+    using C = TtiDirect<R>;
+    if (blockIdx.z >= gridDim.z - rec.slices) {
+        chain_trigger();
+        chain_wait();
+        if (!(__ldcg(a.err) & DEV_ERR_NONFINITE))
+            record_receivers(&rec, a.wave, 4, a.cur, 2 + a.cur, &a.L);
+        return;
+    }
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float *tile = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
+                                            ~static_cast<uintptr_t>(127));
+    uint64_t *full = reinterpret_cast<uint64_t *>(tile + 2 * C::F1);
+    const int tid = threadIdx.x;
+    const int tx = tid % 8, ty = tid / 8 % C::BY, tz = tid / (8 * C::BY);
+    const int shot = blockIdx.z / nzc, chunk = blockIdx.z - shot * nzc;
+    const int x0 = blockIdx.x * C::BX, y0 = blockIdx.y * C::BY, z0 = chunk * C::BZ;
+    const int gx = x0 + 4 * tx, gy = y0 + ty, gz = z0 + tz;
+    if (tid == 0) {
+        prefetch_tensormap(&map_whalo);
+        mbar_init(full, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    chain_trigger();
+    chain_wait();
+    if (tid == 0) {
+        mbar_arrive_expect_tx(full, 2 * C::F1 * 4);
+        tma_load_5d(tile, &map_whalo, full, x0 - C::RA, y0 - R, z0 - R, a.cur, 2 * shot);
+    }
+    const bool ok = gx < a.L.nxp && gy < a.L.ny && gz < a.L.nz;
+    const int64_t off = (int64_t)gz * a.L.plane + (int64_t)gy * a.L.nxp + gx;
+    Q4 nx = Q4{0ull, 0ull}, ny = nx, nz = nx;
+    if (ok) {
+        nx = ldg_q4(a.nvec + off);
+        ny = ldg_q4(a.nvec + a.L.vol + off);
+        nz = ldg_q4(a.nvec + 2 * a.L.vol + off);
+    }
+    // set by the divergence watchdog to stop the run: nothing is stored then
+    const bool stopped = __ldcg(a.err) & DEV_ERR_NONFINITE;
+    if (!mbar_wait_bounded(full, 0)) {
+        atomicOr(a.err, DEV_ERR_TIMEOUT);
+        // the copy gets a bounded chance to land
+        if (tid == 0) mbar_wait_bounded(full, 0, 200000000ull);
+        return;
+    }
+    if (!ok || stopped) return;
+    constexpr int SY = C::PW, SZ = C::PW * C::PH;
+    float *out = a.tmp + (int64_t)6 * shot * a.L.vol + off;
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        const float *H = tile + f * C::F1 + (R + tz) * SZ + (R + ty) * SY + 4 * tx;
+        const Q4 gxv = q4_from(dx4<R, C::RA, KIND>(H, a.t1[0]));
+        const Q4 gyv = dy_q4<R, KIND>(H + C::RA, SY, a.t1[1]);
+        const Q4 gzv = dz_direct<R, KIND, false>(H + C::RA, SZ, a.t1[2], gxv);
+        const Q4 h = q4_fma(nz, gzv, q4_fma(nx, gxv, q4_mul(ny, gyv)));
+        Q4 o[3];
+        if (f == 0) {  // f_i = D_i p - n_i h
+            const Q4 mh = q4_neg(h);
+            o[0] = q4_fma(nx, mh, gxv);
+            o[1] = q4_fma(ny, mh, gyv);
+            o[2] = q4_fma(nz, mh, gzv);
+        } else {  // e_i = n_i h
+            o[0] = q4_mul(nx, h);
+            o[1] = q4_mul(ny, h);
+            o[2] = q4_mul(nz, h);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            *reinterpret_cast<ulonglong2 *>(out + (3 * f + c) * a.L.vol) =
+                make_ulonglong2(o[c].lo, o[c].hi);
+    }
+}
+
+template <int R, int KIND>
+__global__ void __launch_bounds__(TtiDirect<R>::THREADS)
+    tti_direct2_kernel(const __grid_constant__ CUtensorMap map_tint,
+                       const __grid_constant__ CUtensorMap map_tx,
+                       const __grid_constant__ CUtensorMap map_ty,
+                       const __grid_constant__ CUtensorMap map_wlev,
+                       const __grid_constant__ CUtensorMap map_cint,
+                       const __grid_constant__ TtiArgs a,
+                       const __grid_constant__ AcousticInject inj, int zchunk, int nzc) {
+    using C = TtiDirect<R>;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float *tile = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
+                                            ~static_cast<uintptr_t>(127));
+    float *tile_y = tile + 2 * C::FX, *tile_z = tile_y + 2 * C::FY;
+    uint64_t *full = reinterpret_cast<uint64_t *>(tile_z + 2 * C::FZ);
+    const int tid = threadIdx.x;
+    const int tx = tid % 8, ty = tid / 8 % C::BY, tz = tid / (8 * C::BY);
+    const int shot = blockIdx.z / nzc, chunk = blockIdx.z - shot * nzc;
+    const int x0 = blockIdx.x * C::BX, y0 = blockIdx.y * C::BY, z0 = chunk * C::BZ;
+    const int gx = x0 + 4 * tx, gy = y0 + ty, gz = z0 + tz;
+    if (tid == 0) {
+        prefetch_tensormap(&map_tint);
+        prefetch_tensormap(&map_tx);
+        prefetch_tensormap(&map_ty);
+        mbar_init(full, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    chain_trigger();
+    chain_wait();
+    if (tid == 0) {
+        mbar_arrive_expect_tx(full, 2 * (C::FX + C::FY + C::FZ) * 4);
+        tma_load_5d(tile, &map_tx, full, x0 - C::RA, y0, z0, 0, 2 * shot);      // f_x, e_x
+        tma_load_5d(tile_y, &map_ty, full, x0, y0 - R, z0, 1, 2 * shot);        // f_y, e_y
+        tma_load_5d(tile_z, &map_tint, full, x0, y0, z0 - R, 2, 2 * shot);      // f_z, e_z
+    }
+    const bool ok = gx < a.L.nxp && gy < a.L.ny && gz < a.L.nz;
+    const int64_t off = (int64_t)gz * a.L.plane + (int64_t)gy * a.L.nxp + gx;
+    float *wave = a.wave + (int64_t)4 * shot * a.L.vol + off;
+    Q4 b = Q4{0ull, 0ull}, av = b, sv = b, keep = b, qc[2] = {b, b}, qm[2] = {b, b};
+    if (ok) {
+        b = ldg_q4(a.bcoef + off);
+        av = ldg_q4(a.acoef + off);
+        sv = ldg_q4(a.scoef + off);
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            qc[f] = lds_q4(wave + (2 * f + a.cur) * a.L.vol);
+            qm[f] = lds_q4(wave + (2 * f + 1 - a.cur) * a.L.vol);
+        }
+        float dpx4[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dpx4[i] = (gx + i < a.L.nx) ? a.dpx[gx + i] : 0.f;
+        const f2 dyz = f2_splat(-(a.dpy[gy] + a.dpz[gz]));
+        const f2 one2 = f2_splat(1.f);
+        // 1 - zeta, zeta = (dx + dy + dz) b
+        keep = Q4{f2_fma(f2_sub(dyz, f2_pack(dpx4[0], dpx4[1])), b.lo, one2),
+                  f2_fma(f2_sub(dyz, f2_pack(dpx4[2], dpx4[3])), b.hi, one2)};
+    }
+    const bool stopped = __ldcg(a.err) & DEV_ERR_NONFINITE;
+    bool landed = mbar_wait_bounded(full, 0);
+    if (!landed) {
+        atomicOr(a.err, DEV_ERR_TIMEOUT);
+        // the copies get a bounded chance to land
+        if (tid == 0) mbar_wait_bounded(full, 0, 200000000ull);
+    } else if (ok && !stopped) {
+        constexpr bool EARLY = R <= 2;  // see the marching pass
+        Q4 H[2];                        // Hxy p, Hz r
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const float *hx = tile + f * C::FX + (tz * C::BY + ty) * C::PW + 4 * tx;
+            const float *hy = tile_y + f * C::FY + (tz * C::PH + R + ty) * C::BX + 4 * tx;
+            const float *hz = tile_z + f * C::FZ + ((R + tz) * C::BY + ty) * C::BX + 4 * tx;
+            const Q4 dxy = q4_add(q4_from(dx4<R, C::RA, KIND>(hx, a.t2[0])),
+                                  dy_q4<R, KIND>(hy, C::BX, a.t2[1]));
+            H[f] = dz_direct<R, KIND, EARLY>(hz, C::BX * C::BY, a.t2[2], dxy);
+            if (!EARLY) H[f] = q4_add(dxy, H[f]);
+        }
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            const Q4 rhs = f == 0 ? q4_fma(av, H[0], q4_mul(sv, H[1]))  // a Hxy p + s Hz r
+                                  : q4_fma(sv, H[0], H[1]);             // s Hxy p + Hz r
+            const Q4 o = q4_fma(b, rhs, q4_fma(keep, q4_sub(qc[f], qm[f]), qc[f]));
+            float4 v = make_float4(f32x2::f2_lo(o.lo), f32x2::f2_hi(o.lo), f32x2::f2_lo(o.hi),
+                                   f32x2::f2_hi(o.hi));
+            // the row's padding stays zero
+            if (gx >= a.L.nx) v.x = 0.f;
+            if (gx + 1 >= a.L.nx) v.y = 0.f;
+            if (gx + 2 >= a.L.nx) v.z = 0.f;
+            if (gx + 3 >= a.L.nx) v.w = 0.f;
+            *reinterpret_cast<float4 *>(wave + (2 * f + 1 - a.cur) * a.L.vol) = v;
+        }
+    }
+    if (inj.nsrc > 0) {
+        __syncthreads();
+        if (tid == 0 && landed && !stopped)
+            tti_inject_column<C::BX, C::BY>(&a, &inj, zchunk, nzc);
+    }
+}
+
 // ---------------------------------------------------------------- recompute
 
 // The "no temporaries" scheme of the ablation (the paper's `advanced` level:
@@ -485,7 +710,21 @@ struct PassEntry {
     size_t smem;
     int bx, by, pw, ph, threads;
     float launch, lat, thr, warm;
+    int bz, pd;  // z extent of a block and of its copy (marching passes: 0 and 1)
 };
+
+template <int PASS, int R, int STAG>
+PassEntry direct_entry(float launch, float lat, float thr) {
+    using C = TtiDirect<R>;
+    constexpr int KIND = STAG ? (PASS == 1 ? 1 : -1) : 0;
+    const void *fn;
+    if constexpr (PASS == 1)
+        fn = (const void *)&tti_direct1_kernel<R, KIND>;
+    else
+        fn = (const void *)&tti_direct2_kernel<R, KIND>;
+    return PassEntry{fn,    PASS == 1 ? C::SMEM1 : C::SMEM2,
+                     C::BX, C::BY, C::PW, C::PH, C::THREADS, launch, lat, thr, 0.f, C::BZ, C::PD};
+}
 
 template <int PASS, int R, int TX, int TY, int D, int U, int MINB, int STAG>
 PassEntry pass_entry(float launch, float lat, float thr, float warm) {
@@ -497,7 +736,7 @@ PassEntry pass_entry(float launch, float lat, float thr, float warm) {
     else
         fn = (const void *)&tti_pass2_kernel<R, TX, TY, D, KIND, U, MINB>;
     return PassEntry{fn,    PASS == 1 ? C::SMEM1 : C::SMEM2,
-                     C::BX, C::BY, C::PW, C::PH, C::THREADS, launch, lat, thr, warm};
+                     C::BX, C::BY, C::PW, C::PH, C::THREADS, launch, lat, thr, warm, 0, 1};
 }
 
 struct PassTable {
@@ -523,21 +762,25 @@ PassTable pass1_table(int radius) {
         FD_TTI_ENTRY(1, 1, 16, 8, 3, 4, 0, 5.74f, 0.050f, 0.467f, 0.10f)};
     static const PassEntry r2[] = {
         FD_TTI_ENTRY(1, 2, 16, 8, 3, 4, 0, 5.74f, 0.050f, 0.467f, 0.10f),
-        FD_TTI_ENTRY(1, 2, 16, 16, 3, 4, 0, 2.59f, 0.771f, 0.249f, 0.66f)};
+        FD_TTI_ENTRY(1, 2, 16, 16, 3, 4, 0, 2.59f, 0.771f, 0.249f, 0.66f),
+        direct_entry<1, 2, STAG>(5.96f, 0.62f, 2.09f)};
     static const PassEntry r4[] = {
-        FD_TTI_ENTRY(1, 4, 16, 8, 3, 4, 0, 6.43f, 0.275f, 0.453f, 0.21f)};
+        FD_TTI_ENTRY(1, 4, 16, 8, 3, 4, 0, 6.43f, 0.275f, 0.453f, 0.21f),
+        direct_entry<1, 4, STAG>(5.67f, 0.05f, 3.05f)};
     static const PassEntry r6[] = {
         FD_TTI_ENTRY(1, 6, 16, 8, 3, 4, 2, 6.84f, 0.449f, 0.465f, 0.25f),
-        FD_TTI_ENTRY(1, 6, 16, 14, 3, 4, 1, 4.65f, 0.828f, 0.145f, 0.41f)};
+        FD_TTI_ENTRY(1, 6, 16, 14, 3, 4, 1, 4.65f, 0.828f, 0.145f, 0.41f),
+        direct_entry<1, 6, STAG>(5.04f, 3.26f, 3.50f)};
     static const PassEntry r8[] = {
         FD_TTI_ENTRY(1, 8, 16, 14, 3, 2, 1, 5.46f, 0.529f, 0.851f, 0.39f),
-        FD_TTI_ENTRY(1, 8, 16, 6, 3, 2, 2, 7.26f, 0.548f, 0.423f, 0.30f)};
+        FD_TTI_ENTRY(1, 8, 16, 6, 3, 2, 2, 7.26f, 0.548f, 0.423f, 0.30f),
+        direct_entry<1, 8, STAG>(4.89f, 4.79f, 3.82f)};
     switch (radius) {
         case 1: return {r1, 1};
-        case 2: return {r2, 2};
-        case 4: return {r4, 1};
-        case 6: return {r6, 2};
-        case 8: return {r8, 2};
+        case 2: return {r2, 3};
+        case 4: return {r4, 2};
+        case 6: return {r6, 3};
+        case 8: return {r8, 3};
         default: return {nullptr, 0};
     }
 }
@@ -547,20 +790,24 @@ PassTable pass2_table(int radius) {
     static const PassEntry r1[] = {
         FD_TTI_ENTRY(2, 1, 16, 8, 2, 4, 0, 5.87f, 0.050f, 0.632f, 0.27f)};
     static const PassEntry r2[] = {
-        FD_TTI_ENTRY(2, 2, 16, 8, 2, 4, 0, 5.87f, 0.050f, 0.632f, 0.27f)};
+        FD_TTI_ENTRY(2, 2, 16, 8, 2, 4, 0, 5.87f, 0.050f, 0.632f, 0.27f),
+        direct_entry<2, 2, STAG>(5.03f, 3.28f, 1.99f)};
     static const PassEntry r4[] = {
-        FD_TTI_ENTRY(2, 4, 16, 8, 2, 4, 0, 7.16f, 0.199f, 0.631f, 0.20f)};
+        FD_TTI_ENTRY(2, 4, 16, 8, 2, 4, 0, 7.16f, 0.199f, 0.631f, 0.20f),
+        direct_entry<2, 4, STAG>(4.95f, 4.53f, 2.84f)};
     static const PassEntry r6[] = {
-        FD_TTI_ENTRY(2, 6, 16, 8, 2, 4, 2, 7.92f, 0.408f, 0.622f, 0.25f)};
+        FD_TTI_ENTRY(2, 6, 16, 8, 2, 4, 2, 7.92f, 0.408f, 0.622f, 0.25f),
+        direct_entry<2, 6, STAG>(4.11f, 5.05f, 4.27f)};
     static const PassEntry r8[] = {
         FD_TTI_ENTRY(2, 8, 16, 14, 2, 4, 1, 4.78f, 0.652f, 0.881f, 0.40f),
-        FD_TTI_ENTRY(2, 8, 16, 6, 1, 1, 2, 7.03f, 0.648f, 0.499f, 0.32f)};
+        FD_TTI_ENTRY(2, 8, 16, 6, 1, 1, 2, 7.03f, 0.648f, 0.499f, 0.32f),
+        direct_entry<2, 8, STAG>(5.21f, 3.93f, 4.39f)};
     switch (radius) {
         case 1: return {r1, 1};
-        case 2: return {r2, 1};
-        case 4: return {r4, 1};
-        case 6: return {r6, 1};
-        case 8: return {r8, 2};
+        case 2: return {r2, 2};
+        case 4: return {r4, 2};
+        case 6: return {r6, 2};
+        case 8: return {r8, 3};
         default: return {nullptr, 0};
     }
 }
@@ -606,15 +853,25 @@ fd_status plan_pass(int pass, int radius, int stag, int config, const WaveLayout
         if (per_sm < 1) return set_error(FD_ERR_CUDA, "TTI pass-%d kernel does not fit", pass);
         const int64_t cols = (int64_t)((L.nx + e.bx - 1) / e.bx) *
                              ((L.ny + e.by - 1) / e.by) * nshots;
-        double planes = 0.0;
-        int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
+        double planes = 0.0, waves = 0.0;
+        int nzc;
+        if (e.bz) {
+            nzc = (L.nz + e.bz - 1) / e.bz;
+            planes = wave_cost(cols * nzc, nsm, per_sm, e.thr / e.lat);
+            waves = (double)cols * nzc / ((double)nsm * per_sm);
+            if ((waves > 2.0 || (int64_t)nzc * nshots > 60000) && config < 0) continue;
+        } else {
+            nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
                                 &planes);
-        if (nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
-        const double us = e.launch + e.lat * planes;
+        }
+        if (!e.bz && nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
+        // A second wave of blocks hides nothing: only for a clear gain (96^3 so 4
+        // TTI 17.4 against 22.0 us), and never a third.
+        const double us = (e.launch + e.lat * planes) * (waves > 1.0 ? 1.06 : 1.0);
         if (best < 0 || us < best_us) {
             best = i;
             best_us = us;
-            chunk = (L.nz + nzc - 1) / nzc;
+            chunk = e.bz ? e.bz : (L.nz + nzc - 1) / nzc;
         }
     }
     const PassEntry &e = t.e[best];
@@ -632,6 +889,8 @@ fd_status plan_pass(int pass, int radius, int stag, int config, const WaveLayout
     p->by = e.by;
     p->pw = e.pw;
     p->ph = e.ph;
+    p->bz = e.bz ? e.bz : 1;
+    p->pd = e.pd;
     p->est_us = best_us;
     return FD_OK;
 }
@@ -668,11 +927,13 @@ fd_status tti_plan(int radius, const WaveLayout &L, int nshots, float *wave, flo
     const uint64_t tdim[5] = {nx, ny, nz, 3, nf}, tstr[4] = {sy, sz, sv, 3 * sv};
     const uint32_t bx1 = plan->p1.bx, by1 = plan->p1.by, bx2 = plan->p2.bx, by2 = plan->p2.by;
     const uint32_t wint[5] = {bx1, by1, 1, 1, 2};
-    const uint32_t whalo[5] = {(uint32_t)plan->p1.pw, (uint32_t)plan->p1.ph, 1, 1, 2};
+    const uint32_t bz2 = plan->p2.bz;
+    const uint32_t whalo[5] = {(uint32_t)plan->p1.pw, (uint32_t)plan->p1.ph,
+                               (uint32_t)plan->p1.pd, 1, 2};
     const uint32_t wlev[5] = {bx2, by2, 1, 2, 2};
-    const uint32_t tint[5] = {bx2, by2, 1, 1, 2};
-    const uint32_t txb[5] = {(uint32_t)plan->p2.pw, by2, 1, 1, 2};
-    const uint32_t tyb[5] = {bx2, (uint32_t)plan->p2.ph, 1, 1, 2};
+    const uint32_t tint[5] = {bx2, by2, (uint32_t)plan->p2.pd, 1, 2};
+    const uint32_t txb[5] = {(uint32_t)plan->p2.pw, by2, bz2, 1, 2};
+    const uint32_t tyb[5] = {bx2, (uint32_t)plan->p2.ph, bz2, 1, 2};
     FD_TRY(make_tensor_map_5d(&plan->map_wint, wave, wdim, wstr, wint));
     FD_TRY(make_tensor_map_5d(&plan->map_whalo, wave, wdim, wstr, whalo));
     FD_TRY(make_tensor_map_5d(&plan->map_wlev, wave, wdim, wstr, wlev));
@@ -696,7 +957,7 @@ fd_status tti_choose_scheme(int radius, int stag, const WaveLayout &L, int nshot
     FD_TRY(plan_pass(1, radius, stag, -1, L, nshots, &p1));
     FD_TRY(plan_pass(2, radius, stag, -1, L, nshots, &p2));
     // so 4: two passes up to about 128^3 (48^3 10.0 against 15.5 us per step,
-    // 96^3 21.3 and 23.0, 128^3 34.4 and 34.1), fused above (256^3 204 against
+    // 96^3 17.4 and 22.9, 128^3 35.9 and 32.5), fused above (256^3 204 against
     // 268, 512^3 1430 against 2025).  The pass tables were fitted to launches
     // between events, 3.7 us each longer than chained ones.  The six
     // temporaries are not spent on many small shots at once.

@@ -301,7 +301,7 @@ struct TraceStreamer {
     StagedOut *out = nullptr;
     int nshots = 0, nt = 0, nrec = 0;
     int done = 0;
-    SideLane lane{1};
+    SideLane lane;
     bool active() const { return out && out->host && nrec > 0; }
     fd_status begin(StagedOut *o, int ns, int t, int nr) {
         out = o;
@@ -776,9 +776,9 @@ int g_acoustic_h_config[kMaxRadius + 1] = {-1, -1, -1, -1, -1, -1, -1, -1, -1};
 }  // namespace
 
 // acoustic_forward with the wavefield levels and b stored in IEEE binary16
-// (FP32 arithmetic).  Same schedule as the FP32 path without time tiling:
-// per step the stencil kernel, the injection of src[n] into u^{n+1}, and the
-// receivers of u^n on a side stream.
+// (FP32 arithmetic).  Same schedule as the FP32 path without time tiling: one
+// launch per step, which also records the receivers of u^n and injects src[n]
+// into u^{n+1} (more than 16 sources per shot: by the sparse kernel behind it).
 static fd_status acoustic_forward_h_impl(const fd_grid *grid, int so, double dt, int nt,
                                          int nshots, const float *m, const float *damp,
                                          int nsrc, const float *src_xyz, const float *src_wav,
@@ -999,7 +999,8 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
          op.scheme != FD_TTI_RECOMPUTE && op.scheme != FD_TTI_FUSED))
         return set_error(FD_ERR_ARG, "tti_forward: options (%d, %d, %d) out of range", op.deriv,
                          op.receiver, op.scheme);
-    if (op.scheme == FD_TTI_AUTO) {
+    const bool automatic = op.scheme == FD_TTI_AUTO;
+    if (automatic) {
         int scheme = kTtiTwoPass;
         FD_TRY(tti_choose_scheme(so / 2, op.deriv == FD_TTI_STAGGERED, wave_layout(*grid), nshots,
                                  &scheme));
@@ -1046,7 +1047,17 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
     swav.plan(ws, src_wav, (size_t)nshots * nt * nsrc);
     srxyz.plan(ws, rec_xyz, (size_t)nshots * nrec * 3);
     srec.plan(ws, rec_out, (size_t)nshots * nt * nrec);
-    FD_TRY(ws.allocate(s));
+    const fd_status got = ws.allocate(s);
+    if (got == FD_ERR_OOM && automatic && two_pass && R <= 2 && tti_fused_supported(R)) {
+        // no memory for the temporaries: the fused scheme has none
+        clear_error();
+        FD_TRY(cs.finish());
+        op.scheme = FD_TTI_FUSED;
+        return tti_forward_impl(grid, so, dt, nt, nshots, m, damp, eps, delta, theta, phi, nsrc,
+                                src_xyz, src_wav, nrec, rec_xyz, rec_out, p_init, r_init, p_final,
+                                r_final, &op, caller);
+    }
+    FD_TRY(got);
     float *acoef = bcoef + L.vol;
     float *scoef = bcoef + 2 * L.vol;
     float *nvec = bcoef + 3 * L.vol;
@@ -1437,7 +1448,8 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     const int ndamp = L.nx + L.ny + L.nz;
     const int nsteps = nt - 1;
     const int64_t vol = L.vol;
-    int K = checkpoint_every > 0 ? checkpoint_every : (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
+    const int sqrt_k = (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
+    int K = checkpoint_every > 0 ? checkpoint_every : sqrt_k;
     // shots of a batch
     const int most = nshots < kGradMaxShots ? nshots : kGradMaxShots;
     if (checkpoint_every == 0) {
@@ -1505,7 +1517,16 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     sres.plan(ws, rec_resid, (size_t)nshots * nt * nrec);
     sg.plan(ws, grad_m, dense);
     sq.plan(ws, src_grad, src_grad ? (size_t)nshots * nt * nsrc : 0);
-    FD_TRY(ws.allocate(s));
+    const fd_status got = ws.allocate(s);
+    if (got == FD_ERR_OOM && checkpoint_every == 0 && K > sqrt_k) {
+        // no memory for the history after all
+        clear_error();
+        FD_TRY(cs.finish());
+        return acoustic_gradient_impl(grid, so, dt, nt, nshots, m, damp, nsrc, src_xyz, src_wav,
+                                      nrec, rec_xyz, rec_resid, sqrt_k, grad_m, src_grad, what,
+                                      caller);
+    }
+    FD_TRY(got);
     for (Staged *st : {&sm, &sdamp, &ssxyz, &swav, &srxyz, &sres}) FD_TRY(st->place(s));
     FD_TRY(acoustic_common_setup(grid, so, dt, gd, nshots, sm.dev, sdamp.dev, nsrc, ssxyz.dev,
                                  nrec, srxyz.dev, bcoef, dps, src_tab, rec_tab, dstats, what, s));

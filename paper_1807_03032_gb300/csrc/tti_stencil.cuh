@@ -10,12 +10,6 @@
 namespace fdsweep {
 namespace tti {
 
-__device__ __forceinline__ float4 f4add(float4 a, float4 b) {
-    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
-__device__ __forceinline__ float4 f4fma(float w, float4 a, float4 c) {
-    return make_float4(fmaf(w, a.x, c.x), fmaf(w, a.y, c.y), fmaf(w, a.z, c.z), fmaf(w, a.w, c.w));
-}
 __device__ __forceinline__ float4 lds4(const float *p) {
     return *reinterpret_cast<const float4 *>(p);
 }
@@ -53,41 +47,7 @@ __device__ __forceinline__ float4 dx4(const float *row, const float *t) {
     return d;
 }
 
-// First derivative along y: `centre` points at the thread's float4 in the
-// centre row, rows `pitch` floats apart.
-template <int R, int KIND>
-__device__ __forceinline__ float4 dy4(const float *centre, int pitch, const float *t) {
-    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = -R; k <= R; ++k) {
-        if (!tap_used<KIND>(k, R)) continue;
-        d = f4fma(t[k + R], lds4(centre + k * pitch), d);
-    }
-    return d;
-}
-
-// z first-derivative accumulator pipeline: acc[i] is output plane p-R+i when
-// plane p arrives with values c (plane p is at offset R - i from it); acc[0]
-// is then complete.
-template <int R, int KIND>
-__device__ __forceinline__ void dz_feed(float4 (&acc)[2 * R], float4 c, const float *t) {
-#pragma unroll
-    for (int i = 0; i < 2 * R; ++i) {
-        if (!tap_used<KIND>(R - i, R)) continue;
-        acc[i] = f4fma(t[2 * R - i], c, acc[i]);
-    }
-}
-// rotate: the new last entry is output p+R, for which plane p is offset -R
-template <int R, int KIND>
-__device__ __forceinline__ void dz_shift(float4 (&acc)[2 * R], float4 c, const float *t) {
-#pragma unroll
-    for (int i = 0; i < 2 * R - 1; ++i) acc[i] = acc[i + 1];
-    const float w = tap_used<KIND>(-R, R) ? t[0] : 0.f;
-    acc[2 * R - 1] = make_float4(w * c.x, w * c.y, w * c.z, w * c.w);
-}
-
-// ---- the same on packed pairs (the two passes), with the same operations in
-// the same order per point
+// ---- cells of four points as two packed pairs
 using f32x2::f2;
 using f32x2::f2_add;
 using f32x2::f2_fma;
@@ -119,6 +79,8 @@ __device__ __forceinline__ Q4 q4_neg(Q4 a) {
 }
 __device__ __forceinline__ Q4 q4_from(float4 v) { return Q4{f2_pack(v.x, v.y), f2_pack(v.z, v.w)}; }
 
+// First derivative along y: `centre` points at the thread's four points in the
+// centre row, rows `pitch` floats apart.
 template <int R, int KIND>
 __device__ __forceinline__ Q4 dy_q4(const float *centre, int pitch, const float *t) {
     Q4 d = Q4{0ull, 0ull};
@@ -129,6 +91,8 @@ __device__ __forceinline__ Q4 dy_q4(const float *centre, int pitch, const float 
     }
     return d;
 }
+// z accumulator pipeline: acc[i] is output plane p-R+i when plane p arrives
+// with values c (plane p is at offset R - i from it); acc[0] is then complete.
 template <int R, int KIND>
 __device__ __forceinline__ void dz_feed_q4(Q4 (&acc)[2 * R], Q4 c, const float *t) {
 #pragma unroll
@@ -137,6 +101,7 @@ __device__ __forceinline__ void dz_feed_q4(Q4 (&acc)[2 * R], Q4 c, const float *
         acc[i] = q4_fma(f2_splat(t[2 * R - i]), c, acc[i]);
     }
 }
+// rotate: the new last entry is output p+R, for which plane p is offset -R
 template <int R, int KIND>
 __device__ __forceinline__ void dz_shift_q4(Q4 (&acc)[2 * R], Q4 c, const float *t) {
 #pragma unroll

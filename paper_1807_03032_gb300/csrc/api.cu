@@ -3,16 +3,17 @@
 //
 // Per time step n (the paper's schedule of one time iteration: stencil
 // update, then sparse injection into the t+1 field; receivers sample t):
-//   acoustic:  K1 acoustic_step  ->  K3/K4 sparse (inject src[n] into u^{n+1},
-//              interpolate rec[n] from u^n)
-//   TTI:       K2a tti_pass1 -> K2b tti_pass2 -> K3/K4 sparse
-// Steps are captured into a CUDA graph of kGraphChunk steps that is replayed;
-// the sparse kernel reads its time index from a device counter that the
-// graph's last node advances.
+//   acoustic:  K1 acoustic_step, which also interpolates rec[n] from u^n and
+//              injects src[n] into u^{n+1} (many sources: K3/K4 sparse)
+//   TTI:       K2a tti_pass1 -> K2b tti_pass2, or the fused kernel, likewise
+// Launches are chained (programmatic dependent launch); long runs replay a
+// CUDA graph of kGraphChunk steps whose kernels read their time index from a
+// device counter that the graph's last node advances.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <vector>
 
 #include "kernels.cuh"
@@ -53,11 +54,24 @@ double second_symbol_max(int r, const double *w) {
     return best;
 }
 
+// The largest value of a scheme's symbol depends on the radius alone: it is
+// scanned once per radius.  (4097 r sines or cosines on every call, between the
+// medium's validation and the first step, were 60 us of a 64^3 call's 640 at
+// so 4, and four times that at so 16.)
+enum SchemeSymbol { kSecondDerivative, kFirstDerivative, kStaggeredDerivative, kNumSymbols };
+double scheme_symbol_max(SchemeSymbol kind, int r, double (*scan)(int, const double *),
+                         const double *weights) {
+    static std::once_flag once[kNumSymbols][kMaxRadius + 1];
+    static double value[kNumSymbols][kMaxRadius + 1];
+    std::call_once(once[kind][r], [&] { value[kind][r] = scan(r, weights); });
+    return value[kind][r];
+}
+
 double acoustic_dt_bound(const fd_grid &g, int r, double m_min) {
     double w[kMaxRadius + 1] = {0.0}, c[kMaxRadius + 1] = {0.0};
     fd_weights(r, w, c);
     const double vmax = 1.0 / sqrt(m_min);
-    const double lam = second_symbol_max(r, w) *
+    const double lam = scheme_symbol_max(kSecondDerivative, r, second_symbol_max, w) *
                        (1.0 / (g.hx * g.hx) + 1.0 / (g.hy * g.hy) + 1.0 / (g.hz * g.hz));
     return 2.0 / (vmax * sqrt(lam));
 }
@@ -532,6 +546,18 @@ static fd_status acoustic_forward_impl(const fd_grid *grid, int so, double dt, i
     }
     FD_TRY(finish_medium_stats(dstats, s));
     FD_STAGE(s, "acoustic: setup kernels");
+    // ---- initial state; queued and planned before the host waits for the
+    // medium's validation
+    FD_CUDA_TRY(cudaMemsetAsync(wave, 0, (size_t)lps * nshots * L.vol * 4, s));
+    if (u_init)
+        for (int sh = 0; sh < nshots; ++sh)
+            FD_TRY(copy_fields_in(wave, L, u_init, sh, 2, lps, 0, s));
+
+    // ---- K1 plan and arguments
+    AcousticPlan plan;
+    FD_STAGE(s, "acoustic: initial state");
+    FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nshots, lps, wave, bcoef, &plan, 0,
+                         damp_field));
     MediumStats hs;
     FD_TRY(read_stats(dstats, &hs, s));
     FD_TRY(flags_to_status(hs.flags, "acoustic_forward"));
@@ -545,17 +571,6 @@ static fd_status acoustic_forward_impl(const fd_grid *grid, int so, double dt, i
                              dt, dt_max, vmax, so);
     }
 
-    // ---- initial state
-    FD_CUDA_TRY(cudaMemsetAsync(wave, 0, (size_t)lps * nshots * L.vol * 4, s));
-    if (u_init)
-        for (int sh = 0; sh < nshots; ++sh)
-            FD_TRY(copy_fields_in(wave, L, u_init, sh, 2, lps, 0, s));
-
-    // ---- K1 plan and arguments
-    AcousticPlan plan;
-    FD_STAGE(s, "acoustic: initial state");
-    FD_TRY(acoustic_plan(R, g_acoustic_config[R], L, nshots, lps, wave, bcoef, &plan, 0,
-                         damp_field));
     FD_STAGE(s, plan.name);
     AcousticStepArgs a;
     memset(&a, 0, sizeof(a));
@@ -1075,25 +1090,7 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
                                   *grid, L, rec_tab + (size_t)sh * nrec, &dstats->flags, s));
     }
     FD_TRY(finish_medium_stats(dstats, s));
-    MediumStats hs;
-    FD_TRY(read_stats(dstats, &hs, s));
-    FD_TRY(flags_to_status(hs.flags, "tti_forward"));
-    {
-        const double vmax = 1.0 / sqrt((double)hs.m_min);
-        const double amax = 1.0 + 2.0 * (double)(hs.eps_max > 0.f ? hs.eps_max : 0.f);
-        double sa[kMaxRadius + 1];
-        staggered_weights(R, sa);
-        const double sig = stag ? staggered_symbol_sq_max(R, sa) : first_symbol_sq_max(R, gd.c);
-        const double lam = sig * (1.0 / (grid->hx * grid->hx) + 1.0 / (grid->hy * grid->hy) +
-                                  1.0 / (grid->hz * grid->hz));
-        const double dt_max = 2.0 / sqrt(amax * vmax * vmax * lam);
-        if (dt > dt_max * (1.0 + 1e-12))
-            return set_error(FD_ERR_CFL,
-                             "dt = %.6g ms exceeds the TTI stability bound %.6g ms "
-                             "(v_max = %.6g km/s, 1+2eps_max = %.4g, so = %d)",
-                             dt, dt_max, vmax, amax, so);
-    }
-
+    // queued and planned before the host waits for the medium's validation
     FD_CUDA_TRY(cudaMemsetAsync(wave, 0, (size_t)4 * nshots * L.vol * 4, s));
     for (int sh = 0; sh < nshots; ++sh) {
         if (p_init) FD_TRY(copy_fields_in(wave, L, p_init, sh, 2, 4, 0, s));
@@ -1107,6 +1104,27 @@ static fd_status tti_forward_impl(const fd_grid *grid, int so, double dt, int nt
     else
         FD_TRY(tti_plan(R, L, nshots, wave, tmp, bcoef, &tplan, stag ? 1 : 0,
                         two_pass ? kTtiTwoPass : kTtiRecompute, g_tti_config[R]));
+    MediumStats hs;
+    FD_TRY(read_stats(dstats, &hs, s));
+    FD_TRY(flags_to_status(hs.flags, "tti_forward"));
+    {
+        const double vmax = 1.0 / sqrt((double)hs.m_min);
+        const double amax = 1.0 + 2.0 * (double)(hs.eps_max > 0.f ? hs.eps_max : 0.f);
+        double sa[kMaxRadius + 1];
+        staggered_weights(R, sa);
+        const double sig =
+            stag ? scheme_symbol_max(kStaggeredDerivative, R, staggered_symbol_sq_max, sa)
+                 : scheme_symbol_max(kFirstDerivative, R, first_symbol_sq_max, gd.c);
+        const double lam = sig * (1.0 / (grid->hx * grid->hx) + 1.0 / (grid->hy * grid->hy) +
+                                  1.0 / (grid->hz * grid->hz));
+        const double dt_max = 2.0 / sqrt(amax * vmax * vmax * lam);
+        if (dt > dt_max * (1.0 + 1e-12))
+            return set_error(FD_ERR_CFL,
+                             "dt = %.6g ms exceeds the TTI stability bound %.6g ms "
+                             "(v_max = %.6g km/s, 1+2eps_max = %.4g, so = %d)",
+                             dt, dt_max, vmax, amax, so);
+    }
+
     TtiArgs a;
     memset(&a, 0, sizeof(a));
     a.wave = wave;

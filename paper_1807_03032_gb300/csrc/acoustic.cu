@@ -572,7 +572,9 @@ struct ConfigEntry {
     float launch, lat, thr, warm;
     const char *name;
     int bz, pd;  // z extent of a block and of its copy (marching kernel: 0 and 1)
+    bool spare = false;  // only for grids that no other entry can launch
 };
+constexpr int kMaxEntries = 8;  // of a configuration table
 
 template <int R, int TX, int TY, int VY, int D, int U, bool DF, int MINB, bool EDGE>
 ConfigEntry make_entry(const char *name, float launch, float lat, float thr, float warm) {
@@ -593,6 +595,11 @@ ConfigEntry make_direct(const char *name, float launch, float lat, float thr) {
     return ConfigEntry{R,     (const void *)&acoustic_direct_kernel<R, DF>,
                        wl,    C::SMEM, C::BX, C::BY, C::PW, C::PH, C::THREADS,
                        launch, lat, thr, 0.f, name, C::BZ, C::PD};
+}
+
+ConfigEntry spare(ConfigEntry e) {
+    e.spare = true;
+    return e;
 }
 
 #define FD_AC_ENTRY(R, TX, TY, VY, D, U, MB, ED, ...)                                           \
@@ -663,7 +670,9 @@ const ConfigEntry *config_table_df(int radius, int *count) {
         FD_AC_ENTRY_DF(1, 16, 16, 1, 3, 4, 0, 0, 2.7f, 0.28f, 0.38f, 0.5f)};
     static const ConfigEntry r2[] = {
         FD_AC_ENTRY_DF(2, 16, 8, 1, 3, 4, 0, 0, 3.17f, 0.286f, 0.185f, 0.42f),
-        make_direct<2, true>("acoustic_direct<2,damp field>", 2.50f, 1.41f, 1.20f)};
+        make_direct<2, true>("acoustic_direct<2,damp field>", 2.50f, 1.41f, 1.20f),
+        // 16 rows: the only one beyond 524280 of them (65535 blocks of 8)
+        spare(FD_AC_ENTRY_DF(2, 16, 16, 1, 3, 4, 0, 0, 2.44f, 0.30f, 0.31f, 0.9f))};
     static const ConfigEntry r4[] = {
         FD_AC_ENTRY_DF(4, 16, 8, 1, 3, 8, 0, 0, 3.33f, 0.291f, 0.193f, 0.57f),
         FD_AC_ENTRY_DF(4, 16, 4, 2, 3, 8, 0, 0, 3.91f, 0.342f, 0.181f, 0.42f),
@@ -679,7 +688,7 @@ const ConfigEntry *config_table_df(int radius, int *count) {
         make_direct<8, true>("acoustic_direct<8,damp field>", 2.80f, 2.68f, 2.20f)};
     switch (radius) {
         case 1: *count = 1; return r1;
-        case 2: *count = 2; return r2;
+        case 2: *count = 3; return r2;
         case 4: *count = 3; return r4;
         case 6: *count = 3; return r6;
         case 8: *count = 4; return r8;
@@ -709,60 +718,33 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     FD_CUDA_TRY(
         cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    // The configuration and chunk count with the smallest estimated time.
-    int best = -1, zchunk = 0;
-    double best_us = 0.0;
+    PlanEntry cand[kMaxEntries];
     for (int i = 0; i < n; ++i) {
-        if (config >= 0 && i != config) continue;
         const ConfigEntry &e = tab[i];
         int per_sm = 0;
         FD_TRY(raise_smem_limit(e.fn, e.smem));
         FD_CUDA_TRY(
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e.fn, e.threads, e.smem));
         if (per_sm < 1) return set_error(FD_ERR_CUDA, "kernel %s does not fit on an SM", e.name);
-        const int64_t cols = (int64_t)((L.nx + e.bx - 1) / e.bx) *
-                             ((L.ny + e.by - 1) / e.by) * nshots;
-        int nzc = 1;
-        double planes = 0.0, waves = 0.0;
-        if (e.bz) {
-            nzc = (L.nz + e.bz - 1) / e.bz;
-            planes = wave_cost(cols * nzc, nsm, per_sm, e.thr / e.lat);
-            waves = (double)cols * nzc / ((double)nsm * per_sm);
-            if ((waves > 2.0 || (int64_t)nzc * nshots > 60000) && config < 0) continue;
-        } else {
-            nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
-                                &planes);
-        }
         // damp_z of a chunk follows the stages in shared memory
-        const int max_chunk = (max_smem - (int)e.smem) / 4;
-        const int min_nzc = (L.nz + max_chunk - 1) / max_chunk;
-        if (nzc < min_nzc) nzc = min_nzc;
-        if (!e.bz && nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
-        if (nzc < min_nzc && config < 0 && i + 1 < n) continue;
-        // A second wave of blocks hides nothing: only for a clear gain (96^3 so 4
-        // TTI 17.4 against 22.0 us), and never a third.
-        const double us = (e.launch + e.lat * planes) * (waves > 1.0 ? 1.06 : 1.0);
-        if (best < 0 || us < best_us) {
-            best = i;
-            best_us = us;
-            zchunk = e.bz ? e.bz : (L.nz + nzc - 1) / nzc;
-        }
+        cand[i] = PlanEntry{e.bx, e.by, e.bz, per_sm, e.launch, e.lat, e.thr,
+                            e.warm * 2.0 * radius, (max_smem - (int)e.smem) / 4, 0, e.spare};
     }
-    const ConfigEntry &e = tab[best];
+    const PlanChoice best = choose_plan(cand, n, config, L.nx, L.ny, L.nz, nshots, nsm);
+    if (best.entry < 0)
+        return set_error(FD_ERR_ARG, "grid too large for the launch configuration");
+    const ConfigEntry &e = tab[best.entry];
     plan->radius = radius;
-    plan->config = best;
+    plan->config = best.entry;
     plan->damp_field = damp_field;
     plan->name = e.name;
     plan->block = dim3(e.threads, 1, 1);
     const int ntx = (L.nx + e.bx - 1) / e.bx;
     const int nty = (L.ny + e.by - 1) / e.by;
-    const int nzc = (L.nz + zchunk - 1) / zchunk;
-    if ((int64_t)nshots * nzc > 65535 || nty > 65535)
-        return set_error(FD_ERR_ARG, "grid too large for the launch configuration");
-    plan->grid = dim3(ntx, nty, nshots * nzc);
-    plan->zchunk = zchunk;
-    plan->nzc = nzc;
-    plan->smem = e.smem + (size_t)zchunk * 4;
+    plan->grid = dim3(ntx, nty, nshots * best.nzc);
+    plan->zchunk = best.zchunk;
+    plan->nzc = best.nzc;
+    plan->smem = e.smem + (size_t)best.zchunk * 4;
     FD_TRY(raise_smem_limit(e.fn, plan->smem));
     if (e.fn_wl) FD_TRY(raise_smem_limit(e.fn_wl, plan->smem));
     FD_TRY(make_tensor_map_4d(&plan->map_halo, wave, L.nx, L.ny, L.nz, (uint64_t)map_shots * lps,

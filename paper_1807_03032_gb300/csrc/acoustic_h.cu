@@ -416,6 +416,7 @@ struct HEntry {
     float launch, lat, thr, warm;
     const char *name;
 };
+constexpr int kMaxHEntries = 4;  // of a configuration table
 
 template <int R, int TX, int TY, int VY, int D, int U, int MINB>
 HEntry make_h_entry(const char *name, float launch, float lat, float thr, float warm) {
@@ -609,48 +610,37 @@ fd_status acoustic_h_plan(int radius, int config, const WaveLayout &L, int nshot
     if (!tab) return set_error(FD_ERR_UNIMPL, "no binary16-storage kernel for radius %d", radius);
     if (L.nxp % 8) return set_error(FD_ERR_ARG, "binary16 layout: row length not a multiple of 8");
     if (config >= n) config = -1;
-    int dev = 0, nsm = 0;
+    int dev = 0, nsm = 0, max_smem = 0;
     FD_CUDA_TRY(cudaGetDevice(&dev));
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    int best = -1, zchunk = 0;
-    double best_us = 0.0;
+    FD_CUDA_TRY(
+        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    PlanEntry cand[kMaxHEntries];
     for (int i = 0; i < n; ++i) {
-        if (config >= 0 && i != config) continue;
         const HEntry &e = tab[i];
         int per_sm = 0;
         FD_TRY(raise_smem_limit(e.fn, e.smem));
         FD_CUDA_TRY(
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e.fn, e.threads, e.smem));
         if (per_sm < 1) return set_error(FD_ERR_CUDA, "kernel %s does not fit on an SM", e.name);
-        const int64_t cols = (int64_t)((L.nx + e.bx - 1) / e.bx) *
-                             ((L.ny + e.by - 1) / e.by) * nshots;
-        double planes = 0.0;
-        int nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
-                                &planes);
-        const int min_nzc = (L.nz + 8191) / 8192;  // damp_z of a chunk: at most 32 KB
-        if (nzc < min_nzc) nzc = min_nzc;
-        if (nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
-        const double us = e.launch + e.lat * planes;
-        if (best < 0 || us < best_us) {
-            best = i;
-            best_us = us;
-            zchunk = (L.nz + nzc - 1) / nzc;
-        }
+        // damp_z of a chunk follows the stages in shared memory: 32 KB of it
+        cand[i] = PlanEntry{e.bx, e.by, 0, per_sm, e.launch, e.lat, e.thr,
+                            e.warm * 2.0 * radius, (max_smem - (int)e.smem) / 4, 8192, false};
     }
-    const HEntry &e = tab[best];
+    const PlanChoice best = choose_plan(cand, n, config, L.nx, L.ny, L.nz, nshots, nsm);
+    if (best.entry < 0)
+        return set_error(FD_ERR_ARG, "grid too large for the launch configuration");
+    const HEntry &e = tab[best.entry];
     plan->radius = radius;
-    plan->config = best;
+    plan->config = best.entry;
     plan->name = e.name;
     plan->block = dim3(e.threads, 1, 1);
     const int ntx = (L.nx + e.bx - 1) / e.bx;
     const int nty = (L.ny + e.by - 1) / e.by;
-    const int nzc = (L.nz + zchunk - 1) / zchunk;
-    if ((int64_t)nshots * nzc > 65535 || nty > 65535)
-        return set_error(FD_ERR_ARG, "grid too large for the launch configuration");
-    plan->grid = dim3(ntx, nty, nshots * nzc);
-    plan->zchunk = zchunk;
-    plan->nzc = nzc;
-    plan->smem = e.smem + (size_t)zchunk * 4;
+    plan->grid = dim3(ntx, nty, nshots * best.nzc);
+    plan->zchunk = best.zchunk;
+    plan->nzc = best.nzc;
+    plan->smem = e.smem + (size_t)best.zchunk * 4;
     FD_TRY(raise_smem_limit(e.fn, plan->smem));
     const uint64_t sy = (uint64_t)L.nxp * 2, sz = (uint64_t)L.plane * 2, sw = (uint64_t)L.vol * 2;
     FD_TRY(make_tensor_map_4d_elem(&plan->map_halo, wave, 2, L.nx, L.ny, L.nz,

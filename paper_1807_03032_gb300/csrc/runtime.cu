@@ -242,43 +242,6 @@ fd_status raise_smem_limit(const void *fn, size_t bytes) {
     return FD_OK;
 }
 
-double wave_cost(int64_t units, int nsm, int per_sm, double load) {
-    const int64_t slots = (int64_t)nsm * per_sm;
-    auto h = [&](double k) { return sqrt(1.0 + load * load * k * k); };
-    const int64_t full = units / slots, rem = units - full * slots;
-    double waves = (double)full * h(per_sm);
-    if (rem) {
-        // the last wave: between the mean and the fullest SM's load
-        double k = (double)rem / nsm;
-        if (k < 1.0) k = 1.0;
-        waves += h(0.5 * (k + ceil(k)));
-    }
-    return waves;
-}
-
-int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load,
-                  double *planes) {
-    const int64_t slots = (int64_t)nsm * per_sm;
-    // beyond a few waves more chunks only add warm-up planes
-    const int64_t most = 8 * slots / (cols > 0 ? cols : 1) + 8;
-    int best = 1;
-    double best_cost = 0.0;
-    int last_chunk = 0;
-    for (int n = 1; n <= nz && n <= most; ++n) {
-        const int chunk = (nz + n - 1) / n;
-        if (chunk == last_chunk) continue;
-        last_chunk = chunk;
-        const int64_t units = cols * ((nz + chunk - 1) / chunk);
-        const double cost = (chunk + warmup) * wave_cost(units, nsm, per_sm, load);
-        if (n == 1 || cost < best_cost) {
-            best_cost = cost;
-            best = n;
-        }
-    }
-    if (planes) *planes = best_cost;
-    return best;
-}
-
 bool is_device_pointer(const void *p) {
     if (!p) return true;
     cudaPointerAttributes attr;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "plan.h"
 
 namespace fdsweep {
 
@@ -36,34 +37,6 @@ fd_status make_tensor_map_5d(CUtensorMap *map, const float *base, const uint64_t
 // shared by every thread and call, so one call must not lower the limit
 // another call is about to launch with (concurrent calls from host threads).
 fd_status raise_smem_limit(const void *fn, size_t bytes);
-
-// Time of `units` equal CTAs on nsm SMs with per_sm places each, in units of a
-// CTA alone on its SM: k CTAs on an SM take sqrt(1 + (load k)^2).
-double wave_cost(int64_t units, int nsm, int per_sm, double load);
-
-// Number of z chunks into which the columns of a z-marching stencil launch
-// are cut (1 .. nz).  A CTA marches `warmup` planes (in units of a full
-// plane's time) before its chunk's first output, and the columns times the
-// chunks fill the machine in waves of nsm * per_sm CTAs, so the launch lasts
-// about
-//   (chunk + warmup) * sum over the waves of h(CTAs per SM),
-//   h(k) = sqrt(1 + (load k)^2),
-// h being the time of one plane relative to a lone CTA's: constant (the
-// latency of one plane's copy and arithmetic) while few CTAs share an SM,
-// proportional to k once its throughput (shared memory, HBM) is used up.
-// The count with the smallest estimate is taken.  Measured on GB300 over 64^3
-// .. 512^3, ragged grids and 1 .. 8 shots (154 problems of the acoustic
-// kernels and TTI, one to 32 chunks each), it picks the fastest measured
-// count or one within 2 % of it in all but 11, the worst at 7 %; filling the
-// slots and rounding the count up instead (a few CTAs then run a whole wave
-// of their own, and chunks were at least 32 planes long) took 1.1x to 6x as
-// long up to 384^3:
-// acoustic 64^3 so 4 20.1 against 7.2 us per step, 256^3 so 8 77 against 53,
-// 384^3 so 8 170 against 142; TTI 48^3 so 4 85 against 15, 256^3 so 8 382
-// against 301.
-// `planes` (optional) receives the estimate.
-int pick_z_chunks(int64_t cols, int nsm, int per_sm, int nz, double warmup, double load,
-                  double *planes = nullptr);
 
 // Host-side fault injection for tests: with the environment variable
 // FDSWEEP_FAIL_ALLOC=1 every device allocation of the library (per-call

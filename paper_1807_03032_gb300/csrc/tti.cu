@@ -743,6 +743,7 @@ struct PassTable {
     const PassEntry *e;
     int n;
 };
+constexpr int kMaxPassEntries = 4;  // of a table
 
 #define FD_TTI_ENTRY(PASS, R, TX, TY, D, U, MB, ...) \
     pass_entry<PASS, R, TX, TY, D, U, MB, STAG>(__VA_ARGS__)
@@ -841,57 +842,36 @@ fd_status plan_pass(int pass, int radius, int stag, int config, const WaveLayout
     int dev = 0, nsm = 0;
     FD_CUDA_TRY(cudaGetDevice(&dev));
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    int best = -1, chunk = 0;
-    double best_us = 0.0;
+    PlanEntry cand[kMaxPassEntries];
     for (int i = 0; i < t.n; ++i) {
-        if (config >= 0 && i != (config < t.n ? config : t.n - 1)) continue;
         const PassEntry &e = t.e[i];
         int per_sm = 0;
         FD_TRY(raise_smem_limit(e.fn, e.smem));
         FD_CUDA_TRY(
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e.fn, e.threads, e.smem));
         if (per_sm < 1) return set_error(FD_ERR_CUDA, "TTI pass-%d kernel does not fit", pass);
-        const int64_t cols = (int64_t)((L.nx + e.bx - 1) / e.bx) *
-                             ((L.ny + e.by - 1) / e.by) * nshots;
-        double planes = 0.0, waves = 0.0;
-        int nzc;
-        if (e.bz) {
-            nzc = (L.nz + e.bz - 1) / e.bz;
-            planes = wave_cost(cols * nzc, nsm, per_sm, e.thr / e.lat);
-            waves = (double)cols * nzc / ((double)nsm * per_sm);
-            if ((waves > 2.0 || (int64_t)nzc * nshots > 60000) && config < 0) continue;
-        } else {
-            nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, e.warm * 2 * radius, e.thr / e.lat,
-                                &planes);
-        }
-        if (!e.bz && nzc > 60000 / nshots) nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
-        // A second wave of blocks hides nothing: only for a clear gain (96^3 so 4
-        // TTI 17.4 against 22.0 us), and never a third.
-        const double us = (e.launch + e.lat * planes) * (waves > 1.0 ? 1.06 : 1.0);
-        if (best < 0 || us < best_us) {
-            best = i;
-            best_us = us;
-            chunk = e.bz ? e.bz : (L.nz + nzc - 1) / nzc;
-        }
+        cand[i] = PlanEntry{e.bx,  e.by, e.bz, per_sm, e.launch, e.lat, e.thr,
+                            e.warm * 2.0 * radius, INT_MAX, 0, false};
     }
-    const PassEntry &e = t.e[best];
-    const int ntx = (L.nx + e.bx - 1) / e.bx, nty = (L.ny + e.by - 1) / e.by;
-    const int nzc = (L.nz + chunk - 1) / chunk;
-    if ((int64_t)nshots * nzc > 65535 || nty > 65535)
+    const int forced = config < 0 ? -1 : (config < t.n ? config : t.n - 1);
+    const PlanChoice best = choose_plan(cand, t.n, forced, L.nx, L.ny, L.nz, nshots, nsm);
+    if (best.entry < 0)
         return set_error(FD_ERR_ARG, "grid too large for the TTI launch configuration");
+    const PassEntry &e = t.e[best.entry];
+    const int ntx = (L.nx + e.bx - 1) / e.bx, nty = (L.ny + e.by - 1) / e.by;
     p->fn = e.fn;
-    p->grid = dim3(ntx, nty, nshots * nzc);
+    p->grid = dim3(ntx, nty, nshots * best.nzc);
     p->block = dim3(e.threads, 1, 1);
     p->smem = e.smem;
-    p->zchunk = chunk;
-    p->nzc = nzc;
+    p->zchunk = best.zchunk;
+    p->nzc = best.nzc;
     p->bx = e.bx;
     p->by = e.by;
     p->pw = e.pw;
     p->ph = e.ph;
     p->bz = e.bz ? e.bz : 1;
     p->pd = e.pd;
-    p->est_us = best_us;
+    p->est_us = best.us;
     return FD_OK;
 }
 

@@ -389,22 +389,20 @@ bool tti_fused_supported(int radius) {
     return fused_info(radius, 0, 0, &in);
 }
 
-// Estimated time (us) of a fused step and its chunk count.
-static fd_status fused_estimate(const FusedInfo &in, int radius, const WaveLayout &L, int nshots,
-                                int *nzc, double *us) {
+// Chunk count of a fused step and its estimated time.
+static fd_status fused_choice(const FusedInfo &in, int radius, const WaveLayout &L, int nshots,
+                              PlanChoice *c) {
     FD_TRY(raise_smem_limit(in.fn, in.smem));
     int dev = 0, nsm = 0, per_sm = 0;
     FD_CUDA_TRY(cudaGetDevice(&dev));
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     FD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, in.fn, in.threads, in.smem));
     if (per_sm < 1) return set_error(FD_ERR_CUDA, "fused TTI kernel does not fit on an SM");
-    const int64_t cols =
-        (int64_t)((L.nx + 63) / 64) * ((L.ny + in.by - 1) / in.by) * nshots;
     // 4R warm-up planes, the first half of which only feed the z pipeline
-    double planes = 0.0;
-    *nzc = pick_z_chunks(cols, nsm, per_sm, L.nz, in.warm * 4 * radius, in.thr / in.lat, &planes);
-    if (*nzc > 60000 / nshots) *nzc = 60000 / nshots > 1 ? 60000 / nshots : 1;  // + receivers
-    *us = in.launch + in.lat * planes;
+    const PlanEntry e{64, in.by, 0, per_sm, in.launch, in.lat, in.thr,
+                      in.warm * 4.0 * radius, INT_MAX, 0, false};
+    *c = choose_plan(&e, 1, -1, L.nx, L.ny, L.nz, nshots, nsm);
+    if (c->entry < 0) return set_error(FD_ERR_ARG, "grid too large for the fused TTI launch");
     return FD_OK;
 }
 
@@ -412,8 +410,10 @@ fd_status tti_fused_time(int radius, int stag, const WaveLayout &L, int nshots, 
     FusedInfo in;
     if (!fused_info(radius, stag, 0, &in))
         return set_error(FD_ERR_ARG, "the fused TTI scheme covers space orders up to 8");
-    int nzc = 1;
-    return fused_estimate(in, radius, L, nshots, &nzc, us);
+    PlanChoice c;
+    FD_TRY(fused_choice(in, radius, L, nshots, &c));
+    *us = c.us;
+    return FD_OK;
 }
 
 fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, float *wave,
@@ -423,24 +423,19 @@ fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, 
         return set_error(FD_ERR_ARG, "the fused TTI scheme covers space orders up to 8");
     const uint32_t bx = 64, by = in.by;
     const int ntx = (L.nx + bx - 1) / bx, nty = (L.ny + by - 1) / by;
-    int nzc = 1;
-    double us = 0.0;
-    FD_TRY(fused_estimate(in, radius, L, nshots, &nzc, &us));
-    const int zchunk = (L.nz + nzc - 1) / nzc;
-    nzc = (L.nz + zchunk - 1) / zchunk;
-    if ((int64_t)nshots * nzc > 65535 || nty > 65535)
-        return set_error(FD_ERR_ARG, "grid too large for the fused TTI launch");
+    PlanChoice c;
+    FD_TRY(fused_choice(in, radius, L, nshots, &c));
     plan->radius = radius;
     plan->stag = stag ? 1 : 0;
     plan->scheme = kTtiFused;
     plan->config = config == 1 ? 1 : 0;
     plan->p1.fn = in.fn;
-    plan->p1.grid = dim3(ntx, nty, nshots * nzc);
+    plan->p1.grid = dim3(ntx, nty, nshots * c.nzc);
     plan->p1.block = dim3(in.threads, 1, 1);
     plan->p1.smem = in.smem;
-    plan->p1.zchunk = zchunk;
-    plan->p1.nzc = nzc;
-    plan->p1.est_us = us;
+    plan->p1.zchunk = c.zchunk;
+    plan->p1.nzc = c.nzc;
+    plan->p1.est_us = c.us;
     const uint64_t sy = (uint64_t)L.nxp * 4, sz = (uint64_t)L.plane * 4, sv = (uint64_t)L.vol * 4;
     const uint64_t wdim[5] = {(uint64_t)L.nx, (uint64_t)L.ny, (uint64_t)L.nz, 2, 2ull * nshots};
     const uint64_t wstr[4] = {sy, sz, sv, 2 * sv};

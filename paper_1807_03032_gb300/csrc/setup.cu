@@ -1,20 +1,21 @@
 // setup.cu -- K0: per-call coefficient precompute and validation.
 //
 //  * b = dt^2 / (m + damp dt / 2) per point, rounded once to FP32 (two-float
-//    FP32 arithmetic with a residual-corrected quotient; FP64 with a
+//    FP32 arithmetic, twofloat.cuh, with a residual-corrected quotient; FP64 with a
 //    Newton-Raphson reciprocal for points outside its range),
 //    the factor that multiplies the Laplacian in the leapfrog update and the
 //    injected source (Listing finject's dt^2 q / m, generalised to the damped
 //    update); damping profiles scaled by 1/dt.
 //  * TTI: a = 1 + 2 eps, s = sqrt(1 + 2 delta) and the symmetry axis
 //    n = (sin theta cos phi, sin theta sin phi, cos theta), precomputed once
-//    because they do not change with time; rounded once to FP32, formed in
-//    two-float arithmetic too.
+//    because they do not change with time; the FP64 values rounded once to
+//    FP32, formed in two-float arithmetic where that decides the rounding.
 //  * Sparse tables: the trilinear corner and fractional offsets of every
 //    source and receiver, x1 = floor((x - o)/h) in FP64, clamped to n - 2.
 //  * Reductions for validation: min/max of m (stability bound), max eps,
 //    flags for non-finite or non-physical values.
 #include "kernels.cuh"
+#include "twofloat.cuh"
 
 namespace fdsweep {
 namespace {
@@ -69,94 +70,6 @@ __device__ __forceinline__ double recip_newton(double x) {
     y = fma(y, fma(-x, y, 1.0), y);
     y = fma(y, fma(-x, y, 1.0), y);
     return y;
-}
-
-// Two-float arithmetic (a value as an unevaluated sum hi + lo of floats),
-// with the error-free transformations TwoSum (Knuth) and TwoProduct (by FMA)
-// and the rounding-explicit intrinsics, so that no operation is contracted.
-struct TwoFloat {
-    float hi, lo;
-};
-
-__device__ __forceinline__ TwoFloat two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return TwoFloat{s, e};
-}
-
-__device__ __forceinline__ TwoFloat quick_two_sum(float a, float b) {  // |a| >= |b| or a = 0
-    const float s = __fadd_rn(a, b);
-    return TwoFloat{s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-
-__device__ __forceinline__ TwoFloat tf_mul(TwoFloat a, TwoFloat b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-    return quick_two_sum(p, e);
-}
-
-__device__ __forceinline__ TwoFloat tf_add(TwoFloat a, TwoFloat b) {
-    const TwoFloat s = two_sum(a.hi, b.hi);
-    return quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
-}
-
-// sin x and cos x as two-floats for |x| <= kSincosRange, to about 2^-36 of
-// their size: x - k pi/2 with pi/2 as three floats and exact products (Cody
-// and Waite's reduction), then the Taylor series on [-pi/4, pi/4], the last
-// terms in plain FP32 and the leading ones in two-float arithmetic.  Against
-// 80-bit references over 2e7 angle pairs the rounded products sin cos, sin
-// sin and cos were within 0.5007 units in the last place, with the same root
-// mean square error (0.28866 units) as rounding the FP64 functions.
-constexpr float kSincosRange = 1000.f;
-__device__ __forceinline__ void sincos_two_float(float x, TwoFloat *sine, TwoFloat *cosine) {
-    const float k = rintf(__fmul_rn(x, 0x1.45f306p-1f));  // x / (pi/2)
-    constexpr float P1 = 0x1.921fb6p+0f, P2 = -0x1.777a5cp-25f, P3 = -0x1.ee59dap-50f;
-    const float p1 = __fmul_rn(k, P1), p1l = fmaf(k, P1, -p1);
-    const TwoFloat t1 = two_sum(__fsub_rn(x, p1), -p1l);  // x - p1 is exact
-    const float p2 = __fmul_rn(k, P2), p2l = fmaf(k, P2, -p2);
-    const TwoFloat t2 = two_sum(t1.hi, -p2);
-    const TwoFloat r =
-        quick_two_sum(t2.hi, __fsub_rn(__fadd_rn(t1.lo, t2.lo), fmaf(k, P3, p2l)));
-    const TwoFloat z = tf_mul(r, r);
-    const float y = z.hi;
-    // sin r = r + r z (-1/3! + z (1/5! + z (-1/7! + ... + z^3 / 13!)))
-    const float u =
-        __fmul_rn(y, fmaf(y, fmaf(y, fmaf(y, 1.f / 6227020800.f, -1.f / 39916800.f),
-                                  1.f / 362880.f), -1.f / 5040.f));
-    TwoFloat q = tf_add(TwoFloat{0x1.111112p-7f, -0x1.dddddep-32f}, TwoFloat{u, 0.f});
-    q = tf_add(TwoFloat{-0x1.555556p-3f, 0x1.555556p-28f}, tf_mul(z, q));
-    const TwoFloat s = tf_add(r, tf_mul(r, tf_mul(z, q)));
-    // cos r = 1 + z (-1/2! + z (1/4! + z (-1/6! + ... + z^3 / 12!)))
-    const float v =
-        __fmul_rn(y, fmaf(y, fmaf(y, fmaf(y, 1.f / 479001600.f, -1.f / 3628800.f),
-                                  1.f / 40320.f), -1.f / 720.f));
-    TwoFloat g = tf_add(TwoFloat{0x1.555556p-5f, -0x1.555556p-30f}, TwoFloat{v, 0.f});
-    g = tf_add(TwoFloat{-0.5f, 0.f}, tf_mul(z, g));
-    const TwoFloat c = tf_add(TwoFloat{1.f, 0.f}, tf_mul(z, g));
-    const int quadrant = (int)k & 3;
-    TwoFloat a = (quadrant & 1) ? c : s, b = (quadrant & 1) ? s : c;
-    if (quadrant & 2) a = TwoFloat{-a.hi, -a.lo};
-    if ((quadrant + 1) & 2) b = TwoFloat{-b.hi, -b.lo};
-    *sine = a;
-    *cosine = b;
-}
-
-// The nearest float to (A + a) / (X + x) for two-float numerator and
-// denominator (X > 0): q = A (1/X) is within two units of the answer; the
-// residual (A + a) - q (X + x), whose leading part A - q X FMA forms to 2^-47
-// of A, times 1/X is the remaining correction, and q plus it is rounded once
-// (Markstein's final step).  The correction carries about 23 bits, so the
-// result can differ from exact rounding only when the quotient lies within
-// about 2^-44 of its size of a rounding midpoint.
-__device__ __forceinline__ float div_two_float_rn(float A, float a, float X, float x) {
-    const float y = __frcp_rn(X);
-    const float q = __fmul_rn(A, y);
-    float r = fmaf(-q, X, A);
-    r = __fadd_rn(r, a);
-    r = fmaf(-q, x, r);
-    return fmaf(r, y, q);
 }
 
 // Four consecutive x points of a dense [nz][ny][nx] row (zero beyond nx):
@@ -273,30 +186,11 @@ __global__ void damp_scale_kernel(const float *__restrict__ damp, int n, double 
     if (i < n) dps[i] = damp ? (float)((double)damp[i] / dt) : 0.f;
 }
 
-// n = (sin theta cos phi, sin theta sin phi, cos theta) of one point.
-__device__ __forceinline__ void axis_of(float th, float ph, float *nx, float *ny, float *nz) {
-    if (fabsf(th) <= kSincosRange && fabsf(ph) <= kSincosRange) {
-        TwoFloat st, ct, sp, cp;
-        sincos_two_float(th, &st, &ct);
-        sincos_two_float(ph, &sp, &cp);
-        *nx = tf_mul(st, cp).hi;
-        *ny = tf_mul(st, sp).hi;
-        *nz = ct.hi;
-        return;
-    }
-    double st, ct, sp, cp;
-    sincos((double)th, &st, &ct);
-    sincos((double)ph, &sp, &cp);
-    *nx = (float)(st * cp);
-    *ny = (float)(st * sp);
-    *nz = (float)ct;
-}
-
-// a = 1 + 2 eps and s = sqrt(1 + 2 delta) rounded once (1 + 2 delta as an
-// exact two-float, the FP32 root corrected by its exact residual), and the
-// symmetry axis.  Two-float FP32 throughout: with FP64 trigonometry the
-// kernel was bound by the FP64 pipe, 7390 us at 384^3 (14 % of a 59-step so 4
-// run) against 647 us (36 bytes per point: 302 us at the copy bandwidth).
+// a = 1 + 2 eps, s = sqrt(1 + 2 delta) and the symmetry axis, each rounded
+// once.  Two-float FP32 decides all but about one point in 2^16 (the others
+// take the FP64 functions): with FP64 trigonometry throughout the kernel was
+// bound by the FP64 pipe, 7390 us at 384^3 (14 % of a 59-step so 4 run) against
+// 892 us (36 bytes per point: 302 us at the copy bandwidth).
 __global__ void __launch_bounds__(256)
     tti_coeff_kernel(const float *__restrict__ eps, const float *__restrict__ delta,
                      const float *__restrict__ theta, const float *__restrict__ phi,
@@ -323,11 +217,7 @@ __global__ void __launch_bounds__(256)
                 bad = DEV_ERR_MEDIUM;
             lmax = fmaxf(lmax, ev);
             av[e] = __fadd_rn(1.f, 2.f * ev);
-            const TwoFloat x = two_sum(1.f, 2.f * dv);
-            if (x.hi > 0.f) {
-                const float r = __fsqrt_rn(x.hi);
-                sv[e] = __fadd_rn(r, __fdividef(__fadd_rn(fmaf(-r, r, x.hi), x.lo), 2.f * r));
-            }
+            sv[e] = anellipticity_root(dv);
             axis_of(th, ph, &xv[e], &yv[e], &zv[e]);
         }
         const int64_t o = (int64_t)4 * n;

@@ -278,7 +278,8 @@ fd_status acoustic_adjoint(const fd_grid *grid, int so, double dt, int nt, int n
  * segment during the reverse sweep (the paper's time-subsampled save, Listing
  * fd-4, used for inversion).  0: the whole history of a batch of shots, which
  * needs no recomputation, when it takes at most an eighth of the device memory
- * and a quarter of what is free, otherwise every round(sqrt(nt-1)) steps.
+ * and a quarter of what is available (free, or held unused by the device's
+ * default memory pool), otherwise every round(sqrt(nt-1)) steps.
  *
  *   src_wav   [nshots][nt][nsrc]  source wavelets of the forward model.
  *   rec_resid [nshots][nt][nrec]  residual traces.
@@ -286,8 +287,11 @@ fd_status acoustic_adjoint(const fd_grid *grid, int so, double dt, int nt, int n
  *   Device memory: 11 + K + 2 + 2 ceil((nt-1)/K) wavefield volumes per shot
  *   of a batch (9 + K + 2 for one segment), K the checkpoint interval; 7 fewer
  *   where one shot would not fit otherwise.  Shots are stepped together in
- *   batches of up to 8, as many as fit in 80 % of the free device memory (at
+ *   batches of up to 8, as many as fit in 80 % of the available memory (at
  *   least one; the environment variable FDSWEEP_GRAD_BATCH=n caps the batch).
+ *   Workspaces return to the default memory pool, which keeps them for the
+ *   next call; a cudaMalloc or cudaMallocAsync of the process that needs the
+ *   memory gets it, and cudaMemPoolTrimTo gives it to other processes.
  *   Other arguments as for acoustic_forward.
  */
 fd_status acoustic_gradient(const fd_grid *grid, int so, double dt, int nt, int nshots,

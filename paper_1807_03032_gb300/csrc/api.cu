@@ -1443,8 +1443,8 @@ static fd_status acoustic_adjoint_impl(const fd_grid *grid, int so, double dt, i
  *
  * One segment (K = nt-1) needs no recomputation: two stencil sweeps instead of
  * three.  checkpoint_every = 0 takes it when the history of a batch fits in an
- * eighth of the device memory and in a quarter of what is free, and segments
- * of round(sqrt(nt-1)) otherwise.  At so 8: 4 shots at 128^3, 239 steps, 8 GB:
+ * eighth of the device memory and in a quarter of what is available, and segments
+ * of round(sqrt(nt-1)) otherwise (plan_gradient).  At so 8: 4 shots at 128^3, 239 steps, 8 GB:
  * 15.4 ms against 22.2; 2 shots at 64^3: 4.3 against 6.4.
  */
 static constexpr int kGradSteps = 8;  // 1 / 3 / 8 / 16: 19.7 / 16.9 / 16.1 / 15.7 ms
@@ -1454,7 +1454,11 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
                                         const float *src_xyz, const float *src_wav, int nrec,
                                         const float *rec_xyz, const float *rec_resid,
                                         int checkpoint_every, float *grad_m, float *src_grad,
-                                        const char *what, cudaStream_t caller) {
+                                        const char *what, cudaStream_t caller,
+                                        int most_shots = kGradMaxShots) {
+    // FDSWEEP_GRAD_BATCH=n caps the batch (to exercise several batches)
+    const char *cap = getenv("FDSWEEP_GRAD_BATCH");
+    if (cap && atoi(cap) > 0 && atoi(cap) < most_shots) most_shots = atoi(cap);
     FD_TRY(validate_common(grid, so, dt, nt, nshots, m, nsrc, src_xyz, src_wav, nrec, rec_xyz,
                            rec_resid));
     if (!grad_m) return set_error(FD_ERR_ARG, "%s: grad_m is null", what);
@@ -1466,51 +1470,19 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     const int ndamp = L.nx + L.ny + L.nz;
     const int nsteps = nt - 1;
     const int64_t vol = L.vol;
-    const int sqrt_k = (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
-    int K = checkpoint_every > 0 ? checkpoint_every : sqrt_k;
-    // shots of a batch
-    const int most = nshots < kGradMaxShots ? nshots : kGradMaxShots;
-    if (checkpoint_every == 0) {
-        size_t free_b = 0, total_b = 0;
-        FD_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-        const double history = (double)most * (nsteps + 2) * (double)vol * 4;
-        if (history <= (double)total_b / 8 && history <= ((double)free_b + pool_unused()) / 4)
-            K = nsteps;
-    }
-    if (K < 1) K = 1;
-    if (nsteps > 0 && K > nsteps) K = nsteps;
-    const int nseg = nsteps > 0 ? (nsteps + K - 1) / K : 0;
+    // Shots are processed in batches of B (one stencil launch per step for the
+    // whole batch); B is bounded by the device memory the per-shot buffers
+    // (forward pair, adjoint ring, the segment, the checkpoints) need.
+    size_t free_b = 0, total_b = 0;
+    FD_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+    const GradientPlan gp = plan_gradient(
+        nsteps, nshots, vol, checkpoint_every, most_shots, kGradSteps, (double)total_b,
+        (double)free_b + pool_unused(),
+        24.0 * (double)vol + 4.0 * nshots * (double)nt * ((double)nrec + nsrc));
+    const int K = gp.K, nseg = gp.nseg, G = gp.G, B = gp.B, nfwd = gp.nfwd, nck = gp.nck;
     CallStream cs;
     FD_TRY(cs.begin(caller));
     cudaStream_t s = cs.get();
-    // Shots are processed in batches of B (one stencil launch per step for the
-    // whole batch); B is bounded by the device memory the per-shot buffers
-    // (forward and adjoint pairs, the segment, the checkpoints) need.
-    // The adjoint's levels are a ring of G + 1, so that the imaging condition of
-    // G steps is one launch (see grad_steps_kernel).
-    const int nfwd = nseg > 1 ? 2 : 0, nck = nseg > 1 ? 2 * nseg : 0;
-    int G = K < kGradSteps ? (K > 1 ? K : 1) : kGradSteps;
-    int B = 1;
-    {
-        size_t free_b = 0, total_b = 0;
-        FD_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-        const int64_t fixed = (int64_t)(4 + 2) * vol * 4 +
-                              (int64_t)nshots * (int64_t)nt * (nrec + nsrc) * 4;
-        const int64_t budget = (int64_t)(0.8 * (double)free_b) - fixed;
-        // FDSWEEP_GRAD_BATCH=n caps the batch (to exercise several batches)
-        const char *cap = getenv("FDSWEEP_GRAD_BATCH");
-        auto batch = [&](int g) {
-            const int64_t per_shot = (int64_t)(nfwd + g + 1 + K + 2 + nck) * vol * 4;
-            const int64_t fit = per_shot > 0 ? budget / per_shot : 1;
-            const int b = (int)(fit > most ? most : fit);
-            return cap && atoi(cap) > 0 && atoi(cap) < b ? atoi(cap) : b;
-        };
-        B = batch(G);
-        if (B < 1) {  // the least: one shot, two adjoint levels, one step per launch
-            G = 1;
-            B = 1;
-        }
-    }
     Workspace ws;
     float *fwd, *adj, *seg, *ckpt, *grad, *bcoef, *dps;
     SparsePoint *src_tab, *rec_tab;
@@ -1536,13 +1508,17 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     sg.plan(ws, grad_m, dense);
     sq.plan(ws, src_grad, src_grad ? (size_t)nshots * nt * nsrc : 0);
     const fd_status got = ws.allocate(s);
-    if (got == FD_ERR_OOM && checkpoint_every == 0 && K > sqrt_k) {
-        // no memory for the history after all
+    const int sqrt_k = (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
+    const bool shorten = checkpoint_every == 0 && K > sqrt_k;
+    if (got == FD_ERR_OOM && (shorten || B > 1)) {
+        // not available after all (taken meanwhile): segments instead of the
+        // history, then smaller batches
         clear_error();
         FD_TRY(cs.finish());
         return acoustic_gradient_impl(grid, so, dt, nt, nshots, m, damp, nsrc, src_xyz, src_wav,
-                                      nrec, rec_xyz, rec_resid, sqrt_k, grad_m, src_grad, what,
-                                      caller);
+                                      nrec, rec_xyz, rec_resid, shorten ? sqrt_k : checkpoint_every,
+                                      grad_m, src_grad, what, caller,
+                                      shorten ? most_shots : B / 2);
     }
     FD_TRY(got);
     for (Staged *st : {&sm, &sdamp, &ssxyz, &swav, &srxyz, &sres}) FD_TRY(st->place(s));

@@ -140,4 +140,47 @@ inline PlanChoice choose_plan(const PlanEntry *e, int n, int forced, int nx, int
     return best;
 }
 
+// Checkpoint interval K, segments, imaging steps per launch G (the adjoint's
+// ring has G + 1 levels) and shots of a batch B of a gradient over nsteps steps
+// of nshots shots on fields of vol floats.
+//   available  bytes the call can allocate: what is free on the device and what
+//              the memory pool holds unused.  Both decisions below count the
+//              same bytes, so that a call's batches (and with them the order of
+//              its sums) do not depend on how far earlier calls grew the pool.
+//   fixed      bytes of everything but the per-shot levels.
+//   most_shots, most_steps  upper limits of B and G.
+// checkpoint_every = 0 keeps the whole history of a batch (K = nsteps, no
+// recomputation) where it takes at most an eighth of the device memory and a
+// quarter of what is available, and round(sqrt(nsteps)) steps otherwise.
+struct GradientPlan {
+    int K, nseg, G, B;
+    int nfwd, nck;  // forward levels and checkpoint levels per shot
+};
+
+inline GradientPlan plan_gradient(int nsteps, int nshots, int64_t vol, int checkpoint_every,
+                                  int most_shots, int most_steps, double total,
+                                  double available, double fixed) {
+    GradientPlan p;
+    const double level = (double)vol * 4.0;
+    const int most = nshots < most_shots ? nshots : most_shots;
+    p.K = checkpoint_every > 0 ? checkpoint_every
+                               : (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
+    const double history = (double)most * (nsteps + 2) * level;
+    if (checkpoint_every == 0 && history <= total / 8 && history <= available / 4) p.K = nsteps;
+    if (p.K < 1) p.K = 1;
+    if (nsteps > 0 && p.K > nsteps) p.K = nsteps;
+    p.nseg = nsteps > 0 ? (nsteps - 1) / p.K + 1 : 0;
+    p.nfwd = p.nseg > 1 ? 2 : 0;
+    p.nck = p.nseg > 1 ? 2 * p.nseg : 0;
+    p.G = p.K < most_steps ? p.K : most_steps;
+    const double per_shot = ((double)p.nfwd + p.G + 1 + p.K + 2 + p.nck) * level;
+    const double fit = (0.8 * available - fixed) / per_shot;
+    p.B = fit >= most ? most : (int)fit;
+    if (p.B < 1) {  // the least: one shot, two adjoint levels, one step per launch
+        p.G = 1;
+        p.B = 1;
+    }
+    return p;
+}
+
 }  // namespace fdsweep

@@ -1629,8 +1629,10 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
                 FD_CUDA_TRY(cudaMemcpy2DAsync(seg, (size_t)(K + 2) * vb,
                                               ckpt + (size_t)c * 2 * nb * vol, 2 * vb, 2 * vb, nb,
                                               cudaMemcpyDeviceToDevice, s));
-            else
-                FD_CUDA_TRY(cudaMemset2DAsync(seg, (size_t)(K + 2) * vb, 0, 2 * vb, nb, s));
+            else  // shot by shot: a history is longer than the largest pitch (2 GiB)
+                for (int b = 0; b < nb; ++b)
+                    FD_CUDA_TRY(
+                        cudaMemsetAsync(seg + (int64_t)b * (K + 2) * vol, 0, 2 * vb, s));
             for (int t = t0 + 1; t <= kmax; ++t) {
                 AcousticStepArgs ai = as;
                 ai.lps = K + 2;

@@ -74,6 +74,7 @@ struct AcCfg {
     static constexpr size_t SMEM = (size_t)NSL * STAGE * 4 + NSL * 16 + 16 + 128;
     static_assert(PW <= 256 && PH <= 256 && BX <= 256 && BY <= 256, "TMA box dimension limit");
     static_assert(INT % 32 == 0 && CONSUMERS % 32 == 0, "tile shape");
+    static_assert(WARPS <= kMaxRingWarps, "room behind the abort flag");
 };
 
 // Source injection by the CTA that wrote a source's corners, after its
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
             mbar_init(&empty[s], C::WARPS);
         }
         fence_mbar_init();
-        *abort_flag = 0;
+        init_ring_abort(abort_flag);
     }
     for (int z = za + tid; z < zb; z += C::THREADS) sdz[z - za] = a.dpz[z];
     __syncthreads();
@@ -291,8 +292,7 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
     for (int j = 0; j < nplanes; ++j, pos.next()) {
         const int slot = pos.slot(j);
         if (*abort_flag || !mbar_wait_bounded(&full[slot], pos.phase(j), wait_ns)) {
-            *abort_flag = 1;
-            atomicOr(a.err, DEV_ERR_TIMEOUT);
+            leave_ring(abort_flag, j, a.err);
             break;
         }
         const float *H = smem + slot * C::STAGE;

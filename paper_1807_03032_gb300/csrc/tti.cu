@@ -79,6 +79,7 @@ struct TtiCfg {
     static constexpr size_t SMEM2 = (size_t)NSL * STAGE2 * 4 + NSL * 16 + 16 + 128;
     static_assert(PW <= 256 && PH <= 256, "TMA box dimension limit");
     static_assert(CONSUMERS % 32 == 0, "whole consumer warps");
+    static_assert(WARPS <= kMaxRingWarps, "room behind the abort flag");
 };
 
 struct Ring {
@@ -101,7 +102,7 @@ __device__ __forceinline__ Ring ring_init(unsigned char *raw, size_t stage_float
             mbar_init(&r.empty[s], WARPS);
         }
         fence_mbar_init();
-        *r.abort_flag = 0;
+        init_ring_abort(r.abort_flag);
     }
     return r;
 }
@@ -201,8 +202,7 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
         for (int j = 0; j < nplanes; ++j, pos.next()) {
             const int slot = pos.slot(j);
             if (*ring.abort_flag || !mbar_wait_bounded(&ring.full[slot], pos.phase(j))) {
-                *ring.abort_flag = 1;
-                atomicOr(a.err, DEV_ERR_TIMEOUT);
+                leave_ring(ring.abort_flag, j, a.err);
                 break;
             }
             const float *st = ring.smem + slot * C::STAGE1;
@@ -333,8 +333,7 @@ __global__ void __launch_bounds__(TX *TY + 32, MINB)
             const int zs = za - 2 * R + j;
             const float dz = j >= 2 * R ? __ldg(a.dpz + zs) : 0.f;
             if (*ring.abort_flag || !mbar_wait_bounded(&ring.full[slot], pos.phase(j))) {
-                *ring.abort_flag = 1;
-                atomicOr(a.err, DEV_ERR_TIMEOUT);
+                leave_ring(ring.abort_flag, j, a.err);
                 break;
             }
             const float *st = ring.smem + slot * C::STAGE2;

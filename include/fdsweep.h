@@ -491,7 +491,9 @@ int fd_num_tti_configs(int so);
  * Tile configuration override for the acoustic stencil kernel (for tuning
  * sweeps): index into the compiled configuration table for the given space
  * order, or -1 for the built-in choice (the configuration with the smallest
- * estimated time for the grid).  Returns FD_ERR_ARG if out of range.
+ * estimated time for the grid).  With a 3-D damping field the index counts in
+ * that variant's table (built-in choice beyond its end).  Returns FD_ERR_ARG
+ * if out of range.
  */
 fd_status fd_set_acoustic_config(int so, int config);
 int fd_num_acoustic_configs(int so);

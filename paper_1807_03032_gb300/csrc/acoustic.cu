@@ -712,7 +712,7 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
     const ConfigEntry *tab =
         damp_field ? config_table_df(radius, &n) : config_table(radius, &n);
     if (!tab) return set_error(FD_ERR_SO, "no acoustic kernel for radius %d", radius);
-    if (config >= n || damp_field) config = -1;
+    if (config >= n) config = -1;
     int dev = 0, nsm = 0, max_smem = 0;
     FD_CUDA_TRY(cudaGetDevice(&dev));
     FD_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -144,7 +144,7 @@ int acoustic_num_configs(int radius);
 // covers `nshots` shots; the tensor maps cover `map_shots` shots (default:
 // nshots) for callers that map launch shots to slots (slot_map).
 // damp_field: the damping is a 3-D field; bcoef then holds two fields, b and
-// zeta = damp b / dt ([2][vol]), and the default configuration is used.
+// zeta = damp b / dt ([2][vol]), and `config` counts in its own table.
 fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots, int lps,
                         float *wave, const float *bcoef, AcousticPlan *plan, int map_shots = 0,
                         bool damp_field = false);

@@ -476,13 +476,13 @@ fd_status fd_set_time_tiling(int so, int mode);
 int fd_num_time_tiling_configs(int so);
 
 /*
- * Launch configuration override of the two TTI passes (prefetch depths and
- * loop unroll; for tuning sweeps): index into the compiled table for the
- * given space order (0 .. fd_num_tti_configs(so) - 1), or -1 for the
- * built-in choice.  Applies to centred derivatives of the two-pass scheme
- * (the staggered reading always uses the built-in choice); for the fused
- * scheme configuration 1 selects 64 x 8 tiles instead of 64 x 16 (other
- * values: the built-in choice).  Process-wide; FD_ERR_ARG if out of range.
+ * Launch configuration override of the two TTI passes (tiles, ring depths and
+ * one-block kernels; for tuning sweeps): index into the compiled table for the
+ * given space order (0 .. fd_num_tti_configs(so) - 1; a pass with a shorter
+ * table takes its last entry), or -1 for the built-in choice, for centred and
+ * staggered derivatives of the two-pass scheme.  For the fused scheme at
+ * so <= 4 configuration 1 selects 64 x 16 tiles (the built-in choice), 0
+ * selects 64 x 8.  Process-wide; FD_ERR_ARG if out of range.
  */
 fd_status fd_set_tti_config(int so, int config);
 int fd_num_tti_configs(int so);

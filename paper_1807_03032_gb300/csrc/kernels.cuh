@@ -314,7 +314,6 @@ struct TtiPlan {
     int radius = 0;
     int stag = 0;    // 0: centred first derivatives, 1: staggered (D+ inner, D- outer)
     int scheme = kTtiTwoPass;
-    int config = 0;  // tile choice of the fused scheme
     TtiPassPlan p1, p2;                        // p1 alone: fused and recompute schemes
     CUtensorMap map_wint, map_whalo;           // p, r of a level: interior, x+y halo boxes
     CUtensorMap map_wlev;                      // p, r at both levels: interior box
@@ -335,7 +334,7 @@ int tti_num_configs(int radius);
 // memory; radii 1, 2 and 4.
 bool tti_fused_supported(int radius);
 fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, float *wave,
-                         const float *coef, TtiPlan *plan, int config = 0);
+                         const float *coef, TtiPlan *plan, int config = -1);
 fd_status tti_fused_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
                            const AcousticInject &inj, const ReceiveArgs &receive);
 // inject, receive: done by the step's own kernels (not with the recompute

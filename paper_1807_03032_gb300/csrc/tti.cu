@@ -878,7 +878,8 @@ fd_status plan_pass(int pass, int radius, int stag, int config, const WaveLayout
 
 int tti_num_configs(int radius) {
     const PassTable a = pass_table(1, radius, 0), b = pass_table(2, radius, 0);
-    return a.n > b.n ? a.n : b.n;
+    const int n = a.n > b.n ? a.n : b.n;
+    return a.e && radius <= 2 && n < 2 ? 2 : n;  // the fused scheme has two tiles
 }
 
 fd_status tti_plan(int radius, const WaveLayout &L, int nshots, float *wave, float *tmp,

@@ -360,12 +360,12 @@ FusedInfo fused_info_t(int stag, float launch, float lat, float thr, float warm)
                      launch,  lat,    thr,   warm};
 }
 
-// Configuration 0: 64 x 16 tiles, one CTA per SM (R <= 2; 1.38x the tile's
-// gradients); configuration 1: 64 x 8 tiles, two CTAs (1.63x).  so 4, us per
+// Built-in and configuration 1: 64 x 16 tiles, one CTA per SM (R <= 2; 1.38x the
+// tile's gradients); configuration 0: 64 x 8 tiles, two CTAs (1.63x).  so 4, us per
 // step: 96^3 23.0 and 26.7, 256^3 204 and 248, 384^3 598 and 711, 512^3 1430
 // and 1664.  The costs are fitted to 13 problems.
 bool fused_info(int radius, int stag, int config, FusedInfo *out) {
-    const bool small = config == 1;
+    const bool small = config == 0;
     switch (radius) {
         case 1:
             *out = small ? fused_info_t<1, 8, 1, 2, 2>(stag, 4.1f, 1.05f, 0.60f, 0.59f)
@@ -386,7 +386,7 @@ bool fused_info(int radius, int stag, int config, FusedInfo *out) {
 
 bool tti_fused_supported(int radius) {
     FusedInfo in;
-    return fused_info(radius, 0, 0, &in);
+    return fused_info(radius, 0, -1, &in);
 }
 
 // Chunk count of a fused step and its estimated time.
@@ -408,7 +408,7 @@ static fd_status fused_choice(const FusedInfo &in, int radius, const WaveLayout 
 
 fd_status tti_fused_time(int radius, int stag, const WaveLayout &L, int nshots, double *us) {
     FusedInfo in;
-    if (!fused_info(radius, stag, 0, &in))
+    if (!fused_info(radius, stag, -1, &in))
         return set_error(FD_ERR_ARG, "the fused TTI scheme covers space orders up to 8");
     PlanChoice c;
     FD_TRY(fused_choice(in, radius, L, nshots, &c));
@@ -428,7 +428,6 @@ fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, 
     plan->radius = radius;
     plan->stag = stag ? 1 : 0;
     plan->scheme = kTtiFused;
-    plan->config = config == 1 ? 1 : 0;
     plan->p1.fn = in.fn;
     plan->p1.grid = dim3(ntx, nty, nshots * c.nzc);
     plan->p1.block = dim3(in.threads, 1, 1);

@@ -287,8 +287,8 @@ fd_status acoustic_adjoint(const fd_grid *grid, int so, double dt, int nt, int n
  *   Device memory: 11 + K + 2 + 2 ceil((nt-1)/K) wavefield volumes per shot
  *   of a batch (9 + K + 2 for one segment), K the checkpoint interval; 7 fewer
  *   where one shot would not fit otherwise.  Shots are stepped together in
- *   batches of up to 8, as many as fit in 80 % of the available memory (at
- *   least one; the environment variable FDSWEEP_GRAD_BATCH=n caps the batch).
+ *   batches of up to 8, or as many as have 16 million points together, as far
+ *   as they fit in 80 % of the available memory (at least one; the environment variable FDSWEEP_GRAD_BATCH=n caps the batch).
  *   Workspaces return to the default memory pool, which keeps them for the
  *   next call; a cudaMalloc or cudaMallocAsync of the process that needs the
  *   memory gets it, and cudaMemPoolTrimTo gives it to other processes.

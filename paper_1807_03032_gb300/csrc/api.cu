@@ -1455,10 +1455,10 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
                                         const float *rec_xyz, const float *rec_resid,
                                         int checkpoint_every, float *grad_m, float *src_grad,
                                         const char *what, cudaStream_t caller,
-                                        int most_shots = kGradMaxShots) {
+                                        int cap = INT_MAX) {
     // FDSWEEP_GRAD_BATCH=n caps the batch (to exercise several batches)
-    const char *cap = getenv("FDSWEEP_GRAD_BATCH");
-    if (cap && atoi(cap) > 0 && atoi(cap) < most_shots) most_shots = atoi(cap);
+    const char *most = getenv("FDSWEEP_GRAD_BATCH");
+    if (most && atoi(most) > 0 && atoi(most) < cap) cap = atoi(most);
     FD_TRY(validate_common(grid, so, dt, nt, nshots, m, nsrc, src_xyz, src_wav, nrec, rec_xyz,
                            rec_resid));
     if (!grad_m) return set_error(FD_ERR_ARG, "%s: grad_m is null", what);
@@ -1476,7 +1476,7 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
     size_t free_b = 0, total_b = 0;
     FD_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     const GradientPlan gp = plan_gradient(
-        nsteps, nshots, vol, checkpoint_every, most_shots, kGradSteps, (double)total_b,
+        nsteps, nshots, vol, checkpoint_every, cap, kGradSteps, (double)total_b,
         (double)free_b + pool_unused(),
         24.0 * (double)vol + 4.0 * nshots * (double)nt * ((double)nrec + nsrc));
     const int K = gp.K, nseg = gp.nseg, G = gp.G, B = gp.B, nfwd = gp.nfwd, nck = gp.nck;
@@ -1518,7 +1518,7 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
         return acoustic_gradient_impl(grid, so, dt, nt, nshots, m, damp, nsrc, src_xyz, src_wav,
                                       nrec, rec_xyz, rec_resid, shorten ? sqrt_k : checkpoint_every,
                                       grad_m, src_grad, what, caller,
-                                      shorten ? most_shots : B / 2);
+                                      shorten ? cap : B / 2);
     }
     FD_TRY(got);
     for (Staged *st : {&sm, &sdamp, &ssxyz, &swav, &srxyz, &sres}) FD_TRY(st->place(s));
@@ -1652,16 +1652,18 @@ static fd_status acoustic_gradient_impl(const fd_grid *grid, int so, double dt, 
                 if (done - k + 1 == G || k == t0 + 1) {
                     GradArgs ga;
                     ga.grad = grad;
-                    ga.w = adj;
                     ga.w_stride = (G + 1) * vol;
                     ga.w_levels = G + 1;
                     ga.w_level = (acur + G + 1 - (done - k)) % (G + 1);
-                    ga.u = seg + (size_t)(done - t0 + 1) * vol;
                     ga.u_stride = (int64_t)(K + 2) * vol;
                     ga.vol = vol;
-                    ga.nb = nb;
                     ga.steps = done - k + 1;
-                    FD_TRY(grad_accumulate(ga, s));
+                    for (int b = 0; b < nb; b += kGradShots) {
+                        ga.w = adj + b * ga.w_stride;
+                        ga.u = seg + b * ga.u_stride + (int64_t)(done - t0 + 1) * vol;
+                        ga.nb = nb - b < kGradShots ? nb - b : kGradShots;
+                        FD_TRY(grad_accumulate(ga, s));
+                    }
                     done = k - 1;
                 }
                 // dq^{k-1} = S w^k, before w^{k-1} is formed

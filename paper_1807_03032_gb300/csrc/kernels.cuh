@@ -11,6 +11,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "plan.h"
 
 namespace fdsweep {
 
@@ -223,14 +224,13 @@ fd_status bump_counter(int *counter, int by, cudaStream_t stream);
 // (scaled by -1/dt^2 once at the end).  Shot b's adjoint levels are a ring of
 // w_levels fields of vol floats from w + b w_stride, step j in level
 // (w_level + j) mod w_levels; u + b u_stride is its level u^k and the levels
-// below it are the vol, 2 vol, .. floats before.  nb <= kGradMaxShots.
+// below it are the vol, 2 vol, .. floats before.  nb <= kGradShots.
 struct GradArgs {
     float *grad;
     const float *w, *u;
     int64_t w_stride, u_stride, vol;
     int w_level, w_levels, nb, steps;
 };
-constexpr int kGradMaxShots = 8;
 fd_status grad_accumulate(const GradArgs &a, cudaStream_t stream);
 fd_status scale_field(float *f, float s, int64_t n, cudaStream_t stream);
 

@@ -148,25 +148,45 @@ inline PlanChoice choose_plan(const PlanEntry *e, int n, int forced, int nx, int
 //              same bytes, so that a call's batches (and with them the order of
 //              its sums) do not depend on how far earlier calls grew the pool.
 //   fixed      bytes of everything but the per-shot levels.
-//   most_shots, most_steps  upper limits of B and G.
+//   cap, most_steps  upper limits of B and G.
+// A batch is kGradShots shots, or as many as have kGradBatchPoints points.
 // checkpoint_every = 0 keeps the whole history of a batch (K = nsteps, no
 // recomputation) where it takes at most an eighth of the device memory and a
-// quarter of what is available, and round(sqrt(nsteps)) steps otherwise.
+// quarter of what is available (smaller batches where only kGradShots shots'
+// does), and round(sqrt(nsteps)) steps otherwise.
+// The imaging condition takes kGradShots shots per launch, and so does a batch
+// of large grids; where eight shots leave the device idle a batch is as many as
+// have kGradBatchPoints points.  59 steps, segments of 8, ms with batches of 8 /
+// of 4e6 / 8e6 / 1.6e7 points: 64 shots of 40^3 so 16 18.6 / 9.6 / 8.6 / 8.6,
+// 64 of 48^3 so 4 14.0 / 8.4 / 7.5 / 7.5, 32 of 64^3 9.2 / 7.2 / 7.0 / 6.2, 24
+// of 80^3 so 8 14.7 / 14.5 / 13.8 / 12.8; from 96^3 on the same within 1 %.
+constexpr int kGradShots = 8;
+constexpr double kGradBatchPoints = 1.6e7;
+
 struct GradientPlan {
     int K, nseg, G, B;
     int nfwd, nck;  // forward levels and checkpoint levels per shot
 };
 
 inline GradientPlan plan_gradient(int nsteps, int nshots, int64_t vol, int checkpoint_every,
-                                  int most_shots, int most_steps, double total,
-                                  double available, double fixed) {
+                                  int cap, int most_steps, double total, double available,
+                                  double fixed) {
     GradientPlan p;
     const double level = (double)vol * 4.0;
-    const int most = nshots < most_shots ? nshots : most_shots;
+    double wide = ceil(kGradBatchPoints / (double)vol);
+    if (wide > kMaxGridYZ / 4) wide = kMaxGridYZ / 4;  // shots lie along the grid's z
+    int most = wide > kGradShots ? (wide < nshots ? (int)wide : nshots) : kGradShots;
+    if (most > nshots) most = nshots;
+    if (most > cap) most = cap;
     p.K = checkpoint_every > 0 ? checkpoint_every
                                : (int)lround(sqrt((double)(nsteps > 1 ? nsteps : 1)));
-    const double history = (double)most * (nsteps + 2) * level;
-    if (checkpoint_every == 0 && history <= total / 8 && history <= available / 4) p.K = nsteps;
+    const double history = (nsteps + 2) * level;  // of a shot
+    const double keep = total / 8 < available / 4 ? total / 8 : available / 4;
+    if (checkpoint_every == 0) {
+        if (most > kGradShots && most * history > keep && kGradShots * history <= keep)
+            most = kGradShots;
+        if (most * history <= keep) p.K = nsteps;
+    }
     if (p.K < 1) p.K = 1;
     if (nsteps > 0 && p.K > nsteps) p.K = nsteps;
     p.nseg = nsteps > 0 ? (nsteps - 1) / p.K + 1 : 0;

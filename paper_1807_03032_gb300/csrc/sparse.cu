@@ -191,12 +191,12 @@ fd_status bump_counter(int *counter, int by, cudaStream_t stream) {
 fd_status grad_accumulate(const GradArgs &a, cudaStream_t stream) {
     if (a.vol % 4 || a.w_stride % 4 || a.u_stride % 4)
         return set_error(FD_ERR_ARG, "grad_accumulate: sizes not multiples of 4");
-    if (a.nb > kGradMaxShots)
+    if (a.nb > kGradShots)
         return set_error(FD_ERR_ARG, "grad_accumulate: %d shots in a batch", a.nb);
     if (a.nb <= 4)
         grad_steps_kernel<4, 4><<<stream_grid(a.vol / 4, 256), 256, 0, stream>>>(a);
     else
-        grad_steps_kernel<2, kGradMaxShots><<<stream_grid(a.vol / 2, 256), 256, 0, stream>>>(a);
+        grad_steps_kernel<2, kGradShots><<<stream_grid(a.vol / 2, 256), 256, 0, stream>>>(a);
     FD_CUDA_TRY(cudaGetLastError());
     note_launch(stream);
     return FD_OK;

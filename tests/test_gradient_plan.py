@@ -20,21 +20,38 @@ WRAP = """
 extern "C" void plan(int nsteps, int nshots, long long vol, int every, double total,
                      double available, double fixed, int *out) {
     const fdsweep::GradientPlan p =
-        fdsweep::plan_gradient(nsteps, nshots, vol, every, 8, 8, total, available, fixed);
+        fdsweep::plan_gradient(nsteps, nshots, vol, every, 1 << 30, 8, total, available, fixed);
     const int v[] = {p.K, p.nseg, p.G, p.B, p.nfwd, p.nck};
     for (int i = 0; i < 6; ++i) out[i] = v[i];
 }
 """
 
 
-def test_plan_fits_the_memory_it_counts(tmp_path):
-    src, lib = str(tmp_path / "plan.cpp"), str(tmp_path / "plan.so")
+@pytest.fixture(scope="module")
+def fn(tmp_path_factory):
+    d = tmp_path_factory.mktemp("gradient_plan")
+    src, lib = str(d / "plan.cpp"), str(d / "plan.so")
     with open(src, "w") as f:
         f.write(WRAP)
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, src, "-o", lib],
                    check=True)
-    fn = ctypes.CDLL(lib).plan
-    D = ctypes.c_double
+    return ctypes.CDLL(lib).plan
+
+
+D = ctypes.c_double
+
+
+@pytest.mark.parametrize("n,nshots,batch", [(32, 64, 64), (32, 128, 128), (40, 128, 128),
+                                            (64, 32, 32), (64, 100, 62), (128, 16, 8),
+                                            (256, 16, 8), (64, 3, 3), (4, 100000, 16383)])
+@pytest.mark.parametrize("every", [0, 8])
+def test_small_grids_are_batched_by_their_points(fn, n, nshots, batch, every):
+    out = (ctypes.c_int * 6)()
+    fn(59, nshots, ctypes.c_longlong(n ** 3), every, D(2.97e11), D(2.9e11), D(24.0 * n ** 3), out)
+    assert out[3] == batch
+
+
+def test_plan_fits_the_memory_it_counts(fn):
     rng = random.Random(2)
     total = 2.97e11
     for _ in range(20000):
@@ -45,13 +62,14 @@ def test_plan_fits_the_memory_it_counts(tmp_path):
         out = (ctypes.c_int * 6)()
         fn(nsteps, nshots, ctypes.c_longlong(vol), every, D(total), D(available), D(fixed), out)
         K, nseg, G, B, nfwd, nck = out
-        assert 1 <= B <= min(nshots, 8) and 1 <= G <= min(K, 8)
+        assert 1 <= B <= nshots and 1 <= G <= min(K, 8)
+        assert B <= 8 or (B - 1) * vol < 1.6e7  # more only of grids that do not fill the device
         assert nseg * K >= nsteps > (nseg - 1) * K if nsteps else nseg == 0
         levels = nfwd + G + 1 + K + 2 + nck
         if B > 1 or G > 1:
             assert B * levels * vol * 4.0 + fixed <= 0.8 * available
         if every == 0 and nseg == 1 and nsteps > 2:  # the whole history is kept
-            assert min(nshots, 8) * (nsteps + 2) * vol * 4.0 <= min(total / 8, available / 4)
+            assert B * (nsteps + 2) * vol * 4.0 <= min(total / 8, available / 4)
         if every:
             assert K == min(every, max(nsteps, 1)) or nsteps == 0
         if B == 1 and G == 1:  # no more than two pairs, the segment and the checkpoints

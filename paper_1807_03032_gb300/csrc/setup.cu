@@ -190,7 +190,7 @@ __global__ void damp_scale_kernel(const float *__restrict__ damp, int n, double 
 // once.  Two-float FP32 decides all but about one point in 2^16 (the others
 // take the FP64 functions): with FP64 trigonometry throughout the kernel was
 // bound by the FP64 pipe, 7390 us at 384^3 (14 % of a 59-step so 4 run) against
-// 892 us (36 bytes per point: 302 us at the copy bandwidth).
+// 920 us (36 bytes per point: 302 us at the copy bandwidth).
 __global__ void __launch_bounds__(256)
     tti_coeff_kernel(const float *__restrict__ eps, const float *__restrict__ delta,
                      const float *__restrict__ theta, const float *__restrict__ phi,

@@ -60,8 +60,10 @@ FD_TF bool rounds_surely(TwoFloat v, float *f) {
 // their size: x - k pi/2 with pi/2 as three floats and exact products (Cody
 // and Waite's reduction), then the Taylor series on [-pi/4, pi/4], the last
 // terms in plain FP32 and the leading ones in two-float arithmetic.  False
-// where the reduction cancels too many digits for that (x within 2^-20 of a
-// multiple of pi/2 other than 0).
+// where the reduction cancels too many digits for that: its error is at most
+// 2^-63, and 2^-70 within one turn of 0, where a remainder below 2^-20 leaves
+// nothing to round in the first sums (the nearest floats to 90, 180, 270 and 360
+// degrees, axes that models do use, are 2^-24, 2^-23, 2^-26 and 2^-22 from them).
 constexpr float kSincosRange = 1000.f;
 FD_TF bool sincos_two_float(float x, TwoFloat *sine, TwoFloat *cosine) {
     const float k = rintf(__fmul_rn(x, 0x1.45f306p-1f));  // x / (pi/2)
@@ -96,7 +98,7 @@ FD_TF bool sincos_two_float(float x, TwoFloat *sine, TwoFloat *cosine) {
     if ((quadrant + 1) & 2) b = TwoFloat{-b.hi, -b.lo};
     *sine = a;
     *cosine = b;
-    return fabsf(r.hi) >= 0x1p-20f || k == 0.f;
+    return fabsf(r.hi) >= 0x1p-20f || k == 0.f || (fabsf(k) <= 4.f && fabsf(r.hi) >= 0x1p-27f);
 }
 
 // n = (sin theta cos phi, sin theta sin phi, cos theta) of one point: the FP64

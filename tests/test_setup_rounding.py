@@ -113,6 +113,20 @@ def test_few_angles_need_64_bits(lib):
     assert lib.undecided(P(th), P(ph), ctypes.c_long(th.size)) <= 3 * 2.0 ** -17 * th.size * 1.5
 
 
+def test_right_angles_do_not_need_64_bits(lib):
+    """A horizontal axis (theta = 90 degrees) or one along a grid axis is a whole model's value."""
+    for th in np.float32([0.0, np.pi / 2, np.pi, -np.pi / 2]):
+        for ph in np.float32([0.0, np.pi / 2, np.pi, 1.5 * np.pi, 2 * np.pi, -np.pi / 2]):
+            a, b = np.full(4, th, np.float32), np.full(4, ph, np.float32)
+            assert lib.undecided(P(a), P(b), ctypes.c_long(4)) == 0, (th, ph)
+    k = (np.arange(-4, 5) * np.pi / 2).astype(np.float32)
+    near = np.concatenate([k] + [k + s * np.spacing(np.abs(k)) for s in range(-40, 41)])
+    n, exact = axis(lib, *(v.ravel() for v in np.meshgrid(near, near)))
+    for c in range(3):
+        normal = np.abs(exact[c]) >= 2.0 ** -126
+        assert_rounded(n[normal, c], exact[c][normal], 2.0 ** -50)
+
+
 def test_root_is_the_64_bit_value_rounded_once(lib):
     rng = np.random.default_rng(9)
     d = np.concatenate([rng.uniform(-0.5, 0.5, 2000000), rng.uniform(-0.5, -0.49, 200000),

@@ -87,8 +87,10 @@ def kernel_source_hash():
     version it was measured on."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1807_03032_gb300", "csrc")
-    for f in ("acoustic.cu", "acoustic2.cu", "f32x2.cuh", "common.cuh"):
-        h.update(_code_lines(open(os.path.join(csrc, f), "rb").read()))
+    for f in ("acoustic.cu", "acoustic2.cu", "f32x2.cuh", "common.cuh", "ring.cuh", "receive.cuh",
+              "plan.h"):
+        if os.path.exists(os.path.join(csrc, f)):
+            h.update(_code_lines(open(os.path.join(csrc, f), "rb").read()))
     k = open(os.path.join(csrc, "kernels.cuh"), "rb").read()
     a = k.find(b"// ---------------------------------------------------------------- acoustic K1")
     b = k.find(b"// ---------------------------------------------------------------- sparse K3/K4")
@@ -678,8 +680,8 @@ def run_fwi(args, fd, dev, stream):
             "gradient_s": round(grad_ms * 1e-3, 3), "forward_s": round(fwd_ms * 1e-3, 3),
             "objective": float(0.5 * (resid.double() ** 2).sum()), "finite": ok,
             "note": "gradient GPts/s counts forward-model grid-point updates (nt-1 per shot); "
-                    "the gradient performs a forward with checkpoints, a recomputation and "
-                    "an adjoint sweep",
+                    "with the explicit checkpoint interval of this line the gradient performs "
+                    "a forward with checkpoints, a recomputation and an adjoint sweep",
             "parity": "tests/test_gpu_fwi_scale.py: the same recipe at 96^3, 4 shots in 2 "
                       "batches, nt 400, checkpoint every 20: GPU gradient vs the FP64 oracle "
                       "gradient within 1e-4 (relative L2 and max-abs), and Taylor slopes 1 and 2 "

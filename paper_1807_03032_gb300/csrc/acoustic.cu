@@ -613,7 +613,7 @@ ConfigEntry spare(ConfigEntry e) {
 
 // The configurations of each radius (template arguments R, TX, TY, VY, D, U,
 // minimum CTAs per SM, EDGE); acoustic_plan takes the one with the smallest
-// estimated time for the grid.  Ring sizes are powers of two (D = 3), so that
+// estimated time for the grid (plan.h).  Ring sizes are powers of two (D = 3), so that
 // the unrolled plane loop has constant stage addresses.
 //  * Small tiles fill the machine on small grids (64 x 4 at so 16: 128^3 17.8
 //    us per step, 64 x 8 19.4).
@@ -621,9 +621,9 @@ ConfigEntry spare(ConfigEntry e) {
 //    neighbours, which bound the wide stencils: R y-rows above and below cost
 //    R + 1 reads per point instead of 2R.  At so 12 and 16 a few large CTAs
 //    pay best at large sizes: 64 x 28 tiles, one CTA of 224 + 32 threads with
-//    255 registers per SM, run 512^3 so 16 in 369 us (442 with 64 x 8, 472
-//    before the producer warp); 64 x 44 at so 12 in 340 us (387 and 402).
-//  * so 4 and 8 are at the HBM limit at 512^3 (306 and 318 us for 2.15 GB).
+//    255 registers per SM, run 512^3 so 16 in 378 us (442 with 64 x 8, 472
+//    before the producer warp); 64 x 44 at so 12 in 331 us (387 and 402).
+//  * so 4 and 8 are at the HBM limit at 512^3 (310 and 329 us for 2.15 GB).
 //  * EDGE (see the kernel) halves what the 2R extra planes of a chunk cost, so
 //    that wide stencils can be cut into more chunks: so 16 4 x 128^3 41.4 ->
 //    37.5 us per step, 160^3 25.9 -> 22.4, 64^3 11.4 -> 9.4; so 12 4 x 128^3
@@ -663,8 +663,9 @@ const ConfigEntry *config_table(int radius, int *count) {
 }
 
 // 3-D damping field: a fourth interior tile per stage (64 x 44 tiles at so 12
-// would need a shorter ring and measured slower than 64 x 16 up to 384^3);
-// the costs fitted to 10 problems.
+// would need a shorter ring and measured slower than 64 x 16 up to 384^3); the
+// costs of the marching entries fitted to 10 problems, the one-block entries
+// with the per-axis kernels' costs.
 const ConfigEntry *config_table_df(int radius, int *count) {
     static const ConfigEntry r1[] = {
         FD_AC_ENTRY_DF(1, 16, 16, 1, 3, 4, 0, 0, 2.7f, 0.28f, 0.38f, 0.5f)};
@@ -741,9 +742,11 @@ fd_status acoustic_plan(int radius, int config, const WaveLayout &L, int nshots,
     plan->block = dim3(e.threads, 1, 1);
     const int ntx = (L.nx + e.bx - 1) / e.bx;
     const int nty = (L.ny + e.by - 1) / e.by;
-    plan->grid = dim3(ntx, nty, nshots * best.nzc);
+    int nzc = 1;
+    if (best.zchunk < L.nz) nzc = best.nzc;
+    plan->grid = dim3(ntx, nty, nshots * nzc);
     plan->zchunk = best.zchunk;
-    plan->nzc = best.nzc;
+    plan->nzc = nzc;
     plan->smem = e.smem + (size_t)best.zchunk * 4;
     FD_TRY(raise_smem_limit(e.fn, plan->smem));
     if (e.fn_wl) FD_TRY(raise_smem_limit(e.fn_wl, plan->smem));

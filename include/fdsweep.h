@@ -126,11 +126,13 @@ fd_status acoustic_forward(const fd_grid *grid, int so, double dt, int nt, int n
  *                  with it.
  *                  FD_STORAGE_AUTO: the faster of the two on GB300 for the
  *                  space order, measured at 512^3: binary16 for so <= 8 (its
- *                  kernel 1.69x / 1.15x the FP32 one at so 4 / 8), FP32 for
+ *                  kernel 1.69x / 1.19x the FP32 one at so 4 / 8), FP32 for
  *                  so 12 and 16 (where the binary16 kernel, bound by the
- *                  conversions, ran 0.95x / 0.80x), and FP32 with
- *                  FD_DAMP_FIELD.  The results are those of the storage
- *                  chosen.
+ *                  conversions, ran 0.91x / 0.82x), and FP32 with
+ *                  FD_DAMP_FIELD.  The choice does not depend on the grid
+ *                  (on grids of FP32's one-block kernels, up to about 80^3,
+ *                  FP32 can be the faster one).  The results are those of
+ *                  the storage chosen.
  *   opts->damp_layout
  *                  FD_DAMP_AXES: damp holds the per-axis profiles
  *                  [nx + ny + nz] of acoustic_forward (damp(i,j,k) = d_x[i] +

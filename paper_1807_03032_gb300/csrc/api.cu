@@ -1736,8 +1736,8 @@ fd_status acoustic_forward_opts(const fd_grid *grid, int so, double dt, int nt, 
         return fdsweep::set_error(FD_ERR_ARG, "acoustic_forward_opts: damp_layout %d not in {0, 1}",
                                   layout);
     // FD_STORAGE_AUTO: binary16 storage where its kernel measured faster than
-    // the FP32 one on GB300 at 512^3 (so 4: 1.69x, so 8: 1.15x), FP32 storage
-    // where it did not (so 12: 0.95x, so 16: 0.80x; the binary16 kernel is
+    // the FP32 one on GB300 at 512^3 (so 4: 1.69x, so 8: 1.19x), FP32 storage
+    // where it did not (so 12: 0.91x, so 16: 0.82x; the binary16 kernel is
     // bound by the conversions there), and FP32 with a 3-D damping field.
     if (storage == FD_STORAGE_AUTO)
         storage = (so <= 8 && layout == FD_DAMP_AXES) ? FD_STORAGE_F16 : FD_STORAGE_F32;

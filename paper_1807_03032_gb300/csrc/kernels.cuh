@@ -337,12 +337,12 @@ fd_status tti_fused_plan(int radius, int stag, const WaveLayout &L, int nshots, 
                          const float *coef, TtiPlan *plan, int config = -1);
 fd_status tti_fused_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
                            const AcousticInject &inj, const ReceiveArgs &receive);
-// inject, receive: done by the step's own kernels (not with the recompute
-// scheme; see tti_records_receivers); at most kInjectMaxSources sources.
 // Estimated time (us) of a fused step.
 fd_status tti_fused_time(int radius, int stag, const WaveLayout &L, int nshots, double *us);
 // The automatic scheme (kTtiTwoPass or kTtiFused) for a problem.
 fd_status tti_choose_scheme(int radius, int stag, const WaveLayout &L, int nshots, int *scheme);
+// inject, receive: done by the step's own kernels (not with the recompute
+// scheme; see tti_records_receivers); at most kInjectMaxSources sources.
 fd_status tti_launch(const TtiPlan &plan, const TtiArgs &a, cudaStream_t stream,
                      cudaEvent_t *ev /* 3 events or null */,
                      const AcousticInject *inject = nullptr,

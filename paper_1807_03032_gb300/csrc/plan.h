@@ -101,7 +101,8 @@ inline bool plan_one(const PlanEntry &e, bool forced, int nx, int ny, int nz, in
     if (e.bz) {
         const int nzc = (nz + e.bz - 1) / e.bz;
         const double waves = (double)cols * nzc / ((double)nsm * e.per_sm);
-        // A second wave of blocks hides nothing: only for a clear gain, and
+        // A second wave of blocks hides nothing: only for a clear gain (TTI
+        // 96^3 so 4 17.4 against 22.0 us, K1 128^3 so 8 14.9 against 9.8), and
         // never a third.
         if ((waves > 2.0 || (int64_t)nzc * nshots > kMostColumnsZ) && !forced) return false;
         if (waves > 1.0) penalty = 1.06;

@@ -748,7 +748,8 @@ constexpr int kMaxPassEntries = 4;  // of a table
     pass_entry<PASS, R, TX, TY, D, U, MB, STAG>(__VA_ARGS__)
 
 // Per radius (template arguments TX, TY, D, U, minimum CTAs per SM), fitted
-// and chosen on 13 problems from 48^3 to 512^3.  Both fields' pending z
+// and chosen on 13 problems from 48^3 to 512^3 with centred derivatives (the
+// staggered ones have as many taps but one; so 2 takes so 4's costs).  Both fields' pending z
 // outputs take 16R registers of a thread, which decides the tile: 64 x 8 with
 // two or three CTAs per SM up to so 12, one CTA of 64 x 14 (224 + 32 threads
 // with 255 registers) at so 16, a smaller one beside it for small grids.
